@@ -117,20 +117,20 @@ def _rows(case, n, seed):
     return synth.make_cache(w, "cuda")
 
 
-def prepare(case, seed):
-    ctx = fk.Context()
-    st = dict(case=case, ctx=ctx)
+def _inputs(case, seed):
+    """The full cache, the rows to append, the lengths and the queries of a case, from the seed alone."""
+    st = dict(case=case)
     st["k"], st["v"] = _rows(case, case["capacity"], 10 * seed + 1)
     op = case["op"]
     if op == "cycle":
         n_in = case["capacity"] - case["sink"]
         st["new_k"], st["new_v"] = _rows(case, n_in - case["kept"], 10 * seed + 2)
         st["lens"] = [case["sink"] + case["kept"]] * case["batch"]
-        pairs = [(n_in, case["kept"])]
+        st["pairs"] = [(n_in, case["kept"])] * case["batch"]
     elif op == "ragged":
         st["lens"] = _lens(case)
         st["kept"] = [(n - case["sink"]) // 2 for n in st["lens"]]
-        pairs = [(n - case["sink"], kept) for n, kept in zip(st["lens"], st["kept"])]
+        st["pairs"] = [(n - case["sink"], kept) for n, kept in zip(st["lens"], st["kept"])]
     else:
         n_new = case.get("n_new", 1)
         st["new_k"], st["new_v"] = _rows(case, n_new, 10 * seed + 2)
@@ -141,10 +141,17 @@ def prepare(case, seed):
         size = (case["layers"], case["batch"], heads, case["head_dim"]) if op == "decode" else \
             (case["layers"], case["batch"], heads, n_new, case["head_dim"])
         st["q"] = torch.randn(size, generator=gen, device="cuda").to(DTYPES[case["dtype"]])
+        st["pairs"] = []
+    return st
+
+
+def prepare(case, seed):
+    st = _inputs(case, seed)
+    ctx = st["ctx"] = fk.Context()
+    if "q" in st:
         st["out"] = torch.empty_like(st["q"])
-        pairs = []
     layout = fk.layout_of(st["k"])
-    for n_in, kept in pairs:  # the tables of these lengths, kept by the context
+    for n_in, kept in dict.fromkeys(st["pairs"]):  # the tables of these lengths, kept by the context
         ctx.plan(n_in, kept, layout.dtype, ctx.resolve_variant(layout, n_in, kept))
     return st
 
@@ -197,3 +204,53 @@ def tolerance(case):
     and operands, one rounding of the result), the attention 2e-3 (fp16 scores, bf16 weights and result), the
     fp32 compression 4e-7 or less -- but sums of thousands of fp32 terms in another order differ by several times that."""
     return {"rel": 1e-2} if case["dtype"] == "bf16" else {"rel": 5e-6}
+
+
+def _projection(n_in, kept):
+    """The compression of one column as a matrix: sqrt(kept / n_in) * IDCT_kept * (first kept rows of DCT-II_n_in), 64 bits."""
+    t = torch.arange(kept, device="cuda")
+
+    def rows(n):  # cos(pi (2 i + 1) t / 2 n), orthonormal, the angle reduced in whole numbers
+        i = torch.arange(n, device="cuda")
+        c = torch.cos(((2 * i[None, :] + 1) * t[:, None] % (4 * n)).double() * (math.pi / (2 * n))) * math.sqrt(2 / n)
+        c[0] *= math.sqrt(0.5)
+        return c
+    return math.sqrt(kept / n_in) * rows(kept).T @ rows(n_in)
+
+
+def _rope(x, positions, base=10000.0):
+    """Channel c with channel c + d/2, turned by position * base^(-2c/d); x ends in [position, channel]."""
+    h = x.shape[-1] // 2
+    angle = positions.double()[:, None] * base ** (-torch.arange(h, device="cuda").double() / h)
+    cos, sin = torch.cos(angle), torch.sin(angle)
+    return torch.cat([x[..., :h] * cos - x[..., h:] * sin, x[..., h:] * cos + x[..., :h] * sin], dim=-1)
+
+
+def exact(case, seed):
+    """What ``run`` returns for these inputs, by plain torch in 64 bits."""
+    st = _inputs(case, seed)
+    k, v, sink, op = st["k"].double(), st["v"].double(), case["sink"], case["op"]
+    for b, (n_in, kept) in enumerate(st["pairs"]):
+        p = _projection(n_in, kept)
+        for cache in (k, v):
+            for layer in range(case["layers"]):
+                cache[b, layer, :, sink:sink + kept] = p @ cache[b, layer, :, sink:sink + n_in]
+    if op == "ragged":
+        return k, v
+    for b, at in enumerate(st["lens"] if op == "cycle" else st["before"]):
+        for cache, new in ((k, st["new_k"]), (v, st["new_v"])):
+            cache[b, :, :, at:at + new.shape[3]] = new[b].double()
+    if op == "cycle":
+        return k, v
+    n_new, group, d = case.get("n_new", 1), case["group"], case["head_dim"]
+    q = st["q"].reshape(case["layers"], case["batch"], case["kv_heads"], group, n_new, d)
+    out = torch.empty(q.shape, dtype=torch.float64, device="cuda")
+    for b, n in enumerate(_lens(case)):
+        at = torch.arange(n, device="cuda")
+        unseen = at[None, :] > at[n - n_new:, None]  # a query sees the rows up to its own
+        for layer in range(case["layers"]):
+            for head in range(case["kv_heads"]):
+                keys, queries = _rope(k[b, layer, head, :n], at), _rope(q[layer, b, head].double(), at[n - n_new:])
+                scores = (queries @ keys.T / math.sqrt(d)).masked_fill_(unseen, -math.inf)
+                out[layer, b, head] = torch.softmax(scores, dim=-1) @ v[b, layer, head, :n]
+    return out.reshape(st["q"].shape), k, v
