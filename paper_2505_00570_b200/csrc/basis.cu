@@ -107,35 +107,64 @@ __global__ void build_folded_basis_kernel(__nv_bfloat16* __restrict__ out, int32
     }
 }
 
-// Second fold.  For even L the even-t part Pe is, up to a factor, the basis of the compression of
+// Four blocks.  For even L the even-t part Pe is, up to a factor, the basis of the compression of
 // N/2 rows to L/2 (t = 2t': cos(pi t' (2m+1) / (2 (L/2))) cos(pi t' (2n+1) / (2 (N/2)))), so it has the same
 // symmetries one level down: with N' = N/2, L' = L/2, n < N'/2, m < ceil(L'/2)
 //     Pee[m][n] = (Pe[m][n] + Pe[m][N'-1-n]) / 2,   Peo[m][n] = (Pe[m][n] - Pe[m][N'-1-n]) / 2,
 //     s_m = Pee uu + Peo uv,   s_{L'-1-m} = Pee uu - Peo uv,     uu_n = u_n + u_{N'-1-n},  uv_n = u_n - u_{N'-1-n}.
-// Planes: 0 = Pee, 1 = Peo (columns n < N'/2), 2 = Po[m][.], 3 = Po[L'-1-m][.] (columns n < N'), rows m < ceil(L'/2).
-__global__ void build_folded2_basis_kernel(__nv_bfloat16* __restrict__ out, int32_t n_in, int32_t n_keep, int32_t ld,
-                                           int32_t rows_pad)
+// The odd-t part, t = 2t'+1, has the frequencies of a DCT-IV, z_t' = sum_n v_n cos((2t'+1)(2n+1) phi), phi = pi / (4N').
+// Neighbours t' = 2k and 2k - 1 are the cosine of a sum and of a difference of (2n+1) 4k phi and (2n+1) phi, so
+//     z_2k = C_k - S_k,  z_{2k-1} = C_k + S_k,   C_k = sum_n cos((2n+1) phi) v_n cos(pi k (2n+1) / N'),  S_k with sines,
+// and under n -> N'-1-n the first factor changes cosine and sine while the second keeps (changes) its sign:
+//     C_k = sum_{n < N'/2} p_n cos(pi k (2n+1) / N'),  p_n = cos(theta_n) v_n + sin(theta_n) v_{N'-1-n},
+//     S_k = sum_{n < N'/2} q_n sin(pi k (2n+1) / N'),  q_n = sin(theta_n) v_n - cos(theta_n) v_{N'-1-n},  theta_n = (2n+1) phi.
+// (The splitting of a DCT-IV into two transforms of half its length by plane rotations: Wang, "Fast algorithms for
+// the discrete W transform and for the discrete Fourier transform", 1984.)  The inverse of length L' is the transpose
+// of the same: with theta'_m = pi (2m+1) / (4L'), d_m = cos(theta'_m) A_m + sin(theta'_m) B_m and
+// d_{L'-1-m} = sin(theta'_m) A_m - cos(theta'_m) B_m,
+//     A = PA p,  PA[m][n] = (1/N) [D(a+) + D(a-)],   B = PB q,  PB[m][n] = (1/N) [D(a-) - D(a+)],
+//     a± = (2m+1) N' ± (2n+1) L',   D(a) = sin((2K+1) pi a / (2N'L')) / sin(pi a / (2N'L')),   K = floor((L'-1) / 2),
+// because the retained t' < L' pair up.  For even L' the last one, t' = L'-1 = 2K' - 1 with K' = L'/2, has lost its
+// partner: z = C_K' + S_K' both go to B, with weight (2/N) (-1)^m.
+// Planes: 0 = Pee, 1 = Peo, 2 = PA, 3 = PB in columns n < N'/2 and, for even L', the weights of p in B behind them.
+__global__ void build_quad_basis_kernel(__nv_bfloat16* __restrict__ out, float2* __restrict__ turns, int32_t n_in, int32_t n_keep,
+                                        int32_t ld, int32_t rows_pad)
 {
     const int64_t plane = (int64_t)rows_pad * ld;
     const int64_t N = n_in, L = n_keep, Nh = N / 2, Lh = L / 2, Nq = Nh / 2, Lq = (Lh + 1) / 2;
+    const int64_t K1 = 2 * ((Lh - 1) / 2) + 1, unit = 2 * Nh * Lh;  // 2K+1; angles are integer multiples of pi / unit
     auto pe = [&](int64_t m, int64_t n) { return 0.5 * (basis_entry(m, n, N, L, 0) + basis_entry(m, N - 1 - n, N, L, 0)); };
-    auto po = [&](int64_t m, int64_t n) { return 0.5 * (basis_entry(m, n, N, L, 0) - basis_entry(m, N - 1 - n, N, L, 0)); };
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < plane; i += (int64_t)gridDim.x * blockDim.x) {
+    auto series = [&](int64_t a) {
+        if (a == 0) return (double)K1;
+        return sinpi((double)((K1 * a) % (2 * unit)) / (double)unit) / sinpi((double)a / (double)unit);
+    };
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = i0; i < plane; i += step) {
         const int64_t m = i / ld, n = i % ld;
-        double pee = 0.0, peo = 0.0, p_lo = 0.0, p_hi = 0.0;
+        double pee = 0.0, peo = 0.0, pa = 0.0, pb = 0.0;
         if (m < Lq && n < Nq) {
             const double a = pe(m, n), b = pe(m, Nh - 1 - n);
             pee = 0.5 * (a + b);
             peo = 0.5 * (a - b);
+            const int64_t u = (2 * m + 1) * Nh, w = (2 * n + 1) * Lh;
+            const double plus = series(u + w), minus = series(u - w);
+            pa = (plus + minus) / (double)N;
+            pb = (minus - plus) / (double)N;
         }
-        if (m < Lq && n < Nh) {
-            p_lo = po(m, n);
-            p_hi = po(Lh - 1 - m, n);
+        if (m < Lq && n < 2 * Nq && Lh % 2 == 0) {  // the component without a partner
+            const int64_t k = (Lh / 2 * (2 * (n % Nq) + 1)) % (2 * Nh);
+            const double x = (double)k / (double)Nh, weight = (m % 2 ? -2.0 : 2.0) / (double)N;
+            pb += weight * (n < Nq ? sinpi(x) : cospi(x));
         }
         out[i] = __double2bfloat16(pee);
         out[plane + i] = __double2bfloat16(peo);
-        out[2 * plane + i] = __double2bfloat16(p_lo);
-        out[3 * plane + i] = __double2bfloat16(p_hi);
+        out[2 * plane + i] = __double2bfloat16(pa);
+        out[3 * plane + i] = __double2bfloat16(pb);
+    }
+    for (int64_t n = i0; n < Nq; n += step) {
+        double sn, cs;
+        sincospi((double)(2 * n + 1) / (double)(4 * Nh), &sn, &cs);
+        turns[n] = make_float2((float)cs, (float)sn);
     }
 }
 
@@ -169,12 +198,12 @@ cudaError_t launch_build_dct_folded(__nv_bfloat16* out, int32_t n_in, int32_t ld
     return cudaGetLastError();
 }
 
-cudaError_t launch_build_folded2_basis(__nv_bfloat16* out, int32_t n_in, int32_t n_keep, int32_t ld, int32_t rows_pad,
-                                       cudaStream_t stream)
+cudaError_t launch_build_quad_basis(__nv_bfloat16* out, float2* turns, int32_t n_in, int32_t n_keep, int32_t ld, int32_t rows_pad,
+                                    cudaStream_t stream)
 {
     const int64_t total = (int64_t)rows_pad * ld;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 148 * 32));
-    build_folded2_basis_kernel<<<(unsigned)blocks, 256, 0, stream>>>(out, n_in, n_keep, ld, rows_pad);
+    build_quad_basis_kernel<<<(unsigned)blocks, 256, 0, stream>>>(out, turns, n_in, n_keep, ld, rows_pad);
     return cudaGetLastError();
 }
 

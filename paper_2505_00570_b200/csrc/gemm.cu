@@ -10,10 +10,12 @@
 // which is the same linear map with half the multiply-adds.  (For odd N the middle row enters u
 // once and v as zero; for odd L the middle output row has d = 0 and is written once.)
 // For even L the even part Pe is itself the basis of a compression of N/2 rows to L/2, so where N is a
-// multiple of 4 it is folded once more (uu, uv; Pee, Peo; see MODE_FOLD2 and basis.cu): three quarters
-// of these multiply-adds again.  The two-level form is what a plain compression of such lengths
-// runs (the paper's 4092 -> 2046 and 4096 -> 2048); the description below is the one-level form, which
-// serves every other length, retained bands, ragged batches and the power spectrum.
+// multiple of 4 it is folded once more (uu, uv; Pee, Peo); and the odd part Po, whose frequencies are
+// those of a DCT-IV, splits by a rotation of its mirrored rows into two blocks of the same quarter size
+// (p, q; PA, PB; see MODE_QUAD and basis.cu): four blocks of ceil(L/4) x N/4, half of these multiply-adds
+// again.  The four-block form is what a plain compression of such lengths runs (the paper's
+// 4092 -> 2046 and 4096 -> 2048); the description below is the one-level form, which serves every other
+// length, retained bands, ragged batches and the power spectrum.
 //
 // Two kernels per call:
 //   fold_kernel         reads every non-sink cache row once and writes U and V (bf16) to a scratch
@@ -64,6 +66,11 @@ constexpr int B_BYTES = 2 * B_CHUNK_BYTES;         // 16 KB: this CTA's 128 of t
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;     // 32 KB per CTA
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
 constexpr int NUM_THREADS = 320;                   // 10 warps
+// MODE_QUAD: three warpgroups (producer and MMA issuer | epilogue | epilogue) that share the registers unevenly.  The
+// shares add up to what the block is launched with: 40 + 2 * 232 = 3 * 168.
+constexpr int QUAD_THREADS = 384, QUAD_LAUNCH_REGS = 168, QUAD_CONTROL_REGS = 40, QUAD_EPILOGUE_REGS = 232;
+static_assert(QUAD_CONTROL_REGS + 2 * QUAD_EPILOGUE_REGS <= 3 * QUAD_LAUNCH_REGS, "a larger sum would wait for registers for ever");
+constexpr size_t PARK_BYTES_PER_CTA = (size_t)BM * 256 * 4;  // MODE_QUAD: the pairs (s, s') of one tile, two bf16 each
 constexpr int EPI_WARPS = 8;
 constexpr unsigned long long LANDING_NS = 1000000ull;        // 1 ms: far longer than any copy in flight needs
 
@@ -79,9 +86,11 @@ struct GemmParams {
     int32_t basis_rows_pad;     // row offset of the Po plane inside the basis tensor map
     int32_t pair0, pair_count;  // (batch, layer, kv_head) triples covered by this launch
     int32_t m_pairs, k_steps;   // tiles of 256 folded rows per (batch, layer, kv_head); slices per phase
-    // two-level fold only: ceil(L / 4) = twice-folded output rows, N / 4 = rows of uu (and of uv), slices of
-    // the two short phases
-    int32_t rows_quarter, n_quarter, k_steps_short;
+    // four-block form only: ceil(L / 4) = rows of a block, N / 4 = rows of each of its four inputs, slices of
+    // the first three phases and of the last one, where the pairs (s, s') wait, whether rows take 32-byte stores
+    int32_t rows_quarter, n_quarter, k_steps_short, k_steps_last;
+    uint4* park;
+    int32_t wide_rows;
     int32_t sink;
     int32_t mirror_sign;        // +1: y[L-1-m] = s - d;  -1: y[L-1-m] = d - s (a retained band that starts at an odd component)
     // power-spectrum mode only: per tensor [layers][kv_heads][n_in] sums, the weight of one squared value
@@ -357,12 +366,14 @@ __global__ void __launch_bounds__(256) fold_kernel(const CacheView view, const F
     }
 }
 
-// Two levels of folding at once (n_in a multiple of 4; see basis.cu): with N' = n_in / 2 and n < N' / 2 the
-// four rows n, N-1-n, N'-1-n and N'+n give u_n, u_{N'-1-n}, v_n, v_{N'-1-n}, and from the two u's
-// uu_n = u_n + u_{N'-1-n}, uv_n = u_n - u_{N'-1-n} (sums in fp32, rounded once).  Plane 0 of a matrix holds uu
-// (rows 0 .. N'/2 - 1) followed by uv (rows N'/2 .. N' - 1), plane 1 holds v: the same bytes as one level.
-__device__ __forceinline__ void fold8x2(const uint4& a, const uint4& b, const uint4& c, const uint4& d, uint4* uu, uint4* uv,
-                                        uint4* v1, uint4* v2)
+// The four-block fold (n_in a multiple of 4; see basis.cu): with N' = n_in / 2 and n < N' / 2 the four rows
+// n, N-1-n, N'-1-n and N'+n give u_n, u_{N'-1-n}, v_n, v_{N'-1-n}; from the two u's come
+// uu_n = u_n + u_{N'-1-n}, uv_n = u_n - u_{N'-1-n}, from the two v's, turned by theta_n = pi (2n+1) / (4 N'),
+// p_n = cos v_n + sin v_{N'-1-n}, q_n = sin v_n - cos v_{N'-1-n} (all in fp32, rounded once).  Plane 0 of a
+// matrix holds uu (rows 0 .. N'/2 - 1) followed by uv (rows N'/2 .. N' - 1), plane 1 holds q followed by p: the same
+// bytes as one level.
+__device__ __forceinline__ void fold8_quad(const uint4& a, const uint4& b, const uint4& c, const uint4& d, float2 cs, uint4* uu,
+                                           uint4* uv, uint4* p, uint4* q)
 {
     const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w}, cw[4] = {c.x, c.y, c.z, c.w},
                    dw[4] = {d.x, d.y, d.z, d.w};
@@ -374,30 +385,33 @@ __device__ __forceinline__ void fold8x2(const uint4& a, const uint4& b, const ui
         const float c0 = __uint_as_float(cw[i] << 16), c1 = __uint_as_float(cw[i] & 0xffff0000u);
         const float d0 = __uint_as_float(dw[i] << 16), d1 = __uint_as_float(dw[i] & 0xffff0000u);
         const float p0 = a0 + b0, p1 = a1 + b1, q0 = c0 + d0, q1 = c1 + d1;  // u_n, u_{N'-1-n}
+        const float r0 = a0 - b0, r1 = a1 - b1, s0 = c0 - d0, s1 = c1 - d1;  // v_n, v_{N'-1-n}
         o[0][i] = pack_bf16(p0 + q0, p1 + q1);
         o[1][i] = pack_bf16(p0 - q0, p1 - q1);
-        o[2][i] = pack_bf16(a0 - b0, a1 - b1);
-        o[3][i] = pack_bf16(c0 - d0, c1 - d1);
+        o[2][i] = pack_bf16(fmaf(cs.x, r0, cs.y * s0), fmaf(cs.x, r1, cs.y * s1));
+        o[3][i] = pack_bf16(fmaf(cs.y, r0, -cs.x * s0), fmaf(cs.y, r1, -cs.x * s1));
     }
     *uu = make_uint4(o[0][0], o[0][1], o[0][2], o[0][3]);
     *uv = make_uint4(o[1][0], o[1][1], o[1][2], o[1][3]);
-    *v1 = make_uint4(o[2][0], o[2][1], o[2][2], o[2][3]);
-    *v2 = make_uint4(o[3][0], o[3][1], o[3][2], o[3][3]);
+    *p = make_uint4(o[2][0], o[2][1], o[2][2], o[2][3]);
+    *q = make_uint4(o[3][0], o[3][1], o[3][2], o[3][3]);
 }
 
 // Block (x, y) as in fold_kernel; job.n_half = N' rows per plane; a thread folds two vectors per round.
-__global__ void __launch_bounds__(256) fold2_kernel(const CacheView view, const FoldJob job)
+// `turns`: (cos, sin) of theta_n, n < N' / 2.
+__global__ void __launch_bounds__(256) fold_quad_kernel(const CacheView view, const FoldJob job, const float2* __restrict__ turns)
 {
     const uint32_t pt = blockIdx.x;
     const char* x = static_cast<const char*>(tensor_base(view, pt & 1)) +
                     (matrix_offset(view, job.pair0 + (int32_t)(pt >> 1)) + (int64_t)job.sink * view.stride_token) * 2;
     const int64_t row_bytes = view.stride_token * 2;
     const int32_t n_quarter = job.n_half / 2;
-    const uint32_t total = (uint32_t)n_quarter * 16u;                // vectors of uu (= of uv)
+    const uint32_t total = (uint32_t)n_quarter * 16u;                // vectors of uu (= of uv, q, p)
     uint4* plane0 = job.dst + (int64_t)pt * 2 * ((int64_t)job.n_half * 16);
     uint4* plane1 = plane0 + (int64_t)job.n_half * 16;
     for (uint32_t c0 = blockIdx.y * 512u; c0 < total; c0 += gridDim.y * 512u) {
         uint4 a[2], b[2], c[2], d[2];
+        float2 cs[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const uint32_t i = c0 + j * 256u + threadIdx.x;
@@ -407,19 +421,19 @@ __global__ void __launch_bounds__(256) fold2_kernel(const CacheView view, const 
                 b[j] = __ldcs(reinterpret_cast<const uint4*>(x + (job.n_in - 1 - n) * row_bytes) + (i & 15u));
                 c[j] = __ldcs(reinterpret_cast<const uint4*>(x + (job.n_half - 1 - n) * row_bytes) + (i & 15u));
                 d[j] = __ldcs(reinterpret_cast<const uint4*>(x + (job.n_half + n) * row_bytes) + (i & 15u));
+                cs[j] = __ldg(turns + n);
             }
         }
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const uint32_t i = c0 + j * 256u + threadIdx.x;
             if (i < total) {
-                const int32_t n = (int32_t)(i >> 4);
-                uint4 uu, uv, v1, v2;
-                fold8x2(a[j], b[j], c[j], d[j], &uu, &uv, &v1, &v2);
+                uint4 uu, uv, p, q;
+                fold8_quad(a[j], b[j], c[j], d[j], cs[j], &uu, &uv, &p, &q);
                 __stcs(plane0 + i, uu);
                 __stcs(plane0 + total + i, uv);
-                __stcs(plane1 + i, v1);
-                __stcs(plane1 + (int64_t)(job.n_half - 1 - n) * 16 + (i & 15u), v2);
+                __stcs(plane1 + i, q);
+                __stcs(plane1 + total + i, p);
             }
         }
     }
@@ -477,13 +491,15 @@ __global__ void __launch_bounds__(256) fold_ragged_kernel(const CacheView view, 
 //   cache (map_x = K tensor, map_v = V tensor, 5-D maps over the non-sink rows), there is one
 //   accumulator and one tile per (batch, layer, kv_head).  The tile's rows are stored only after
 //   every slice of its matrices has been read, so writing in place is safe here too.
-// MODE_FOLD2: two levels of the symmetry fold (n_in a multiple of 4, n_keep even).  A tile is 256
-//   twice-folded rows m < ceil(L/4) and runs four phases: a = Pee uu and b = Peo uv (N/4 deep), then
-//   d = Po v for rows m and d' = Po v for the mirrored rows L/2-1-m (N/2 deep), alternating between the
-//   two halves of tensor memory.  The epilogue parks a, turns it with b into the pair s = a + b,
-//   s' = a - b (kept as two bf16 in the register a occupied) and stores y_m = s + d, y_{L-1-m} = s - d,
-//   y_{L/2-1-m} = s' + d', y_{L/2+m} = s' - d': three quarters of the multiply-adds of MODE_FOLD.
-constexpr int MODE_FOLD = 0, MODE_SPECTRUM = 1, MODE_DIRECT = 2, MODE_RAGGED = 3, MODE_FOLD2 = 4;
+// MODE_QUAD: the four-block form (n_in a multiple of 4, n_keep even).  A tile is 256 rows m < ceil(L/4) of all
+//   four blocks and runs four phases, each N/4 deep, alternating between the two halves of tensor memory:
+//   a = Pee uu, b = Peo uv, A = PA p, B = PB q (for even L/2 one retained component couples p into B: the last
+//   phase then runs on through p, with that component's column weights as its basis).  The epilogue
+//   parks a in registers, turns it with b into the pair s = a + b, s' = a - b (two bf16 in a 32-bit word), which waits
+//   in a work area of this CTA that stays in L2 -- the accumulators of a tile would need twice the tensor memory there is --,
+//   parks A, and turns it with B by theta'_m = pi (2m+1) / (2L) into d = cos A + sin B and d' = sin A - cos B:
+//   y_m = s + d, y_{L-1-m} = s - d, y_{L/2-1-m} = s' + d', y_{L/2+m} = s' - d'.
+constexpr int MODE_FOLD = 0, MODE_SPECTRUM = 1, MODE_DIRECT = 2, MODE_RAGGED = 3, MODE_QUAD = 4;
 
 // Ragged mode: a role walks its tiles in increasing order, so the sequence a tile belongs to is
 // found by moving a cursor forward; the table is read only when a tile crosses into a new sequence.
@@ -529,15 +545,38 @@ __device__ __forceinline__ TileCtx tile_ctx(const GemmParams& prm, int32_t tile,
     return t;
 }
 
+// Registers of the calling warpgroup from here on (every warp of it executes this).
+template <int REGS, bool MORE>
+__device__ __forceinline__ void set_registers()
+{
+    if constexpr (MORE)
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS));
+    else
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS));
+}
+
+// 16 channels of one output row: one 32-byte store where every row is 32-byte aligned, else two of 16 bytes.
+__device__ __forceinline__ void store_row16(__nv_bfloat16* dst, const uint32_t (&v)[8], bool wide)
+{
+    if (wide) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                     "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                     : "memory");
+    } else {
+        reinterpret_cast<uint4*>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<uint4*>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    }
+}
+
 template <int MODE>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+__global__ void __launch_bounds__(MODE == MODE_QUAD ? QUAD_THREADS : NUM_THREADS, 1)
 freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_x,
                    const __grid_constant__ CUtensorMap map_v, const CacheView view, const GemmParams prm)
 {
     constexpr bool SPECTRUM = MODE == MODE_SPECTRUM;
-    constexpr bool FOLD2 = MODE == MODE_FOLD2;
-    constexpr int PHASES = MODE == MODE_DIRECT ? 1 : FOLD2 ? 4 : 2;
-    constexpr int USES = FOLD2 ? 2 : 1;  // times a tile fills each half of tensor memory
+    constexpr bool QUAD = MODE == MODE_QUAD;
+    constexpr int PHASES = MODE == MODE_DIRECT ? 1 : QUAD ? 4 : 2;
+    constexpr int USES = QUAD ? 2 : 1;  // times a tile fills each half of tensor memory
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // 128-byte swizzle atoms need 1024-byte alignment
@@ -582,97 +621,104 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
 
-    if (warp == 0) {
-        // ---------------- TMA producer (both CTAs) ----------------
-        if (lane == 0) {
-            uint32_t it = 0;  // global slice counter: stage = it % STAGES, phase = it / STAGES
-            bool alive = true;
-            SeqCursor cursor;
-            for (int32_t tile = cluster; tile < total_tiles && alive; tile += n_clusters) {
-                const TileCtx tc = tile_ctx<MODE>(prm, tile, &map_p, &map_x, cursor);
-                const int32_t pair_local = tc.pair_local;
-                const int32_t m0 = (tc.m_tile * 2 + (int32_t)rank) * BM;
-                const int32_t pair = tc.pair;  // direct mode: coordinates inside the cache tensor
-                const int32_t head = pair % view.kv_heads, layer = (pair / view.kv_heads) % view.layers,
-                              seq = pair / (view.kv_heads * view.layers);
-                for (int eo = 0; eo < PHASES && alive; ++eo) {
-                    // rank 0: K channels, rank 1: V.  Two-level fold: phases 0, 1 read uu and uv (both in plane 0,
-                    // uv n_quarter rows down), phases 2, 3 read v (plane 1)
-                    const int32_t plane = (pair_local * 2 + (int32_t)rank) * 2 + (FOLD2 ? eo >> 1 : eo);
-                    const int32_t row0 = (FOLD2 && eo == 1) ? prm.n_quarter : 0;
-                    const int32_t phase_steps = (FOLD2 && eo < 2) ? prm.k_steps_short : tc.k_steps;
-                    for (int32_t ks = 0; ks < phase_steps; ++ks, ++it) {
-                        const int s = it % STAGES;
-                        if (it >= STAGES &&
-                            !mbar_wait(empty_bar(s), ((it / STAGES) - 1) & 1, abort_flag, prm.status, ERR_EMPTY_WAIT, prm.wait_limit_ns)) {
-                            alive = false;
-                            break;
-                        }
-                        const uint32_t stage = base + s * STAGE_BYTES;
-                        const uint32_t leader_full = cluster_addr(full_bar(s), 0);
-                        if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
-                        const int32_t k0 = ks * BK;
-                        tma_load_2d(stage, tc.map_p, leader_full, k0, eo * tc.basis_rows_pad + m0);
-                        if constexpr (MODE == MODE_DIRECT) {
-                            const CUtensorMap* cache = rank ? &map_v : &map_x;
-                            tma_load_5d(stage + A_BYTES, cache, leader_full, 0, k0, head, layer, seq);
-                            tma_load_5d(stage + A_BYTES + B_CHUNK_BYTES, cache, leader_full, 64, k0, head, layer, seq);
-                        } else {
-                            tma_load_3d(stage + A_BYTES, tc.map_x, leader_full, 0, row0 + k0, plane);
-                            tma_load_3d(stage + A_BYTES + B_CHUNK_BYTES, tc.map_x, leader_full, 64, row0 + k0, plane);
+    constexpr int FIRST_EPI_WARP = QUAD ? 4 : 2;
+    // One setmaxnreg per warpgroup, inside the branch that only this warpgroup takes: where branches meet, ptxas
+    // assumes the fewest registers.
+    if (warp < FIRST_EPI_WARP) {
+        if constexpr (QUAD) set_registers<QUAD_CONTROL_REGS, false>();
+        if (warp == 0) {
+            // ---------------- TMA producer (both CTAs) ----------------
+            if (lane == 0) {
+                uint32_t it = 0;  // global slice counter: stage = it % STAGES, phase = it / STAGES
+                bool alive = true;
+                SeqCursor cursor;
+                for (int32_t tile = cluster; tile < total_tiles && alive; tile += n_clusters) {
+                    const TileCtx tc = tile_ctx<MODE>(prm, tile, &map_p, &map_x, cursor);
+                    const int32_t pair_local = tc.pair_local;
+                    const int32_t m0 = (tc.m_tile * 2 + (int32_t)rank) * BM;
+                    const int32_t pair = tc.pair;  // direct mode: coordinates inside the cache tensor
+                    const int32_t head = pair % view.kv_heads, layer = (pair / view.kv_heads) % view.layers,
+                                  seq = pair / (view.kv_heads * view.layers);
+                    for (int eo = 0; eo < PHASES && alive; ++eo) {
+                        // rank 0: K channels, rank 1: V.  Four blocks: phases 0, 1 read uu and uv (both in plane 0, uv
+                        // n_quarter rows down), phases 2, 3 read p (n_quarter rows down in plane 1) and q
+                        const int32_t plane = (pair_local * 2 + (int32_t)rank) * 2 + (QUAD ? eo >> 1 : eo);
+                        const int32_t row0 = (QUAD && (eo == 1 || eo == 2)) ? prm.n_quarter : 0;
+                        const int32_t phase_steps = !QUAD ? tc.k_steps : eo < 3 ? prm.k_steps_short : prm.k_steps_last;
+                        for (int32_t ks = 0; ks < phase_steps; ++ks, ++it) {
+                            const int s = it % STAGES;
+                            if (it >= STAGES &&
+                                !mbar_wait(empty_bar(s), ((it / STAGES) - 1) & 1, abort_flag, prm.status, ERR_EMPTY_WAIT, prm.wait_limit_ns)) {
+                                alive = false;
+                                break;
+                            }
+                            const uint32_t stage = base + s * STAGE_BYTES;
+                            const uint32_t leader_full = cluster_addr(full_bar(s), 0);
+                            if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
+                            const int32_t k0 = ks * BK;
+                            tma_load_2d(stage, tc.map_p, leader_full, k0, eo * tc.basis_rows_pad + m0);
+                            if constexpr (MODE == MODE_DIRECT) {
+                                const CUtensorMap* cache = rank ? &map_v : &map_x;
+                                tma_load_5d(stage + A_BYTES, cache, leader_full, 0, k0, head, layer, seq);
+                                tma_load_5d(stage + A_BYTES + B_CHUNK_BYTES, cache, leader_full, 64, k0, head, layer, seq);
+                            } else {
+                                tma_load_3d(stage + A_BYTES, tc.map_x, leader_full, 0, row0 + k0, plane);
+                                tma_load_3d(stage + A_BYTES + B_CHUNK_BYTES, tc.map_x, leader_full, 64, row0 + k0, plane);
+                            }
                         }
                     }
                 }
+                if (*abort_flag) {  // let the copies in flight land before this CTA's shared memory goes away
+                    const unsigned long long t0 = global_timer_ns();
+                    while (global_timer_ns() - t0 < LANDING_NS) __nanosleep(1000);
+                }
             }
-            if (*abort_flag) {  // let the copies in flight land before this CTA's shared memory goes away
-                const unsigned long long t0 = global_timer_ns();
-                while (global_timer_ns() - t0 < LANDING_NS) __nanosleep(1000);
-            }
-        }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer (leader CTA only) ----------------
-        if (lane == 0 && rank == 0) {
-            uint32_t it = 0, tile_no = 0;
-            bool alive = true;
-            SeqCursor cursor;
-            for (int32_t tile = cluster; tile < total_tiles && alive; tile += n_clusters, ++tile_no) {
-                const int32_t tile_steps = tile_ctx<MODE>(prm, tile, &map_p, &map_x, cursor).k_steps;
-                for (int eo = 0; eo < PHASES && alive; ++eo) {
-                    const int acc = eo & 1;                                   // half of tensor memory
-                    const uint32_t use = tile_no * USES + (uint32_t)(eo >> 1);  // how often that half was filled before
-                    const int32_t k_steps = (FOLD2 && eo < 2) ? prm.k_steps_short : tile_steps;
-                    if (use > 0) {  // both CTAs' epilogues must have read what this half held last
-                        if (!mbar_wait(acc_empty_bar(acc), (use - 1) & 1, abort_flag, prm.status, ERR_ACC_EMPTY_WAIT, prm.wait_limit_ns)) {
-                            alive = false;
-                            break;
+        } else if (warp == 1) {
+            // ---------------- MMA issuer (leader CTA only) ----------------
+            if (lane == 0 && rank == 0) {
+                uint32_t it = 0, tile_no = 0;
+                bool alive = true;
+                SeqCursor cursor;
+                for (int32_t tile = cluster; tile < total_tiles && alive; tile += n_clusters, ++tile_no) {
+                    const int32_t tile_steps = tile_ctx<MODE>(prm, tile, &map_p, &map_x, cursor).k_steps;
+                    for (int eo = 0; eo < PHASES && alive; ++eo) {
+                        const int acc = eo & 1;                                   // half of tensor memory
+                        const uint32_t use = tile_no * USES + (uint32_t)(eo >> 1);  // how often that half was filled before
+                        const int32_t k_steps = !QUAD ? tile_steps : eo < 3 ? prm.k_steps_short : prm.k_steps_last;
+                        if (use > 0) {  // both CTAs' epilogues must have read what this half held last
+                            if (!mbar_wait(acc_empty_bar(acc), (use - 1) & 1, abort_flag, prm.status, ERR_ACC_EMPTY_WAIT, prm.wait_limit_ns)) {
+                                alive = false;
+                                break;
+                            }
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         }
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        for (int32_t ks = 0; ks < k_steps; ++ks, ++it) {
+                            const int s = it % STAGES;
+                            if (!mbar_wait(full_bar(s), (it / STAGES) & 1, abort_flag, prm.status, ERR_FULL_WAIT, prm.wait_limit_ns)) {
+                                alive = false;
+                                break;
+                            }
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            const uint32_t a0 = base + s * STAGE_BYTES, b0 = a0 + A_BYTES;
+    #pragma unroll
+                            for (int kk = 0; kk < BK / 16; ++kk) {
+                                // A: 128 rows per CTA, 8-row groups 1 KB apart; 16 k-elements = 32 bytes inside the swizzled row
+                                const uint64_t ad = smem_desc(a0 + kk * 32, 16, 1024);
+                                // B: per CTA 2 chunks of 64 channels 8 KB apart (leading offset), 8-row groups 1 KB apart
+                                const uint64_t bd = smem_desc(b0 + kk * 2048, B_CHUNK_BYTES, 1024);
+                                umma_bf16(tmem_base + acc * 256, ad, bd, (ks | kk) != 0);
+                            }
+                            umma_commit_both(empty_bar(s));  // frees the stage in both CTAs when these MMAs have read it
+                        }
+                        if (alive) umma_commit_both(acc_full_bar(acc));
                     }
-                    for (int32_t ks = 0; ks < k_steps; ++ks, ++it) {
-                        const int s = it % STAGES;
-                        if (!mbar_wait(full_bar(s), (it / STAGES) & 1, abort_flag, prm.status, ERR_FULL_WAIT, prm.wait_limit_ns)) {
-                            alive = false;
-                            break;
-                        }
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t a0 = base + s * STAGE_BYTES, b0 = a0 + A_BYTES;
-#pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk) {
-                            // A: 128 rows per CTA, 8-row groups 1 KB apart; 16 k-elements = 32 bytes inside the swizzled row
-                            const uint64_t ad = smem_desc(a0 + kk * 32, 16, 1024);
-                            // B: per CTA 2 chunks of 64 channels 8 KB apart (leading offset), 8-row groups 1 KB apart
-                            const uint64_t bd = smem_desc(b0 + kk * 2048, B_CHUNK_BYTES, 1024);
-                            umma_bf16(tmem_base + acc * 256, ad, bd, (ks | kk) != 0);
-                        }
-                        umma_commit_both(empty_bar(s));  // frees the stage in both CTAs when these MMAs have read it
-                    }
-                    if (alive) umma_commit_both(acc_full_bar(acc));
                 }
             }
         }
     } else {
+        if constexpr (QUAD) set_registers<QUAD_EPILOGUE_REGS, true>();
         // ---------------- epilogue (both CTAs, each on its own 128 rows) ----------------
-        const int ew = warp - 2, quarter = warp % 4, tensor = ew / 4;  // tensor: 0 = K columns, 1 = V columns
+        const int ew = warp - FIRST_EPI_WARP, quarter = warp % 4, tensor = ew / 4;  // tensor: 0 = K columns, 1 = V columns
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + tensor * 128;
         const uint32_t leader_s_empty = cluster_addr(acc_empty_bar(0), 0), leader_d_empty = cluster_addr(acc_empty_bar(1), 0);
         uint32_t tile_no = 0;
@@ -733,13 +779,15 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                 }
                 if (!alive) break;
             }
-        } else if constexpr (FOLD2) {
+        } else if constexpr (QUAD) {
             const uint32_t leader_empty[2] = {leader_s_empty, leader_d_empty};
             auto release = [&](int acc) {
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(leader_empty[acc]);
             };
+            // this thread's 32 vectors of the work area: vector i of lane l at (i * 32 + l), so that a warp's access is dense
+            uint4* park = prm.park + ((size_t)blockIdx.x * EPI_WARPS + ew) * (32 * 32) + lane;
             for (int32_t tile = cluster; tile < total_tiles; tile += n_clusters, ++tile_no) {
                 const uint32_t use = 2 * tile_no;
                 // a = Pee uu: park this thread's row (128 columns) in registers
@@ -752,7 +800,7 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                 tmem_ld32<96>(lane_addr + 96, s);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                 release(0);
-                // b = Peo uv: s = a + b (low half of the register) and s' = a - b (high half), both bf16
+                // b = Peo uv: s = a + b (low half of a word) and s' = a - b (high half), both bf16, go to the work area
                 if (!mbar_wait(acc_full_bar(1), use & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
@@ -760,11 +808,15 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                     uint32_t b[16];
                     tmem_ld16(lane_addr + 256 + c * 16, b);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    uint32_t w[16];
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const float av = __uint_as_float(s[c * 16 + j]), bv = __uint_as_float(b[j]);
-                        s[c * 16 + j] = pack_bf16(av + bv, av - bv);
+                        w[j] = pack_bf16(av + bv, av - bv);
                     }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        __stcg(park + (c * 4 + j) * 32, make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]));
                 }
                 release(1);
 
@@ -772,46 +824,65 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                 const int32_t m = (tc.m_tile * 2 + (int32_t)rank) * BM + quarter * 32 + lane;
                 const int32_t mh = tc.rows_half - 1 - m;  // the row whose even part is s'
                 const bool row_ok = m < prm.rows_quarter;
+                const bool second_ok = row_ok && mh != m;  // the middle row of an odd L/2 is its own mirror
+                float ct, st;                              // theta'_m = pi (2m+1) / (2L)
+                sincospif((float)(2 * m + 1) / (float)(2 * tc.n_keep), &st, &ct);
                 __nv_bfloat16* mat = static_cast<__nv_bfloat16*>(tensor_base(view, tensor)) +
                                      matrix_offset(view, tc.pair) + (int64_t)prm.sink * view.stride_token;
-                bool alive = true;
+                __nv_bfloat16* rows[4] = {mat + (int64_t)m * view.stride_token, mat + (int64_t)(tc.n_keep - 1 - m) * view.stride_token,
+                                          mat + (int64_t)mh * view.stride_token, mat + (int64_t)(tc.rows_half + m) * view.stride_token};
+                // A = PA p: park it
+                if (!mbar_wait(acc_full_bar(0), (use + 1) & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                tmem_ld32<0>(lane_addr + 0, s);
+                tmem_ld32<32>(lane_addr + 32, s);
+                tmem_ld32<64>(lane_addr + 64, s);
+                tmem_ld32<96>(lane_addr + 96, s);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                release(0);
+                // B = PB q: turn (A, B), combine with (s, s') and store the four rows
+                if (!mbar_wait(acc_full_bar(1), (use + 1) & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    // d = Po v of rows m (half 0) or of the mirrored rows L/2-1-m (half 1): rows r and L-1-r
-                    if (!mbar_wait(acc_full_bar(half), (use + 1) & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) {
-                        alive = false;
-                        break;
+                for (int c = 0; c < 8; ++c) {
+                    uint32_t b[16];
+                    tmem_ld16(lane_addr + 256 + c * 16, b);
+                    uint32_t w[16];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        // volatile: hoisting the loads of every chunk to the front would cost more registers than there are
+                        asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                     : "=r"(w[4 * j]), "=r"(w[4 * j + 1]), "=r"(w[4 * j + 2]), "=r"(w[4 * j + 3])
+                                     : "l"(park + (c * 4 + j) * 32)
+                                     : "memory");
                     }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const int32_t r = half ? mh : m;
-                    const bool store = row_ok && !(half && mh == m);  // the middle row of an odd L/2 comes out of half 0
-                    uint4* out_p = reinterpret_cast<uint4*>(mat + (int64_t)r * view.stride_token);
-                    uint4* out_m = reinterpret_cast<uint4*>(mat + (int64_t)(tc.n_keep - 1 - r) * view.stride_token);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (c == 7) release(1);
+                    uint32_t y[4][8];
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        uint32_t d[16];
-                        tmem_ld16(lane_addr + half * 256 + c * 16, d);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                        if (store) {
-                            uint32_t p[8], q[8];
+                    for (int j = 0; j < 8; ++j) {
+                        float lo[4], hi[4];
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const uint32_t w0 = s[c * 16 + 2 * j], w1 = s[c * 16 + 2 * j + 1];
-                                const float s0 = __uint_as_float(half ? w0 & 0xffff0000u : w0 << 16);
-                                const float s1 = __uint_as_float(half ? w1 & 0xffff0000u : w1 << 16);
-                                const float d0 = __uint_as_float(d[2 * j]), d1 = __uint_as_float(d[2 * j + 1]);
-                                p[j] = pack_bf16(s0 + d0, s1 + d1);
-                                q[j] = pack_bf16(s0 - d0, s1 - d1);
-                            }
-                            out_p[2 * c] = make_uint4(p[0], p[1], p[2], p[3]);
-                            out_p[2 * c + 1] = make_uint4(p[4], p[5], p[6], p[7]);
-                            out_m[2 * c] = make_uint4(q[0], q[1], q[2], q[3]);
-                            out_m[2 * c + 1] = make_uint4(q[4], q[5], q[6], q[7]);
+                        for (int e = 0; e < 2; ++e) {
+                            const uint32_t word = w[2 * j + e];
+                            const float s0 = __uint_as_float(word << 16), s1 = __uint_as_float(word & 0xffff0000u);
+                            const float A = __uint_as_float(s[c * 16 + 2 * j + e]), B = __uint_as_float(b[2 * j + e]);
+                            const float d0 = fmaf(ct, A, st * B), d1 = fmaf(st, A, -ct * B);
+                            float(&o)[4] = e ? hi : lo;
+                            o[0] = s0 + d0; o[1] = s0 - d0; o[2] = s1 + d1; o[3] = s1 - d1;
                         }
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) y[r][j] = pack_bf16(lo[r], hi[r]);
                     }
-                    release(half);
+                    if (row_ok) {
+                        store_row16(rows[0] + c * 16, y[0], prm.wide_rows);
+                        store_row16(rows[1] + c * 16, y[1], prm.wide_rows);
+                    }
+                    if (second_ok) {
+                        store_row16(rows[2] + c * 16, y[2], prm.wide_rows);
+                        store_row16(rows[3] + c * 16, y[3], prm.wide_rows);
+                    }
                 }
-                if (!alive) break;
             }
         } else
         for (int32_t tile = cluster; tile < total_tiles; tile += n_clusters, ++tile_no) {
@@ -926,14 +997,14 @@ bool encode_basis_map(CUtensorMap* map, const Basis& basis)
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The four planes of the twice-folded basis stacked: 4 * fold2_rows_pad rows x fold_ld columns.
-bool encode_basis2_map(CUtensorMap* map, const Basis& basis)
+// The four blocks of the basis stacked: 4 * quad_rows_pad rows x fold_ld columns.
+bool encode_quad_map(CUtensorMap* map, const Basis& basis)
 {
-    const cuuint64_t dims[2] = {(cuuint64_t)basis.fold_ld, (cuuint64_t)4 * basis.fold2_rows_pad};
+    const cuuint64_t dims[2] = {(cuuint64_t)basis.fold_ld, (cuuint64_t)4 * basis.quad_rows_pad};
     const cuuint64_t strides[1] = {(cuuint64_t)basis.fold_ld * 2};
     const cuuint32_t box[2] = {BK, BM};
     const cuuint32_t elem[2] = {1, 1};
-    return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, basis.fold2, dims, strides, box, elem,
+    return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, basis.quad, dims, strides, box, elem,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -949,6 +1020,10 @@ bool encode_scratch_map(CUtensorMap* map, void* scratch, int32_t n_half, int32_t
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+
+// 64-row slices of one phase of the four-block form; the last phase runs on through p where L/2 is even.
+int32_t quad_steps(int32_t n_in) { return (n_in / 4 + BK - 1) / BK; }
+int32_t quad_last_steps(int32_t n_in, int32_t n_keep) { return n_keep / 2 % 2 ? quad_steps(n_in) : (n_in / 2 + BK - 1) / BK; }
 
 constexpr size_t kRaggedScratchLimit = size_t(64) << 30;  // a ragged batch is folded whole: beyond this it goes sequence by sequence
 constexpr size_t kFoldBufferBytes = size_t(2304) << 20;  // scratch for the folded inputs: a 7B-shaped cache of 4096 tokens fits in one pass
@@ -980,7 +1055,7 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(freqkv_gemm_kernel<MODE_RAGGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(freqkv_gemm_kernel<MODE_FOLD2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+            e = cudaFuncSetAttribute(freqkv_gemm_kernel<MODE_QUAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
         if (e != cudaSuccess) {
             state->last_error = "cudaFuncSetAttribute(max dynamic shared memory)";
             return e;
@@ -997,6 +1072,13 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
+        // the register shares of MODE_QUAD are of what its block is launched with
+        cudaFuncAttributes fa;
+        const cudaError_t ae = cudaFuncGetAttributes(&fa, freqkv_gemm_kernel<MODE_QUAD>);
+        if (ae != cudaSuccess || fa.numRegs < QUAD_LAUNCH_REGS) {
+            state->last_error = "the four-block kernel was not built with the registers it shares out";
+            return ae != cudaSuccess ? ae : cudaErrorLaunchOutOfResources;
+        }
         int n = 0;
         const cudaError_t q = cudaOccupancyMaxActiveClusters(&n, freqkv_gemm_kernel<MODE_FOLD>, &cfg);
         if (q != cudaSuccess || n < 1) {
@@ -1005,6 +1087,14 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
         }
         state->max_clusters = std::min(n, sm_count / 2);
         state->attr_set = true;
+    }
+    if (basis.quad && !state->park) {  // once: it depends on the device alone
+        const cudaError_t e = cudaMalloc(&state->park, (size_t)2 * state->max_clusters * PARK_BYTES_PER_CTA);
+        if (e != cudaSuccess) {
+            state->park = nullptr;
+            state->last_error = "cudaMalloc(work area of the four-block epilogue)";
+            return e;
+        }
     }
     const int32_t n_half = (basis.n_in + 1) / 2;
     const size_t per_pair = (size_t)4 * n_half * 128 * 2;  // K and V, U and V planes
@@ -1035,16 +1125,16 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
     const cudaError_t prepared = gemm_prepare(state, view.mats_per_tensor, basis, sm_count);
     if (prepared != cudaSuccess) return prepared;
     const int32_t n_half = (basis.n_in + 1) / 2, rows_half = (basis.n_keep + 1) / 2;
-    // two levels of folding where the basis has them (lengths that halve twice; not for the spectrum's basis)
+    // the four-block form where the basis has it (gemm_quad; not the spectrum's basis)
     const int32_t rows_quarter = (rows_half + 1) / 2;
-    const bool fold2 = basis.fold2 != nullptr && !spectrum && gemm_fold_levels(basis.n_in, basis.n_keep, basis.first) == 2;
-    const int32_t m_pairs = ((fold2 ? rows_quarter : rows_half) + 2 * BM - 1) / (2 * BM);  // tiles of 256 folded rows
+    const bool quad = basis.quad != nullptr && !spectrum;
+    const int32_t m_pairs = ((quad ? rows_quarter : rows_half) + 2 * BM - 1) / (2 * BM);  // tiles of 256 folded rows
     const int32_t pairs = view.mats_per_tensor;
     const size_t per_pair = (size_t)4 * n_half * 128 * 2;
     // One pass when the folded inputs fit the scratch buffer, else several passes of `chunk` pairs.
     const int64_t chunk = std::min<int64_t>(std::max<int64_t>(1, (int64_t)(kFoldBufferBytes / per_pair)), pairs);
     CUtensorMap map_p;
-    if (!(fold2 ? encode_basis2_map(&map_p, basis) : encode_basis_map(&map_p, basis))) {
+    if (!(quad ? encode_quad_map(&map_p, basis) : encode_basis_map(&map_p, basis))) {
         state->last_error = "tensor map encoding rejected the basis";
         return cudaErrorInvalidValue;
     }
@@ -1056,9 +1146,9 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
         job.n_half = n_half;
         job.sink = sink;
         job.dst = static_cast<uint4*>(state->scratch);
-        if (fold2) {
+        if (quad) {
             const unsigned fold_y = (unsigned)std::min<int64_t>(((int64_t)(n_half / 2) * 16 + 511) / 512, 64);
-            fold2_kernel<<<dim3((unsigned)job.pair_count * 2, fold_y), 256, 0, stream>>>(view, job);
+            fold_quad_kernel<<<dim3((unsigned)job.pair_count * 2, fold_y), 256, 0, stream>>>(view, job, basis.turns);
         } else {
             const unsigned fold_y = (unsigned)std::min<int64_t>(((int64_t)n_half * 16 + 1023) / 1024, 64);
             fold_kernel<<<dim3((unsigned)job.pair_count * 2, fold_y), 256, 0, stream>>>(view, job);
@@ -1076,10 +1166,14 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
         GemmParams prm;
         prm.n_keep = basis.n_keep;
         prm.rows_half = rows_half;
-        prm.basis_rows_pad = fold2 ? basis.fold2_rows_pad : basis.fold_rows_pad;
+        prm.basis_rows_pad = quad ? basis.quad_rows_pad : basis.fold_rows_pad;
         prm.rows_quarter = rows_quarter;
         prm.n_quarter = n_half / 2;
-        prm.k_steps_short = (n_half / 2 + BK - 1) / BK;
+        prm.k_steps_short = quad_steps(basis.n_in);
+        prm.k_steps_last = quad_last_steps(basis.n_in, basis.n_keep);
+        prm.park = static_cast<uint4*>(state->park);
+        prm.wide_rows = (((uintptr_t)view.base[0] | (uintptr_t)view.base[1]) & 31) == 0 &&
+                        ((view.stride_token | view.stride_head | view.stride_layer | view.stride_batch) & 15) == 0;
         prm.pair0 = job.pair0;
         prm.pair_count = job.pair_count;
         prm.m_pairs = m_pairs;
@@ -1099,7 +1193,7 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
         const int clusters = std::min<int32_t>(tiles, state->max_clusters);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(2 * clusters));
-        cfg.blockDim = dim3(NUM_THREADS);
+        cfg.blockDim = dim3(quad ? QUAD_THREADS : NUM_THREADS);
         cfg.dynamicSmemBytes = SMEM_BYTES;
         cfg.stream = stream;
         cudaLaunchAttribute attr[1];
@@ -1111,7 +1205,7 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
         cfg.numAttrs = 1;
         if (hooks.before) hooks.before(hooks.user, stream);
         e = spectrum ? cudaLaunchKernelEx(&cfg, freqkv_gemm_kernel<MODE_SPECTRUM>, map_p, map_x, map_x, view, prm)
-            : fold2  ? cudaLaunchKernelEx(&cfg, freqkv_gemm_kernel<MODE_FOLD2>, map_p, map_x, map_x, view, prm)
+            : quad   ? cudaLaunchKernelEx(&cfg, freqkv_gemm_kernel<MODE_QUAD>, map_p, map_x, map_x, view, prm)
                      : cudaLaunchKernelEx(&cfg, freqkv_gemm_kernel<MODE_FOLD>, map_p, map_x, map_x, view, prm);
         if (hooks.after) hooks.after(hooks.user, stream);
         if (e != cudaSuccess) {
@@ -1284,10 +1378,9 @@ static bool encode_cache_map(CUtensorMap* map, const CacheView& view, int tensor
 
 bool gemm_is_direct(int32_t n_keep) { return n_keep <= 2 * BM; }
 
-// Levels of the symmetry fold a plain compression of these lengths runs: 0 = none (the direct mode), 2 where
-// the lengths halve twice (n_in a multiple of 4, n_keep even, the lowest components kept) and the second level
-// means fewer 64-row slices per matrix pair (tiles are 256 rows high: with few kept rows it can leave its
-// last tile nearly empty and save nothing), else 1.
+// Levels of the mirror symmetry alone: 0 = none (the direct mode), 2 where the lengths halve twice (n_in a
+// multiple of 4, n_keep even, the lowest components kept) and a second level would mean fewer 64-row slices per
+// matrix pair (tiles are 256 rows high: with few kept rows it can leave its last tile nearly empty), else 1.
 int32_t gemm_fold_levels(int32_t n_in, int32_t n_keep, int32_t first)
 {
     if (gemm_is_direct(n_keep)) return 0;
@@ -1297,6 +1390,20 @@ int32_t gemm_fold_levels(int32_t n_in, int32_t n_keep, int32_t first)
     const int64_t slices2 =
         (int64_t)((rows_quarter + 2 * BM - 1) / (2 * BM)) * 2 * ((n_half / 2 + BK - 1) / BK + (n_half + BK - 1) / BK);
     return slices2 < slices1 ? 2 : 1;
+}
+
+// The four-block form: where the lengths allow it (as for two levels) and it means fewer 64-row slices per matrix pair
+// than one level -- 4092 -> 2046: 128 of them instead of 256, 3000 -> 1500: 96 instead of 144.  Compression and append of a
+// 7B-shaped cache (2048 matrices, 4092 -> 2046) 2.52 ms with two levels of the mirror symmetry alone, 2.21 ms with the
+// four blocks; 8B-shaped (4096 matrices, 8188 -> 4094) 15.4 and 12.5 ms; error against 64 bits 1.7e-3 both.
+bool gemm_quad(int32_t n_in, int32_t n_keep, int32_t first)
+{
+    if (gemm_is_direct(n_keep) || first != 0 || n_in % 4 != 0 || n_keep % 2 != 0) return false;
+    const int32_t rows_half = n_keep / 2, rows_quarter = (rows_half + 1) / 2;
+    const int64_t slices1 = (int64_t)((rows_half + 2 * BM - 1) / (2 * BM)) * 2 * ((n_in / 2 + BK - 1) / BK);
+    const int64_t slices4 =
+        (int64_t)((rows_quarter + 2 * BM - 1) / (2 * BM)) * (3 * quad_steps(n_in) + quad_last_steps(n_in, n_keep));
+    return slices4 < slices1;
 }
 
 cudaError_t launch_gemm_direct(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink,
@@ -1376,6 +1483,8 @@ void gemm_release(GemmState* state)
     if (state->scratch) cudaFree(state->scratch);
     state->scratch = nullptr;
     state->scratch_bytes = 0;
+    if (state->park) cudaFree(state->park);
+    state->park = nullptr;
 }
 
 }  // namespace freqkv

@@ -13,6 +13,7 @@ struct GemmState {
     int max_clusters = 0;     // CTA pairs that can be resident at once
     void* scratch = nullptr;  // folded inputs U, V: [pairs][K|V][U|V][ceil(n_in/2)][128] bf16 per pass
     size_t scratch_bytes = 0;
+    void* park = nullptr;     // four-block form: (s, s') of the tile each CTA works on (19 MB on 74 CTA pairs)
     void* ragged_meta = nullptr;  // tensor maps, shapes and fold jobs of a ragged batch (device)
     size_t ragged_meta_bytes = 0;
     unsigned long long wait_limit_ns = 2000000000ull;  // bound of every mbarrier wait inside the kernel (2 s)
@@ -40,8 +41,10 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
 cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, int sm_count);
 // At most 256 kept rows: one tile per (batch, layer, kv_head), no fold pass, the dense basis (Basis::dense).
 bool gemm_is_direct(int32_t n_keep);
-// 0, 1 or 2 levels of the symmetry fold for a plain compression of these lengths (see gemm.cu).
+// 0, 1 or 2 levels of the mirror symmetry for a plain compression of these lengths (see gemm.cu).
 int32_t gemm_fold_levels(int32_t n_in, int32_t n_keep, int32_t first);
+// Does a plain compression of these lengths run as four quarter-size blocks?
+bool gemm_quad(int32_t n_in, int32_t n_keep, int32_t first);
 cudaError_t launch_gemm_direct(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink,
                                int32_t* status_dev, int sm_count, const LaunchHooks& hooks, cudaStream_t stream);
 // One sequence of a ragged batch: its index in the cache and the (folded) basis of its lengths.

@@ -251,6 +251,15 @@ def test_gemm_two_fold_levels(ctx, n_in, kept, sink):
     parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM, row_pad=8)
 
 
+@pytest.mark.parametrize("n_in,kept,sink", [(1028, 514, 4), (1032, 516, 0), (2048, 1028, 4), (3000, 1500, 4), (2064, 1026, 1)])
+def test_gemm_four_blocks(ctx, n_in, kept, sink):
+    """The four-block form at its edges: the fewest kept rows it takes, a row more than one tile of 256, even and odd
+    kept / 2 (an even one leaves a component without a partner), inputs that are no whole number of 64-row slices."""
+    w = small(cap=n_in + sink + 3, dtype=torch.bfloat16, sink=sink, outliers=2, B=1, Ly=2, H=2)
+    parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM)
+    parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM, row_pad=8)
+
+
 def test_gemm_batch_layers_heads_and_padding(ctx):
     w = small(cap=333, dtype=torch.bfloat16, sink=4, outliers=2, B=2, Ly=3, H=2)
     parity.check_compress(ctx, w, 330, 163, 4, fk.GEMM)
