@@ -245,15 +245,24 @@ void free_bases(freqkv_ctx* ctx)
         if (kv.second.f32) cudaFree(kv.second.f32);
         if (kv.second.fold) cudaFree(kv.second.fold);
         if (kv.second.dense) cudaFree(kv.second.dense);
+        if (kv.second.f32_fold) cudaFree(kv.second.f32_fold);
     }
     ctx->bases.clear();
     ctx->basis_bytes = 0;
 }
 
+// The folded fp32 product serves fp32 caches that the plain one would; asking for the CUDA-core variant by name
+// keeps the plain one.  One level already halves its multiply-adds; at 100 rows both take 14 us, so below 64, where a
+// call is launch-bound, nothing changes.
+bool fold_f32_applies(const freqkv_ctx* ctx, int32_t dtype, int32_t n_in, int32_t first)
+{
+    return dtype == FREQKV_F32 && first == 0 && n_in >= 64 && ctx->forced != FREQKV_SIMT;
+}
+
 // Projection basis for (n_in, n_keep) holding at least the requested forms: the full fp32 matrix
-// (CUDA-core path) and/or the folded bf16 pair Pe, Po (tensor-core path).
+// (CUDA-core path), the folded bf16 pair Pe, Po (tensor-core path), the folded fp32 planes.
 freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t first, bool need_f32, bool need_fold,
-                        cudaStream_t stream, Basis* out)
+                        cudaStream_t stream, Basis* out, bool need_f32_fold = false)
 {
     const auto key = std::make_tuple(n_in, n_keep, first);
     Basis b;
@@ -262,7 +271,8 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
     // the tensor-core path wants the folded pair, or, for few kept rows, the dense bf16 matrix
     const bool direct = need_fold && first != kDctRows && gemm_is_direct(n_keep);
     const bool make_f32 = need_f32 && !b.f32, make_fold = need_fold && !direct && !b.fold, make_dense = direct && !b.dense;
-    if (make_f32 || make_fold || make_dense) {
+    const bool make_f32_fold = need_f32_fold && !b.f32_fold;
+    if (make_f32 || make_fold || make_dense || make_f32_fold) {
         auto shape = [&](Basis& x) {
             x.n_in = n_in;
             x.n_keep = n_keep;
@@ -272,6 +282,10 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
             x.fold_ld = ((n_in + 1) / 2 + 63) / 64 * 64;
             x.fold_rows_pad = ((n_keep + 1) / 2 + 255) / 256 * 256;
             x.dense_rows_pad = 256;
+            const int32_t blocks = fold_f32_blocks(n_in, n_keep);
+            // four blocks: columns up to n_in / 2 (the last block may run on through p), rows padded to the product's tiles
+            x.f32_fold_k = (n_in / 2 + 1 + 15) / 16 * 16;
+            x.f32_fold_m = ((n_keep + blocks - 1) / blocks + 31) / 32 * 32;
             x.quad_rows_pad = first >= 0 && gemm_quad(n_in, n_keep, first) ? ((n_keep / 2 + 1) / 2 + 255) / 256 * 256 : 0;
         };
         shape(b);
@@ -281,7 +295,10 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
         const size_t turns_elems = b.quad_rows_pad ? (size_t)(n_in / 4) * (sizeof(float2) / 2) : 0;  // counted in bf16
         const size_t fold_elems = fold1_elems + quad_elems + turns_elems;
         const size_t dense_elems = (size_t)256 * b.ld;
-        const size_t want = (make_f32 ? elems * 4 : 0) + (make_fold ? fold_elems * 2 : 0) + (make_dense ? dense_elems * 2 : 0);
+        const int32_t f32_blocks = fold_f32_blocks(n_in, n_keep);
+        const size_t f32_plane_elems = (size_t)f32_blocks * b.f32_fold_k * b.f32_fold_m;
+        const size_t f32_fold_elems = f32_plane_elems + (f32_blocks == 4 ? (size_t)(n_in / 4) * 2 : 0);
+        const size_t want = (make_f32_fold ? f32_fold_elems * 4 : 0) + (make_f32 ? elems * 4 : 0) + (make_fold ? fold_elems * 2 : 0) + (make_dense ? dense_elems * 2 : 0);
         if (ctx->basis_bytes + want > kBasisBudgetBytes) {
             FREQKV_CUDA(ctx, cudaDeviceSynchronize());  // bases may be in use by enqueued kernels
             free_bases(ctx);
@@ -306,8 +323,23 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
                 return cuda_fail(ctx, e, "cudaMalloc(basis)");
             }
         }
+        float* pq = nullptr;
+        if (need_f32_fold && !b.f32_fold) {
+            const cudaError_t e = cudaMalloc(&pq, f32_fold_elems * 4);
+            if (e != cudaSuccess) {
+                if (pf) cudaFree(pf);
+                if (pb) cudaFree(pb);
+                if (pd) cudaFree(pd);
+                return cuda_fail(ctx, e, "cudaMalloc(basis)");
+            }
+        }
         cudaError_t e = cudaSuccess;
-        if (pf) {
+        if (pq) {
+            e = launch_build_fold_f32(pq, reinterpret_cast<float2*>(pq + f32_plane_elems), n_in, n_keep, f32_blocks, b.f32_fold_k,
+                                      b.f32_fold_m, stream);
+            ctx->kernels_launched += 1;
+        }
+        if (e == cudaSuccess && pf) {
             e = launch_build_basis(pf, nullptr, n_in, n_keep, first, b.ld, b.rows_pad, stream);
             ctx->kernels_launched += 1;
         }
@@ -329,7 +361,14 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
             if (pf) cudaFree(pf);
             if (pb) cudaFree(pb);
             if (pd) cudaFree(pd);
+            if (pq) cudaFree(pq);
             return cuda_fail(ctx, e, "build_basis");
+        }
+        if (pq) {
+            b.f32_fold = pq;
+            b.f32_turns = f32_blocks == 4 ? reinterpret_cast<float2*>(pq + f32_plane_elems) : nullptr;
+            b.f32_fold_alloc_elems = (int64_t)f32_fold_elems;
+            ctx->basis_bytes += f32_fold_elems * 4;
         }
         if (pd) { b.dense = pd; ctx->basis_bytes += dense_elems * 2; }
         if (pf) { b.f32 = pf; ctx->basis_bytes += elems * 4; }
@@ -349,7 +388,7 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
 size_t basis_device_bytes(const Basis& b)
 {
     return (b.f32 ? (size_t)b.ld * b.rows_pad * 4 : 0) + (b.fold ? (size_t)b.fold_alloc_elems * 2 : 0) +
-           (b.dense ? (size_t)256 * b.ld * 2 : 0);
+           (b.dense ? (size_t)256 * b.ld * 2 : 0) + (b.f32_fold ? (size_t)b.f32_fold_alloc_elems * 4 : 0);
 }
 
 // Remove the plan of (n_in, n_keep, first) from the cache without freeing it: the caller owns its
@@ -368,6 +407,7 @@ void free_basis(Basis* b)
     if (b->f32) cudaFree(b->f32);
     if (b->fold) cudaFree(b->fold);
     if (b->dense) cudaFree(b->dense);
+    if (b->f32_fold) cudaFree(b->f32_fold);
     *b = Basis();
 }
 
@@ -471,11 +511,12 @@ freqkv_status compress_group(freqkv_ctx* ctx, const freqkv_layout& l, void* k, v
 
     Basis basis;
     const bool gemm = variant == FREQKV_GEMM;
+    const bool folded = !gemm && fold_f32_applies(ctx, l.dtype, n_in, first);
     freqkv_status st = FREQKV_OK;
     if (own_basis)
         basis = *own_basis;
     else
-        st = get_basis(ctx, n_in, n_keep, first, !gemm, gemm, stream, &basis);
+        st = get_basis(ctx, n_in, n_keep, first, !gemm && !folded, gemm, stream, &basis, folded);
     if (st != FREQKV_OK) return st;
 
     if (gemm) {
@@ -495,7 +536,7 @@ freqkv_status compress_group(freqkv_ctx* ctx, const freqkv_layout& l, void* k, v
         return FREQKV_OK;
     }
 
-    const size_t per_mat = (size_t)n_keep * l.head_dim * dtype_size(l.dtype);
+    const size_t per_mat = folded ? fold_f32_scratch_bytes(n_in, n_keep, l.head_dim) : (size_t)n_keep * l.head_dim * dtype_size(l.dtype);
     int64_t chunk = (int64_t)std::max<size_t>(1, kScratchChunkBytes / per_mat);
     chunk = std::min<int64_t>(chunk, n_mat);
     chunk = std::min<int64_t>(chunk, 1 << 30);
@@ -505,6 +546,14 @@ freqkv_status compress_group(freqkv_ctx* ctx, const freqkv_layout& l, void* k, v
     for (int32_t first = 0; first < n_mat; first += (int32_t)chunk) {
         const int32_t count = (int32_t)std::min<int64_t>(chunk, n_mat - first);
         cudaError_t e;
+        if (folded) {
+            TransformTimer timer(ctx, stream);
+            e = launch_fold_f32(view, first, count, basis, sink, scratch, ctx->sm_count, stream);
+            timer.end();
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "fold_f32");
+            ctx->kernels_launched += 2;
+            continue;
+        }
         {
             TransformTimer timer(ctx, stream);
             e = launch_project_simt(view, l.dtype, first, count, basis, sink, scratch, stream);
@@ -672,7 +721,8 @@ freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_
     Basis b;
     const bool gemm = variant == FREQKV_GEMM;
     const bool both = variant == FREQKV_AUTO;
-    return get_basis(ctx, n_in, n_keep, 0, !gemm || both, (gemm || both) && dtype == FREQKV_BF16, stream, &b);
+    const bool folded = !gemm && fold_f32_applies(ctx, dtype, n_in, 0);
+    return get_basis(ctx, n_in, n_keep, 0, (!gemm && !folded) || both, (gemm || both) && dtype == FREQKV_BF16, stream, &b, folded);
 }
 
 freqkv_status freqkv_check_compress(const freqkv_layout* layout, const void* k, const void* v, int32_t cache_len,

@@ -127,45 +127,80 @@ __global__ void build_folded_basis_kernel(__nv_bfloat16* __restrict__ out, int32
 // because the retained t' < L' pair up.  For even L' the last one, t' = L'-1 = 2K' - 1 with K' = L'/2, has lost its
 // partner: z = C_K' + S_K' both go to B, with weight (2/N) (-1)^m.
 // Planes: 0 = Pee, 1 = Peo, 2 = PA, 3 = PB in columns n < N'/2 and, for even L', the weights of p in B behind them.
-__global__ void build_quad_basis_kernel(__nv_bfloat16* __restrict__ out, float2* __restrict__ turns, int32_t n_in, int32_t n_keep,
-                                        int32_t ld, int32_t rows_pad)
+// The entries of the four planes at (m, n), n < N/2 (planes 0 to 2 end at N/4).
+__device__ inline void quad_entries(int64_t m, int64_t n, int64_t N, int64_t L, double (&e)[4])
 {
-    const int64_t plane = (int64_t)rows_pad * ld;
-    const int64_t N = n_in, L = n_keep, Nh = N / 2, Lh = L / 2, Nq = Nh / 2, Lq = (Lh + 1) / 2;
+    const int64_t Nh = N / 2, Lh = L / 2, Nq = Nh / 2, Lq = (Lh + 1) / 2;
     const int64_t K1 = 2 * ((Lh - 1) / 2) + 1, unit = 2 * Nh * Lh;  // 2K+1; angles are integer multiples of pi / unit
-    auto pe = [&](int64_t m, int64_t n) { return 0.5 * (basis_entry(m, n, N, L, 0) + basis_entry(m, N - 1 - n, N, L, 0)); };
+    auto pe = [&](int64_t c) { return 0.5 * (basis_entry(m, c, N, L, 0) + basis_entry(m, N - 1 - c, N, L, 0)); };
     auto series = [&](int64_t a) {
         if (a == 0) return (double)K1;
         return sinpi((double)((K1 * a) % (2 * unit)) / (double)unit) / sinpi((double)a / (double)unit);
     };
-    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = i0; i < plane; i += step) {
-        const int64_t m = i / ld, n = i % ld;
-        double pee = 0.0, peo = 0.0, pa = 0.0, pb = 0.0;
-        if (m < Lq && n < Nq) {
-            const double a = pe(m, n), b = pe(m, Nh - 1 - n);
-            pee = 0.5 * (a + b);
-            peo = 0.5 * (a - b);
-            const int64_t u = (2 * m + 1) * Nh, w = (2 * n + 1) * Lh;
-            const double plus = series(u + w), minus = series(u - w);
-            pa = (plus + minus) / (double)N;
-            pb = (minus - plus) / (double)N;
-        }
-        if (m < Lq && n < 2 * Nq && Lh % 2 == 0) {  // the component without a partner
-            const int64_t k = (Lh / 2 * (2 * (n % Nq) + 1)) % (2 * Nh);
-            const double x = (double)k / (double)Nh, weight = (m % 2 ? -2.0 : 2.0) / (double)N;
-            pb += weight * (n < Nq ? sinpi(x) : cospi(x));
-        }
-        out[i] = __double2bfloat16(pee);
-        out[plane + i] = __double2bfloat16(peo);
-        out[2 * plane + i] = __double2bfloat16(pa);
-        out[3 * plane + i] = __double2bfloat16(pb);
+    e[0] = e[1] = e[2] = e[3] = 0.0;
+    if (m < Lq && n < Nq) {
+        const double a = pe(n), b = pe(Nh - 1 - n);
+        e[0] = 0.5 * (a + b);
+        e[1] = 0.5 * (a - b);
+        const int64_t u = (2 * m + 1) * Nh, w = (2 * n + 1) * Lh;
+        const double plus = series(u + w), minus = series(u - w);
+        e[2] = (plus + minus) / (double)N;
+        e[3] = (minus - plus) / (double)N;
     }
-    for (int64_t n = i0; n < Nq; n += step) {
+    if (m < Lq && n < 2 * Nq && Lh % 2 == 0) {  // the component without a partner
+        const int64_t k = (Lh / 2 * (2 * (n % Nq) + 1)) % (2 * Nh);
+        const double x = (double)k / (double)Nh, weight = (m % 2 ? -2.0 : 2.0) / (double)N;
+        e[3] += weight * (n < Nq ? sinpi(x) : cospi(x));
+    }
+}
+
+__device__ inline void store_turns(float2* turns, int64_t n_in, int64_t i0, int64_t step)
+{
+    for (int64_t n = i0; n < n_in / 4; n += step) {
         double sn, cs;
-        sincospi((double)(2 * n + 1) / (double)(4 * Nh), &sn, &cs);
+        sincospi((double)(2 * n + 1) / (double)(2 * n_in), &sn, &cs);  // theta_n
         turns[n] = make_float2((float)cs, (float)sn);
     }
+}
+
+__global__ void build_quad_basis_kernel(__nv_bfloat16* __restrict__ out, float2* __restrict__ turns, int32_t n_in, int32_t n_keep,
+                                        int32_t ld, int32_t rows_pad)
+{
+    const int64_t plane = (int64_t)rows_pad * ld;
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = i0; i < plane; i += step) {
+        double e[4];
+        quad_entries(i / ld, i % ld, n_in, n_keep, e);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) out[b * plane + i] = __double2bfloat16(e[b]);
+    }
+    store_turns(turns, n_in, i0, step);
+}
+
+// The same blocks, or the two of one level, in fp32 and transposed: [blocks][k_pad][m_pad], zero past the ends.
+__global__ void build_fold_f32_kernel(float* __restrict__ out, float2* __restrict__ turns, int32_t n_in, int32_t n_keep, int32_t blocks,
+                                      int32_t k_pad, int32_t m_pad)
+{
+    const int64_t plane = (int64_t)k_pad * m_pad, N = n_in, L = n_keep;
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = i0; i < plane; i += step) {
+        const int64_t n = i / m_pad, m = i % m_pad;
+        if (blocks == 4) {
+            double e[4];
+            quad_entries(m, n, N, L, e);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) out[b * plane + i] = (float)e[b];
+        } else {
+            double a = 0.0, b = 0.0;
+            if (m < (L + 1) / 2 && n < (N + 1) / 2) {
+                a = basis_entry(m, n, N, L, 0);
+                b = basis_entry(m, N - 1 - n, N, L, 0);
+            }
+            out[i] = (float)(0.5 * (a + b));
+            out[plane + i] = (float)(0.5 * (a - b));
+        }
+    }
+    if (blocks == 4) store_turns(turns, n_in, i0, step);
 }
 
 // The plain orthonormal DCT-II of length N, folded the same way (power-spectrum analysis): plane 0
@@ -204,6 +239,15 @@ cudaError_t launch_build_quad_basis(__nv_bfloat16* out, float2* turns, int32_t n
     const int64_t total = (int64_t)rows_pad * ld;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 148 * 32));
     build_quad_basis_kernel<<<(unsigned)blocks, 256, 0, stream>>>(out, turns, n_in, n_keep, ld, rows_pad);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_build_fold_f32(float* out, float2* turns, int32_t n_in, int32_t n_keep, int32_t blocks, int32_t k_pad,
+                                  int32_t m_pad, cudaStream_t stream)
+{
+    const int64_t total = (int64_t)k_pad * m_pad;
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 148 * 32));
+    build_fold_f32_kernel<<<(unsigned)grid, 256, 0, stream>>>(out, turns, n_in, n_keep, blocks, k_pad, m_pad);
     return cudaGetLastError();
 }
 

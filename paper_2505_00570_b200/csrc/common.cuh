@@ -52,6 +52,12 @@ struct Basis {
     float2* turns = nullptr;
     int32_t quad_rows_pad = 0;
     int64_t fold_alloc_elems = 0;  // bf16 elements of the allocation `fold` points to
+    // Folded fp32 product (foldf32.cu): fold_f32_blocks(n_in, n_keep) planes of f32_fold_k x f32_fold_m, transposed, then
+    // (cos, sin) of theta_n, n < n_in / 4, where there are four.
+    float* f32_fold = nullptr;
+    float2* f32_turns = nullptr;
+    int32_t f32_fold_k = 0, f32_fold_m = 0;
+    int64_t f32_fold_alloc_elems = 0;
     // Tensor-core path for at most 256 kept rows: the whole P in bf16, dense_rows_pad (256) x ld.
     __nv_bfloat16* dense = nullptr;
     int32_t dense_rows_pad = 0;
@@ -68,6 +74,10 @@ cudaError_t launch_build_basis(float* p_f32, __nv_bfloat16* p_bf16, int32_t n_in
 cudaError_t launch_build_quad_basis(__nv_bfloat16* out, float2* turns, int32_t n_in, int32_t n_keep, int32_t ld, int32_t rows_pad,
                                     cudaStream_t stream);
 
+// The folded fp32 basis of foldf32.cu: `blocks` planes of k_pad x m_pad, transposed; `turns` for four blocks.
+cudaError_t launch_build_fold_f32(float* out, float2* turns, int32_t n_in, int32_t n_keep, int32_t blocks, int32_t k_pad,
+                                  int32_t m_pad, cudaStream_t stream);
+
 // Pe and Po of the folded basis (two planes of rows_pad x ld), zero padding elsewhere.
 cudaError_t launch_build_folded_basis(__nv_bfloat16* out, int32_t n_in, int32_t n_keep, int32_t first, int32_t ld,
                                       int32_t rows_pad, cudaStream_t stream);
@@ -78,6 +88,13 @@ cudaError_t launch_build_dct_folded(__nv_bfloat16* out, int32_t n_in, int32_t ld
 // scratch[i - first][m][c] = sum_n P[m][n] * X_i[sink + n][c] for matrices first .. first+count-1.
 cudaError_t launch_project_simt(const CacheView& view, int32_t dtype, int32_t first, int32_t count, const Basis& basis,
                                 int32_t sink, void* scratch, cudaStream_t stream);
+
+// The folded fp32 product (foldf32.cu), in place: matrices first .. first+count-1, scratch of
+// fold_f32_scratch_bytes per matrix.
+int32_t fold_f32_blocks(int32_t n_in, int32_t n_keep);
+size_t fold_f32_scratch_bytes(int32_t n_in, int32_t n_keep, int32_t head_dim);
+cudaError_t launch_fold_f32(const CacheView& view, int32_t first, int32_t count, const Basis& basis, int32_t sink, void* scratch,
+                            int sm_count, cudaStream_t stream);
 
 // cache rows [sink, sink + n_keep) of matrices first .. first+count-1 <- scratch.
 cudaError_t launch_copy_back(const CacheView& view, int32_t dtype, int32_t first, int32_t count, int32_t n_keep,

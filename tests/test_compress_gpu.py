@@ -260,6 +260,16 @@ def test_gemm_four_blocks(ctx, n_in, kept, sink):
     parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM, row_pad=8)
 
 
+@pytest.mark.parametrize("n_in,kept,hd,H", [(68, 34, 128, 2), (65, 33, 8, 1), (67, 1, 128, 1), (252, 64, 72, 3), (510, 254, 128, 2), (1001, 500, 256, 2),
+                                           (1004, 502, 64, 40), (777, 389, 128, 80), (1000, 1000 - 1, 128, 1), (600, 516, 128, 2)])
+def test_folded_fp32(ctx, n_in, kept, hd, H):
+    """The folded fp32 product at its edges: four blocks (even and odd kept / 2) and one level (odd lengths, the middle
+    rows), head sizes that are no whole tile of channels, few matrices (small tiles) and many (large ones), one kept row."""
+    w = small(cap=n_in + 7, hd=hd, sink=3, Ly=1, H=H)
+    parity.check_compress(ctx, w, n_in + 3, kept, 3, fk.AUTO, sample=6)
+    parity.check_compress(ctx, w, n_in + 3, kept, 3, fk.AUTO, sample=6, row_pad=8)
+
+
 def test_gemm_batch_layers_heads_and_padding(ctx):
     w = small(cap=333, dtype=torch.bfloat16, sink=4, outliers=2, B=2, Ly=3, H=2)
     parity.check_compress(ctx, w, 330, 163, 4, fk.GEMM)
