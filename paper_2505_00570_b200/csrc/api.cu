@@ -285,7 +285,7 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
             const int32_t blocks = fold_f32_blocks(n_in, n_keep);
             // four blocks: columns up to n_in / 2 (the last block may run on through p), rows padded to the product's tiles
             x.f32_fold_k = (n_in / 2 + 1 + 15) / 16 * 16;
-            x.f32_fold_m = ((n_keep + blocks - 1) / blocks + 31) / 32 * 32;
+            x.f32_fold_m = ((n_keep + blocks - 1) / blocks + 127) / 128 * 128;
             x.quad_rows_pad = first >= 0 && gemm_quad(n_in, n_keep, first) ? ((n_keep / 2 + 1) / 2 + 255) / 256 * 256 : 0;
         };
         shape(b);
@@ -551,7 +551,7 @@ freqkv_status compress_group(freqkv_ctx* ctx, const freqkv_layout& l, void* k, v
             e = launch_fold_f32(view, first, count, basis, sink, scratch, ctx->sm_count, stream);
             timer.end();
             if (e != cudaSuccess) return cuda_fail(ctx, e, "fold_f32");
-            ctx->kernels_launched += 2;
+            ctx->kernels_launched += 3;
             continue;
         }
         {

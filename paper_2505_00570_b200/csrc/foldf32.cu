@@ -7,17 +7,17 @@
 // and four times shorter than the plain product's.
 //
 //   fold_f32_kernel      reads every non-sink row once and writes the 2 or 4 folded planes to scratch; HBM- or L2-bound.
-//   product_f32_kernel   one CTA computes TM rows x TN channels of every block of one matrix, one block after the
-//                        other (accumulators of all of them stay in registers), then combines them and stores the
-//                        2 or 4 output rows of each folded row straight into the cache: it reads only scratch and
-//                        basis, so that is safe in place, and nothing is copied back.  A thread owns 4 rows x 4
-//                        channels of every block; slices of 16 folded rows come through a ring of cp.async stages (the
-//                        basis is stored transposed, so both operands arrive in the order they are read in).
-//                        Bound by FFMA issue: 16 FFMA for two 16-byte shared-memory loads.
+//   product_f32_kernel   one CTA computes TM rows x TN channels of one block of one matrix; slices of 16 folded rows come
+//                        through a ring of cp.async stages (the basis is stored transposed, so both operands arrive in
+//                        the order they are read in).  Bound by FFMA issue: a thread owns 8 x 8 products, 64 FFMA for
+//                        four 16-byte shared-memory loads, and a warp reads 4 x 8 distinct vectors of each operand.
+//   unfold_f32_kernel    combines the blocks and stores the 2 or 4 output rows of each folded row into the cache.
+// Only the first kernel reads the cache and only the last one writes it: safe in place.
 //
-// Measured against the plain product (64 matrices of 128 channels unless said): 2044 -> 1022 959 -> 253 us, odd lengths
-// 2043 -> 1021 959 -> 443 us, 4000 -> 2000 3655 -> 1131 us, one head 2044 -> 1022 (2 matrices) 107 -> 49 us; error against
-// 64 bits 5.7e-7 -> 2.8e-7.
+// Measured against the plain product (64 matrices of 128 channels unless said): 2044 -> 1022 959 -> 212 us, odd lengths
+// 2043 -> 1021 959 -> 387 us, 4000 -> 2000 3655 -> 1040 us, 2 matrices 2044 -> 1022 107 -> 23 us; error against 64 bits
+// 5.7e-7 -> 2.8e-7.  (All blocks of a tile in one CTA, combined in registers without a third kernel, left a thread 4 x 4
+// products of each and took 253 us.)
 #include <algorithm>
 
 #include "common.cuh"
@@ -67,9 +67,9 @@ __global__ void __launch_bounds__(256) fold_f32_kernel(const CacheView view, int
 struct ProductParams {
     const float* basis;      // [blocks][basis_k][m_pad]: transposed, zero past the ends
     const float* planes;     // [matrix][blocks][rows][head_dim]
-    int32_t first, n_in, n_keep, sink;
-    int32_t m_pad, basis_k;
-    int32_t rows, rows_last;  // folded rows of a plane; rows the last block's product runs over (q, or q and then p)
+    float* out;              // [matrix][blocks][rows_out][head_dim]
+    int32_t head_dim, blocks, m_pad, basis_k;
+    int32_t rows, rows_last, rows_out;  // folded rows of a plane; rows the last block's product runs over (q, or q and then p)
 };
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid)
@@ -78,159 +78,163 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 
-// grid: x = matrix, y = TM folded output rows, z = TN channels.
-template <int BLOCKS, int TM, int TN>
-__global__ void __launch_bounds__((TM / 4) * (TN / 4)) product_f32_kernel(const CacheView view, const ProductParams p)
+// grid: x = matrix * blocks + block, y = TM folded output rows, z = TN channels.  A warp covers 4 M x 8 N products: lane
+// (ly, lx) has rows ly * 4 + 16 i and channels lx * 4 + 32 j, four of each.
+template <int TM, int TN, int M, int N>
+__global__ void __launch_bounds__(TM / M * TN / N) product_f32_kernel(const ProductParams p)
 {
-    constexpr int THREADS = (TM / 4) * (TN / 4);
+    constexpr int THREADS = TM / M * TN / N, WARPS_N = TN / (8 * N);
     constexpr int A_VECS = TK * TM / 4, B_VECS = TK * TN / 4;  // 16-byte vectors of a stage
     __shared__ __align__(16) float As[STAGES][TK][TM];
     __shared__ __align__(16) float Bs[STAGES][TK][TN];
 
-    const int tid = threadIdx.x, ty = tid / (TN / 4), tx = tid % (TN / 4);
+    const int tid = threadIdx.x, warp = tid / 32, ly = tid % 32 / 8, lx = tid % 8;
+    const int ty = warp / WARPS_N * 4 * M + ly * 4, tx = warp % WARPS_N * 8 * N + lx * 4;
     const int32_t m0 = blockIdx.y * TM, c0 = blockIdx.z * TN;
-    const float* planes = p.planes + (size_t)blockIdx.x * BLOCKS * p.rows * view.head_dim;
+    const int32_t block = blockIdx.x % p.blocks, mat = blockIdx.x / p.blocks;
+    // the four blocks' inputs lie in the order uu, uv, q, p: block 2 (PA) reads p, block 3 (PB) q and, where it runs on, p
+    const int32_t plane = p.blocks == 4 && block >= 2 ? 5 - block : block;
+    const int32_t limit = block == p.blocks - 1 ? p.rows_last : p.rows, steps = (limit + TK - 1) / TK;
+    const float* a_src = p.basis + (size_t)block * p.basis_k * p.m_pad + m0;
+    const float* b_src = p.planes + ((size_t)mat * p.blocks + plane) * p.rows * p.head_dim + c0;
 
-    // The product's slices in one sequence over all blocks, so that the ring runs on from block to block.
-    const int32_t steps = (p.rows + TK - 1) / TK, steps_last = (p.rows_last + TK - 1) / TK;
-    // fetch cursor: block and slice of the next stage to fill
-    int32_t f_block = 0, f_step = 0;
+    int32_t next = 0;
     auto fetch = [&](int stage) {
-        if (f_block < BLOCKS) {
-            const int32_t k0 = f_step * TK;
-            // the four blocks' inputs lie in the order uu, uv, q, p: block 2 (PA) reads p, block 3 (PB) q and, where it runs on, p
-            const int32_t plane = BLOCKS == 4 && f_block >= 2 ? 5 - f_block : f_block;
-            const int32_t limit = f_block == BLOCKS - 1 ? p.rows_last : p.rows;
-            const float* a = p.basis + ((size_t)f_block * p.basis_k + k0) * p.m_pad + m0;
-            const float* b = planes + ((size_t)plane * p.rows + k0) * view.head_dim;
+        if (next < steps) {
+            const int32_t k0 = next * TK;
 #pragma unroll
             for (int i = 0; i < (A_VECS + THREADS - 1) / THREADS; ++i) {
                 const int idx = tid + i * THREADS, k = idx / (TM / 4), m = idx % (TM / 4) * 4;
                 if (A_VECS % THREADS == 0 || idx < A_VECS)
-                    cp_async16((uint32_t)__cvta_generic_to_shared(&As[stage][k][m]), a + (size_t)k * p.m_pad + m, true);
+                    cp_async16((uint32_t)__cvta_generic_to_shared(&As[stage][k][m]), a_src + (size_t)(k0 + k) * p.m_pad + m, true);
             }
 #pragma unroll
             for (int i = 0; i < (B_VECS + THREADS - 1) / THREADS; ++i) {
                 const int idx = tid + i * THREADS, k = idx / (TN / 4), c = idx % (TN / 4) * 4;
-                const bool ok = k0 + k < limit && c0 + c < view.head_dim;
+                const bool ok = k0 + k < limit && c0 + c < p.head_dim;
                 if (B_VECS % THREADS == 0 || idx < B_VECS)
-                    cp_async16((uint32_t)__cvta_generic_to_shared(&Bs[stage][k][c]), ok ? b + (size_t)k * view.head_dim + c0 + c : planes, ok);
-            }
-            if (++f_step == (f_block == BLOCKS - 1 ? steps_last : steps)) {
-                f_step = 0;
-                ++f_block;
+                    cp_async16((uint32_t)__cvta_generic_to_shared(&Bs[stage][k][c]), ok ? b_src + (size_t)(k0 + k) * p.head_dim + c : p.planes, ok);
             }
         }
+        ++next;
         asm volatile("cp.async.commit_group;" ::: "memory");  // empty past the end: the count of groups stays in step
     };
 
-    float acc[BLOCKS][4][4] = {};
+    float acc[M][N] = {};
 #pragma unroll
     for (int s = 0; s < STAGES - 1; ++s) fetch(s);
     int stage = 0;
-#pragma unroll
-    for (int blk = 0; blk < BLOCKS; ++blk) {
-        const int32_t n_steps = blk == BLOCKS - 1 ? steps_last : steps;
 #pragma unroll 1
-        for (int32_t st = 0; st < n_steps; ++st) {
-            asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
-            __syncthreads();  // this stage has landed for every thread, and every thread is done with the one refilled next
-            fetch(stage == 0 ? STAGES - 1 : stage - 1);
+    for (int32_t st = 0; st < steps; ++st) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+        __syncthreads();  // this stage has landed for every thread, and every thread is done with the one refilled next
+        fetch(stage == 0 ? STAGES - 1 : stage - 1);
 #pragma unroll
-            for (int k = 0; k < TK; ++k) {
-                const float4 a = *reinterpret_cast<const float4*>(&As[stage][k][ty * 4]);
-                const float4 b = *reinterpret_cast<const float4*>(&Bs[stage][k][tx * 4]);
-                const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+        for (int k = 0; k < TK; ++k) {
+            float a[M], b[N];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < M; i += 4) *reinterpret_cast<float4*>(&a[i]) = *reinterpret_cast<const float4*>(&As[stage][k][ty + i * 4]);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[blk][i][j] = fmaf(av[i], bv[j], acc[blk][i][j]);
-            }
-            stage = stage + 1 == STAGES ? 0 : stage + 1;
+            for (int j = 0; j < N; j += 4) *reinterpret_cast<float4*>(&b[j]) = *reinterpret_cast<const float4*>(&Bs[stage][k][tx + j * 8]);
+#pragma unroll
+            for (int i = 0; i < M; ++i)
+#pragma unroll
+                for (int j = 0; j < N; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        }
+        stage = stage + 1 == STAGES ? 0 : stage + 1;
+    }
+    float* out = p.out + (size_t)blockIdx.x * p.rows_out * p.head_dim;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        const int32_t m = m0 + ty + (i / 4) * 16 + i % 4;
+        if (m >= p.rows_out) continue;
+#pragma unroll
+        for (int j = 0; j < N; j += 4) {
+            const int32_t c = c0 + tx + j * 8;
+            if (c < p.head_dim)
+                *reinterpret_cast<float4*>(out + (size_t)m * p.head_dim + c) = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
         }
     }
+}
 
-    const int32_t c = c0 + tx * 4;
-    if (c >= view.head_dim) return;
-    const int32_t mat = p.first + (int32_t)blockIdx.x, tensor = mat / view.mats_per_tensor;
+// One thread per folded row and four channels; grid as fold_f32_kernel's.
+template <int BLOCKS>
+__global__ void __launch_bounds__(256) unfold_f32_kernel(const CacheView view, int32_t first, int32_t n_keep, int32_t sink,
+                                                         const float4* __restrict__ sums)
+{
+    const uint32_t vecs = (uint32_t)view.head_dim / 4;
+    const int32_t rows_half = (n_keep + 1) / 2, rows_out = BLOCKS == 2 ? rows_half : (rows_half + 1) / 2;
+    const uint32_t plane = (uint32_t)rows_out * vecs;
+    const int32_t mat = first + (int32_t)blockIdx.x, tensor = mat / view.mats_per_tensor;
     float* y = static_cast<float*>(tensor_base(view, tensor)) + matrix_offset(view, mat % view.mats_per_tensor) +
-               (int64_t)p.sink * view.stride_token + c;
-    auto store = [&](int32_t r, const float (&v)[4]) {
-        *reinterpret_cast<float4*>(y + (int64_t)r * view.stride_token) = make_float4(v[0], v[1], v[2], v[3]);
-    };
-    const int32_t rows_half = (p.n_keep + 1) / 2, rows_out = BLOCKS == 2 ? rows_half : (rows_half + 1) / 2;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int32_t m = m0 + ty * 4 + i;
-        if (m >= rows_out) continue;
-        float o0[4], o1[4];
+               (int64_t)sink * view.stride_token;
+    const float4* in = sums + (size_t)blockIdx.x * BLOCKS * plane;
+    for (uint32_t i = blockIdx.y * blockDim.x + threadIdx.x; i < plane; i += gridDim.y * blockDim.x) {
+        const int32_t m = (int32_t)(i / vecs);
+        const uint32_t vec = i - (uint32_t)m * vecs;
+        auto store = [&](int32_t r, const float4& v) { reinterpret_cast<float4*>(y + (int64_t)r * view.stride_token)[vec] = v; };
+        const float4 a = __ldg(in + i), b = __ldg(in + plane + i);
+        const float4 s = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+        const float4 t = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
         if constexpr (BLOCKS == 2) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                o0[j] = acc[0][i][j] + acc[1][i][j];
-                o1[j] = acc[0][i][j] - acc[1][i][j];
-            }
-            store(m, o0);
-            if (p.n_keep - 1 - m != m) store(p.n_keep - 1 - m, o1);
+            store(m, s);
+            if (n_keep - 1 - m != m) store(n_keep - 1 - m, t);
         } else {
-            float ct, st;  // theta'_m = pi (2m+1) / (2L)
-            sincospif((float)(2 * m + 1) / (float)(2 * p.n_keep), &st, &ct);
+            const float4 A = __ldg(in + 2 * plane + i), B = __ldg(in + 3 * plane + i);
+            float cs, sn;  // theta'_m = pi (2m+1) / (2L)
+            sincospif((float)(2 * m + 1) / (float)(2 * n_keep), &sn, &cs);
+            const float4 d = make_float4(fmaf(cs, A.x, sn * B.x), fmaf(cs, A.y, sn * B.y), fmaf(cs, A.z, sn * B.z), fmaf(cs, A.w, sn * B.w));
+            const float4 e = make_float4(fmaf(sn, A.x, -cs * B.x), fmaf(sn, A.y, -cs * B.y), fmaf(sn, A.z, -cs * B.z), fmaf(sn, A.w, -cs * B.w));
+            store(m, make_float4(s.x + d.x, s.y + d.y, s.z + d.z, s.w + d.w));
+            store(n_keep - 1 - m, make_float4(s.x - d.x, s.y - d.y, s.z - d.z, s.w - d.w));
             const int32_t mh = rows_half - 1 - m;
-            float o2[4], o3[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float s0 = acc[0][i][j] + acc[1][i][j], s1 = acc[0][i][j] - acc[1][i][j];
-                const float d0 = fmaf(ct, acc[2][i][j], st * acc[3][i][j]), d1 = fmaf(st, acc[2][i][j], -ct * acc[3][i][j]);
-                o0[j] = s0 + d0;
-                o1[j] = s0 - d0;
-                o2[j] = s1 + d1;
-                o3[j] = s1 - d1;
-            }
-            store(m, o0);
-            store(p.n_keep - 1 - m, o1);
             if (mh != m) {  // the middle row of an odd L/2 is its own mirror
-                store(mh, o2);
-                store(rows_half + m, o3);
+                store(mh, make_float4(t.x + e.x, t.y + e.y, t.z + e.z, t.w + e.w));
+                store(rows_half + m, make_float4(t.x - e.x, t.y - e.y, t.z - e.z, t.w - e.w));
             }
         }
     }
 }
 
-template <int BLOCKS, int TM, int TN>
-void launch_product(const CacheView& view, const ProductParams& p, int32_t count, int32_t rows_out, cudaStream_t stream)
+template <int TM, int TN, int M, int N>
+void launch_product(const ProductParams& p, int32_t count, cudaStream_t stream)
 {
-    const dim3 grid((unsigned)count, (unsigned)((rows_out + TM - 1) / TM), (unsigned)((view.head_dim + TN - 1) / TN));
-    product_f32_kernel<BLOCKS, TM, TN><<<grid, (TM / 4) * (TN / 4), 0, stream>>>(view, p);
+    const dim3 grid((unsigned)(count * p.blocks), (unsigned)((p.rows_out + TM - 1) / TM), (unsigned)((p.head_dim + TN - 1) / TN));
+    product_f32_kernel<TM, TN, M, N><<<grid, TM / M * TN / N, 0, stream>>>(p);
 }
 
 template <int BLOCKS>
 cudaError_t launch_blocks(const CacheView& view, int32_t first, int32_t count, const Basis& basis, int32_t sink, float* scratch,
                           int sm_count, cudaStream_t stream)
 {
+    const int32_t rows_half = (basis.n_keep + 1) / 2;
     ProductParams p;
     p.basis = basis.f32_fold;
     p.planes = scratch;
-    p.first = first;
-    p.n_in = basis.n_in;
-    p.n_keep = basis.n_keep;
-    p.sink = sink;
+    p.head_dim = view.head_dim;
+    p.blocks = BLOCKS;
     p.m_pad = basis.f32_fold_m;
     p.basis_k = basis.f32_fold_k;
     p.rows = (basis.n_in + BLOCKS - 1) / BLOCKS;
     p.rows_last = BLOCKS == 4 && basis.n_keep / 2 % 2 == 0 ? 2 * p.rows : p.rows;
-    const int64_t vecs = (int64_t)p.rows * (view.head_dim / 4);
-    const unsigned fold_y = (unsigned)std::min<int64_t>((vecs + 255) / 256, 64);
-    fold_f32_kernel<BLOCKS><<<dim3((unsigned)count, fold_y), 256, 0, stream>>>(view, first, basis.n_in, sink, basis.f32_turns,
-                                                                             reinterpret_cast<float4*>(scratch));
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const int32_t rows_half = (basis.n_keep + 1) / 2, rows_out = BLOCKS == 2 ? rows_half : (rows_half + 1) / 2;
-    // Large tiles reuse a shared-memory operand twice as often; small ones spread few matrices over more SMs.
-    const int64_t large = (int64_t)count * ((rows_out + 31) / 32) * ((view.head_dim + 63) / 64);
-    if (large >= 2 * sm_count)
-        launch_product<BLOCKS, 32, 64>(view, p, count, rows_out, stream);
+    p.rows_out = BLOCKS == 2 ? rows_half : (rows_half + 1) / 2;
+    p.out = scratch + (size_t)count * BLOCKS * p.rows * view.head_dim;
+    auto share = [&](int32_t rows) { return (unsigned)std::min<int64_t>(((int64_t)rows * (view.head_dim / 4) + 255) / 256, 64); };
+    fold_f32_kernel<BLOCKS><<<dim3((unsigned)count, share(p.rows)), 256, 0, stream>>>(view, first, basis.n_in, sink, basis.f32_turns,
+                                                                                    reinterpret_cast<float4*>(scratch));
+    // 8 x 8 products a thread take the fewest shared-memory loads, 4 x 4 spread few matrices over more SMs (2 matrices of
+    // 2044 -> 1022: 41 and 23 us).  Tiles of 128 rows read the folded inputs least often; where they would leave much of
+    // the last one empty, tiles of 32 (64 matrices of 256 rows a block 212 and 222 us, 16 of 281 rows 75 and 58 us).
+    const int64_t rows128 = (p.rows_out + 127) / 128 * 128, rows32 = (p.rows_out + 31) / 32 * 32;
+    const int64_t large = (int64_t)count * BLOCKS * ((p.rows_out + 127) / 128) * ((view.head_dim + 63) / 64);
+    if (large < 2 * sm_count)
+        launch_product<32, 32, 4, 4>(p, count, stream);
+    else if (rows128 * 10 <= rows32 * 11)
+        launch_product<128, 64, 8, 8>(p, count, stream);
     else
-        launch_product<BLOCKS, 16, 32>(view, p, count, rows_out, stream);
+        launch_product<32, 64, 8, 8>(p, count, stream);
+    unfold_f32_kernel<BLOCKS><<<dim3((unsigned)count, share(p.rows_out)), 256, 0, stream>>>(view, first, basis.n_keep, sink,
+                                                                                         reinterpret_cast<const float4*>(p.out));
     return cudaGetLastError();
 }
 
@@ -241,8 +245,9 @@ int32_t fold_f32_blocks(int32_t n_in, int32_t n_keep) { return n_in % 4 == 0 && 
 
 size_t fold_f32_scratch_bytes(int32_t n_in, int32_t n_keep, int32_t head_dim)
 {
-    const int32_t blocks = fold_f32_blocks(n_in, n_keep);
-    return (size_t)blocks * ((n_in + blocks - 1) / blocks) * head_dim * sizeof(float);
+    const int32_t blocks = fold_f32_blocks(n_in, n_keep), rows_half = (n_keep + 1) / 2;
+    const int32_t rows = (n_in + blocks - 1) / blocks, rows_out = blocks == 2 ? rows_half : (rows_half + 1) / 2;
+    return (size_t)blocks * (rows + rows_out) * head_dim * sizeof(float);  // the folded inputs, the blocks' products
 }
 
 cudaError_t launch_fold_f32(const CacheView& view, int32_t first, int32_t count, const Basis& basis, int32_t sink, void* scratch,
