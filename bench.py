@@ -387,7 +387,7 @@ def run_attend(args, ctx, fk, synth, name, dev, peaks):
     for i in range(max(args.warmup, 3)):
         ctx.attend_decode(k, v, i % layers, q, lens, rope_base=base, out=out)
     torch.cuda.synchronize()
-    ctx.get_timing()
+    _, _, launches0 = ctx.get_timing()
     ctx.set_timing(True)
     a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     a.record()
@@ -395,7 +395,7 @@ def run_attend(args, ctx, fk, synth, name, dev, peaks):
         ctx.attend_decode(k, v, i % layers, q, lens, rope_base=base, out=out)
     b.record()
     torch.cuda.synchronize()
-    n, t_ms, _ = ctx.get_timing()
+    n, t_ms, launches1 = ctx.get_timing()
     ctx.set_timing(False)
     ms = a.elapsed_time(b) / args.steps
     kernel_ms = t_ms / max(n, 1)
@@ -408,10 +408,10 @@ def run_attend(args, ctx, fk, synth, name, dev, peaks):
                        "l2": "%d layers alternate, %.2f GB read per call" % (layers, bytes_per_call / 1e9)},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                          "frac": achieved / peaks["hbm_gbs"], "peak_kind": "copy, of " + peaks["source"],
-                         "kernel": ("attend_mma_kernel" if G >= 2 else "attend_partial_kernel") + " + attend_merge_kernel",
+                         "kernel": "attend_mma_kernel" if G >= 2 else "attend_partial_kernel (+ attend_merge_kernel)",
                          "kernel_ms": kernel_ms,
                          "traffic": load_traffic(name, "attend")},
-            "cpu_baseline": None, "e2e": None, "gpu_launches": 2 * args.steps}
+            "cpu_baseline": None, "e2e": None, "gpu_launches": launches1 - launches0}
 
 
 def run_prefill_attend(args, ctx, fk, synth, name, dev, peaks):

@@ -56,6 +56,7 @@ struct freqkv_ctx {
     double rope_base = 0.0;
     float* attend_partial = nullptr;
     size_t attend_partial_bytes = 0;
+    int32_t* attend_tickets = nullptr;  // per (sequence, kv head): splits finished, zero between calls (see attend_ticket_bytes)
     void* prefill_keys = nullptr;     // rotated keys of one layer, fp16
     size_t prefill_keys_bytes = 0;
     void* prefill_queries = nullptr;  // rotated, scaled queries of one chunk, fp16
@@ -619,9 +620,15 @@ freqkv_status freqkv_create(freqkv_ctx** out, int device)
         return FREQKV_ERR_UNSUPPORTED;
     }
     ctx->sm_count = prop.multiProcessorCount;
+    // zeroed here and not on a call's stream: a call may be under capture
+    const size_t tickets = attend_ticket_bytes(ctx->sm_count);
     if (cudaMalloc(&ctx->status_dev, sizeof(int32_t)) != cudaSuccess ||
-        cudaMemset(ctx->status_dev, 0, sizeof(int32_t)) != cudaSuccess) {
+        cudaMemset(ctx->status_dev, 0, sizeof(int32_t)) != cudaSuccess ||
+        cudaMalloc(&ctx->attend_tickets, tickets) != cudaSuccess || cudaMemset(ctx->attend_tickets, 0, tickets) != cudaSuccess ||
+        cudaStreamSynchronize(nullptr) != cudaSuccess) {  // calls may come on streams that do not wait for this one
         cudaGetLastError();
+        if (ctx->status_dev) cudaFree(ctx->status_dev);
+        if (ctx->attend_tickets) cudaFree(ctx->attend_tickets);
         delete ctx;
         return FREQKV_ERR_ALLOC;
     }
@@ -645,6 +652,7 @@ freqkv_status freqkv_destroy(freqkv_ctx* ctx)
     if (ctx->work_done) cudaEventDestroy(ctx->work_done);
     if (ctx->rope_table) cudaFree(ctx->rope_table);
     if (ctx->attend_partial) cudaFree(ctx->attend_partial);
+    if (ctx->attend_tickets) cudaFree(ctx->attend_tickets);
     if (ctx->prefill_keys) cudaFree(ctx->prefill_keys);
     if (ctx->prefill_queries) cudaFree(ctx->prefill_queries);
     for (int i = 0; i < 3; ++i)
@@ -1101,13 +1109,11 @@ freqkv_status freqkv_attend_decode(freqkv_ctx* ctx, const freqkv_layout* layout,
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     WorkOrder order(ctx, stream);
     if (scale <= 0.f) scale = 1.0f / sqrtf((float)l.head_dim);
-    int32_t max_len = 0;
-    for (int32_t b = 0; b < l.batch; ++b) max_len = std::max(max_len, lens[b]);
     const float2* table = nullptr;
     const freqkv_status ts = rope_table_for(ctx, l.capacity, rope_base, stream, &table);
     if (ts != FREQKV_OK) return ts;
-    const int32_t splits = attend_splits(l.batch, l.kv_heads, max_len, q_heads_per_kv, l.dtype, ctx->sm_count);
-    const size_t need = attend_partial_bytes(splits, l.batch, l.kv_heads * q_heads_per_kv);
+    const AttendPlan plan = attend_plan(l.batch, lens, l.kv_heads, q_heads_per_kv, l.dtype, ctx->sm_count);
+    const size_t need = attend_partial_bytes(plan.splits, l.batch, l.kv_heads * q_heads_per_kv);
     if (need > ctx->attend_partial_bytes) {
         if (ctx->attend_partial) {
             FREQKV_CUDA(ctx, cudaDeviceSynchronize());
@@ -1118,13 +1124,15 @@ freqkv_status freqkv_attend_decode(freqkv_ctx* ctx, const freqkv_layout* layout,
         FREQKV_CUDA(ctx, cudaMalloc(&ctx->attend_partial, need));
         ctx->attend_partial_bytes = need;
     }
+    int32_t launched = 0;
     cudaError_t e;
     {
         TransformTimer timer(ctx, stream);
-        e = launch_attend(l, k, v, layer, q, out, q_heads_per_kv, lens, table, scale, splits, ctx->attend_partial, stream);
+        e = launch_attend(l, k, v, layer, q, out, q_heads_per_kv, lens, table, scale, plan, ctx->attend_partial,
+                          ctx->attend_tickets, &launched, stream);
     }
+    ctx->kernels_launched += launched;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "attend");
-    ctx->kernels_launched += 1 + (l.batch + ATTEND_MAX_BATCH - 1) / ATTEND_MAX_BATCH;
     return FREQKV_OK;
 }
 

@@ -5,8 +5,8 @@
 // and value are row len - 1).  RoPE pairs channel c with channel c + 64 (head_dim 128), angle
 // pos * base^(-2c/128).
 //
-// The work is one pass over the K and V rows of the layer: HBM-bound.  Kernel 1 splits the rows
-// of every (sequence, kv head) over `splits` CTAs; inside a CTA each half-warp walks its own run
+// The work is one pass over the K and V rows of the layer: HBM-bound.  The rows of every (sequence,
+// kv head) are split over CTAs of about `chunk` rows each; inside a CTA each half-warp walks its own run
 // of consecutive rows, four rows per round (all loads first): 16 lanes x 2 x 8 bytes cover the
 // two halves of a bf16 key row, 16 lanes x 16 bytes a value row.  A lane keeps cos/sin of the
 // current row's angle for its four channel pairs and steps them by one row with a fixed rotation
@@ -15,7 +15,10 @@
 // Scores of all G query heads of the kv head are reduced over the 16 lanes by shuffles and fed to
 // a running softmax (base-2 exponent, scale * log2 e folded into the query).  Half-warps, then
 // warps, merge their (max, sum, weighted values) and the CTA writes one partial per query head;
-// kernel 2 merges the partials of the splits, normalises and rounds once to the cache dtype.
+// they are then merged in the order of the splits, normalised and rounded once to the cache dtype.  Where all CTAs are
+// resident at once, the one that finishes a (sequence, kv head) last -- a ticket counter tells -- does that, so a call
+// is one launch; with several waves of CTAs that end (fence, ticket) would hold up the next CTA of every slot, and a
+// second kernel merges instead (16 sequences x 32 heads x 4096 rows: 175 us a layer with it, 183 us with tickets).
 #include <algorithm>
 #include <cmath>
 
@@ -35,13 +38,16 @@ struct AttendParams {
     const void* k;
     const void* v;           // bases of the cache tensors, already moved to the layer
     int64_t stride_batch, stride_head, stride_token;  // elements
-    int32_t kv_heads, splits, batch0;
+    int32_t kv_heads, batch0;
     const void* q;           // [batch, kv_heads * G, 128]
-    float* partial;          // [splits][batch][kv_heads * G][PART]
+    void* out;               // like q
+    float* partial;          // [split][batch][kv_heads * G][PART]
+    int32_t* tickets;        // [batch * kv_heads]: splits finished so far, 0 between launches; null: attend_merge_kernel follows
     const float2* table;     // [rows][64]: cos, sin of row * base^(-2c/128); null = no RoPE
     float qscale;            // scale * log2(e)
     int32_t total_batch;
     int32_t len[ATTEND_MAX_BATCH];
+    uint16_t tiles[ATTEND_MAX_BATCH];  // of 16 rows in one split of each sequence
 };
 
 __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&o)[4])
@@ -121,12 +127,85 @@ __device__ __forceinline__ void rotate(float& lo, float& hi, float2 cs)
     hi = b;
 }
 
-template <typename T, int G>
+__device__ __forceinline__ void store1(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void store1(float* p, float v) { *p = v; }
+
+// Called by every CTA after its threads have written their partials (n_splits > 1): the last CTA of the
+// group merges all of them.  Warps share the heads; with fewer heads than warps, the splits of a head too.
+// `sm`: (NT / 32) * 130 floats of shared memory that nothing else uses any more.
+template <typename T, int G, int NT>
+__device__ __forceinline__ void merge_splits(const AttendParams& p, int32_t b, int32_t h, int32_t n_splits, float* sm)
+{
+    constexpr int WARPS = NT / 32, PER_HEAD = WARPS >= G ? WARPS / G : 1;  // warps per head
+    __shared__ int32_t is_last;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int32_t* t = p.tickets + (int64_t)(p.batch0 + b) * p.kv_heads + h;
+        const int32_t last = atomicAdd(t, 1) == n_splits - 1;
+        if (last) *t = 0;  // for the next launch
+        is_last = last;
+    }
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    const int64_t heads_total = (int64_t)p.total_batch * p.kv_heads * G;
+    const int64_t head0 = ((int64_t)(p.batch0 + b) * p.kv_heads + h) * G;
+#pragma unroll 1
+    for (int g = warp / PER_HEAD; g < G; g += WARPS / PER_HEAD) {
+        const float* base = p.partial + (head0 + g) * PART;
+        float mx = NEG;
+        for (int s = lane; s < n_splits; s += 32) mx = fmaxf(mx, __ldcg(base + s * heads_total * PART));
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float sum = 0.f;
+#pragma unroll 8
+        for (int s = warp % PER_HEAD; s < n_splits; s += PER_HEAD) {
+            const float* pp = base + s * heads_total * PART;
+            const float2 ml = __ldcg(reinterpret_cast<const float2*>(pp));
+            const float4 o = __ldcg(reinterpret_cast<const float4*>(pp + 4) + lane);
+            const float f = ex2(ml.x - mx);
+            sum = fmaf(ml.y, f, sum);
+            acc.x = fmaf(o.x, f, acc.x);
+            acc.y = fmaf(o.y, f, acc.y);
+            acc.z = fmaf(o.z, f, acc.z);
+            acc.w = fmaf(o.w, f, acc.w);
+        }
+        if (PER_HEAD > 1) {
+            float* mine = sm + warp * 130;
+            mine[4 * lane] = acc.x; mine[4 * lane + 1] = acc.y; mine[4 * lane + 2] = acc.z; mine[4 * lane + 3] = acc.w;
+            if (lane == 0) mine[128] = sum;
+            __syncthreads();  // WARPS / PER_HEAD == G: every warp is here exactly once
+            if (warp % PER_HEAD == 0) {
+#pragma unroll
+                for (int w = 1; w < PER_HEAD; ++w) {
+                    const float* other = sm + (warp + w) * 130;
+                    acc.x += other[4 * lane]; acc.y += other[4 * lane + 1]; acc.z += other[4 * lane + 2]; acc.w += other[4 * lane + 3];
+                    sum += other[128];
+                }
+            }
+        }
+        if (warp % PER_HEAD == 0) {
+            T* out = static_cast<T*>(p.out) + (head0 + g) * 128 + 4 * lane;
+            store1(out, acc.x / sum);
+            store1(out + 1, acc.y / sum);
+            store1(out + 2, acc.z / sum);
+            store1(out + 3, acc.w / sum);
+        }
+    }
+}
+
+// TICKETS: the last CTA of a group merges its splits (AttendParams::tickets); else attend_merge_kernel follows.  (As a branch
+// of one kernel the merge cost the calls that do not use it 1 %.)
+template <typename T, int G, bool TICKETS>
 __global__ void __launch_bounds__(THREADS, (G <= 4 ? 2 : 1)) attend_partial_kernel(const AttendParams p)
 {
     constexpr int ROWS = G >= 8 ? 2 : 4;  // rows per round and half-warp (fewer when many query heads need registers)
     __shared__ float sm_ml[8][G][2];
     __shared__ float sm_o[8][G][128];
+    __shared__ float sm_merge[G < 8 ? 8 * 130 : 1];
 
     const int tid = threadIdx.x, warp = tid / 32, l16 = tid % 16, hw = tid / 16;
     const int32_t bh = blockIdx.y, b = bh / p.kv_heads, h = bh % p.kv_heads;
@@ -136,8 +215,8 @@ __global__ void __launch_bounds__(THREADS, (G <= 4 ? 2 : 1)) attend_partial_kern
     const T* V = static_cast<const T*>(p.v) + mat;
 
     // rows of this CTA, then of this half-warp (runs of consecutive rows)
-    const int32_t chunk = (len + p.splits - 1) / p.splits;
-    const int32_t r0 = min(len, (int32_t)blockIdx.x * chunk), r1 = min(len, r0 + chunk);
+    const int32_t rows = p.tiles[b] * 16, r0 = (int32_t)blockIdx.x * rows, r1 = min(len, r0 + rows);
+    if (r0 >= len) return;  // a shorter sequence has fewer splits
     const int32_t per = (r1 - r0 + 15) / 16;
     const int32_t j0 = min(r1, r0 + hw * per), j1 = min(r1, j0 + per);
     const int c0 = 4 * l16;  // this lane's channel pairs: (c0 + i, 64 + c0 + i), i < 4
@@ -283,6 +362,7 @@ __global__ void __launch_bounds__(THREADS, (G <= 4 ? 2 : 1)) attend_partial_kern
         }
     }
     __syncthreads();
+    const int32_t n_splits = (len + rows - 1) / rows;
     for (int idx = tid; idx < G * 128; idx += THREADS) {
         const int g = idx / 128, c = idx % 128;
         float mn = NEG;
@@ -295,12 +375,19 @@ __global__ void __launch_bounds__(THREADS, (G <= 4 ? 2 : 1)) attend_partial_kern
             sum = fmaf(sm_ml[w][g][1], f, sum);
             acc = fmaf(sm_o[w][g][c], f, acc);
         }
+        if (n_splits == 1) {
+            store1(static_cast<T*>(p.out) + (((int64_t)(p.batch0 + b) * p.kv_heads + h) * G + g) * 128 + c, acc / sum);
+            continue;
+        }
         float* out = p.partial + (((int64_t)blockIdx.x * p.total_batch + p.batch0 + b) * p.kv_heads * G + h * G + g) * PART;
         out[4 + c] = acc;
         if (c == 0) {
             out[0] = mn;
             out[1] = sum;
         }
+    }
+    if constexpr (TICKETS) {
+            if (n_splits > 1) merge_splits<T, G, THREADS>(p, b, h, n_splits, sm_merge);
     }
 }
 
@@ -388,7 +475,7 @@ __device__ __forceinline__ uint32_t pack2_f16(float lo, float hi)
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-template <int G>
+template <int G, bool TICKETS>
 __global__ void __launch_bounds__(MMA_THREADS, MMA_CTAS_PER_SM) attend_mma_kernel(const AttendParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -400,14 +487,38 @@ __global__ void __launch_bounds__(MMA_THREADS, MMA_CTAS_PER_SM) attend_mma_kerne
     const __nv_bfloat16* K = static_cast<const __nv_bfloat16*>(p.k) + mat;
     const __nv_bfloat16* V = static_cast<const __nv_bfloat16*>(p.v) + mat;
 
-    const int32_t chunk = (len + p.splits - 1) / p.splits;
-    const int32_t r0 = min(len, (int32_t)blockIdx.x * chunk), r1 = min(len, r0 + chunk);
+    const int32_t rows = p.tiles[b] * 16, r0 = (int32_t)blockIdx.x * rows, r1 = min(len, r0 + rows);
+    if (r0 >= len) return;  // a shorter sequence has fewer splits
     const int32_t n_tiles = (r1 - r0 + TILE_ROWS - 1) / TILE_ROWS;
 
     const uint32_t warp_smem = (uint32_t)__cvta_generic_to_shared(smem) + warp * WARP_TILE_BYTES;
     auto k_tile = [&](int stage) { return warp_smem + stage * 2 * TILE_BYTES; };
     auto v_tile = [&](int stage) { return warp_smem + stage * 2 * TILE_BYTES + TILE_BYTES; };
 
+    const int l16 = lane % 16, hw = lane / 16, c0 = 4 * l16;  // rotation roles, see below
+    // the first tiles' rows and angles travel while the queries are prepared
+    auto prefetch = [&](int32_t tile, int stage) {
+        const int32_t row0 = r0 + tile * TILE_ROWS;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int idx = lane + 32 * i, row = idx >> 4, ch = idx & 15;
+            const bool ok = row0 + row < r1;
+            const int64_t src = (int64_t)min(row0 + row, r1 - 1) * p.stride_token + ch * 8;
+            cp_async16(k_tile(stage) + tile_off(row, ch), K + src, ok);
+            cp_async16(v_tile(stage) + tile_off(row, ch), V + src, ok);
+        }
+    };
+    // One group is committed per ring slot, empty past the last tile, so that "all but the newest
+    // MMA_STAGES - 1 groups" always means "the current tile has landed".
+#pragma unroll
+    for (int j = 0; j < MMA_STAGES - 1; ++j) {
+        if (warp + j * MMA_WARPS < n_tiles) prefetch(warp + j * MMA_WARPS, j);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    float2 cs_next[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        cs_next[i] = p.table ? p.table[(int64_t)min(r0 + warp * TILE_ROWS + 8 * hw, len - 1) * 64 + c0 + i] : make_float2(1.f, 0.f);
     // queries as fp16 B fragments: head gq (zero past G), channels 16 kc + 2 tq (+1) and + 8
     uint32_t qb[8][2];
     {
@@ -436,7 +547,6 @@ __global__ void __launch_bounds__(MMA_THREADS, MMA_CTAS_PER_SM) attend_mma_kerne
     }
 
     // rotation roles: half-warp hw rotates rows 8 hw .. 8 hw + 7 of a tile, lane l16 the pairs 4 l16 .. 4 l16 + 3
-    const int l16 = lane % 16, hw = lane / 16, c0 = 4 * l16;
     float2 step[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) step[i] = p.table ? p.table[64 + c0 + i] : make_float2(1.f, 0.f);
@@ -449,28 +559,6 @@ __global__ void __launch_bounds__(MMA_THREADS, MMA_CTAS_PER_SM) attend_mma_kerne
 #pragma unroll
         for (int i = 0; i < 4; ++i) o[cb][i] = 0.f;
 
-    auto prefetch = [&](int32_t tile, int stage) {
-        const int32_t row0 = r0 + tile * TILE_ROWS;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int idx = lane + 32 * i, row = idx >> 4, ch = idx & 15;
-            const bool ok = row0 + row < r1;
-            const int64_t src = (int64_t)min(row0 + row, r1 - 1) * p.stride_token + ch * 8;
-            cp_async16(k_tile(stage) + tile_off(row, ch), K + src, ok);
-            cp_async16(v_tile(stage) + tile_off(row, ch), V + src, ok);
-        }
-    };
-    // One group is committed per ring slot, empty past the last tile, so that "all but the newest
-    // MMA_STAGES - 1 groups" always means "the current tile has landed".
-#pragma unroll
-    for (int j = 0; j < MMA_STAGES - 1; ++j) {
-        if (warp + j * MMA_WARPS < n_tiles) prefetch(warp + j * MMA_WARPS, j);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    float2 cs_next[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        cs_next[i] = p.table ? p.table[(int64_t)min(r0 + warp * TILE_ROWS + 8 * hw, len - 1) * 64 + c0 + i] : make_float2(1.f, 0.f);
     const int mi = lane >> 3, lr = lane & 7;  // ldmatrix roles: lane supplies row lr of matrix mi
     int stage = 0;
     for (int32_t tile = warp; tile < n_tiles; tile += MMA_WARPS, stage = stage + 1 == MMA_STAGES ? 0 : stage + 1) {
@@ -592,6 +680,7 @@ __global__ void __launch_bounds__(MMA_THREADS, MMA_CTAS_PER_SM) attend_mma_kerne
         }
     }
     __syncthreads();
+    const int32_t n_splits = (len + rows - 1) / rows;
     for (int idx = tid; idx < G * 128; idx += MMA_THREADS) {
         const int g = idx / 128, c = idx % 128;
         float mn = NEG;
@@ -604,6 +693,10 @@ __global__ void __launch_bounds__(MMA_THREADS, MMA_CTAS_PER_SM) attend_mma_kerne
             sum = fmaf(sm_ml[(w * 8 + g) * 2 + 1], f, sum);
             acc = fmaf(sm_o[(w * 8 + g) * 128 + c], f, acc);
         }
+        if (n_splits == 1) {
+            store1(static_cast<__nv_bfloat16*>(p.out) + (((int64_t)(p.batch0 + b) * p.kv_heads + h) * G + g) * 128 + c, acc / sum);
+            continue;
+        }
         float* out = p.partial + (((int64_t)blockIdx.x * p.total_batch + p.batch0 + b) * p.kv_heads * G + h * G + g) * PART;
         out[4 + c] = acc;
         if (c == 0) {
@@ -611,16 +704,24 @@ __global__ void __launch_bounds__(MMA_THREADS, MMA_CTAS_PER_SM) attend_mma_kerne
             out[1] = sum;
         }
     }
+    if constexpr (TICKETS)
+        if (n_splits > 1) merge_splits<__nv_bfloat16, G, MMA_THREADS>(p, b, h, n_splits, reinterpret_cast<float*>(smem));
 }
 
-// One block per (sequence, query head): merge the partials of the splits in one pass, rescaling as
-// the maximum grows (unrolled so that the loads of several splits are in flight), normalise and
-// round once to the cache dtype.
+// One block per (sequence, query head) with several splits: merge them (see attend_partial_kernel's comment).
+struct MergeParams {
+    const float* partial;
+    void* out;
+    int32_t heads;           // query heads of a sequence
+    int64_t head0, heads_total;
+    uint16_t splits[ATTEND_MAX_BATCH];
+};
 template <typename T>
-__global__ void __launch_bounds__(128) attend_merge_kernel(const float* __restrict__ partial, int32_t splits,
-                                                           int64_t heads_total, T* __restrict__ out)
+__global__ void __launch_bounds__(128) attend_merge_kernel(const MergeParams p)
 {
-    const int64_t head = blockIdx.x;
+    const int32_t splits = p.splits[blockIdx.x / p.heads];
+    if (splits == 1) return;  // written by the CTA itself
+    const int64_t heads_total = p.heads_total, head = p.head0 + blockIdx.x;
     const int c = threadIdx.x;
     // launched with programmatic stream serialization: the blocks may start while the kernel that
     // writes the partials is still draining; wait here until that grid has completed and its writes are visible
@@ -628,18 +729,14 @@ __global__ void __launch_bounds__(128) attend_merge_kernel(const float* __restri
     float mn = NEG, sum = 0.f, acc = 0.f;
 #pragma unroll 8
     for (int s = 0; s < splits; ++s) {
-        const float* pp = partial + (s * heads_total + head) * PART;
+        const float* pp = p.partial + (s * heads_total + head) * PART;
         const float m_s = pp[0], l_s = pp[1], o_s = pp[4 + c];
         const float m_new = fmaxf(mn, m_s), fa = ex2(mn - m_new), fb = ex2(m_s - m_new);
         sum = fmaf(sum, fa, l_s * fb);
         acc = fmaf(acc, fa, o_s * fb);
         mn = m_new;
     }
-    const float y = acc / sum;
-    if constexpr (sizeof(T) == 2)
-        out[head * 128 + c] = __float2bfloat16_rn(y);
-    else
-        out[head * 128 + c] = y;
+    store1(static_cast<T*>(p.out) + head * 128 + c, acc / sum);
 }
 
 // cos / sin of pos * base^(-2c/128) in fp64, rounded once.
@@ -654,11 +751,13 @@ __global__ void rope_table_kernel(float2* table, int32_t rows, double base)
     table[i] = make_float2((float)cs, (float)sn);
 }
 
-cudaError_t launch_mma(const AttendParams& prm, int32_t g, int32_t nb, cudaStream_t stream)
+cudaError_t launch_mma(const AttendParams& prm, int32_t g, int32_t nb, int32_t splits, cudaStream_t stream)
 {
     static PerDeviceOnce attrs;
     const cudaError_t attr_error = attrs.run([] {
-        const void* kernels[3] = {(const void*)attend_mma_kernel<2>, (const void*)attend_mma_kernel<4>, (const void*)attend_mma_kernel<8>};
+        const void* kernels[6] = {(const void*)attend_mma_kernel<2, true>,  (const void*)attend_mma_kernel<4, true>,
+                                  (const void*)attend_mma_kernel<8, true>,  (const void*)attend_mma_kernel<2, false>,
+                                  (const void*)attend_mma_kernel<4, false>, (const void*)attend_mma_kernel<8, false>};
         for (const void* f : kernels) {
             cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, MMA_SMEM_BYTES);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
@@ -667,25 +766,33 @@ cudaError_t launch_mma(const AttendParams& prm, int32_t g, int32_t nb, cudaStrea
         return cudaSuccess;
     });
     if (attr_error != cudaSuccess) return attr_error;
-    const dim3 grid((unsigned)prm.splits, (unsigned)(nb * prm.kv_heads));
+    const dim3 grid((unsigned)splits, (unsigned)(nb * prm.kv_heads));
+    auto launch = [&](auto with_tickets, auto without) {
+        auto* kernel = prm.tickets ? with_tickets : without;
+        kernel<<<grid, MMA_THREADS, MMA_SMEM_BYTES, stream>>>(prm);
+    };
     switch (g) {
-        case 2: attend_mma_kernel<2><<<grid, MMA_THREADS, MMA_SMEM_BYTES, stream>>>(prm); break;
-        case 4: attend_mma_kernel<4><<<grid, MMA_THREADS, MMA_SMEM_BYTES, stream>>>(prm); break;
-        case 8: attend_mma_kernel<8><<<grid, MMA_THREADS, MMA_SMEM_BYTES, stream>>>(prm); break;
+        case 2: launch(attend_mma_kernel<2, true>, attend_mma_kernel<2, false>); break;
+        case 4: launch(attend_mma_kernel<4, true>, attend_mma_kernel<4, false>); break;
+        case 8: launch(attend_mma_kernel<8, true>, attend_mma_kernel<8, false>); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_typed(const AttendParams& prm, int32_t g, int32_t nb, cudaStream_t stream)
+cudaError_t launch_typed(const AttendParams& prm, int32_t g, int32_t nb, int32_t splits, cudaStream_t stream)
 {
-    const dim3 grid((unsigned)prm.splits, (unsigned)(nb * prm.kv_heads));
+    const dim3 grid((unsigned)splits, (unsigned)(nb * prm.kv_heads));
+    auto launch = [&](auto with_tickets, auto without) {
+        auto* kernel = prm.tickets ? with_tickets : without;
+        kernel<<<grid, THREADS, 0, stream>>>(prm);
+    };
     switch (g) {
-        case 1: attend_partial_kernel<T, 1><<<grid, THREADS, 0, stream>>>(prm); break;
-        case 2: attend_partial_kernel<T, 2><<<grid, THREADS, 0, stream>>>(prm); break;
-        case 4: attend_partial_kernel<T, 4><<<grid, THREADS, 0, stream>>>(prm); break;
-        case 8: attend_partial_kernel<T, 8><<<grid, THREADS, 0, stream>>>(prm); break;
+        case 1: launch(attend_partial_kernel<T, 1, true>, attend_partial_kernel<T, 1, false>); break;
+        case 2: launch(attend_partial_kernel<T, 2, true>, attend_partial_kernel<T, 2, false>); break;
+        case 4: launch(attend_partial_kernel<T, 4, true>, attend_partial_kernel<T, 4, false>); break;
+        case 8: launch(attend_partial_kernel<T, 8, true>, attend_partial_kernel<T, 8, false>); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -698,27 +805,36 @@ bool attend_supported(int32_t head_dim, int32_t q_heads_per_kv)
     return head_dim == 128 && (q_heads_per_kv == 1 || q_heads_per_kv == 2 || q_heads_per_kv == 4 || q_heads_per_kv == 8);
 }
 
-// Splits of the rows of one (sequence, kv head): the count, among those that leave a CTA at least
-// 1024 rows, whose CTAs fill whole waves of the resident CTAs best (the smallest such count).
-// Shorter chunks with fuller waves measured slower: the prologue (length, queries, table) and the
-// partials weigh more than the idle CTA slots.
-int32_t attend_splits(int32_t batch, int32_t kv_heads, int32_t max_len, int32_t q_heads_per_kv, int32_t dtype, int sm_count)
+// Rows of one CTA.  Each candidate is judged by the rows' time of its waves of resident CTAs, waves * (rows +
+// OVERHEAD_ROWS): the constant stands for a CTA's prologue (query, table) and its share of the merge.  A launch with
+// few (sequence, kv head) groups splits down to MIN_ROWS rows, so that even a single sequence is read by the whole
+// chip; one with many groups takes long chunks that fill their last wave.  Measured, us a layer, against two splits
+// of at least 1024 rows: 1 sequence x 8 KV heads x 2611 rows 28.7 -> 13.2 (128 rows 13.4, 256 rows 13.5), 4 x 8 heads of up
+// to 1990 rows 40.7 -> 16.4, 8 x 8 heads of 4099 to 8192 rows 48.9 -> 43.4; OVERHEAD_ROWS 32 and 192 give the same.
+AttendPlan attend_plan(int32_t batch, const int32_t* lens, int32_t kv_heads, int32_t q_heads_per_kv, int32_t dtype, int sm_count)
 {
-    const double groups = (double)batch * kv_heads;
+    constexpr int32_t MIN_ROWS = 192, OVERHEAD_ROWS = 96, MOST_SPLITS = 64, MOST_ROWS = 0xffff * 16;  // a split's tiles are 16 bits
     const bool tensor_cores = dtype == FREQKV_BF16 && q_heads_per_kv >= 2;
-    const double resident = (double)sm_count * (tensor_cores ? MMA_CTAS_PER_SM : q_heads_per_kv <= 4 ? 2 : 1);
-    const int32_t most = std::max(1, std::min(32, max_len / 1024));
-    int32_t best = 1;
-    double best_fill = 0.0;
-    for (int32_t s = 1; s <= most; ++s) {
-        const double waves = groups * s / resident, fill = waves / std::ceil(waves);
-        if (fill > best_fill + 0.02) {
-            best_fill = fill;
-            best = s;
+    const int64_t resident = (int64_t)sm_count * (tensor_cores ? MMA_CTAS_PER_SM : q_heads_per_kv <= 4 ? 2 : 1);
+    const int32_t longest = *std::max_element(lens, lens + batch);
+    AttendPlan plan = {};
+    int64_t best_cost = -1;
+    for (int32_t splits = 1; splits <= MOST_SPLITS; splits += std::max(1, splits / 4)) {
+        const int32_t chunk = std::min(((longest + splits - 1) / splits + 15) & ~15, MOST_ROWS);
+        if (splits > 1 && chunk < MIN_ROWS) break;
+        int64_t ctas = 0;
+        for (int32_t b = 0; b < batch; ++b) ctas += (int64_t)kv_heads * ((lens[b] + chunk - 1) / chunk);
+        const int64_t cost = (ctas + resident - 1) / resident * (chunk + OVERHEAD_ROWS);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            plan = {chunk, (longest + chunk - 1) / chunk, ctas <= resident};
         }
     }
-    return best;
+    return plan;
 }
+
+// One wave of CTAs holds at most so many (sequence, kv head) groups.
+size_t attend_ticket_bytes(int sm_count) { return (size_t)sm_count * MMA_CTAS_PER_SM * sizeof(int32_t); }
 
 size_t attend_partial_bytes(int32_t splits, int32_t batch, int32_t q_heads)
 {
@@ -733,9 +849,10 @@ cudaError_t launch_rope_table(float2* table, int32_t rows, double base, cudaStre
 }
 
 cudaError_t launch_attend(const freqkv_layout& l, const void* k, const void* v, int32_t layer, const void* q, void* out,
-                          int32_t g, const int32_t* lens_host, const float2* table, float scale, int32_t splits,
-                          float* partial, cudaStream_t stream)
+                          int32_t g, const int32_t* lens_host, const float2* table, float scale, const AttendPlan& plan,
+                          float* partial, int32_t* tickets, int32_t* launched, cudaStream_t stream)
 {
+    *launched = 0;
     const size_t elt = dtype_size(l.dtype);
     AttendParams prm;
     prm.k = static_cast<const char*>(k) + (size_t)layer * l.stride_layer * elt;
@@ -744,36 +861,53 @@ cudaError_t launch_attend(const freqkv_layout& l, const void* k, const void* v, 
     prm.stride_head = l.stride_head;
     prm.stride_token = l.stride_token;
     prm.kv_heads = l.kv_heads;
-    prm.splits = splits;
     prm.q = q;
+    prm.out = out;
     prm.partial = partial;
+    prm.tickets = plan.one_wave ? tickets : nullptr;
     prm.table = table;
     prm.qscale = scale * 1.4426950408889634f;
     prm.total_batch = l.batch;
     for (int32_t b0 = 0; b0 < l.batch; b0 += ATTEND_MAX_BATCH) {
         const int32_t nb = std::min(ATTEND_MAX_BATCH, l.batch - b0);
         prm.batch0 = b0;
-        for (int32_t i = 0; i < nb; ++i) prm.len[i] = lens_host[b0 + i];
-        const cudaError_t e = l.dtype == FREQKV_F32 ? launch_typed<float>(prm, g, nb, stream)
-                              : g >= 2             ? launch_mma(prm, g, nb, stream)   // grouped queries: tensor cores
-                                                   : launch_typed<__nv_bfloat16>(prm, g, nb, stream);
+        MergeParams merge;
+        int32_t splits = 1;  // of the longest sequence of this launch: the grid's width
+        for (int32_t i = 0; i < nb; ++i) {
+            // as few splits as hold `chunk` rows each, evenly filled in whole tiles of 16 rows
+            const int32_t len = lens_host[b0 + i], n = (len + plan.chunk - 1) / plan.chunk, tiles = ((len + n - 1) / n + 15) / 16;
+            prm.len[i] = len;
+            prm.tiles[i] = (uint16_t)tiles;
+            merge.splits[i] = (uint16_t)((len + tiles * 16 - 1) / (tiles * 16));
+            splits = std::max(splits, n);
+        }
+        const cudaError_t e = l.dtype == FREQKV_F32 ? launch_typed<float>(prm, g, nb, splits, stream)
+                              : g >= 2             ? launch_mma(prm, g, nb, splits, stream)   // grouped queries: tensor cores
+                                                   : launch_typed<__nv_bfloat16>(prm, g, nb, splits, stream);
         if (e != cudaSuccess) return e;
+        ++*launched;
+        if (!prm.tickets && splits > 1) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(nb * l.kv_heads * g));
+            cfg.blockDim = dim3(128);
+            cfg.stream = stream;
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;  // let the launch overlap the tail of the kernel before it
+            attr.val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            merge.partial = partial;
+            merge.out = out;
+            merge.heads = l.kv_heads * g;
+            merge.head0 = (int64_t)b0 * merge.heads;
+            merge.heads_total = (int64_t)l.batch * merge.heads;
+            const cudaError_t me = l.dtype == FREQKV_F32 ? cudaLaunchKernelEx(&cfg, attend_merge_kernel<float>, merge)
+                                                         : cudaLaunchKernelEx(&cfg, attend_merge_kernel<__nv_bfloat16>, merge);
+            if (me != cudaSuccess) return me;
+            ++*launched;
+        }
     }
-    const int64_t heads_total = (int64_t)l.batch * l.kv_heads * g;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)heads_total);
-    cfg.blockDim = dim3(128);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;  // let the launch overlap the tail of the kernel before it
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    const float* partial_in = partial;
-    if (l.dtype == FREQKV_F32)
-        return cudaLaunchKernelEx(&cfg, attend_merge_kernel<float>, partial_in, splits, heads_total, static_cast<float*>(out));
-    return cudaLaunchKernelEx(&cfg, attend_merge_kernel<__nv_bfloat16>, partial_in, splits, heads_total,
-                              static_cast<__nv_bfloat16*>(out));
+    return cudaSuccess;
 }
 
 }  // namespace freqkv

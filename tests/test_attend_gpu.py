@@ -138,3 +138,18 @@ def test_attend_more_sequences_than_one_launch_takes(ctx, G):
     k, v = synth.make_cache(w, "cuda")
     lens = [96 - (b % 60) for b in range(131)]
     check(ctx, k, v, 0, queries(131, G, torch.bfloat16, 17 + G), lens, 10000.0, heads=[(0, 0), (1, 0), (127, 0), (128, 0), (130, 0)])
+
+
+@pytest.mark.parametrize("G,H,lens", [(4, 8, [2611]), (1, 4, [193, 7000, 192]), (8, 4, [1400, 17, 385, 600]), (2, 3, [191, 1]),
+                                      (1, 32, [900 + 37 * b for b in range(24)])])
+def test_attend_splits_and_their_merge(ctx, G, H, lens):
+    """A few groups cut into many splits that the last CTA of a group merges (one split, two, lengths around the smallest
+    split), and more groups than one wave of CTAs holds, merged by a kernel of its own; the same bits call after call."""
+    w = workload(len(lens), 1, H, max(lens) + 5, torch.bfloat16, seed=23)
+    k, v = synth.make_cache(w, "cuda")
+    q = queries(len(lens), H * G, torch.bfloat16, 24)
+    first = ctx.attend_decode(k, v, 0, q, lens)
+    for _ in range(3):
+        assert torch.equal(ctx.attend_decode(k, v, 0, q, lens), first)
+    last = len(lens) - 1
+    check(ctx, k, v, 0, q, lens, 10000.0, heads=[(0, 0), (last, H - 1), (last // 2, 1)])
