@@ -150,17 +150,28 @@ def workload_numbers(w, cache_len, kept, sink, first=0):
     e = 2 if w.dtype == torch.bfloat16 else 4
     m = w.n_matrices
     n_in = cache_len - sink
-    # Multiply-adds the tensor-core variant executes.  One level of the symmetry fold: even and odd parts,
-    # ceil(L/2) x ceil(N/2) each.  Where the lengths halve twice (N a multiple of 4, L even, the lowest
-    # components kept) the even part is folded again: ceil(L/4) rows x (N/4 + N/4 + N/2 + N/2) columns.
+    # Multiply-adds the mirror symmetry leaves.  One level: even and odd parts, ceil(L/2) x ceil(N/2) each.  Where the
+    # lengths halve twice (N a multiple of 4, L even, the lowest components kept) the even part folds again:
+    # ceil(L/4) rows x (N/4 + N/4 + N/2 + N/2) columns.
     from paper_2505_00570_b200 import binding as _fk
-    fold_levels = _fk.gemm_fold_levels(n_in, kept, first)   # the library's own rule (0 = no fold pass: few kept rows)
+    fold_levels = _fk.gemm_fold_levels(n_in, kept, first)   # 0 = no fold pass: few kept rows
     if fold_levels == 2:
         folded = 2.0 * ((kept // 2 + 1) // 2) * 3 * (n_in // 2) * w.head_dim * m
     else:
         folded = 2.0 * 2 * ((kept + 1) // 2) * ((n_in + 1) // 2) * w.head_dim * m
+    # What the library executes: where N is a multiple of 4, L even and the lowest components are kept, four blocks of
+    # ceil(L/4) x N/4 (the last N/2 deep for even L/2) if that means fewer 64-row slices of 256-row tiles than one level.
+    def slices(rows, steps):
+        return -(-rows // 256) * steps
+    q, tail = -(-(n_in // 4) // 64), -(-(n_in // 2) // 64) if kept // 2 % 2 == 0 else -(-(n_in // 4) // 64)
+    four = (first == 0 and n_in % 4 == 0 and kept % 2 == 0 and kept > 256 and
+            slices((kept // 2 + 1) // 2, 3 * q + tail) < slices((kept + 1) // 2, 2 * -(-(n_in // 2) // 64)))
+    executed = 2.0 * 2 * ((kept + 1) // 2) * ((n_in + 1) // 2) * w.head_dim * m
+    if four:
+        executed = 2.0 * ((kept // 2 + 1) // 2) * (4 if kept // 2 % 2 else 5) * (n_in // 4) * w.head_dim * m
     return {
         "fold_levels": fold_levels,
+        "executed_flops": executed,
         "matrices": m,
         "cache_in_bytes": m * cache_len * w.head_dim * e,
         "algorithmic_bytes": m * (n_in + kept) * w.head_dim * e,   # read N' rows, write L rows
@@ -658,7 +669,7 @@ def main():
     peaks = load_peaks()
     kernel_ms = t_ms / max(t_launches, 1)                  # average duration of one launch of the dominant kernel
     per_call = max(t_launches, 1) / args.steps             # launches per compression (large caches take several passes)
-    for key in ("folded_flops", "projection_flops", "algorithmic_bytes"):
+    for key in ("executed_flops", "projection_flops", "algorithmic_bytes"):
         nums[key + "_per_launch"] = nums[key] / per_call
     if chosen == fk.GEMM and kept <= 256:
         # few kept rows: the tensor-core variant reads the cache directly (no fold pass, one tile per
@@ -667,7 +678,7 @@ def main():
         roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "peak_kind": "copy, of " + peaks["source"]}
     elif chosen == fk.GEMM:
-        achieved = nums["folded_flops_per_launch"] / (kernel_ms * 1e-3) / 1e12
+        achieved = nums["executed_flops_per_launch"] / (kernel_ms * 1e-3) / 1e12
         # the burst figure is the denominator for a timed region of under a second, the sustained
         # one (power cap reached) for longer loops; both fractions are printed
         burst = ms_total < 1000.0
@@ -677,12 +688,12 @@ def main():
                 "frac": achieved / peak, "peak_kind": ("burst" if burst else "sustained") + ", of " + peaks["source"],
                 "frac_of_burst_peak": achieved / peaks["bf16_tflops"],
                 "frac_of_sustained_peak": achieved / peaks["bf16_tflops_sustained"],
-                "flops_per_launch": nums["folded_flops_per_launch"], "fold_levels": nums["fold_levels"],
+                "flops_per_launch": nums["executed_flops_per_launch"],
                 "dense_equivalent_flops_per_launch": nums["projection_flops_per_launch"],
                 # the fold pass the kernel cannot run without: its time (compress call minus the
                 # timed kernel) and the bytes it moves (every non-sink row read once, written once)
                 "fold_ms": fold_ms, "fold_bytes": 2 * nums["matrices"] * (cache_len - sink) * w.head_dim * 2,
-                "frac_of_burst_peak_whole_call": nums["folded_flops"] / (compress_ms * 1e-3) / 1e12 / peaks["bf16_tflops"]}
+                "frac_of_burst_peak_whole_call": nums["executed_flops"] / (compress_ms * 1e-3) / 1e12 / peaks["bf16_tflops"]}
     elif chosen == fk.FDCT:
         achieved = nums["algorithmic_bytes_per_launch"] / (kernel_ms * 1e-3) / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",

@@ -831,7 +831,7 @@ freqkv_status freqkv_power_spectrum(freqkv_ctx* ctx, const freqkv_layout* layout
     hooks.user = &timer;
     hooks.before = [](void* u, cudaStream_t) { static_cast<TransformTimer*>(u)->begin(); };
     hooks.after = [](void* u, cudaStream_t) { static_cast<TransformTimer*>(u)->end(); };
-    const cudaError_t e = launch_gemm(&ctx->gemm, view, basis, sink, ctx->status_dev, ctx->sm_count, hooks, stream, &out);
+    const cudaError_t e = launch_gemm_spectrum(&ctx->gemm, view, basis, sink, ctx->status_dev, ctx->sm_count, hooks, stream, out);
     if (e != cudaSuccess) return cuda_fail(ctx, e, ctx->gemm.last_error ? ctx->gemm.last_error : "launch_gemm");
     ctx->kernels_launched += ctx->gemm.kernels_last_call;
     return FREQKV_OK;

@@ -20,7 +20,7 @@
 // Two kernels per call:
 //   fold_kernel         reads every non-sink cache row once and writes U and V (bf16) to a scratch
 //                       buffer, one plane of ceil(N/2) x 128 per (matrix, u|v); HBM-bound.
-//   freqkv_gemm_kernel  persistent, one CTA per SM, CTAs paired into clusters of two that share
+//   freqkv_fold_gemm_kernel  persistent, one CTA per SM, CTAs paired into clusters of two that share
 //                       every MMA (tcgen05 cta_group::2).  A cluster works on output tiles of 256
 //                       folded rows x 256 columns (the K matrix and the V matrix of one (batch,
 //                       layer, kv_head) side by side, so K and V share every instruction): CTA r
@@ -35,7 +35,7 @@
 //                 of 6 stages of 32 KB; the bytes of both CTAs complete the leader's barrier;
 //     warp 1      MMA issuer (leader CTA only): 4 tcgen05.mma (256 x 256 x 16) per stage, commits
 //                 multicast to the barriers of both CTAs;
-//     warps 2-9   epilogue: when S is complete they park it in registers (which frees that half
+//     warps 4-11  epilogue: when S is complete they park it in registers (which frees that half
 //                 of tensor memory for the next tile while D is still accumulating); when D is
 //                 complete they form s + d and s - d, round to bf16 (nearest even) and store rows
 //                 m and L-1-m straight into the cache.  Both steps overlap the MMAs of the
@@ -65,55 +65,55 @@ constexpr int B_CHUNK_BYTES = BK * 128;            // 8 KB: 64 rows x 64 channel
 constexpr int B_BYTES = 2 * B_CHUNK_BYTES;         // 16 KB: this CTA's 128 of the 256 columns
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;     // 32 KB per CTA
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
-constexpr int NUM_THREADS = 320;                   // 10 warps
-// MODE_QUAD: three warpgroups (producer and MMA issuer | epilogue | epilogue) that share the registers unevenly.  The
-// shares add up to what the block is launched with: 40 + 2 * 232 = 3 * 168.
-constexpr int QUAD_THREADS = 384, QUAD_LAUNCH_REGS = 168, QUAD_CONTROL_REGS = 40, QUAD_EPILOGUE_REGS = 232;
-static_assert(QUAD_CONTROL_REGS + 2 * QUAD_EPILOGUE_REGS <= 3 * QUAD_LAUNCH_REGS, "a larger sum would wait for registers for ever");
-constexpr size_t PARK_BYTES_PER_CTA = (size_t)BM * 256 * 4;  // MODE_QUAD: the pairs (s, s') of one tile, two bf16 each
+constexpr int NUM_THREADS = 320;                   // direct and spectrum modes: 10 warps
+// The kernel of the folded forms: three warpgroups (producer and MMA issuer | epilogue | epilogue) that share the
+// registers unevenly.  The shares add up to what the block is launched with: 40 + 2 * 232 = 3 * 168.
+constexpr int FOLD_THREADS = 384, FOLD_LAUNCH_REGS = 168, CONTROL_REGS = 40, EPILOGUE_REGS = 232;
+static_assert(CONTROL_REGS + 2 * EPILOGUE_REGS <= 3 * FOLD_LAUNCH_REGS, "a larger sum would wait for registers for ever");
+constexpr size_t PARK_BYTES_PER_CTA = (size_t)BM * 256 * 8;  // four blocks: the pairs (s, s') of one tile, bf16 or fp32
 constexpr int EPI_WARPS = 8;
 constexpr unsigned long long LANDING_NS = 1000000ull;        // 1 ms: far longer than any copy in flight needs
 
 constexpr uint32_t ERR_FULL_WAIT = 1u, ERR_EMPTY_WAIT = 2u, ERR_ACC_FULL_WAIT = 4u, ERR_ACC_EMPTY_WAIT = 8u;
 
-struct RaggedSeq {
-    int32_t tile0, pair0, n_keep, rows_half, basis_rows_pad, k_steps, m_pairs, pad;
+// The matrices of one sequence (or of one pass of a uniform call): how they fold and what their tiles are.
+struct FoldSeq {
+    int32_t tile0;              // first tile in the launch
+    int32_t pair0;              // first (batch, layer, kv_head) triple
+    int32_t n_half, n_keep, rows_half;
+    int32_t quad;               // four blocks instead of one level
+    int32_t basis_rows_pad;     // row offset of one basis plane to the next inside the basis tensor map
+    int32_t k_steps, k_last;    // slices per phase; of the fourth phase of four
+    int32_t m_pairs;            // tiles of 256 folded rows per triple
+};
+
+struct FoldParams {
+    int32_t sink;
+    int32_t mirror_sign;        // +1: y[L-1-m] = s - d;  -1: y[L-1-m] = d - s (a retained band that starts at an odd component)
+    int32_t wide_rows;          // every row is 32-byte aligned
+    int32_t total_tiles;
+    uint4* park;                // four blocks: work area of (s, s')
+    int32_t* status;
+    unsigned long long wait_limit_ns;  // bound of every mbarrier wait
+    FoldSeq seq;                // uniform calls
+    // ragged batches: one entry per sequence, sorted by decreasing work, and one past the end that holds the total of
+    // tiles; two tensor maps per sequence (basis, planes)
+    const FoldSeq* seqs;
+    const CUtensorMap* seq_maps;
 };
 
 struct GemmParams {
     int32_t n_keep;             // L
-    int32_t rows_half;          // ceil(L / 2): folded output rows
     int32_t basis_rows_pad;     // row offset of the Po plane inside the basis tensor map
     int32_t pair0, pair_count;  // (batch, layer, kv_head) triples covered by this launch
     int32_t m_pairs, k_steps;   // tiles of 256 folded rows per (batch, layer, kv_head); slices per phase
-    // four-block form only: ceil(L / 4) = rows of a block, N / 4 = rows of each of its four inputs, slices of
-    // the first three phases and of the last one, where the pairs (s, s') wait, whether rows take 32-byte stores
-    int32_t rows_quarter, n_quarter, k_steps_short, k_steps_last;
-    uint4* park;
-    int32_t wide_rows;
     int32_t sink;
-    int32_t mirror_sign;        // +1: y[L-1-m] = s - d;  -1: y[L-1-m] = d - s (a retained band that starts at an odd component)
     // power-spectrum mode only: per tensor [layers][kv_heads][n_in] sums, the weight of one squared value
     float* spectrum[2];
     float spectrum_scale;
     int32_t n_in;
     int32_t* status;
     unsigned long long wait_limit_ns;  // bound of every mbarrier wait
-    // ragged mode only: per-sequence shapes (sorted by decreasing work, tile0 = running sum of tiles,
-    // one entry past the end holds the total) and two tensor maps per sequence (basis, folded inputs)
-    const RaggedSeq* seqs;
-    const CUtensorMap* seq_maps;
-    int32_t n_seqs;
-};
-
-// What one tile (256 folded output rows x K|V of one (batch, layer, kv_head)) works on.
-struct TileCtx {
-    const CUtensorMap* map_p;   // basis
-    const CUtensorMap* map_x;   // folded inputs
-    int32_t pair;               // (batch, layer, kv_head) triple inside the cache view
-    int32_t pair_local;         // ... inside the scratch planes its tensor map covers
-    int32_t m_tile;             // which 256 folded rows
-    int32_t n_keep, rows_half, basis_rows_pad, k_steps;
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -323,14 +323,14 @@ __device__ __forceinline__ void fold8(const uint4& a, const uint4& b, uint4* u, 
 struct FoldJob {
     int32_t pair0, pair_count, n_in, n_half, sink;
     uint4* dst;
+    const float2* turns;  // four blocks: (cos, sin) of theta_n; null: one level
 };
 
-// Block (x, y): matrix x of the job (pair_local * 2 + tensor), y-th share of its n_half * 16 vectors.
+// One level: matrix pt of the job (pair_local * 2 + tensor), the y-th of gridDim.y shares of its n_half * 16 vectors.
 // The matrix arithmetic is done once per thread; each thread then folds four vectors per round,
 // all eight loads first.  Reads and writes are streaming (each byte is touched once).
-__global__ void __launch_bounds__(256) fold_kernel(const CacheView view, const FoldJob job)
+__device__ __forceinline__ void fold_one_level(const CacheView& view, const FoldJob& job, uint32_t pt)
 {
-    const uint32_t pt = blockIdx.x;
     const char* x = static_cast<const char*>(tensor_base(view, pt & 1)) +
                     (matrix_offset(view, job.pair0 + (int32_t)(pt >> 1)) + (int64_t)job.sink * view.stride_token) * 2;
     const int64_t row_bytes = view.stride_token * 2;
@@ -397,11 +397,9 @@ __device__ __forceinline__ void fold8_quad(const uint4& a, const uint4& b, const
     *q = make_uint4(o[3][0], o[3][1], o[3][2], o[3][3]);
 }
 
-// Block (x, y) as in fold_kernel; job.n_half = N' rows per plane; a thread folds two vectors per round.
-// `turns`: (cos, sin) of theta_n, n < N' / 2.
-__global__ void __launch_bounds__(256) fold_quad_kernel(const CacheView view, const FoldJob job, const float2* __restrict__ turns)
+// Four blocks: as fold_one_level; job.n_half = N' rows per plane; a thread folds two vectors per round.
+__device__ __forceinline__ void fold_four_blocks(const CacheView& view, const FoldJob& job, uint32_t pt, const float2* __restrict__ turns)
 {
-    const uint32_t pt = blockIdx.x;
     const char* x = static_cast<const char*>(tensor_base(view, pt & 1)) +
                     (matrix_offset(view, job.pair0 + (int32_t)(pt >> 1)) + (int64_t)job.sink * view.stride_token) * 2;
     const int64_t row_bytes = view.stride_token * 2;
@@ -439,111 +437,36 @@ __global__ void __launch_bounds__(256) fold_quad_kernel(const CacheView view, co
     }
 }
 
-// The same for a ragged batch in one launch: every sequence has the same number of matrices, so
-// block x belongs to job x / mats_per_seq.
-__global__ void __launch_bounds__(256) fold_ragged_kernel(const CacheView view, const FoldJob* jobs, int32_t mats_per_seq)
+// Block x: matrix x of the job, or, of a ragged batch (every sequence has the same number of matrices), of job x / mats_per_seq.
+__global__ void __launch_bounds__(256) fold_kernel(const CacheView view, const FoldJob job) { fold_one_level(view, job, blockIdx.x); }
+
+// (`turns` = job.turns as a parameter of its own: read through the struct it costs 83 registers instead of 80, one block an SM
+// less, and 0.02 ms of a 7B-shaped fold.)
+__global__ void __launch_bounds__(256) fold_quad_kernel(const CacheView view, const FoldJob job, const float2* __restrict__ turns)
 {
-    const FoldJob job = jobs[blockIdx.x / mats_per_seq];
-    const uint32_t pt = blockIdx.x % mats_per_seq;
-    const char* x = static_cast<const char*>(tensor_base(view, pt & 1)) +
-                    (matrix_offset(view, job.pair0 + (int32_t)(pt >> 1)) + (int64_t)job.sink * view.stride_token) * 2;
-    const int64_t row_bytes = view.stride_token * 2;
-    const uint32_t total = (uint32_t)job.n_half * 16u;
-    uint4* u_plane = job.dst + (int64_t)pt * 2 * total;
-    for (uint32_t c0 = blockIdx.y * 1024u; c0 < total; c0 += gridDim.y * 1024u) {
-        uint4 a[4], b[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t i = c0 + j * 256u + threadIdx.x;
-            if (i < total) {
-                const int32_t n = (int32_t)(i >> 4), nr = job.n_in - 1 - n;
-                a[j] = __ldcs(reinterpret_cast<const uint4*>(x + n * row_bytes) + (i & 15u));
-                b[j] = __ldcs(reinterpret_cast<const uint4*>(x + nr * row_bytes) + (i & 15u));
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t i = c0 + j * 256u + threadIdx.x;
-            if (i < total) {
-                const int32_t n = (int32_t)(i >> 4);
-                uint4 u, v;
-                fold8(a[j], b[j], &u, &v);
-                if (job.n_in - 1 - n == n) {
-                    u = a[j];
-                    v = make_uint4(0u, 0u, 0u, 0u);
-                }
-                __stcs(u_plane + i, u);
-                __stcs(u_plane + total + i, v);
-            }
-        }
-    }
+    fold_four_blocks(view, job, blockIdx.x, turns);
 }
 
-// MODE_FOLD: the compression above.
-// MODE_RAGGED: MODE_FOLD over sequences of different lengths in one launch: a tile looks up its
-//   sequence (shapes, basis and folded-input tensor maps) in a table built on the host.
+__global__ void __launch_bounds__(256, 4) fold_ragged_kernel(const CacheView view, const FoldJob* jobs, int32_t mats_per_seq)
+{
+    const FoldJob job = jobs[blockIdx.x / mats_per_seq];
+    if (job.turns)
+        fold_four_blocks(view, job, blockIdx.x % mats_per_seq, job.turns);
+    else
+        fold_one_level(view, job, blockIdx.x % mats_per_seq);
+}
+
+// The other two uses of the same tiles:
 // MODE_SPECTRUM: the basis holds the even and the odd rows of the plain N-point DCT-II instead of
 //   Pe and Po, so S and D are the components z_2m and z_2m+1 themselves; the epilogue squares them,
 //   sums over the 128 channels of its tensor and adds the sum to the power spectrum of its
 //   (layer, kv head).  Nothing is written to the cache.
-// MODE_DIRECT: for at most 256 kept rows (small retaining ratios) the fold pass would cost more
+// MODE_DIRECT: for at most 256 kept rows (small retaining ratios) the fold would cost more
 //   than it saves: the basis is the plain L x N matrix P, the input slices come straight from the
 //   cache (map_x = K tensor, map_v = V tensor, 5-D maps over the non-sink rows), there is one
 //   accumulator and one tile per (batch, layer, kv_head).  The tile's rows are stored only after
 //   every slice of its matrices has been read, so writing in place is safe here too.
-// MODE_QUAD: the four-block form (n_in a multiple of 4, n_keep even).  A tile is 256 rows m < ceil(L/4) of all
-//   four blocks and runs four phases, each N/4 deep, alternating between the two halves of tensor memory:
-//   a = Pee uu, b = Peo uv, A = PA p, B = PB q (for even L/2 one retained component couples p into B: the last
-//   phase then runs on through p, with that component's column weights as its basis).  The epilogue
-//   parks a in registers, turns it with b into the pair s = a + b, s' = a - b (two bf16 in a 32-bit word), which waits
-//   in a work area of this CTA that stays in L2 -- the accumulators of a tile would need twice the tensor memory there is --,
-//   parks A, and turns it with B by theta'_m = pi (2m+1) / (2L) into d = cos A + sin B and d' = sin A - cos B:
-//   y_m = s + d, y_{L-1-m} = s - d, y_{L/2-1-m} = s' + d', y_{L/2+m} = s' - d'.
-constexpr int MODE_FOLD = 0, MODE_SPECTRUM = 1, MODE_DIRECT = 2, MODE_RAGGED = 3, MODE_QUAD = 4;
-
-// Ragged mode: a role walks its tiles in increasing order, so the sequence a tile belongs to is
-// found by moving a cursor forward; the table is read only when a tile crosses into a new sequence.
-struct SeqCursor {
-    int32_t idx = -1, end_tile = 0;
-    RaggedSeq s;
-};
-
-template <int MODE>
-__device__ __forceinline__ TileCtx tile_ctx(const GemmParams& prm, int32_t tile, const CUtensorMap* map_p, const CUtensorMap* map_x,
-                                            SeqCursor& cur)
-{
-    TileCtx t;
-    if constexpr (MODE == MODE_RAGGED) {
-        while (tile >= cur.end_tile) {
-            ++cur.idx;
-            cur.s = prm.seqs[cur.idx];
-            cur.end_tile = __ldg(&prm.seqs[cur.idx + 1].tile0);
-        }
-        const RaggedSeq& s = cur.s;
-        const int32_t lo = cur.idx;
-        const int32_t local = tile - s.tile0;
-        t.map_p = prm.seq_maps + 2 * lo;
-        t.map_x = prm.seq_maps + 2 * lo + 1;
-        t.pair_local = local / s.m_pairs;
-        t.m_tile = local % s.m_pairs;
-        t.pair = s.pair0 + t.pair_local;
-        t.n_keep = s.n_keep;
-        t.rows_half = s.rows_half;
-        t.basis_rows_pad = s.basis_rows_pad;
-        t.k_steps = s.k_steps;
-    } else {
-        t.map_p = map_p;
-        t.map_x = map_x;
-        t.pair_local = tile / prm.m_pairs;
-        t.m_tile = tile % prm.m_pairs;
-        t.pair = prm.pair0 + t.pair_local;
-        t.n_keep = prm.n_keep;
-        t.rows_half = prm.rows_half;
-        t.basis_rows_pad = prm.basis_rows_pad;
-        t.k_steps = prm.k_steps;
-    }
-    return t;
-}
+constexpr int MODE_SPECTRUM = 1, MODE_DIRECT = 2;
 
 // Registers of the calling warpgroup from here on (every warp of it executes this).
 template <int REGS, bool MORE>
@@ -568,15 +491,353 @@ __device__ __forceinline__ void store_row16(__nv_bfloat16* dst, const uint32_t (
     }
 }
 
+// ---- the product of the folded forms ----
+
+// Ragged batches: a role walks its tiles in increasing order, so the sequence a tile belongs to is found by moving a
+// cursor forward; the table in global memory is read only when a tile crosses into a new sequence.
+struct SeqCursor {
+    int32_t idx = -1, end_tile = 0;
+    FoldSeq s;
+};
+template <bool RAGGED>
+__device__ __forceinline__ const FoldSeq& seq_of_tile(const FoldParams& prm, int32_t tile, SeqCursor& cur)
+{
+    if constexpr (RAGGED) {
+        while (tile >= cur.end_tile) {
+            ++cur.idx;
+            cur.s = prm.seqs[cur.idx];
+            cur.end_tile = __ldg(&prm.seqs[cur.idx + 1].tile0);
+        }
+        return cur.s;
+    } else {
+        return prm.seq;
+    }
+}
+
+// FORM_ONE_LEVEL, FORM_FOUR_BLOCKS, FORM_FOUR_BLOCKS_WIDE: the compression of one pair of lengths; WIDE keeps the pairs (s, s')
+//   below in fp32, for lengths at which one level, whose sums never leave fp32, is the alternative.
+// FORM_RAGGED: sequences of different lengths in one launch: a tile looks up its sequence (shapes, tensor
+//   maps) in a table built on the host; one-level and four-block sequences mix (FoldSeq::quad).
+// Four blocks (n_in a multiple of 4, n_keep even): a tile is 256 rows m < ceil(L/4) of all
+//   four blocks and runs four phases, each N/4 deep, alternating between the two halves of tensor memory:
+//   a = Pee uu, b = Peo uv, A = PA p, B = PB q (for even L/2 one retained component couples p into B: the last
+//   phase then runs on through p, with that component's column weights as its basis).  The epilogue
+//   parks a in registers, turns it with b into the pair s = a + b, s' = a - b (two bf16 in a word, or two words), which waits
+//   in a work area of this CTA that stays in L2 -- the accumulators of a tile would need twice the tensor memory there is --,
+//   parks A, and turns it with B by theta'_m = pi (2m+1) / (2L) into d = cos A + sin B and d' = sin A - cos B:
+//   y_m = s + d, y_{L-1-m} = s - d, y_{L/2-1-m} = s' + d', y_{L/2+m} = s' - d'.
+constexpr int FORM_ONE_LEVEL = 0, FORM_FOUR_BLOCKS = 1, FORM_RAGGED = 2, FORM_FOUR_BLOCKS_WIDE = 3;
+
+template <int FORM>
+__global__ void __launch_bounds__(FOLD_THREADS, 1)
+freqkv_fold_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_x, const CacheView view,
+                        const __grid_constant__ FoldParams prm)
+{
+    constexpr bool RAGGED = FORM == FORM_RAGGED, WIDE = FORM == FORM_RAGGED || FORM == FORM_FOUR_BLOCKS_WIDE;
+    constexpr bool FOUR = FORM == FORM_FOUR_BLOCKS || FORM == FORM_FOUR_BLOCKS_WIDE;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;  // 128-byte swizzle atoms need 1024-byte alignment
+    uint8_t* aligned = smem_raw + (base - raw);
+    const uint32_t bar0 = base + STAGES * STAGE_BYTES;
+    // barrier slots (same offsets in both CTAs): full[0..S) -- used in the leader only --, empty[S..2S), then
+    // s_full, s_empty, d_full, d_empty (the two *_empty used in the leader only)
+    auto full_bar = [&](int s) { return bar0 + 8u * s; };
+    auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
+    auto acc_full_bar = [&](int eo) { return bar0 + 8u * (2 * STAGES + 2 * eo); };
+    auto acc_empty_bar = [&](int eo) { return bar0 + 8u * (2 * STAGES + 2 * eo + 1); };
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(aligned + STAGES * STAGE_BYTES + 8 * (2 * STAGES + 4));
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const uint32_t rank = cluster_rank();  // 0 = leader of the pair
+    const int32_t cluster = blockIdx.x / 2, n_clusters = gridDim.x / 2;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(full_bar(s), 1);   // the leader's producer arrives; both producers' bytes are counted
+            mbar_init(empty_bar(s), 1);  // one multicast commit
+        }
+        for (int eo = 0; eo < 2; ++eo) {
+            mbar_init(acc_full_bar(eo), 1);               // one multicast commit
+            mbar_init(acc_empty_bar(eo), 2 * EPI_WARPS);  // the epilogue warps of both CTAs
+        }
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {  // tensor memory of the pair: all 512 columns in each CTA
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync_all();  // the peer's barriers exist before anything signals them
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = *tmem_slot;
+
+    // One setmaxnreg per warpgroup, inside the branch that only this warpgroup takes: where branches meet, ptxas
+    // assumes the fewest registers.
+    if (warp < 4) {
+        set_registers<CONTROL_REGS, false>();
+        if (warp == 0) {
+            // ---------------- TMA producer (both CTAs) ----------------
+            if (lane == 0) {
+                uint32_t it = 0;  // global slice counter: stage = it % STAGES, phase = it / STAGES
+                bool alive = true;
+                SeqCursor cursor;
+                for (int32_t tile = cluster; tile < prm.total_tiles && alive; tile += n_clusters) {
+                    const FoldSeq& s = seq_of_tile<RAGGED>(prm, tile, cursor);
+                    const CUtensorMap* mp = RAGGED ? prm.seq_maps + 2 * cursor.idx : &map_p;
+                    const CUtensorMap* mx = RAGGED ? prm.seq_maps + 2 * cursor.idx + 1 : &map_x;
+                    const int32_t local = tile - s.tile0, pair = local / s.m_pairs;
+                    const int32_t m0 = (local % s.m_pairs * 2 + (int32_t)rank) * BM;
+                    const bool quad = RAGGED ? s.quad != 0 : FOUR;
+                    const int32_t phases = quad ? 4 : 2;
+                    for (int eo = 0; eo < phases && alive; ++eo) {
+                        // rank 0: K channels, rank 1: V.  Four blocks: phases 0, 1 read uu and uv (both in plane 0, uv
+                        // n_half / 2 rows down), phases 2, 3 read p (n_half / 2 rows down in plane 1) and q
+                        const int32_t plane = (pair * 2 + (int32_t)rank) * 2 + (quad ? eo >> 1 : eo);
+                        const int32_t row0 = (quad && (eo == 1 || eo == 2)) ? s.n_half / 2 : 0;
+                        const int32_t steps = eo == 3 ? s.k_last : s.k_steps;
+                        for (int32_t ks = 0; ks < steps; ++ks, ++it) {
+                            const int st = it % STAGES;
+                            if (it >= STAGES &&
+                                !mbar_wait(empty_bar(st), ((it / STAGES) - 1) & 1, abort_flag, prm.status, ERR_EMPTY_WAIT, prm.wait_limit_ns)) {
+                                alive = false;
+                                break;
+                            }
+                            const uint32_t stage = base + st * STAGE_BYTES;
+                            const uint32_t leader_full = cluster_addr(full_bar(st), 0);
+                            if (rank == 0) mbar_expect_tx(full_bar(st), 2 * STAGE_BYTES);
+                            const int32_t k0 = ks * BK;
+                            tma_load_2d(stage, mp, leader_full, k0, eo * s.basis_rows_pad + m0);
+                            tma_load_3d(stage + A_BYTES, mx, leader_full, 0, row0 + k0, plane);
+                            tma_load_3d(stage + A_BYTES + B_CHUNK_BYTES, mx, leader_full, 64, row0 + k0, plane);
+                        }
+                    }
+                }
+                if (*abort_flag) {  // let the copies in flight land before this CTA's shared memory goes away
+                    const unsigned long long t0 = global_timer_ns();
+                    while (global_timer_ns() - t0 < LANDING_NS) __nanosleep(1000);
+                }
+            }
+        } else if (warp == 1) {
+            // ---------------- MMA issuer (leader CTA only) ----------------
+            if (lane == 0 && rank == 0) {
+                uint32_t it = 0, phase = 0;  // phase: over all tiles; half of tensor memory = phase % 2
+                bool alive = true;
+                SeqCursor cursor;
+                for (int32_t tile = cluster; tile < prm.total_tiles && alive; tile += n_clusters) {
+                    const FoldSeq& s = seq_of_tile<RAGGED>(prm, tile, cursor);
+                    const int32_t phases = (RAGGED ? s.quad != 0 : FOUR) ? 4 : 2, k_steps = s.k_steps, k_last = s.k_last;
+                    for (int eo = 0; eo < phases && alive; ++eo, ++phase) {
+                        const uint32_t acc = phase & 1, use = phase >> 1;  // use: how often that half was filled before
+                        if (use > 0) {  // both CTAs' epilogues must have read what this half held last
+                            if (!mbar_wait(acc_empty_bar(acc), (use - 1) & 1, abort_flag, prm.status, ERR_ACC_EMPTY_WAIT, prm.wait_limit_ns)) {
+                                alive = false;
+                                break;
+                            }
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        }
+                        const int32_t steps = eo == 3 ? k_last : k_steps;
+                        for (int32_t ks = 0; ks < steps; ++ks, ++it) {
+                            const int st = it % STAGES;
+                            if (!mbar_wait(full_bar(st), (it / STAGES) & 1, abort_flag, prm.status, ERR_FULL_WAIT, prm.wait_limit_ns)) {
+                                alive = false;
+                                break;
+                            }
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            const uint32_t a0 = base + st * STAGE_BYTES, b0 = a0 + A_BYTES;
+#pragma unroll
+                            for (int kk = 0; kk < BK / 16; ++kk) {
+                                // A: 128 rows per CTA, 8-row groups 1 KB apart; 16 k-elements = 32 bytes inside the swizzled row
+                                const uint64_t ad = smem_desc(a0 + kk * 32, 16, 1024);
+                                // B: per CTA 2 chunks of 64 channels 8 KB apart (leading offset), 8-row groups 1 KB apart
+                                const uint64_t bd = smem_desc(b0 + kk * 2048, B_CHUNK_BYTES, 1024);
+                                umma_bf16(tmem_base + acc * 256, ad, bd, (ks | kk) != 0);
+                            }
+                            umma_commit_both(empty_bar(st));  // frees the stage in both CTAs when these MMAs have read it
+                        }
+                        if (alive) umma_commit_both(acc_full_bar(acc));
+                    }
+                }
+            }
+        }
+    } else {
+        set_registers<EPILOGUE_REGS, true>();
+        // ---------------- epilogue (both CTAs, each on its own 128 rows) ----------------
+        const int ew = warp - 4, quarter = warp % 4, tensor = ew / 4;  // tensor: 0 = K columns, 1 = V columns
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + tensor * 128;
+        // this thread's vectors of the work area: vector i of lane l at (i * 32 + l), so that a warp's access is dense
+        uint4* park = prm.park + ((size_t)blockIdx.x * EPI_WARPS + ew) * (64 * 32) + lane;
+        uint32_t phase = 0;  // as the MMA issuer counts
+        // wait for the accumulator that is complete next
+        auto next_full = [&]() -> bool {
+            const bool ok = mbar_wait(acc_full_bar(phase & 1), (phase >> 1) & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            return ok;
+        };
+        // hand it back; both CTAs' warps tell the leader
+        auto release = [&]() {
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(cluster_addr(acc_empty_bar(phase & 1), 0));
+            ++phase;
+        };
+        SeqCursor cursor;
+        for (int32_t tile = cluster; tile < prm.total_tiles; tile += n_clusters) {
+            const FoldSeq& sq = seq_of_tile<RAGGED>(prm, tile, cursor);
+            uint32_t s[128];
+            auto park_all = [&](uint32_t addr) {
+                tmem_ld32<0>(addr + 0, s);
+                tmem_ld32<32>(addr + 32, s);
+                tmem_ld32<64>(addr + 64, s);
+                tmem_ld32<96>(addr + 96, s);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            };
+            // S = Pe U, or a = Pee uu: park this thread's row (128 columns) in registers, hand that half back
+            if (!next_full()) break;
+            park_all(lane_addr + (phase & 1) * 256);
+            release();
+            const int32_t local = tile - sq.tile0, n_keep = sq.n_keep;
+            const int32_t m = (local % sq.m_pairs * 2 + (int32_t)rank) * BM + quarter * 32 + lane;
+            __nv_bfloat16* mat = static_cast<__nv_bfloat16*>(tensor_base(view, tensor)) +
+                                 matrix_offset(view, sq.pair0 + local / sq.m_pairs) + (int64_t)prm.sink * view.stride_token;
+            if (RAGGED ? !sq.quad : FORM == FORM_ONE_LEVEL) {
+                // D = Po V: combine and store rows m and L-1-m
+                if (!next_full()) break;
+                const uint32_t addr = lane_addr + (phase & 1) * 256;
+                const bool row_ok = m < sq.rows_half, mirror_ok = row_ok && n_keep - 1 - m != m;
+                const float sgn = (float)prm.mirror_sign;
+                __nv_bfloat16* out_p = mat + (int64_t)m * view.stride_token;
+                __nv_bfloat16* out_m = mat + (int64_t)(n_keep - 1 - m) * view.stride_token;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    uint32_t d[16];
+                    tmem_ld16(addr + c * 16, d);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (c == 7) release();
+                    uint32_t p[8], q[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float s0 = __uint_as_float(s[c * 16 + 2 * j]), s1 = __uint_as_float(s[c * 16 + 2 * j + 1]);
+                        const float d0 = __uint_as_float(d[2 * j]), d1 = __uint_as_float(d[2 * j + 1]);
+                        p[j] = pack_bf16(s0 + d0, s1 + d1);
+                        q[j] = pack_bf16(sgn * (s0 - d0), sgn * (s1 - d1));
+                    }
+                    if (row_ok) store_row16(out_p + c * 16, p, prm.wide_rows);
+                    if (mirror_ok) store_row16(out_m + c * 16, q, prm.wide_rows);
+                }
+                continue;
+            }
+            // b = Peo uv: s = a + b and s' = a - b go to the work area (bf16: s in the low half of a word)
+            if (!next_full()) break;
+            {
+                const uint32_t addr = lane_addr + (phase & 1) * 256;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    uint32_t b[16];
+                    tmem_ld16(addr + c * 16, b);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if constexpr (WIDE) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const float a0 = __uint_as_float(s[c * 16 + 2 * j]), a1 = __uint_as_float(s[c * 16 + 2 * j + 1]);
+                            const float b0 = __uint_as_float(b[2 * j]), b1 = __uint_as_float(b[2 * j + 1]);
+                            __stcg(reinterpret_cast<float4*>(park) + (c * 8 + j) * 32, make_float4(a0 + b0, a0 - b0, a1 + b1, a1 - b1));
+                        }
+                    } else {
+                        uint32_t w[16];
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            const float av = __uint_as_float(s[c * 16 + j]), bv = __uint_as_float(b[j]);
+                            w[j] = pack_bf16(av + bv, av - bv);
+                        }
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            __stcg(park + (c * 4 + j) * 32, make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]));
+                    }
+                }
+            }
+            release();
+            const int32_t rows_half = sq.rows_half, mh = rows_half - 1 - m;  // mh: the row whose even part is s'
+            const bool row_ok = m < (rows_half + 1) / 2;
+            const bool second_ok = row_ok && mh != m;  // the middle row of an odd L/2 is its own mirror
+            float ct, st;                              // theta'_m = pi (2m+1) / (2L)
+            sincospif((float)(2 * m + 1) / (float)(2 * n_keep), &st, &ct);
+            __nv_bfloat16* rows[4] = {mat + (int64_t)m * view.stride_token, mat + (int64_t)(n_keep - 1 - m) * view.stride_token,
+                                      mat + (int64_t)mh * view.stride_token, mat + (int64_t)(rows_half + m) * view.stride_token};
+            // A = PA p: park it
+            if (!next_full()) break;
+            park_all(lane_addr + (phase & 1) * 256);
+            release();
+            // B = PB q: turn (A, B), combine with (s, s') and store the four rows
+            if (!next_full()) break;
+            const uint32_t addr = lane_addr + (phase & 1) * 256;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                uint32_t b[16];
+                tmem_ld16(addr + c * 16, b);
+                constexpr int WORDS = WIDE ? 32 : 16;  // pairs of 16 columns
+                uint32_t w[WORDS];
+#pragma unroll
+                for (int j = 0; j < WORDS / 4; ++j) {
+                    // volatile: hoisting the loads of every chunk to the front would cost more registers than there are
+                    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(w[4 * j]), "=r"(w[4 * j + 1]), "=r"(w[4 * j + 2]), "=r"(w[4 * j + 3])
+                                 : "l"(park + (c * (WORDS / 4) + j) * 32)
+                                 : "memory");
+                }
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (c == 7) release();
+                uint32_t y[4][8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    float lo[4], hi[4];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float s0 = __uint_as_float(WIDE ? w[(4 * j + 2 * e) % WORDS] : w[2 * j + e] << 16);
+                        const float s1 = __uint_as_float(WIDE ? w[(4 * j + 2 * e + 1) % WORDS] : w[2 * j + e] & 0xffff0000u);
+                        const float A = __uint_as_float(s[c * 16 + 2 * j + e]), B = __uint_as_float(b[2 * j + e]);
+                        const float d0 = fmaf(ct, A, st * B), d1 = fmaf(st, A, -ct * B);
+                        float(&o)[4] = e ? hi : lo;
+                        o[0] = s0 + d0;
+                        o[1] = s0 - d0;
+                        o[2] = s1 + d1;
+                        o[3] = s1 - d1;
+                    }
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) y[r][j] = pack_bf16(lo[r], hi[r]);
+                }
+                if (row_ok) {
+                    store_row16(rows[0] + c * 16, y[0], prm.wide_rows);
+                    store_row16(rows[1] + c * 16, y[1], prm.wide_rows);
+                }
+                if (second_ok) {
+                    store_row16(rows[2] + c * 16, y[2], prm.wide_rows);
+                    store_row16(rows[3] + c * 16, y[3], prm.wide_rows);
+                }
+            }
+        }
+    }
+
+    // Neither CTA may leave (its barriers and tensor memory are used by the other) before both are done.
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync_all();
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));
+    }
+}
+
 template <int MODE>
-__global__ void __launch_bounds__(MODE == MODE_QUAD ? QUAD_THREADS : NUM_THREADS, 1)
+__global__ void __launch_bounds__(NUM_THREADS, 1)
 freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_x,
                    const __grid_constant__ CUtensorMap map_v, const CacheView view, const GemmParams prm)
 {
-    constexpr bool SPECTRUM = MODE == MODE_SPECTRUM;
-    constexpr bool QUAD = MODE == MODE_QUAD;
-    constexpr int PHASES = MODE == MODE_DIRECT ? 1 : QUAD ? 4 : 2;
-    constexpr int USES = QUAD ? 2 : 1;  // times a tile fills each half of tensor memory
+    constexpr int PHASES = MODE == MODE_DIRECT ? 1 : 2;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // 128-byte swizzle atoms need 1024-byte alignment
@@ -596,7 +857,7 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
     const uint32_t rank = cluster_rank();  // 0 = leader of the pair
     const int32_t cluster = blockIdx.x / 2, n_clusters = gridDim.x / 2;
     // tiles of 256 folded rows x 256 columns
-    const int32_t total_tiles = MODE == MODE_RAGGED ? prm.seqs[prm.n_seqs].tile0 : prm.pair_count * prm.m_pairs;
+    const int32_t total_tiles = prm.pair_count * prm.m_pairs;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -621,31 +882,22 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
 
-    constexpr int FIRST_EPI_WARP = QUAD ? 4 : 2;
-    // One setmaxnreg per warpgroup, inside the branch that only this warpgroup takes: where branches meet, ptxas
-    // assumes the fewest registers.
-    if (warp < FIRST_EPI_WARP) {
-        if constexpr (QUAD) set_registers<QUAD_CONTROL_REGS, false>();
+    if (warp < 2) {
         if (warp == 0) {
             // ---------------- TMA producer (both CTAs) ----------------
             if (lane == 0) {
                 uint32_t it = 0;  // global slice counter: stage = it % STAGES, phase = it / STAGES
                 bool alive = true;
-                SeqCursor cursor;
                 for (int32_t tile = cluster; tile < total_tiles && alive; tile += n_clusters) {
-                    const TileCtx tc = tile_ctx<MODE>(prm, tile, &map_p, &map_x, cursor);
-                    const int32_t pair_local = tc.pair_local;
-                    const int32_t m0 = (tc.m_tile * 2 + (int32_t)rank) * BM;
-                    const int32_t pair = tc.pair;  // direct mode: coordinates inside the cache tensor
+                    const int32_t pair_local = tile / prm.m_pairs;
+                    const int32_t m0 = (tile % prm.m_pairs * 2 + (int32_t)rank) * BM;
+                    const int32_t pair = prm.pair0 + pair_local;  // direct mode: coordinates inside the cache tensor
                     const int32_t head = pair % view.kv_heads, layer = (pair / view.kv_heads) % view.layers,
                                   seq = pair / (view.kv_heads * view.layers);
                     for (int eo = 0; eo < PHASES && alive; ++eo) {
-                        // rank 0: K channels, rank 1: V.  Four blocks: phases 0, 1 read uu and uv (both in plane 0, uv
-                        // n_quarter rows down), phases 2, 3 read p (n_quarter rows down in plane 1) and q
-                        const int32_t plane = (pair_local * 2 + (int32_t)rank) * 2 + (QUAD ? eo >> 1 : eo);
-                        const int32_t row0 = (QUAD && (eo == 1 || eo == 2)) ? prm.n_quarter : 0;
-                        const int32_t phase_steps = !QUAD ? tc.k_steps : eo < 3 ? prm.k_steps_short : prm.k_steps_last;
-                        for (int32_t ks = 0; ks < phase_steps; ++ks, ++it) {
+                        // rank 0: K channels, rank 1: V
+                        const int32_t plane = (pair_local * 2 + (int32_t)rank) * 2 + eo;
+                        for (int32_t ks = 0; ks < prm.k_steps; ++ks, ++it) {
                             const int s = it % STAGES;
                             if (it >= STAGES &&
                                 !mbar_wait(empty_bar(s), ((it / STAGES) - 1) & 1, abort_flag, prm.status, ERR_EMPTY_WAIT, prm.wait_limit_ns)) {
@@ -656,14 +908,14 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                             const uint32_t leader_full = cluster_addr(full_bar(s), 0);
                             if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
                             const int32_t k0 = ks * BK;
-                            tma_load_2d(stage, tc.map_p, leader_full, k0, eo * tc.basis_rows_pad + m0);
+                            tma_load_2d(stage, &map_p, leader_full, k0, eo * prm.basis_rows_pad + m0);
                             if constexpr (MODE == MODE_DIRECT) {
                                 const CUtensorMap* cache = rank ? &map_v : &map_x;
                                 tma_load_5d(stage + A_BYTES, cache, leader_full, 0, k0, head, layer, seq);
                                 tma_load_5d(stage + A_BYTES + B_CHUNK_BYTES, cache, leader_full, 64, k0, head, layer, seq);
                             } else {
-                                tma_load_3d(stage + A_BYTES, tc.map_x, leader_full, 0, row0 + k0, plane);
-                                tma_load_3d(stage + A_BYTES + B_CHUNK_BYTES, tc.map_x, leader_full, 64, row0 + k0, plane);
+                                tma_load_3d(stage + A_BYTES, &map_x, leader_full, 0, k0, plane);
+                                tma_load_3d(stage + A_BYTES + B_CHUNK_BYTES, &map_x, leader_full, 64, k0, plane);
                             }
                         }
                     }
@@ -678,13 +930,11 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
             if (lane == 0 && rank == 0) {
                 uint32_t it = 0, tile_no = 0;
                 bool alive = true;
-                SeqCursor cursor;
                 for (int32_t tile = cluster; tile < total_tiles && alive; tile += n_clusters, ++tile_no) {
-                    const int32_t tile_steps = tile_ctx<MODE>(prm, tile, &map_p, &map_x, cursor).k_steps;
                     for (int eo = 0; eo < PHASES && alive; ++eo) {
-                        const int acc = eo & 1;                                   // half of tensor memory
-                        const uint32_t use = tile_no * USES + (uint32_t)(eo >> 1);  // how often that half was filled before
-                        const int32_t k_steps = !QUAD ? tile_steps : eo < 3 ? prm.k_steps_short : prm.k_steps_last;
+                        const int acc = eo;                 // half of tensor memory
+                        const uint32_t use = tile_no;       // how often that half was filled before
+                        const int32_t k_steps = prm.k_steps;
                         if (use > 0) {  // both CTAs' epilogues must have read what this half held last
                             if (!mbar_wait(acc_empty_bar(acc), (use - 1) & 1, abort_flag, prm.status, ERR_ACC_EMPTY_WAIT, prm.wait_limit_ns)) {
                                 alive = false;
@@ -716,13 +966,11 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
             }
         }
     } else {
-        if constexpr (QUAD) set_registers<QUAD_EPILOGUE_REGS, true>();
         // ---------------- epilogue (both CTAs, each on its own 128 rows) ----------------
-        const int ew = warp - FIRST_EPI_WARP, quarter = warp % 4, tensor = ew / 4;  // tensor: 0 = K columns, 1 = V columns
+        const int ew = warp - 2, quarter = warp % 4, tensor = ew / 4;  // tensor: 0 = K columns, 1 = V columns
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + tensor * 128;
         const uint32_t leader_s_empty = cluster_addr(acc_empty_bar(0), 0), leader_d_empty = cluster_addr(acc_empty_bar(1), 0);
         uint32_t tile_no = 0;
-        SeqCursor cursor;
         if constexpr (MODE == MODE_DIRECT) {
             for (int32_t tile = cluster; tile < total_tiles; tile += n_clusters, ++tile_no) {
                 if (!mbar_wait(acc_full_bar(0), tile_no & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) break;
@@ -748,7 +996,7 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(leader_s_empty);
             }
-        } else if constexpr (SPECTRUM) {
+        } else {
             for (int32_t tile = cluster; tile < total_tiles; tile += n_clusters, ++tile_no) {
                 const int32_t pair = prm.pair0 + tile / prm.m_pairs;
                 const int32_t head = pair % view.kv_heads, layer = (pair / view.kv_heads) % view.layers;
@@ -773,169 +1021,12 @@ freqkv_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_const
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(eo ? leader_d_empty : leader_s_empty);
                     const int32_t t = 2 * m + eo;  // S holds the even components, D the odd ones
-                    if (t < prm.n_in && prm.spectrum[tensor])
-                        atomicAdd(prm.spectrum[tensor] + ((int64_t)layer * view.kv_heads + head) * prm.n_in + t,
+                    if (float* out = tensor ? prm.spectrum[1] : prm.spectrum[0]; t < prm.n_in && out)
+                        atomicAdd(out + ((int64_t)layer * view.kv_heads + head) * prm.n_in + t,
                                   sum * prm.spectrum_scale);
                 }
                 if (!alive) break;
             }
-        } else if constexpr (QUAD) {
-            const uint32_t leader_empty[2] = {leader_s_empty, leader_d_empty};
-            auto release = [&](int acc) {
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(leader_empty[acc]);
-            };
-            // this thread's 32 vectors of the work area: vector i of lane l at (i * 32 + l), so that a warp's access is dense
-            uint4* park = prm.park + ((size_t)blockIdx.x * EPI_WARPS + ew) * (32 * 32) + lane;
-            for (int32_t tile = cluster; tile < total_tiles; tile += n_clusters, ++tile_no) {
-                const uint32_t use = 2 * tile_no;
-                // a = Pee uu: park this thread's row (128 columns) in registers
-                if (!mbar_wait(acc_full_bar(0), use & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                uint32_t s[128];
-                tmem_ld32<0>(lane_addr + 0, s);
-                tmem_ld32<32>(lane_addr + 32, s);
-                tmem_ld32<64>(lane_addr + 64, s);
-                tmem_ld32<96>(lane_addr + 96, s);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                release(0);
-                // b = Peo uv: s = a + b (low half of a word) and s' = a - b (high half), both bf16, go to the work area
-                if (!mbar_wait(acc_full_bar(1), use & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    uint32_t b[16];
-                    tmem_ld16(lane_addr + 256 + c * 16, b);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    uint32_t w[16];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float av = __uint_as_float(s[c * 16 + j]), bv = __uint_as_float(b[j]);
-                        w[j] = pack_bf16(av + bv, av - bv);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        __stcg(park + (c * 4 + j) * 32, make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]));
-                }
-                release(1);
-
-                const TileCtx tc = tile_ctx<MODE>(prm, tile, &map_p, &map_x, cursor);
-                const int32_t m = (tc.m_tile * 2 + (int32_t)rank) * BM + quarter * 32 + lane;
-                const int32_t mh = tc.rows_half - 1 - m;  // the row whose even part is s'
-                const bool row_ok = m < prm.rows_quarter;
-                const bool second_ok = row_ok && mh != m;  // the middle row of an odd L/2 is its own mirror
-                float ct, st;                              // theta'_m = pi (2m+1) / (2L)
-                sincospif((float)(2 * m + 1) / (float)(2 * tc.n_keep), &st, &ct);
-                __nv_bfloat16* mat = static_cast<__nv_bfloat16*>(tensor_base(view, tensor)) +
-                                     matrix_offset(view, tc.pair) + (int64_t)prm.sink * view.stride_token;
-                __nv_bfloat16* rows[4] = {mat + (int64_t)m * view.stride_token, mat + (int64_t)(tc.n_keep - 1 - m) * view.stride_token,
-                                          mat + (int64_t)mh * view.stride_token, mat + (int64_t)(tc.rows_half + m) * view.stride_token};
-                // A = PA p: park it
-                if (!mbar_wait(acc_full_bar(0), (use + 1) & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                tmem_ld32<0>(lane_addr + 0, s);
-                tmem_ld32<32>(lane_addr + 32, s);
-                tmem_ld32<64>(lane_addr + 64, s);
-                tmem_ld32<96>(lane_addr + 96, s);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                release(0);
-                // B = PB q: turn (A, B), combine with (s, s') and store the four rows
-                if (!mbar_wait(acc_full_bar(1), (use + 1) & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    uint32_t b[16];
-                    tmem_ld16(lane_addr + 256 + c * 16, b);
-                    uint32_t w[16];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        // volatile: hoisting the loads of every chunk to the front would cost more registers than there are
-                        asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
-                                     : "=r"(w[4 * j]), "=r"(w[4 * j + 1]), "=r"(w[4 * j + 2]), "=r"(w[4 * j + 3])
-                                     : "l"(park + (c * 4 + j) * 32)
-                                     : "memory");
-                    }
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (c == 7) release(1);
-                    uint32_t y[4][8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        float lo[4], hi[4];
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const uint32_t word = w[2 * j + e];
-                            const float s0 = __uint_as_float(word << 16), s1 = __uint_as_float(word & 0xffff0000u);
-                            const float A = __uint_as_float(s[c * 16 + 2 * j + e]), B = __uint_as_float(b[2 * j + e]);
-                            const float d0 = fmaf(ct, A, st * B), d1 = fmaf(st, A, -ct * B);
-                            float(&o)[4] = e ? hi : lo;
-                            o[0] = s0 + d0; o[1] = s0 - d0; o[2] = s1 + d1; o[3] = s1 - d1;
-                        }
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) y[r][j] = pack_bf16(lo[r], hi[r]);
-                    }
-                    if (row_ok) {
-                        store_row16(rows[0] + c * 16, y[0], prm.wide_rows);
-                        store_row16(rows[1] + c * 16, y[1], prm.wide_rows);
-                    }
-                    if (second_ok) {
-                        store_row16(rows[2] + c * 16, y[2], prm.wide_rows);
-                        store_row16(rows[3] + c * 16, y[3], prm.wide_rows);
-                    }
-                }
-            }
-        } else
-        for (int32_t tile = cluster; tile < total_tiles; tile += n_clusters, ++tile_no) {
-            // S = Pe U: park this thread's row (128 columns) in registers, release that half
-            if (!mbar_wait(acc_full_bar(0), tile_no & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            uint32_t s[128];
-            tmem_ld32<0>(lane_addr + 0, s);
-            tmem_ld32<32>(lane_addr + 32, s);
-            tmem_ld32<64>(lane_addr + 64, s);
-            tmem_ld32<96>(lane_addr + 96, s);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(leader_s_empty);
-
-            // D = Po V: combine and store rows m and L-1-m
-            if (!mbar_wait(acc_full_bar(1), tile_no & 1, abort_flag, prm.status, ERR_ACC_FULL_WAIT, prm.wait_limit_ns)) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const TileCtx tc = tile_ctx<MODE>(prm, tile, &map_p, &map_x, cursor);
-            const int32_t m = (tc.m_tile * 2 + (int32_t)rank) * BM + quarter * 32 + lane;
-            const int32_t mr = tc.n_keep - 1 - m;
-            const bool row_ok = m < tc.rows_half;
-            const float sgn = (float)prm.mirror_sign;
-            __nv_bfloat16* mat = static_cast<__nv_bfloat16*>(tensor_base(view, tensor)) +
-                                 matrix_offset(view, tc.pair) + (int64_t)prm.sink * view.stride_token;
-            uint4* out_p = reinterpret_cast<uint4*>(mat + (int64_t)m * view.stride_token);
-            uint4* out_m = reinterpret_cast<uint4*>(mat + (int64_t)mr * view.stride_token);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                uint32_t d[16];
-                tmem_ld16(lane_addr + 256 + c * 16, d);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (row_ok) {
-                    uint32_t p[8], q[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float s0 = __uint_as_float(s[c * 16 + 2 * j]), s1 = __uint_as_float(s[c * 16 + 2 * j + 1]);
-                        const float d0 = __uint_as_float(d[2 * j]), d1 = __uint_as_float(d[2 * j + 1]);
-                        p[j] = pack_bf16(s0 + d0, s1 + d1);
-                        q[j] = pack_bf16(sgn * (s0 - d0), sgn * (s1 - d1));
-                    }
-                    out_p[2 * c] = make_uint4(p[0], p[1], p[2], p[3]);
-                    out_p[2 * c + 1] = make_uint4(p[4], p[5], p[6], p[7]);
-                    if (mr != m) {
-                        out_m[2 * c] = make_uint4(q[0], q[1], q[2], q[3]);
-                        out_m[2 * c + 1] = make_uint4(q[4], q[5], q[6], q[7]);
-                    }
-                }
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(leader_d_empty);
         }
     }
 
@@ -1035,6 +1126,44 @@ bool gemm_supported(int32_t dtype, int32_t head_dim, int32_t n_in, int32_t n_kee
     return dtype == FREQKV_BF16 && head_dim == 128 && n_in >= 1 && n_keep >= 1 && n_keep <= n_in;
 }
 
+// A device buffer of at least `bytes`; earlier launches may still use the one it replaces.
+static cudaError_t grow(void** buffer, size_t* have, size_t bytes)
+{
+    if (bytes <= *have) return cudaSuccess;
+    if (*buffer) {
+        const cudaError_t e = cudaDeviceSynchronize();
+        if (e != cudaSuccess) return e;
+        cudaFree(*buffer);
+        *buffer = nullptr;
+        *have = 0;
+    }
+    const cudaError_t e = cudaMalloc(buffer, bytes);
+    if (e == cudaSuccess)
+        *have = bytes;
+    else
+        *buffer = nullptr;
+    return e;
+}
+
+// A launch of CTA pairs.
+struct PairLaunch {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    PairLaunch(int ctas, int threads, int smem, cudaStream_t stream)
+    {
+        cfg.gridDim = dim3((unsigned)ctas);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = (size_t)smem;
+        cfg.stream = stream;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+};
+
 // Everything a launch needs that is not a stream operation: kernel attributes, the count of
 // resident CTA pairs, the scratch buffer for `pairs` (batch, layer, kv_head) triples of this basis
 // (pairs = 0: none, the direct mode reads the cache itself).
@@ -1047,40 +1176,28 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
         return cudaErrorNotSupported;
     }
     if (!state->attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(freqkv_gemm_kernel<MODE_FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(freqkv_gemm_kernel<MODE_SPECTRUM>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(freqkv_gemm_kernel<MODE_DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(freqkv_gemm_kernel<MODE_RAGGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(freqkv_gemm_kernel<MODE_QUAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e != cudaSuccess) {
-            state->last_error = "cudaFuncSetAttribute(max dynamic shared memory)";
-            return e;
+        const void* kernels[6] = {(const void*)freqkv_gemm_kernel<MODE_SPECTRUM>, (const void*)freqkv_gemm_kernel<MODE_DIRECT>,
+                                  (const void*)freqkv_fold_gemm_kernel<FORM_ONE_LEVEL>, (const void*)freqkv_fold_gemm_kernel<FORM_FOUR_BLOCKS>,
+                                  (const void*)freqkv_fold_gemm_kernel<FORM_FOUR_BLOCKS_WIDE>, (const void*)freqkv_fold_gemm_kernel<FORM_RAGGED>};
+        for (int i = 0; i < 6; ++i) {
+            const cudaError_t e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+            if (e != cudaSuccess) {
+                state->last_error = "cudaFuncSetAttribute(max dynamic shared memory)";
+                return e;
+            }
+        }
+        for (int i = 2; i < 6; ++i) {  // the register shares are of what the block is launched with
+            cudaFuncAttributes fa;
+            const cudaError_t e = cudaFuncGetAttributes(&fa, kernels[i]);
+            if (e != cudaSuccess || fa.numRegs < FOLD_LAUNCH_REGS) {
+                state->last_error = "the kernel of the folded forms was not built with the registers it shares out";
+                return e != cudaSuccess ? e : cudaErrorLaunchOutOfResources;
+            }
         }
         // how many CTA pairs the device can hold at once (one CTA per SM; SMs pair up inside a GPC)
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(2 * (sm_count / 2)));
-        cfg.blockDim = dim3(NUM_THREADS);
-        cfg.dynamicSmemBytes = SMEM_BYTES;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        // the register shares of MODE_QUAD are of what its block is launched with
-        cudaFuncAttributes fa;
-        const cudaError_t ae = cudaFuncGetAttributes(&fa, freqkv_gemm_kernel<MODE_QUAD>);
-        if (ae != cudaSuccess || fa.numRegs < QUAD_LAUNCH_REGS) {
-            state->last_error = "the four-block kernel was not built with the registers it shares out";
-            return ae != cudaSuccess ? ae : cudaErrorLaunchOutOfResources;
-        }
+        PairLaunch launch(2 * (sm_count / 2), FOLD_THREADS, SMEM_BYTES, nullptr);
         int n = 0;
-        const cudaError_t q = cudaOccupancyMaxActiveClusters(&n, freqkv_gemm_kernel<MODE_FOLD>, &cfg);
+        const cudaError_t q = cudaOccupancyMaxActiveClusters(&n, freqkv_fold_gemm_kernel<FORM_ONE_LEVEL>, &launch.cfg);
         if (q != cudaSuccess || n < 1) {
             state->last_error = "cudaOccupancyMaxActiveClusters: no CTA pair fits on this device";
             return q != cudaSuccess ? q : cudaErrorLaunchOutOfResources;
@@ -1099,42 +1216,138 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
     const int32_t n_half = (basis.n_in + 1) / 2;
     const size_t per_pair = (size_t)4 * n_half * 128 * 2;  // K and V, U and V planes
     const int64_t fit = std::max<int64_t>(1, (int64_t)(kFoldBufferBytes / per_pair));
-    const size_t need = (size_t)std::min<int64_t>(fit, pairs) * per_pair;
-    if (need > state->scratch_bytes) {
-        if (state->scratch) {
-            cudaError_t e = cudaDeviceSynchronize();
-            if (e != cudaSuccess) return e;
-            cudaFree(state->scratch);
-            state->scratch = nullptr;
-            state->scratch_bytes = 0;
-        }
-        const cudaError_t e = cudaMalloc(&state->scratch, need);
-        if (e != cudaSuccess) {
-            state->last_error = "cudaMalloc(fold scratch)";
-            return e;
-        }
-        state->scratch_bytes = need;
+    const int64_t pass = std::min<int64_t>(fit, pairs);
+    const cudaError_t e = grow(&state->scratch, &state->scratch_bytes, (size_t)pass * per_pair);
+    if (e != cudaSuccess) state->last_error = "cudaMalloc(fold scratch)";
+    return e;
+}
+
+// The shapes of one sequence: everything but its place in the launch.
+static FoldSeq fold_seq(const Basis& b, int32_t pair0)
+{
+    FoldSeq s = {};
+    s.pair0 = pair0;
+    s.n_half = (b.n_in + 1) / 2;
+    s.n_keep = b.n_keep;
+    s.rows_half = (b.n_keep + 1) / 2;
+    s.quad = b.quad != nullptr;
+    s.basis_rows_pad = s.quad ? b.quad_rows_pad : b.fold_rows_pad;
+    s.k_steps = s.quad ? quad_steps(b.n_in) : (s.n_half + BK - 1) / BK;
+    s.k_last = s.quad ? quad_last_steps(b.n_in, b.n_keep) : 0;
+    const int32_t rows = s.quad ? (s.rows_half + 1) / 2 : s.rows_half;
+    s.m_pairs = (rows + 2 * BM - 1) / (2 * BM);
+    return s;
+}
+
+static FoldParams fold_params(const GemmState* state, const CacheView& view, int32_t sink, int32_t* status_dev)
+{
+    FoldParams prm = {};
+    prm.sink = sink;
+    prm.mirror_sign = 1;
+    prm.wide_rows = (((uintptr_t)view.base[0] | (uintptr_t)view.base[1]) & 31) == 0 &&
+                    ((view.stride_token | view.stride_head | view.stride_layer | view.stride_batch) & 15) == 0;
+    prm.park = static_cast<uint4*>(state->park);
+    prm.status = status_dev;
+    prm.wait_limit_ns = state->wait_limit_ns;
+    return prm;
+}
+
+static FoldJob fold_job(const Basis& b, const FoldSeq& s, int32_t pairs, int32_t sink, void* planes)
+{
+    FoldJob job;
+    job.pair0 = s.pair0;
+    job.pair_count = pairs;
+    job.n_in = b.n_in;
+    job.n_half = s.n_half;
+    job.sink = sink;
+    job.dst = static_cast<uint4*>(planes);
+    job.turns = s.quad ? b.turns : nullptr;
+    return job;
+}
+
+// Blocks per matrix of a fold launch: each takes rounds of 1024 vectors of one level, or 512 of the four blocks.
+static unsigned fold_blocks(int32_t n_half) { return (unsigned)std::min<int64_t>(((int64_t)n_half * 16 + 1023) / 1024, 64); }
+
+// The product, after its fold launch.
+template <int FORM>
+static cudaError_t launch_product(GemmState* state, const CUtensorMap& map_p, const CUtensorMap& map_x, const CacheView& view,
+                                  const FoldParams& prm, const LaunchHooks& hooks, cudaStream_t stream)
+{
+    PairLaunch launch(2 * std::min<int32_t>(prm.total_tiles, state->max_clusters), FOLD_THREADS, SMEM_BYTES, stream);
+    if (hooks.before) hooks.before(hooks.user, stream);
+    const cudaError_t e = cudaLaunchKernelEx(&launch.cfg, freqkv_fold_gemm_kernel<FORM>, map_p, map_x, view, prm);
+    if (hooks.after) hooks.after(hooks.user, stream);
+    if (e != cudaSuccess) {
+        state->last_error = "freqkv_fold_gemm_kernel launch";
+        return e;
     }
+    state->kernels_last_call += 2;
     return cudaSuccess;
 }
 
 cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink, int32_t* status_dev,
-                        int sm_count, const LaunchHooks& hooks, cudaStream_t stream, const SpectrumOut* spectrum)
+                        int sm_count, const LaunchHooks& hooks, cudaStream_t stream)
+{
+    state->kernels_last_call = 0;
+    const cudaError_t prepared = gemm_prepare(state, view.mats_per_tensor, basis, sm_count);
+    if (prepared != cudaSuccess) return prepared;
+    const int32_t pairs = view.mats_per_tensor;
+    FoldSeq seq = fold_seq(basis, 0);
+    const size_t per_pair = (size_t)4 * seq.n_half * 128 * 2;
+    // One pass when the folded inputs fit the scratch buffer, else several passes of `chunk` pairs.
+    const int64_t chunk = std::min<int64_t>(std::max<int64_t>(1, (int64_t)(kFoldBufferBytes / per_pair)), pairs);
+    CUtensorMap map_p;
+    if (!(seq.quad ? encode_quad_map(&map_p, basis) : encode_basis_map(&map_p, basis))) {
+        state->last_error = "tensor map encoding rejected the basis";
+        return cudaErrorInvalidValue;
+    }
+    FoldParams prm = fold_params(state, view, sink, status_dev);
+    prm.mirror_sign = (basis.first & 1) ? -1 : 1;
+    for (int64_t p0 = 0; p0 < pairs; p0 += chunk) {
+        const int32_t count = (int32_t)std::min<int64_t>(chunk, pairs - p0);
+        CUtensorMap map_x;
+        if (!encode_scratch_map(&map_x, state->scratch, seq.n_half, count * 4)) {
+            state->last_error = "tensor map encoding rejected the scratch planes";
+            return cudaErrorInvalidValue;
+        }
+        seq.pair0 = (int32_t)p0;
+        prm.seq = seq;
+        if ((int64_t)count * seq.m_pairs > 0x7fffffff) return cudaErrorInvalidValue;
+        prm.total_tiles = count * seq.m_pairs;
+        const FoldJob job = fold_job(basis, seq, count, sink, state->scratch);
+        const dim3 grid((unsigned)count * 2, fold_blocks(seq.n_half));
+        if (seq.quad)
+            fold_quad_kernel<<<grid, 256, 0, stream>>>(view, job, job.turns);
+        else
+            fold_kernel<<<grid, 256, 0, stream>>>(view, job);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) {
+            state->last_error = "fold_kernel launch";
+            return e;
+        }
+        // lengths that two levels of the mirror symmetry used to serve kept (s, s') in bf16 there, too
+        const bool wide = seq.quad && gemm_fold_levels(basis.n_in, basis.n_keep, basis.first) != 2;
+        e = wide       ? launch_product<FORM_FOUR_BLOCKS_WIDE>(state, map_p, map_x, view, prm, hooks, stream)
+            : seq.quad ? launch_product<FORM_FOUR_BLOCKS>(state, map_p, map_x, view, prm, hooks, stream)
+                       : launch_product<FORM_ONE_LEVEL>(state, map_p, map_x, view, prm, hooks, stream);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// The power spectrum: a fold pass and a pass of the spectrum kernel (two launches per scratch buffer full of planes).
+cudaError_t launch_gemm_spectrum(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink, int32_t* status_dev,
+                                 int sm_count, const LaunchHooks& hooks, cudaStream_t stream, const SpectrumOut& spectrum)
 {
     state->kernels_last_call = 0;
     const cudaError_t prepared = gemm_prepare(state, view.mats_per_tensor, basis, sm_count);
     if (prepared != cudaSuccess) return prepared;
     const int32_t n_half = (basis.n_in + 1) / 2, rows_half = (basis.n_keep + 1) / 2;
-    // the four-block form where the basis has it (gemm_quad; not the spectrum's basis)
-    const int32_t rows_quarter = (rows_half + 1) / 2;
-    const bool quad = basis.quad != nullptr && !spectrum;
-    const int32_t m_pairs = ((quad ? rows_quarter : rows_half) + 2 * BM - 1) / (2 * BM);  // tiles of 256 folded rows
     const int32_t pairs = view.mats_per_tensor;
     const size_t per_pair = (size_t)4 * n_half * 128 * 2;
-    // One pass when the folded inputs fit the scratch buffer, else several passes of `chunk` pairs.
     const int64_t chunk = std::min<int64_t>(std::max<int64_t>(1, (int64_t)(kFoldBufferBytes / per_pair)), pairs);
     CUtensorMap map_p;
-    if (!(quad ? encode_quad_map(&map_p, basis) : encode_basis_map(&map_p, basis))) {
+    if (!encode_basis_map(&map_p, basis)) {
         state->last_error = "tensor map encoding rejected the basis";
         return cudaErrorInvalidValue;
     }
@@ -1146,13 +1359,8 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
         job.n_half = n_half;
         job.sink = sink;
         job.dst = static_cast<uint4*>(state->scratch);
-        if (quad) {
-            const unsigned fold_y = (unsigned)std::min<int64_t>(((int64_t)(n_half / 2) * 16 + 511) / 512, 64);
-            fold_quad_kernel<<<dim3((unsigned)job.pair_count * 2, fold_y), 256, 0, stream>>>(view, job, basis.turns);
-        } else {
-            const unsigned fold_y = (unsigned)std::min<int64_t>(((int64_t)n_half * 16 + 1023) / 1024, 64);
-            fold_kernel<<<dim3((unsigned)job.pair_count * 2, fold_y), 256, 0, stream>>>(view, job);
-        }
+        job.turns = nullptr;
+        fold_kernel<<<dim3((unsigned)job.pair_count * 2, fold_blocks(n_half)), 256, 0, stream>>>(view, job);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) {
             state->last_error = "fold_kernel launch";
@@ -1163,50 +1371,23 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
             state->last_error = "tensor map encoding rejected the scratch planes";
             return cudaErrorInvalidValue;
         }
-        GemmParams prm;
+        GemmParams prm = {};
         prm.n_keep = basis.n_keep;
-        prm.rows_half = rows_half;
-        prm.basis_rows_pad = quad ? basis.quad_rows_pad : basis.fold_rows_pad;
-        prm.rows_quarter = rows_quarter;
-        prm.n_quarter = n_half / 2;
-        prm.k_steps_short = quad_steps(basis.n_in);
-        prm.k_steps_last = quad_last_steps(basis.n_in, basis.n_keep);
-        prm.park = static_cast<uint4*>(state->park);
-        prm.wide_rows = (((uintptr_t)view.base[0] | (uintptr_t)view.base[1]) & 31) == 0 &&
-                        ((view.stride_token | view.stride_head | view.stride_layer | view.stride_batch) & 15) == 0;
+        prm.basis_rows_pad = basis.fold_rows_pad;
         prm.pair0 = job.pair0;
         prm.pair_count = job.pair_count;
-        prm.m_pairs = m_pairs;
+        prm.m_pairs = (rows_half + 2 * BM - 1) / (2 * BM);
         prm.k_steps = (n_half + BK - 1) / BK;
         prm.sink = sink;
-        prm.mirror_sign = (basis.first & 1) ? -1 : 1;
-        prm.spectrum[0] = spectrum ? spectrum->k : nullptr;
-        prm.spectrum[1] = spectrum ? spectrum->v : nullptr;
-        prm.spectrum_scale = spectrum ? spectrum->scale : 0.f;
+        prm.spectrum[0] = spectrum.k;
+        prm.spectrum[1] = spectrum.v;
+        prm.spectrum_scale = spectrum.scale;
         prm.n_in = basis.n_in;
         prm.status = status_dev;
         prm.wait_limit_ns = state->wait_limit_ns;
-        prm.seqs = nullptr;
-        prm.seq_maps = nullptr;
-        prm.n_seqs = 0;
-        const int32_t tiles = job.pair_count * m_pairs;
-        const int clusters = std::min<int32_t>(tiles, state->max_clusters);
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(2 * clusters));
-        cfg.blockDim = dim3(quad ? QUAD_THREADS : NUM_THREADS);
-        cfg.dynamicSmemBytes = SMEM_BYTES;
-        cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        PairLaunch launch(2 * std::min<int32_t>(job.pair_count * prm.m_pairs, state->max_clusters), NUM_THREADS, SMEM_BYTES, stream);
         if (hooks.before) hooks.before(hooks.user, stream);
-        e = spectrum ? cudaLaunchKernelEx(&cfg, freqkv_gemm_kernel<MODE_SPECTRUM>, map_p, map_x, map_x, view, prm)
-            : quad   ? cudaLaunchKernelEx(&cfg, freqkv_gemm_kernel<MODE_QUAD>, map_p, map_x, map_x, view, prm)
-                     : cudaLaunchKernelEx(&cfg, freqkv_gemm_kernel<MODE_FOLD>, map_p, map_x, map_x, view, prm);
+        e = cudaLaunchKernelEx(&launch.cfg, freqkv_gemm_kernel<MODE_SPECTRUM>, map_p, map_x, map_x, view, prm);
         if (hooks.after) hooks.after(hooks.user, stream);
         if (e != cudaSuccess) {
             state->last_error = "freqkv_gemm_kernel launch";
@@ -1217,144 +1398,80 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
     return cudaSuccess;
 }
 
-// A ragged batch in two launches: one fold pass and one tensor-core pass over every sequence,
-// longest first.  Everything that can fail for lack of memory happens before the first launch.
+// A ragged batch in two launches: one fold pass and one tensor-core pass over every sequence, longest first.
+// Everything that can fail for lack of memory happens before the first launch.
 cudaError_t launch_gemm_ragged(GemmState* state, const CacheView& view, const std::vector<RaggedItem>& items_in, int32_t sink,
                                int32_t* status_dev, int sm_count, const LaunchHooks& hooks, cudaStream_t stream)
 {
     state->kernels_last_call = 0;
     if (items_in.empty()) return cudaSuccess;
-    const cudaError_t prepared = gemm_prepare(state, 0, items_in[0].basis, sm_count);
-    if (prepared != cudaSuccess) return prepared;
     const int32_t lh = view.layers * view.kv_heads;  // (layer, kv_head) pairs per sequence
     std::vector<RaggedItem> items = items_in;
     auto work = [](const RaggedItem& it) { return (int64_t)it.basis.n_in * it.basis.n_keep; };
     std::stable_sort(items.begin(), items.end(), [&](const RaggedItem& a, const RaggedItem& b) { return work(a) > work(b); });
     const size_t n = items.size();
-    // scratch: the folded planes of every sequence, back to back
+    for (const RaggedItem& it : items) {
+        const cudaError_t prepared = gemm_prepare(state, 0, it.basis, sm_count);
+        if (prepared != cudaSuccess) return prepared;
+    }
+    // the table's entries; scratch: the folded planes of every sequence, back to back
+    std::vector<FoldSeq> seqs(n + 1);
     std::vector<size_t> offset(n);
-    size_t total = 0;
+    size_t scratch = 0;
+    int64_t tiles = 0;
     int32_t max_half = 0;
     for (size_t i = 0; i < n; ++i) {
-        const int32_t n_half = (items[i].basis.n_in + 1) / 2;
-        offset[i] = total;
-        total += (size_t)lh * 4 * n_half * 256;
-        max_half = std::max(max_half, n_half);
+        FoldSeq& s = seqs[i] = fold_seq(items[i].basis, items[i].batch_index * lh);
+        s.tile0 = (int32_t)tiles;
+        tiles += (int64_t)lh * s.m_pairs;
+        max_half = std::max(max_half, s.n_half);
+        if (tiles > 0x7fffffff || (int64_t)n * 2 * lh > 0x7fffffff) return cudaErrorInvalidValue;
+        offset[i] = scratch;
+        scratch += (size_t)lh * 4 * s.n_half * 256;
     }
-    if (total > kRaggedScratchLimit) {
+    seqs[n].tile0 = (int32_t)tiles;
+    if (scratch > kRaggedScratchLimit) {
         state->last_error = "folded inputs of the ragged batch exceed the scratch limit";
         return cudaErrorMemoryAllocation;
     }
-    if (total > state->scratch_bytes) {
-        if (state->scratch) {
-            const cudaError_t e = cudaDeviceSynchronize();
-            if (e != cudaSuccess) return e;
-            cudaFree(state->scratch);
-            state->scratch = nullptr;
-            state->scratch_bytes = 0;
-        }
-        const cudaError_t e = cudaMalloc(&state->scratch, total);
-        if (e != cudaSuccess) {
-            state->last_error = "cudaMalloc(fold scratch of a ragged batch)";
-            return e;
-        }
-        state->scratch_bytes = total;
-    }
-    // tables: two tensor maps, one shape record and one fold job per sequence
-    const size_t maps_bytes = n * 2 * sizeof(CUtensorMap), seqs_bytes = (n + 1) * sizeof(RaggedSeq), jobs_bytes = n * sizeof(FoldJob);
-    const size_t meta_bytes = maps_bytes + seqs_bytes + jobs_bytes;
-    if (meta_bytes > state->ragged_meta_bytes) {
-        if (state->ragged_meta) {
-            const cudaError_t e = cudaDeviceSynchronize();
-            if (e != cudaSuccess) return e;
-            cudaFree(state->ragged_meta);
-            state->ragged_meta = nullptr;
-            state->ragged_meta_bytes = 0;
-        }
-        const cudaError_t e = cudaMalloc(&state->ragged_meta, meta_bytes);
-        if (e != cudaSuccess) {
-            state->last_error = "cudaMalloc(tables of a ragged batch)";
-            return e;
-        }
-        state->ragged_meta_bytes = meta_bytes;
+    const size_t maps_bytes = n * 2 * sizeof(CUtensorMap), seqs_bytes = ((n + 1) * sizeof(FoldSeq) + 15) / 16 * 16,
+                 jobs_bytes = n * sizeof(FoldJob);
+    cudaError_t e = grow(&state->scratch, &state->scratch_bytes, scratch);
+    if (e == cudaSuccess) e = grow(&state->ragged_meta, &state->ragged_meta_bytes, maps_bytes + seqs_bytes + jobs_bytes);
+    if (e != cudaSuccess) {
+        state->last_error = "cudaMalloc(scratch and tables of a ragged batch)";
+        return e;
     }
     std::vector<CUtensorMap> maps(2 * n);
-    std::vector<RaggedSeq> seqs(n + 1);
     std::vector<FoldJob> jobs(n);
-    int64_t tiles = 0;
     for (size_t i = 0; i < n; ++i) {
-        const Basis& b = items[i].basis;
-        const int32_t n_half = (b.n_in + 1) / 2, rows_half = (b.n_keep + 1) / 2;
         char* planes = static_cast<char*>(state->scratch) + offset[i];
-        if (!encode_basis_map(&maps[2 * i], b) || !encode_scratch_map(&maps[2 * i + 1], planes, n_half, lh * 4)) {
+        const Basis& b = items[i].basis;
+        jobs[i] = fold_job(b, seqs[i], lh, sink, planes);
+        if (!(seqs[i].quad ? encode_quad_map(&maps[2 * i], b) : encode_basis_map(&maps[2 * i], b)) ||
+            !encode_scratch_map(&maps[2 * i + 1], planes, seqs[i].n_half, lh * 4)) {
             state->last_error = "tensor map encoding rejected a sequence of the ragged batch";
             return cudaErrorInvalidValue;
         }
-        RaggedSeq& s = seqs[i];
-        s.tile0 = (int32_t)tiles;
-        s.pair0 = items[i].batch_index * lh;
-        s.n_keep = b.n_keep;
-        s.rows_half = rows_half;
-        s.basis_rows_pad = b.fold_rows_pad;
-        s.k_steps = (n_half + BK - 1) / BK;
-        s.m_pairs = (rows_half + 2 * BM - 1) / (2 * BM);
-        s.pad = 0;
-        tiles += (int64_t)lh * s.m_pairs;
-        FoldJob& j = jobs[i];
-        j.pair0 = s.pair0;
-        j.pair_count = lh;
-        j.n_in = b.n_in;
-        j.n_half = n_half;
-        j.sink = sink;
-        j.dst = reinterpret_cast<uint4*>(planes);
     }
-    if (tiles > 0x7fffffff || (int64_t)n * 2 * lh > 0x7fffffff) return cudaErrorInvalidValue;
-    seqs[n] = RaggedSeq{(int32_t)tiles, 0, 0, 0, 0, 0, 1, 0};
     char* meta = static_cast<char*>(state->ragged_meta);
     // pageable sources: each copy has left its host buffer when the call returns
-    cudaError_t e = cudaMemcpyAsync(meta, maps.data(), maps_bytes, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(meta + maps_bytes, seqs.data(), seqs_bytes, cudaMemcpyHostToDevice, stream);
+    e = cudaMemcpyAsync(meta, maps.data(), maps_bytes, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(meta + maps_bytes, seqs.data(), (n + 1) * sizeof(FoldSeq), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(meta + maps_bytes + seqs_bytes, jobs.data(), jobs_bytes, cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess) return e;
-
-    const unsigned fold_y = (unsigned)std::min<int64_t>(((int64_t)max_half * 16 + 1023) / 1024, 64);
-    fold_ragged_kernel<<<dim3((unsigned)(n * 2 * lh), fold_y), 256, 0, stream>>>(
+    fold_ragged_kernel<<<dim3((unsigned)(n * 2 * lh), fold_blocks(max_half)), 256, 0, stream>>>(
         view, reinterpret_cast<const FoldJob*>(meta + maps_bytes + seqs_bytes), 2 * lh);
     e = cudaGetLastError();
     if (e != cudaSuccess) {
         state->last_error = "fold_ragged_kernel launch";
         return e;
     }
-    GemmParams prm = {};
-    prm.sink = sink;
-    prm.mirror_sign = 1;
-    prm.status = status_dev;
-    prm.wait_limit_ns = state->wait_limit_ns;
+    FoldParams prm = fold_params(state, view, sink, status_dev);
+    prm.total_tiles = (int32_t)tiles;
     prm.seq_maps = reinterpret_cast<const CUtensorMap*>(meta);
-    prm.seqs = reinterpret_cast<const RaggedSeq*>(meta + maps_bytes);
-    prm.n_seqs = (int32_t)n;
-    const int clusters = (int)std::min<int64_t>(tiles, state->max_clusters);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * clusters));
-    cfg.blockDim = dim3(NUM_THREADS);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (hooks.before) hooks.before(hooks.user, stream);
-    e = cudaLaunchKernelEx(&cfg, freqkv_gemm_kernel<MODE_RAGGED>, maps[0], maps[1], maps[1], view, prm);
-    if (hooks.after) hooks.after(hooks.user, stream);
-    if (e != cudaSuccess) {
-        state->last_error = "freqkv_gemm_kernel launch";
-        return e;
-    }
-    state->kernels_last_call = 2;
-    return cudaSuccess;
+    prm.seqs = reinterpret_cast<const FoldSeq*>(meta + maps_bytes);
+    return launch_product<FORM_RAGGED>(state, maps[0], maps[1], view, prm, hooks, stream);
 }
 
 // The non-sink rows of one cache tensor as a 5-D tensor (channel, token, kv_head, layer, batch).
@@ -1434,32 +1551,18 @@ cudaError_t launch_gemm_direct(GemmState* state, const CacheView& view, const Ba
     }
     GemmParams prm = {};
     prm.n_keep = basis.n_keep;
-    prm.rows_half = basis.n_keep;
     prm.basis_rows_pad = 0;
     prm.pair0 = 0;
     prm.pair_count = pairs;
     prm.m_pairs = 1;
     prm.k_steps = (basis.n_in + BK - 1) / BK;
     prm.sink = sink;
-    prm.mirror_sign = 1;
     prm.n_in = basis.n_in;
     prm.status = status_dev;
     prm.wait_limit_ns = state->wait_limit_ns;
-    const int clusters = std::min<int32_t>(pairs, state->max_clusters);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * clusters));
-    cfg.blockDim = dim3(NUM_THREADS);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    PairLaunch launch(2 * std::min<int32_t>(pairs, state->max_clusters), NUM_THREADS, SMEM_BYTES, stream);
     if (hooks.before) hooks.before(hooks.user, stream);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, freqkv_gemm_kernel<MODE_DIRECT>, map_p, map_k, map_v, view, prm);
+    const cudaError_t e = cudaLaunchKernelEx(&launch.cfg, freqkv_gemm_kernel<MODE_DIRECT>, map_p, map_k, map_v, view, prm);
     if (hooks.after) hooks.after(hooks.user, stream);
     if (e != cudaSuccess) {
         state->last_error = "freqkv_gemm_kernel launch";

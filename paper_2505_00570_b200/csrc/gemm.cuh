@@ -13,7 +13,7 @@ struct GemmState {
     int max_clusters = 0;     // CTA pairs that can be resident at once
     void* scratch = nullptr;  // folded inputs U, V: [pairs][K|V][U|V][ceil(n_in/2)][128] bf16 per pass
     size_t scratch_bytes = 0;
-    void* park = nullptr;     // four-block form: (s, s') of the tile each CTA works on (19 MB on 74 CTA pairs)
+    void* park = nullptr;     // four-block form: (s, s') of the tile each CTA works on (38 MB on 74 CTA pairs)
     void* ragged_meta = nullptr;  // tensor maps, shapes and fold jobs of a ragged batch (device)
     size_t ragged_meta_bytes = 0;
     unsigned long long wait_limit_ns = 2000000000ull;  // bound of every mbarrier wait inside the kernel (2 s)
@@ -37,7 +37,10 @@ struct SpectrumOut {
 
 bool gemm_supported(int32_t dtype, int32_t head_dim, int32_t n_in, int32_t n_keep);
 cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink, int32_t* status_dev,
-                        int sm_count, const LaunchHooks& hooks, cudaStream_t stream, const SpectrumOut* spectrum = nullptr);
+                        int sm_count, const LaunchHooks& hooks, cudaStream_t stream);
+// The power spectrum of the rows (basis: the plain DCT's, folded).
+cudaError_t launch_gemm_spectrum(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink, int32_t* status_dev,
+                                 int sm_count, const LaunchHooks& hooks, cudaStream_t stream, const SpectrumOut& spectrum);
 cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, int sm_count);
 // At most 256 kept rows: one tile per (batch, layer, kv_head), no fold pass, the dense basis (Basis::dense).
 bool gemm_is_direct(int32_t n_keep);
