@@ -74,15 +74,17 @@ constexpr size_t kBasisBudgetBytes = size_t(12) << 30;  // plan cache is flushed
 
 struct DeviceGuard {
     int prev = -1;
-    bool ok = true;
+    bool ok = true, changed = false;
     explicit DeviceGuard(int dev)
     {
         if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; return; }
-        if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
+        if (prev == dev) return;
+        changed = true;
+        if (cudaSetDevice(dev) != cudaSuccess) ok = false;
     }
     ~DeviceGuard()
     {
-        if (prev >= 0) cudaSetDevice(prev);
+        if (changed) cudaSetDevice(prev);
     }
 };
 
