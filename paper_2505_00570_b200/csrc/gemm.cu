@@ -12,10 +12,10 @@
 // For even L the even part Pe is itself the basis of a compression of N/2 rows to L/2, so where N is a
 // multiple of 4 it is folded once more (uu, uv; Pee, Peo); and the odd part Po, whose frequencies are
 // those of a DCT-IV, splits by a rotation of its mirrored rows into two blocks of the same quarter size
-// (p, q; PA, PB; see MODE_QUAD and basis.cu): four blocks of ceil(L/4) x N/4, half of these multiply-adds
+// (p, q; PA, PB; see freqkv_fold_gemm_kernel and basis.cu): four blocks of ceil(L/4) x N/4, half of these multiply-adds
 // again.  The four-block form is what a plain compression of such lengths runs (the paper's
-// 4092 -> 2046 and 4096 -> 2048); the description below is the one-level form, which serves every other
-// length, retained bands, ragged batches and the power spectrum.
+// 4092 -> 2046 and 4096 -> 2048), alone or in a ragged batch; the description below is the one-level form, which serves
+// every other length, retained bands and the power spectrum.
 //
 // Two kernels per call:
 //   fold_kernel         reads every non-sink cache row once and writes U and V (bf16) to a scratch

@@ -1,6 +1,6 @@
 // CUDA-core (fp32 FFMA) execution of the compression Y = P X (Section 3.3, Eq. 2-3): the
-// generic path for every shape and the only one that meets the fp32 tolerance for caches whose
-// lengths are not powers of two.  One CTA computes a 64-row x 64-channel tile of one matrix's
+// generic path for every shape (fp32 caches whose lengths are not powers of two take the folded product of
+// foldf32.cu unless this one is asked for).  One CTA computes a 64-row x 64-channel tile of one matrix's
 // output with a classic shared-memory tiled product; results go to a scratch buffer and a
 // second kernel copies them over rows [sink, sink + L) of the cache, because every output row
 // depends on every input row of the same matrix and the two ranges overlap.
