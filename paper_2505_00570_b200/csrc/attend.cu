@@ -50,15 +50,37 @@ struct AttendParams {
     uint16_t tiles[ATTEND_MAX_BATCH];  // of 16 rows in one split of each sequence
 };
 
+// Loads of queries, keys and values.  The kernel may start while the grid that writes them still runs (see wait_for_previous_grid),
+// so they are not constant for its whole life, which the read-only path (ld.global.nc, __ldg) asks for.  volatile: the loads stay
+// behind the wait and in the order they are written in, all of a round first -- 4 layers of 16 x 32 heads x 4096 rows take
+// 714 us with them as with __ldg, but plain loads, which ptxas moves next to their uses, 5 % more.
+__device__ __forceinline__ uint2 load(const uint2* p)
+{
+    uint2 v;
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 load(const uint4* p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 load(const float4* p)
+{
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&o)[4])
 {
-    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+    const uint2 u = load(reinterpret_cast<const uint2*>(p));
     o[0] = __uint_as_float(u.x << 16); o[1] = __uint_as_float(u.x & 0xffff0000u);
     o[2] = __uint_as_float(u.y << 16); o[3] = __uint_as_float(u.y & 0xffff0000u);
 }
 __device__ __forceinline__ void load4(const float* p, float (&o)[4])
 {
-    const float4 u = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 u = load(reinterpret_cast<const float4*>(p));
     o[0] = u.x; o[1] = u.y; o[2] = u.z; o[3] = u.w;
 }
 // One lane's share of a cache row as loaded: 4 + 4 key channels (c0.., 64 + c0..) and 8 value channels.
@@ -76,16 +98,16 @@ struct RawRow<float> {
 
 __device__ __forceinline__ void fetch(RawRow<__nv_bfloat16>& r, const __nv_bfloat16* krow, const __nv_bfloat16* vrow)
 {
-    r.klo = __ldg(reinterpret_cast<const uint2*>(krow));
-    r.khi = __ldg(reinterpret_cast<const uint2*>(krow + 64));
-    r.v = __ldg(reinterpret_cast<const uint4*>(vrow));
+    r.klo = load(reinterpret_cast<const uint2*>(krow));
+    r.khi = load(reinterpret_cast<const uint2*>(krow + 64));
+    r.v = load(reinterpret_cast<const uint4*>(vrow));
 }
 __device__ __forceinline__ void fetch(RawRow<float>& r, const float* krow, const float* vrow)
 {
-    r.klo = __ldg(reinterpret_cast<const float4*>(krow));
-    r.khi = __ldg(reinterpret_cast<const float4*>(krow + 64));
-    r.v0 = __ldg(reinterpret_cast<const float4*>(vrow));
-    r.v1 = __ldg(reinterpret_cast<const float4*>(vrow) + 1);
+    r.klo = load(reinterpret_cast<const float4*>(krow));
+    r.khi = load(reinterpret_cast<const float4*>(krow + 64));
+    r.v0 = load(reinterpret_cast<const float4*>(vrow));
+    r.v1 = load(reinterpret_cast<const float4*>(vrow) + 1);
 }
 __device__ __forceinline__ void unpack2(uint2 u, float (&o)[4])
 {

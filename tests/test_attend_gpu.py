@@ -153,3 +153,38 @@ def test_attend_splits_and_their_merge(ctx, G, H, lens):
         assert torch.equal(ctx.attend_decode(k, v, 0, q, lens), first)
     last = len(lens) - 1
     check(ctx, k, v, 0, q, lens, 10000.0, heads=[(0, 0), (last, H - 1), (last // 2, 1)])
+
+
+@pytest.mark.parametrize("dtype,G,H,lens", [(torch.bfloat16, 4, 8, [2611]), (torch.bfloat16, 1, 8, [1800, 333, 1900]), (torch.float32, 1, 4, [900, 1500]),
+                                            (torch.bfloat16, 1, 32, [900 + 37 * b for b in range(24)]),
+                                            (torch.bfloat16, 4, 32, [500 + 50 * b for b in range(24)])])
+def test_attend_back_to_back_launches_with_different_contents(ctx, dtype, G, H, lens):
+    """A chain of calls that nothing waits between, as a model enqueues them: a token is appended, then every layer attends
+    over lengths of its own with the layer before's output as its queries, merged by tickets or by a kernel of its own.  A launch that
+    read its inputs or merged its partials before the one in front of it was done would differ from the same chain with a
+    synchronisation after every call."""
+    layers, B = 3, len(lens)
+    w = workload(B, layers, H, max(lens) + 8, dtype, seed=31)
+    k0, v0 = synth.make_cache(w, "cuda")
+    q0 = queries(B, H * G, dtype, 32)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(33)
+    rows = [torch.randn(B, layers, H, 1, 128, generator=gen, device="cuda").to(dtype) for _ in range(2)]
+
+    def chain(wait):
+        k, v, q, outs, n = k0.clone(), v0.clone(), q0, [], lens
+        torch.cuda.synchronize()
+        for _ in range(4):
+            n = ctx.append(k, v, rows[0], rows[1], n)
+            for layer in range(layers):
+                wait()
+                q = ctx.attend_decode(k, v, layer, q, [max(1, x - 100 * layer) for x in n], scale=0.02)
+                outs.append(q)
+                wait()
+        torch.cuda.synchronize()
+        return torch.stack(outs)
+
+    apart = chain(torch.cuda.synchronize)
+    assert torch.isfinite(apart.float()).all() and not torch.equal(apart[0], apart[3])
+    for _ in range(3):
+        assert torch.equal(chain(lambda: None), apart)
