@@ -1114,7 +1114,10 @@ freqkv_status freqkv_attend_decode(freqkv_ctx* ctx, const freqkv_layout* layout,
     const float2* table = nullptr;
     const freqkv_status ts = rope_table_for(ctx, l.capacity, rope_base, stream, &table);
     if (ts != FREQKV_OK) return ts;
-    const AttendPlan plan = attend_plan(l.batch, lens, l.kv_heads, q_heads_per_kv, l.dtype, ctx->sm_count);
+    AttendPlan plan = attend_plan(l.batch, lens, l.kv_heads, q_heads_per_kv, l.dtype, ctx->sm_count);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    FREQKV_CUDA(ctx, cudaStreamIsCapturing(stream, &capture));
+    plan.captured = capture != cudaStreamCaptureStatusNone;
     const size_t need = attend_partial_bytes(plan.splits, l.batch, l.kv_heads * q_heads_per_kv);
     if (need > ctx->attend_partial_bytes) {
         if (ctx->attend_partial) {

@@ -787,10 +787,8 @@ __global__ void rope_table_kernel(float2* table, int32_t rows, double base)
 // A model's layers are attended one call after the other: letting a launch's set-up overlap the tail of the one before
 // took 8 layers of 8 x 8 heads from 366 to 348 us, 8 layers of 12 x 4 short ones from 162 to 151 us.  Not under capture: as an
 // edge of a graph it made 32 layers of one sequence slower (12.9 against 14.3 us a layer).
-void launch_attention(void (*kernel)(const AttendParams), dim3 grid, int threads, int smem, cudaStream_t stream, const AttendParams& prm)
+void launch_attention(void (*kernel)(const AttendParams), dim3 grid, int threads, int smem, cudaStream_t stream, const AttendParams& prm, bool overlap)
 {
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) return;  // the caller reads the error
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
@@ -800,11 +798,11 @@ void launch_attention(void (*kernel)(const AttendParams), dim3 grid, int threads
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    cfg.numAttrs = overlap ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, prm);
 }
 
-cudaError_t launch_mma(const AttendParams& prm, int32_t g, int32_t nb, int32_t splits, cudaStream_t stream)
+cudaError_t launch_mma(const AttendParams& prm, int32_t g, int32_t nb, int32_t splits, bool overlap, cudaStream_t stream)
 {
     static PerDeviceOnce attrs;
     const cudaError_t attr_error = attrs.run([] {
@@ -822,7 +820,7 @@ cudaError_t launch_mma(const AttendParams& prm, int32_t g, int32_t nb, int32_t s
     const dim3 grid((unsigned)splits, (unsigned)(nb * prm.kv_heads));
     auto launch = [&](auto with_tickets, auto without) {
         auto* kernel = prm.tickets ? with_tickets : without;
-        launch_attention(kernel, grid, MMA_THREADS, MMA_SMEM_BYTES, stream, prm);
+        launch_attention(kernel, grid, MMA_THREADS, MMA_SMEM_BYTES, stream, prm, overlap);
     };
     switch (g) {
         case 2: launch(attend_mma_kernel<2, true>, attend_mma_kernel<2, false>); break;
@@ -834,12 +832,12 @@ cudaError_t launch_mma(const AttendParams& prm, int32_t g, int32_t nb, int32_t s
 }
 
 template <typename T>
-cudaError_t launch_typed(const AttendParams& prm, int32_t g, int32_t nb, int32_t splits, cudaStream_t stream)
+cudaError_t launch_typed(const AttendParams& prm, int32_t g, int32_t nb, int32_t splits, bool overlap, cudaStream_t stream)
 {
     const dim3 grid((unsigned)splits, (unsigned)(nb * prm.kv_heads));
     auto launch = [&](auto with_tickets, auto without) {
         auto* kernel = prm.tickets ? with_tickets : without;
-        launch_attention(kernel, grid, THREADS, 0, stream, prm);
+        launch_attention(kernel, grid, THREADS, 0, stream, prm, overlap);
     };
     switch (g) {
         case 1: launch(attend_partial_kernel<T, 1, true>, attend_partial_kernel<T, 1, false>); break;
@@ -917,7 +915,10 @@ cudaError_t launch_attend(const freqkv_layout& l, const void* k, const void* v, 
     prm.q = q;
     prm.out = out;
     prm.partial = partial;
-    prm.tickets = plan.one_wave ? tickets : nullptr;
+    // A captured launch takes no tickets: its replays are not ordered with this context's other calls, and a counter that two
+    // overlapping launches left off zero would spoil every later call.
+    const bool overlap = !plan.captured;
+    prm.tickets = plan.one_wave && !plan.captured ? tickets : nullptr;
     prm.table = table;
     prm.qscale = scale * 1.4426950408889634f;
     prm.total_batch = l.batch;
@@ -934,9 +935,9 @@ cudaError_t launch_attend(const freqkv_layout& l, const void* k, const void* v, 
             merge.splits[i] = (uint16_t)((len + tiles * 16 - 1) / (tiles * 16));
             splits = std::max(splits, n);
         }
-        const cudaError_t e = l.dtype == FREQKV_F32 ? launch_typed<float>(prm, g, nb, splits, stream)
-                              : g >= 2             ? launch_mma(prm, g, nb, splits, stream)   // grouped queries: tensor cores
-                                                   : launch_typed<__nv_bfloat16>(prm, g, nb, splits, stream);
+        const cudaError_t e = l.dtype == FREQKV_F32 ? launch_typed<float>(prm, g, nb, splits, overlap, stream)
+                              : g >= 2             ? launch_mma(prm, g, nb, splits, overlap, stream)   // grouped queries: tensor cores
+                                                   : launch_typed<__nv_bfloat16>(prm, g, nb, splits, overlap, stream);
         if (e != cudaSuccess) return e;
         ++*launched;
         if (!prm.tickets && splits > 1) {

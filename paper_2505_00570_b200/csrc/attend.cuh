@@ -12,6 +12,7 @@ struct AttendPlan {
     int32_t chunk;    // most rows of one CTA
     int32_t splits;   // of the longest sequence
     bool one_wave;    // all CTAs are resident at once
+    bool captured;    // the launches go into a graph: no tickets, no overlap with the launch before
 };
 AttendPlan attend_plan(int32_t batch, const int32_t* lens, int32_t kv_heads, int32_t q_heads_per_kv, int32_t dtype, int sm_count);
 // Work areas: one ticket per (sequence, kv head) of a call whose CTAs are all resident, zero before the first launch and

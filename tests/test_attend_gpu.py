@@ -188,3 +188,43 @@ def test_attend_back_to_back_launches_with_different_contents(ctx, dtype, G, H, 
     assert torch.isfinite(apart.float()).all() and not torch.equal(apart[0], apart[3])
     for _ in range(3):
         assert torch.equal(chain(lambda: None), apart)
+
+
+@pytest.mark.parametrize("G,H,lens", [(4, 8, [2611]), (1, 4, [193, 1700, 192]), (1, 32, [900 + 37 * b for b in range(24)])])
+def test_attend_captured_into_a_graph(G, H, lens):
+    """A decode step of three layers captured and replayed, with eager calls of the same context between the replays: the eager
+    calls keep their bits, the replays theirs, new queries are read at each replay.  A captured call merges its splits by a launch of
+    its own, never by the ticket counters, which must be zero between the context's calls and which no replay may leave in
+    another state.  The two merges sum the splits in another order: fp32 rounding, which can move the one rounding to bf16 by a
+    step (2^-8 of the value, stated twice that; values near zero by their fp32 share)."""
+    ctx, B = fk.Context(0), len(lens)
+    w = workload(B, 3, H, max(lens) + 5, torch.bfloat16, seed=41)
+    k, v = synth.make_cache(w, "cuda")
+    q, q2 = queries(B, H * G, torch.bfloat16, 42), queries(B, H * G, torch.bfloat16, 43)
+    stream = torch.cuda.Stream()
+    step = lambda: torch.stack([ctx.attend_decode(k, v, layer, q, lens) for layer in range(3)])  # noqa: E731
+    near = lambda a, b: torch.allclose(a.float(), b.float(), rtol=2.0 ** -7, atol=1e-5 * b.float().abs().max().item())  # noqa: E731
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        want = step()
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        before = ctx.get_timing()[2]
+        with torch.cuda.graph(graph, stream=stream):
+            out = step()
+        assert ctx.get_timing()[2] - before == 6     # per layer: the attention and the merge
+        graph.replay()
+        first = out.clone()
+        assert near(first, want)
+        for i in range(4):
+            graph.replay()
+            got = out.clone()
+            assert torch.equal(got, first) and torch.equal(step(), want), i
+        q.copy_(q2)
+        graph.replay()
+        got, want = out.clone(), step()
+        assert near(got, want) and not near(got, first)
+        check(ctx, k, v, 1, q, lens, 10000.0, heads=[(0, 0), (B - 1, H - 1)])
+        stream.synchronize()
+        del graph
+    ctx.close()
