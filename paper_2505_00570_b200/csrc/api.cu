@@ -54,9 +54,9 @@ struct freqkv_ctx {
     float2* rope_table = nullptr;
     int32_t rope_rows = 0;
     double rope_base = 0.0;
-    float* attend_partial = nullptr;
-    size_t attend_partial_bytes = 0;
-    int32_t* attend_tickets = nullptr;  // per (sequence, kv head): splits finished, zero between calls (see attend_ticket_bytes)
+    void* attend_work = nullptr;  // attend_ticket_bytes of tickets, then the splits' partials
+    size_t attend_work_bytes = 0;
+    bool attend_tickets_clear = false;  // zeroed on a stream that later calls are ordered behind
     void* prefill_keys = nullptr;     // rotated keys of one layer, fp16
     size_t prefill_keys_bytes = 0;
     void* prefill_queries = nullptr;  // rotated, scaled queries of one chunk, fp16
@@ -622,15 +622,10 @@ freqkv_status freqkv_create(freqkv_ctx** out, int device)
         return FREQKV_ERR_UNSUPPORTED;
     }
     ctx->sm_count = prop.multiProcessorCount;
-    // zeroed here and not on a call's stream: a call may be under capture
-    const size_t tickets = attend_ticket_bytes(ctx->sm_count);
     if (cudaMalloc(&ctx->status_dev, sizeof(int32_t)) != cudaSuccess ||
-        cudaMemset(ctx->status_dev, 0, sizeof(int32_t)) != cudaSuccess ||
-        cudaMalloc(&ctx->attend_tickets, tickets) != cudaSuccess || cudaMemset(ctx->attend_tickets, 0, tickets) != cudaSuccess ||
-        cudaStreamSynchronize(nullptr) != cudaSuccess) {  // calls may come on streams that do not wait for this one
+        cudaMemset(ctx->status_dev, 0, sizeof(int32_t)) != cudaSuccess) {
         cudaGetLastError();
         if (ctx->status_dev) cudaFree(ctx->status_dev);
-        if (ctx->attend_tickets) cudaFree(ctx->attend_tickets);
         delete ctx;
         return FREQKV_ERR_ALLOC;
     }
@@ -653,8 +648,7 @@ freqkv_status freqkv_destroy(freqkv_ctx* ctx)
         if (ctx->stage[i]) cudaFree(ctx->stage[i]);
     if (ctx->work_done) cudaEventDestroy(ctx->work_done);
     if (ctx->rope_table) cudaFree(ctx->rope_table);
-    if (ctx->attend_partial) cudaFree(ctx->attend_partial);
-    if (ctx->attend_tickets) cudaFree(ctx->attend_tickets);
+    if (ctx->attend_work) cudaFree(ctx->attend_work);
     if (ctx->prefill_keys) cudaFree(ctx->prefill_keys);
     if (ctx->prefill_queries) cudaFree(ctx->prefill_queries);
     for (int i = 0; i < 3; ++i)
@@ -1118,23 +1112,30 @@ freqkv_status freqkv_attend_decode(freqkv_ctx* ctx, const freqkv_layout* layout,
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     FREQKV_CUDA(ctx, cudaStreamIsCapturing(stream, &capture));
     plan.captured = capture != cudaStreamCaptureStatusNone;
-    const size_t need = attend_partial_bytes(plan.splits, l.batch, l.kv_heads * q_heads_per_kv);
-    if (need > ctx->attend_partial_bytes) {
-        if (ctx->attend_partial) {
+    const size_t tickets = attend_ticket_bytes(ctx->sm_count);
+    const size_t need = tickets + attend_partial_bytes(plan.splits, l.batch, l.kv_heads * q_heads_per_kv);
+    if (need > ctx->attend_work_bytes) {
+        if (ctx->attend_work) {
             FREQKV_CUDA(ctx, cudaDeviceSynchronize());
-            cudaFree(ctx->attend_partial);
-            ctx->attend_partial = nullptr;
-            ctx->attend_partial_bytes = 0;
+            cudaFree(ctx->attend_work);
+            ctx->attend_work = nullptr;
+            ctx->attend_work_bytes = 0;
         }
-        FREQKV_CUDA(ctx, cudaMalloc(&ctx->attend_partial, need));
-        ctx->attend_partial_bytes = need;
+        ctx->attend_tickets_clear = false;
+        FREQKV_CUDA(ctx, cudaMalloc(&ctx->attend_work, need));
+        ctx->attend_work_bytes = need;
+    }
+    if (plan.one_wave && !plan.captured && !ctx->attend_tickets_clear) {
+        FREQKV_CUDA(ctx, cudaMemsetAsync(ctx->attend_work, 0, tickets, stream));
+        ctx->attend_tickets_clear = true;
     }
     int32_t launched = 0;
     cudaError_t e;
     {
         TransformTimer timer(ctx, stream);
-        e = launch_attend(l, k, v, layer, q, out, q_heads_per_kv, lens, table, scale, plan, ctx->attend_partial,
-                          ctx->attend_tickets, &launched, stream);
+        e = launch_attend(l, k, v, layer, q, out, q_heads_per_kv, lens, table, scale, plan,
+                          reinterpret_cast<float*>(static_cast<char*>(ctx->attend_work) + tickets),
+                          static_cast<int32_t*>(ctx->attend_work), &launched, stream);
     }
     ctx->kernels_launched += launched;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "attend");

@@ -884,8 +884,8 @@ AttendPlan attend_plan(int32_t batch, const int32_t* lens, int32_t kv_heads, int
     return plan;
 }
 
-// One wave of CTAs holds at most so many (sequence, kv head) groups.
-size_t attend_ticket_bytes(int sm_count) { return (size_t)sm_count * MMA_CTAS_PER_SM * sizeof(int32_t); }
+// One wave of CTAs holds at most so many (sequence, kv head) groups; whole 256 bytes, so that what follows is aligned.
+size_t attend_ticket_bytes(int sm_count) { return ((size_t)sm_count * MMA_CTAS_PER_SM * sizeof(int32_t) + 255) & ~(size_t)255; }
 
 size_t attend_partial_bytes(int32_t splits, int32_t batch, int32_t q_heads)
 {

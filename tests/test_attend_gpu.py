@@ -228,3 +228,16 @@ def test_attend_captured_into_a_graph(G, H, lens):
         stream.synchronize()
         del graph
     ctx.close()
+
+
+def test_context_creation_does_not_wait_for_enqueued_work():
+    """A context is created while a kernel of 0.2 s or so runs on the default stream: creation returns before it ends."""
+    fk.Context(0).close()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(400_000_000)
+    done = torch.cuda.Event()
+    done.record()
+    ctx = fk.Context(0)
+    assert not done.query()
+    torch.cuda.synchronize()
+    ctx.close()
