@@ -856,6 +856,8 @@ bool attend_supported(int32_t head_dim, int32_t q_heads_per_kv)
     return head_dim == 128 && (q_heads_per_kv == 1 || q_heads_per_kv == 2 || q_heads_per_kv == 4 || q_heads_per_kv == 8);
 }
 
+constexpr int32_t MIN_ROWS = 192, MOST_SPLITS = 64;
+
 // Rows of one CTA.  Each candidate is judged by the rows' time of its waves of resident CTAs, waves * (rows +
 // OVERHEAD_ROWS): the constant stands for a CTA's prologue (query, table) and its share of the merge.  A launch with
 // few (sequence, kv head) groups splits down to MIN_ROWS rows, so that even a single sequence is read by the whole
@@ -864,7 +866,7 @@ bool attend_supported(int32_t head_dim, int32_t q_heads_per_kv)
 // to 1990 rows 40.7 -> 16.4, 8 x 8 heads of 4099 to 8192 rows 48.9 -> 43.4; OVERHEAD_ROWS 32 and 192 give the same.
 AttendPlan attend_plan(int32_t batch, const int32_t* lens, int32_t kv_heads, int32_t q_heads_per_kv, int32_t dtype, int sm_count)
 {
-    constexpr int32_t MIN_ROWS = 192, OVERHEAD_ROWS = 96, MOST_SPLITS = 64, MOST_ROWS = 0xffff * 16;  // a split's tiles are 16 bits
+    constexpr int32_t OVERHEAD_ROWS = 96, MOST_ROWS = 0xffff * 16;  // a split's tiles are 16 bits
     const bool tensor_cores = dtype == FREQKV_BF16 && q_heads_per_kv >= 2;
     const int64_t resident = (int64_t)sm_count * (tensor_cores ? MMA_CTAS_PER_SM : q_heads_per_kv <= 4 ? 2 : 1);
     const int32_t longest = *std::max_element(lens, lens + batch);
@@ -883,6 +885,8 @@ AttendPlan attend_plan(int32_t batch, const int32_t* lens, int32_t kv_heads, int
     }
     return plan;
 }
+
+int32_t attend_most_splits(int32_t longest) { return std::max(1, std::min(longest / MIN_ROWS + 1, MOST_SPLITS)); }
 
 // One wave of CTAs holds at most so many (sequence, kv head) groups; whole 256 bytes, so that what follows is aligned.
 size_t attend_ticket_bytes(int sm_count) { return ((size_t)sm_count * MMA_CTAS_PER_SM * sizeof(int32_t) + 255) & ~(size_t)255; }

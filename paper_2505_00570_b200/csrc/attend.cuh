@@ -15,6 +15,8 @@ struct AttendPlan {
     bool captured;    // the launches go into a graph: no tickets, no overlap with the launch before
 };
 AttendPlan attend_plan(int32_t batch, const int32_t* lens, int32_t kv_heads, int32_t q_heads_per_kv, int32_t dtype, int sm_count);
+// No plan for lengths up to `longest` has more splits (unless rows beyond what 64 CTAs can take force them).
+int32_t attend_most_splits(int32_t longest);
 // Work areas: one ticket per (sequence, kv head) of a call whose CTAs are all resident, zero before the first launch and
 // after every launch; the splits' partials.
 size_t attend_ticket_bytes(int sm_count);
