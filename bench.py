@@ -159,16 +159,11 @@ def workload_numbers(w, cache_len, kept, sink, first=0):
         folded = 2.0 * ((kept // 2 + 1) // 2) * 3 * (n_in // 2) * w.head_dim * m
     else:
         folded = 2.0 * 2 * ((kept + 1) // 2) * ((n_in + 1) // 2) * w.head_dim * m
-    # What the library executes: where N is a multiple of 4, L even and the lowest components are kept, four blocks of
-    # ceil(L/4) x N/4 (the last N/2 deep for even L/2) if that means fewer 64-row slices of 256-row tiles than one level.
-    def slices(rows, steps):
-        return -(-rows // 256) * steps
-    q, tail = -(-(n_in // 4) // 64), -(-(n_in // 2) // 64) if kept // 2 % 2 == 0 else -(-(n_in // 4) // 64)
-    four = (first == 0 and n_in % 4 == 0 and kept % 2 == 0 and kept > 256 and
-            slices((kept // 2 + 1) // 2, 3 * q + tail) < slices((kept + 1) // 2, 2 * -(-(n_in // 2) // 64)))
-    executed = 2.0 * 2 * ((kept + 1) // 2) * ((n_in + 1) // 2) * w.head_dim * m
-    if four:
-        executed = 2.0 * ((kept // 2 + 1) // 2) * (4 if kept // 2 % 2 else 5) * (n_in // 4) * w.head_dim * m
+    # What the library executes: one level, or four blocks of ceil(L/4) x N/4 (the last N/2 deep for even L/2), or the
+    # dense product for few kept rows.
+    blocks = _fk.gemm_blocks(n_in, kept, m // 2, first)
+    executed = {1: 2.0 * kept * n_in, 2: 2.0 * 2 * ((kept + 1) // 2) * ((n_in + 1) // 2),
+                4: 2.0 * ((kept // 2 + 1) // 2) * (4 if kept // 2 % 2 else 5) * (n_in // 4)}[blocks] * w.head_dim * m
     return {
         "fold_levels": fold_levels,
         "executed_flops": executed,

@@ -50,8 +50,9 @@ typedef enum { FREQKV_BF16 = 0, FREQKV_F32 = 1 } freqkv_dtype;
  *   GEMM  the DCT-II -> truncate -> IDCT -> rescale chain folded into one precomputed
  *         kept_len x n_in projection basis and run on the tcgen05 tensor cores (bf16 caches,
  *         head_dim 128 only); halved by the even/odd symmetry of the cosines after a fold pass
- *         over the cache (folded twice, to three eighths, where n_in is a multiple of 4 and
- *         kept_len even), or, for kept_len <= 256, straight from the cache without that pass;
+ *         over the cache (to a quarter where n_in is a multiple of 4, kept_len even and the call
+ *         large enough, see freqkv_gemm_blocks), or, for kept_len <= 256, straight from the cache
+ *         without that pass;
  *   FDCT  fast transform, O(N log N) (Appendix A: the DCT "can be computed using the FFT"): for
  *         bf16 caches the transform pair is factored into four small dense stages that run on
  *         the tensor cores, in place with no scratch, for every n_in = N1 N2 and kept_len = L1 L2
@@ -354,13 +355,18 @@ freqkv_status freqkv_fast_plan_apply_host(int32_t n_in, int32_t n_keep, int32_t 
 /* Host-only: how many levels of the even/odd mirror symmetry (Appendix A's cosines are even or odd
  * under n -> N-1-n) pay for variant GEMM in a compression of n_in rows to kept_len components
  * starting at first_component: 0 = none (kept_len <= 256: straight from the cache), 1, or 2 (n_in a
- * multiple of 4, kept_len even, first_component 0, and fewer 64-row slices that way).  With one level the
- * multiply-adds per matrix are 2 * ceil(L/2) * ceil(N/2) * head_dim, with two
- * 3 * ceil(L/4) * (N/2) * head_dim; where N is a multiple of 4, L even and the lowest components are kept, the
- * library splits the odd part as well and executes 4 * ceil(L/4) * (N/4) * head_dim (5 instead of 4 for
- * even L/2).  -1 for invalid lengths.  Retained bands that start higher and the power spectrum
- * always use one level. */
+ * multiple of 4, kept_len even, first_component 0, and fewer 64-row slices of 256-row tiles that way).  With one
+ * level the multiply-adds per matrix are 2 * ceil(L/2) * ceil(N/2) * head_dim, with two of the mirror symmetry alone
+ * 3 * ceil(L/4) * (N/2) * head_dim.  -1 for invalid lengths.  Retained bands that start higher and the power
+ * spectrum always use one level.  (Where this says 2 the library can split the odd part as well: freqkv_gemm_blocks.) */
 int32_t freqkv_gemm_fold_levels(int32_t n_in, int32_t kept_len, int32_t first_component);
+
+/* Host-only: in how many blocks variant GEMM runs such a compression of `triples` (batch, layer, kv_head) triples:
+ * 1 = the dense kept_len x n_in product straight from the cache (kept_len <= 256); 2 = one level of the mirror
+ * symmetry; 4 = both levels and the odd part split by a rotation, 4 * ceil(L/4) * (N/4) * head_dim multiply-adds per
+ * matrix (5 instead of 4 for even L/2), for lengths of two levels where there is work enough for its longer
+ * tiles.  A ragged batch asks for somewhat more work.  -1 for invalid arguments. */
+int32_t freqkv_gemm_blocks(int32_t n_in, int32_t kept_len, int32_t first_component, int64_t triples);
 
 /* Text of the most recent CUDA failure or device-status report seen by this context (owned by
  * the context, valid until its next call); "" if none. */

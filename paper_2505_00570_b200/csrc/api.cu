@@ -1459,6 +1459,12 @@ int32_t freqkv_gemm_fold_levels(int32_t n_in, int32_t kept_len, int32_t first_co
     return gemm_fold_levels(n_in, kept_len, first_component);
 }
 
+int32_t freqkv_gemm_blocks(int32_t n_in, int32_t kept_len, int32_t first_component, int64_t triples)
+{
+    if (n_in < 1 || kept_len < 1 || kept_len > n_in || first_component < 0 || first_component > n_in - kept_len || triples < 1) return -1;
+    return gemm_blocks(n_in, kept_len, first_component, triples, false);
+}
+
 const char* freqkv_last_error(freqkv_ctx* ctx) { return ctx ? ctx->last_error.c_str() : ""; }
 
 const char* freqkv_status_string(freqkv_status status)

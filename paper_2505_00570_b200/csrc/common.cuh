@@ -45,7 +45,7 @@ struct Basis {
     // m < ceil(n_keep/2), n < ceil(n_in/2), bf16, two planes of fold_rows_pad x fold_ld (see basis.cu).
     __nv_bfloat16* fold = nullptr;
     int32_t fold_ld = 0, fold_rows_pad = 0;
-    // The four-block form, where the lengths take it (gemm_quad): four planes of quad_rows_pad x fold_ld -- Pee, Peo,
+    // The four-block form, where the lengths can take it (gemm_quad; a call chooses by its matrices, gemm_blocks): four planes of quad_rows_pad x fold_ld -- Pee, Peo,
     // PA, PB -- stored behind the two planes above in the same allocation, then (cos, sin) of theta_n, n < n_in / 4
     // (see basis.cu).
     __nv_bfloat16* quad = nullptr;

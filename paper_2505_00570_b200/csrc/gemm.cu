@@ -14,8 +14,8 @@
 // those of a DCT-IV, splits by a rotation of its mirrored rows into two blocks of the same quarter size
 // (p, q; PA, PB; see freqkv_fold_gemm_kernel and basis.cu): four blocks of ceil(L/4) x N/4, half of these multiply-adds
 // again.  The four-block form is what a plain compression of such lengths runs (the paper's
-// 4092 -> 2046 and 4096 -> 2048), alone or in a ragged batch; the description below is the one-level form, which serves
-// every other length, retained bands and the power spectrum.
+// 4092 -> 2046 and 4096 -> 2048) where there is work enough (gemm_blocks), alone or in a ragged batch; the description below
+// is the one-level form, which serves everything else, retained bands and the power spectrum among it.
 //
 // Two kernels per call:
 //   fold_kernel         reads every non-sink cache row once and writes U and V (bf16) to a scratch
@@ -514,10 +514,10 @@ __device__ __forceinline__ const FoldSeq& seq_of_tile(const FoldParams& prm, int
     }
 }
 
-// FORM_ONE_LEVEL, FORM_FOUR_BLOCKS, FORM_FOUR_BLOCKS_WIDE: the compression of one pair of lengths; WIDE keeps the pairs (s, s')
-//   below in fp32, for lengths at which one level, whose sums never leave fp32, is the alternative.
+// FORM_ONE_LEVEL, FORM_FOUR_BLOCKS: the compression of one pair of lengths.
 // FORM_RAGGED: sequences of different lengths in one launch: a tile looks up its sequence (shapes, tensor
-//   maps) in a table built on the host; one-level and four-block sequences mix (FoldSeq::quad).
+//   maps) in a table built on the host; one-level and four-block sequences mix (FoldSeq::quad).  The pairs (s, s') below stay in
+//   fp32 here.
 // Four blocks (n_in a multiple of 4, n_keep even): a tile is 256 rows m < ceil(L/4) of all
 //   four blocks and runs four phases, each N/4 deep, alternating between the two halves of tensor memory:
 //   a = Pee uu, b = Peo uv, A = PA p, B = PB q (for even L/2 one retained component couples p into B: the last
@@ -526,18 +526,18 @@ __device__ __forceinline__ const FoldSeq& seq_of_tile(const FoldParams& prm, int
 //   in a work area of this CTA that stays in L2 -- the accumulators of a tile would need twice the tensor memory there is --,
 //   parks A, and turns it with B by theta'_m = pi (2m+1) / (2L) into d = cos A + sin B and d' = sin A - cos B:
 //   y_m = s + d, y_{L-1-m} = s - d, y_{L/2-1-m} = s' + d', y_{L/2+m} = s' - d'.
-constexpr int FORM_ONE_LEVEL = 0, FORM_FOUR_BLOCKS = 1, FORM_RAGGED = 2, FORM_FOUR_BLOCKS_WIDE = 3;
+constexpr int FORM_ONE_LEVEL = 0, FORM_FOUR_BLOCKS = 1, FORM_RAGGED = 2;
 
 template <int FORM>
 __global__ void __launch_bounds__(FOLD_THREADS, 1)
 freqkv_fold_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_x, const CacheView view,
                         const __grid_constant__ FoldParams prm)
 {
-    constexpr bool RAGGED = FORM == FORM_RAGGED, WIDE = FORM == FORM_RAGGED || FORM == FORM_FOUR_BLOCKS_WIDE;
+    constexpr bool RAGGED = FORM == FORM_RAGGED, WIDE = RAGGED;
     // The next 16 columns (and their pairs) leave tensor memory while these are combined and stored, where the registers allow
     // it (2997 -> 749 1.50 -> 1.48 ms with the append, 64 matrices 1497 -> 749 44.1 -> 42.1 us; with fp32 pairs 57 -> 61 us).
     constexpr bool AHEAD = !WIDE;
-    constexpr bool FOUR = FORM == FORM_FOUR_BLOCKS || FORM == FORM_FOUR_BLOCKS_WIDE;
+    constexpr bool FOUR = FORM == FORM_FOUR_BLOCKS;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // 128-byte swizzle atoms need 1024-byte alignment
@@ -1193,17 +1193,17 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
         return cudaErrorNotSupported;
     }
     if (!state->attr_set) {
-        const void* kernels[6] = {(const void*)freqkv_gemm_kernel<MODE_SPECTRUM>, (const void*)freqkv_gemm_kernel<MODE_DIRECT>,
+        const void* kernels[5] = {(const void*)freqkv_gemm_kernel<MODE_SPECTRUM>, (const void*)freqkv_gemm_kernel<MODE_DIRECT>,
                                   (const void*)freqkv_fold_gemm_kernel<FORM_ONE_LEVEL>, (const void*)freqkv_fold_gemm_kernel<FORM_FOUR_BLOCKS>,
-                                  (const void*)freqkv_fold_gemm_kernel<FORM_FOUR_BLOCKS_WIDE>, (const void*)freqkv_fold_gemm_kernel<FORM_RAGGED>};
-        for (int i = 0; i < 6; ++i) {
+                                  (const void*)freqkv_fold_gemm_kernel<FORM_RAGGED>};
+        for (int i = 0; i < 5; ++i) {
             const cudaError_t e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
             if (e != cudaSuccess) {
                 state->last_error = "cudaFuncSetAttribute(max dynamic shared memory)";
                 return e;
             }
         }
-        for (int i = 2; i < 6; ++i) {  // the register shares are of what the block is launched with
+        for (int i = 2; i < 5; ++i) {  // the register shares are of what the block is launched with
             cudaFuncAttributes fa;
             const cudaError_t e = cudaFuncGetAttributes(&fa, kernels[i]);
             if (e != cudaSuccess || fa.numRegs < FOLD_LAUNCH_REGS) {
@@ -1240,14 +1240,14 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
 }
 
 // The shapes of one sequence: everything but its place in the launch.
-static FoldSeq fold_seq(const Basis& b, int32_t pair0)
+static FoldSeq fold_seq(const Basis& b, int32_t pair0, bool quad)
 {
     FoldSeq s = {};
     s.pair0 = pair0;
     s.n_half = (b.n_in + 1) / 2;
     s.n_keep = b.n_keep;
     s.rows_half = (b.n_keep + 1) / 2;
-    s.quad = b.quad != nullptr;
+    s.quad = quad;
     s.basis_rows_pad = s.quad ? b.quad_rows_pad : b.fold_rows_pad;
     s.k_steps = s.quad ? quad_steps(b.n_in) : (s.n_half + BK - 1) / BK;
     s.k_last = s.quad ? quad_last_steps(b.n_in, b.n_keep) : 0;
@@ -1309,10 +1309,10 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
     const cudaError_t prepared = gemm_prepare(state, view.mats_per_tensor, basis, sm_count);
     if (prepared != cudaSuccess) return prepared;
     const int32_t pairs = view.mats_per_tensor;
-    FoldSeq seq = fold_seq(basis, 0);
-    const size_t per_pair = (size_t)4 * seq.n_half * 128 * 2;
+    const size_t per_pair = (size_t)4 * ((basis.n_in + 1) / 2) * 128 * 2;
     // One pass when the folded inputs fit the scratch buffer, else several passes of `chunk` pairs.
     const int64_t chunk = std::min<int64_t>(std::max<int64_t>(1, (int64_t)(kFoldBufferBytes / per_pair)), pairs);
+    FoldSeq seq = fold_seq(basis, 0, basis.quad && gemm_blocks(basis.n_in, basis.n_keep, basis.first, chunk, false) == 4);
     CUtensorMap map_p;
     if (!(seq.quad ? encode_quad_map(&map_p, basis) : encode_basis_map(&map_p, basis))) {
         state->last_error = "tensor map encoding rejected the basis";
@@ -1342,11 +1342,8 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
             state->last_error = "fold_kernel launch";
             return e;
         }
-        // lengths that two levels of the mirror symmetry used to serve kept (s, s') in bf16 there, too
-        const bool wide = seq.quad && gemm_fold_levels(basis.n_in, basis.n_keep, basis.first) != 2;
-        e = wide       ? launch_product<FORM_FOUR_BLOCKS_WIDE>(state, map_p, map_x, view, prm, hooks, stream)
-            : seq.quad ? launch_product<FORM_FOUR_BLOCKS>(state, map_p, map_x, view, prm, hooks, stream)
-                       : launch_product<FORM_ONE_LEVEL>(state, map_p, map_x, view, prm, hooks, stream);
+        e = seq.quad ? launch_product<FORM_FOUR_BLOCKS>(state, map_p, map_x, view, prm, hooks, stream)
+                     : launch_product<FORM_ONE_LEVEL>(state, map_p, map_x, view, prm, hooks, stream);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1438,7 +1435,9 @@ cudaError_t launch_gemm_ragged(GemmState* state, const CacheView& view, const st
     int64_t tiles = 0;
     int32_t max_half = 0;
     for (size_t i = 0; i < n; ++i) {
-        FoldSeq& s = seqs[i] = fold_seq(items[i].basis, items[i].batch_index * lh);
+        const Basis& b = items[i].basis;
+        const bool quad = b.quad && gemm_blocks(b.n_in, b.n_keep, 0, (int64_t)n * lh, true) == 4;
+        FoldSeq& s = seqs[i] = fold_seq(b, items[i].batch_index * lh, quad);
         s.tile0 = (int32_t)tiles;
         tiles += (int64_t)lh * s.m_pairs;
         max_half = std::max(max_half, s.n_half);
@@ -1526,18 +1525,30 @@ int32_t gemm_fold_levels(int32_t n_in, int32_t n_keep, int32_t first)
     return slices2 < slices1 ? 2 : 1;
 }
 
-// The four-block form: where the lengths allow it (as for two levels) and it means fewer 64-row slices per matrix pair
-// than one level -- 4092 -> 2046: 128 of them instead of 256, 3000 -> 1500: 96 instead of 144.  Compression and append of a
-// 7B-shaped cache (2048 matrices, 4092 -> 2046) 2.52 ms with two levels of the mirror symmetry alone, 2.21 ms with the
-// four blocks; 8B-shaped (4096 matrices, 8188 -> 4094) 15.4 and 12.5 ms; error against 64 bits 1.7e-3 both.
-bool gemm_quad(int32_t n_in, int32_t n_keep, int32_t first)
+bool gemm_quad(int32_t n_in, int32_t n_keep, int32_t first) { return gemm_fold_levels(n_in, n_keep, first) == 2; }
+
+// One level or four blocks, for lengths that halve twice.  Four blocks are half the multiply-adds, but a tile of theirs stands for
+// twice the output rows, and its epilogue -- four phases, the pairs' way through L2 -- outlasts its slices where these are few.  So
+// both forms are counted in slices of their longest CTA pair, with a tile of four blocks costing as many more as its epilogue
+// adds: 30, and 60 in a ragged launch, whose pairs are fp32 (8 more for the first of them).  Compression alone in us, one level and four blocks:
+//   512 matrices 1028 -> 514 109, 125; 2048 -> 1024 181, 203; 4092 -> 1022 329, 319; 4096 -> 2048 468, 436; 4092 -> 2046 476, 406;
+//   8188 -> 4094 1707, 1100.  80 matrices 4096 -> 2048 95, 103; 2200 -> 1650 60, 66; 8 matrices 4092 -> 2046 34, 42; 8188 -> 4094 55, 62.
+//   Ragged, 512 matrices of 1028 -> 514 127, 152; 4096 -> 2048 463, 477; 4092 -> 2046 465, 444; 8188 -> 4094 1590, 1094.
+// Compression and append of a 7B-shaped cache (2048 matrices, 4092 -> 2046) 2.52 ms with two levels of the mirror symmetry alone,
+// 2.21 ms with the four blocks; 8B-shaped (4096 matrices, 8188 -> 4094) 15.4 and 12.5 ms; error against 64 bits 1.7e-3 both.
+// (Where a second level means no fewer slices -- kept rows 1026 to 1536 when both lengths halve: two tiles instead of three --
+// four blocks lost up to a third: 512 matrices 2400 -> 1200 251, 331; 16 matrices 2052 -> 1026 25, 37.)
+int32_t gemm_blocks(int32_t n_in, int32_t n_keep, int32_t first, int64_t triples, bool ragged)
 {
-    if (gemm_is_direct(n_keep) || first != 0 || n_in % 4 != 0 || n_keep % 2 != 0) return false;
+    if (gemm_is_direct(n_keep)) return 1;
+    if (!gemm_quad(n_in, n_keep, first)) return 2;
+    constexpr int64_t CLUSTERS = 74;  // CTA pairs of a B200
     const int32_t rows_half = n_keep / 2, rows_quarter = (rows_half + 1) / 2;
-    const int64_t slices1 = (int64_t)((rows_half + 2 * BM - 1) / (2 * BM)) * 2 * ((n_in / 2 + BK - 1) / BK);
-    const int64_t slices4 =
-        (int64_t)((rows_quarter + 2 * BM - 1) / (2 * BM)) * (3 * quad_steps(n_in) + quad_last_steps(n_in, n_keep));
-    return slices4 < slices1;
+    const int64_t tiles2 = (rows_half + 2 * BM - 1) / (2 * BM), tiles4 = (rows_quarter + 2 * BM - 1) / (2 * BM);
+    const int64_t slices2 = 2 * ((n_in / 2 + BK - 1) / BK), slices4 = 3 * quad_steps(n_in) + quad_last_steps(n_in, n_keep);
+    const int64_t waves2 = (triples * tiles2 + CLUSTERS - 1) / CLUSTERS, waves4 = (triples * tiles4 + CLUSTERS - 1) / CLUSTERS;
+    const int64_t cost4 = ragged ? waves4 * (slices4 + 60) + 8 : waves4 * (slices4 + 30);
+    return cost4 < waves2 * slices2 ? 4 : 2;
 }
 
 cudaError_t launch_gemm_direct(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink,

@@ -46,8 +46,10 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
 bool gemm_is_direct(int32_t n_keep);
 // 0, 1 or 2 levels of the mirror symmetry for a plain compression of these lengths (see gemm.cu).
 int32_t gemm_fold_levels(int32_t n_in, int32_t n_keep, int32_t first);
-// Does a plain compression of these lengths run as four quarter-size blocks?
+// Can a plain compression of these lengths run as four quarter-size blocks?
 bool gemm_quad(int32_t n_in, int32_t n_keep, int32_t first);
+// Blocks that a launch of so many (batch, layer, kv_head) triples runs: 4, 2 (one level), or 1 (the direct mode).
+int32_t gemm_blocks(int32_t n_in, int32_t n_keep, int32_t first, int64_t triples, bool ragged);
 cudaError_t launch_gemm_direct(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink,
                                int32_t* status_dev, int sm_count, const LaunchHooks& hooks, cudaStream_t stream);
 // One sequence of a ragged batch: its index in the cache and the (folded) basis of its lengths.

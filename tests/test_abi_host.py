@@ -184,3 +184,20 @@ def test_fold_level_rule():
     assert fk.gemm_fold_levels(3000, 1500) == 1            # 375 twice-folded rows fill two tiles as badly as 750 fill three
     assert fk.gemm_fold_levels(4092, 40) == 0 and fk.gemm_fold_levels(4092, 256) == 0
     assert fk.gemm_fold_levels(0, 0) == -1 and fk.gemm_fold_levels(10, 11) == -1 and fk.gemm_fold_levels(10, 5, -1) == -1
+
+
+def test_gemm_blocks():
+    """One level or four blocks by the lengths and the work: the paper's shapes run four, a few matrices, short lengths and lengths
+    whose quarter rows fill two tiles as badly as their half rows three run one level; every answer follows the rules' terms."""
+    for n, kept, triples, want in [(4092, 2046, 1024, 4), (4096, 2048, 1024, 4), (8188, 4094, 2048, 4), (8188, 4094, 20, 4), (4092, 2046, 4, 2), (8188, 4094, 4, 2),
+                                   (1028, 514, 256, 2), (2048, 1024, 256, 2), (2400, 1200, 256, 2), (3000, 1500, 2048, 2), (6140, 1534, 256, 2),
+                                   (2200, 1650, 256, 4), (4092, 2045, 1024, 2), (4094, 2046, 1024, 2), (4092, 256, 1024, 1), (4092, 40, 1, 1)]:
+        assert fk.gemm_blocks(n, kept, triples) == want, (n, kept, triples)
+    assert fk.gemm_blocks(4092, 2046, 1024, 2046) == 2     # another band of components
+    for n in range(1, 4000, 37):
+        for kept in {1, n // 4, n // 2, n} - {0}:
+            got = fk.gemm_blocks(n, kept, 1024)
+            assert (got == 1) == (kept <= 256) and (got < 4 or fk.gemm_fold_levels(n, kept) == 2)
+    for bad in [(0, 0, 1), (10, 11, 1), (10, 5, 0)]:
+        assert fk.gemm_blocks(*bad) == -1
+    assert fk.gemm_blocks(10, 5, 1, -1) == -1 and fk.gemm_blocks(10, 5, 1, 6) == -1

@@ -243,7 +243,7 @@ def test_gemm_lengths(ctx, n_in, kept, sink):
 
 @pytest.mark.parametrize("n_in,kept,sink", [(2048, 1024, 0), (4092, 2728, 4), (1396, 698, 4), (4092, 2046, 4), (2732, 1366, 0)])
 def test_gemm_two_fold_levels(ctx, n_in, kept, sink):
-    """Lengths that halve twice (n_in a multiple of 4, kept even) run the symmetry fold at two levels: a whole
+    """Lengths that halve twice (n_in a multiple of 4, kept even), in calls too small for four blocks: a whole
     number of 256-row tiles (2048 -> 1024), a ragged last tile (2728 kept rows: 682 twice-folded ones), an odd
     kept / 2 whose middle row is its own mirror (698, 2046, 1366), several sequences, layers and heads, padded rows."""
     w = small(cap=n_in + sink + 3, dtype=torch.bfloat16, sink=sink, outliers=2, B=2, Ly=2, H=3)
@@ -253,11 +253,69 @@ def test_gemm_two_fold_levels(ctx, n_in, kept, sink):
 
 @pytest.mark.parametrize("n_in,kept,sink", [(1028, 514, 4), (1032, 516, 0), (2048, 1028, 4), (3000, 1500, 4), (2064, 1026, 1)])
 def test_gemm_four_blocks(ctx, n_in, kept, sink):
-    """The four-block form at its edges: the fewest kept rows it takes, a row more than one tile of 256, even and odd
-    kept / 2 (an even one leaves a component without a partner), inputs that are no whole number of 64-row slices."""
+    """Lengths the four blocks could take at their edges, in calls too small for them: the fewest kept rows, a row more than one
+    tile of 256, even and odd kept / 2, inputs that are no whole number of 64-row slices."""
     w = small(cap=n_in + sink + 3, dtype=torch.bfloat16, sink=sink, outliers=2, B=1, Ly=2, H=2)
     parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM)
     parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM, row_pad=8)
+
+
+@pytest.mark.parametrize("n_in,kept,sink,H", [(2044, 1022, 4, 20), (4096, 1024, 0, 20), (3076, 1538, 4, 10), (4096, 2048, 4, 10), (2200, 1650, 1, 10), (8188, 4094, 4, 5)])
+def test_gemm_runs_four_blocks(ctx, n_in, kept, sink, H):
+    """Calls that run four blocks, at the edges of their tiles: one whole tile of 256 quarter rows (511 and 512 half rows), a tile and
+    129 rows, two whole tiles, four; even and odd kept / 2 (an even one leaves a component without a partner, so the last phase
+    runs on; the middle row of an odd one is its own mirror); rows that are 16- but not 32-byte aligned."""
+    assert fk.gemm_blocks(n_in, kept, 2 * H) == 4
+    w = small(cap=n_in + sink + 3, dtype=torch.bfloat16, sink=sink, outliers=2, B=1, Ly=2, H=H)
+    parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM, sample=6)
+    parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM, row_pad=8, sample=6)
+
+
+@pytest.mark.parametrize("pairs,n_in,kept", [(256, 2400, 1200), (256, 1028, 514), (8, 4092, 2046)])
+def test_one_level_where_it_is_faster(ctx, pairs, n_in, kept):
+    """Lengths and sizes of call at which four blocks cost 15 to 35 % more than one level of the fold, which a retained band above
+    the lowest component always runs: the compression takes no longer than such a band (median of alternating
+    runs; the two launch the same work)."""
+    ctx.set_variant(fk.AUTO)
+    k, v = (torch.randn(1, 1, pairs, n_in, 128, device="cuda").bfloat16() for _ in range(2))
+    times = {0: [], 1: []}
+    for i in range(40):
+        for first in (0, 1):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            torch.cuda._sleep(200_000)  # the launches wait on the device: no host time between the events
+            a.record()
+            ctx.compress_band(k, v, n_in, kept, 0, first)
+            b.record()
+            b.synchronize()
+            if i >= 5:
+                times[first].append(a.elapsed_time(b))
+            k.fill_(1.0)
+            v.fill_(1.0)
+    low, band = (float(np.median(times[f])) for f in (0, 1))
+    assert low <= 1.08 * band, f"{1e3 * low:.1f} us against {1e3 * band:.1f} us"
+
+
+@pytest.mark.parametrize("row_pad", [0, 8])
+def test_ragged_batch_mixes_four_blocks_and_one_level(ctx, row_pad):
+    """Sequences of four blocks with even kept / 2 (their last phase runs on through p) and with odd, beside one-level ones: phase
+    counts and depths change from tile to tile.  Whole rows and rows that are 16- but not 32-byte aligned; against the oracle and,
+    sequence by sequence, against the call on its own, which keeps the four blocks' pairs in bf16."""
+    w = small(cap=8200, dtype=torch.bfloat16, sink=4, B=4, Ly=2, H=10, outliers=2)
+    (_, k), (_, v) = parity.guarded_cache(w, torch.device("cuda"), fill_len=8200, row_pad=row_pad)
+    k_in, v_in = k.clone(), v.clone()
+    lens, kept = [8196, 523, 8192, 3002], [4096, 259, 4094, 1499]
+    ctx.set_variant(fk.AUTO)
+    assert ctx.compress_ragged(k, v, lens, kept, 4) == [4 + x for x in kept] and ctx.last_device_status() == fk.OK
+    for b in range(4):
+        one_k, one_v = k_in[b:b + 1].clone(), v_in[b:b + 1].clone()
+        ctx.compress(one_k, one_v, lens[b], kept[b], 4)
+        for t_in, t_out, one in ((k_in, k, one_k), (v_in, v, one_v)):
+            assert torch.equal(t_out[b, :, :, :4], t_in[b, :, :, :4]) and torch.equal(t_out[b, :, :, 4 + kept[b]:], t_in[b, :, :, 4 + kept[b]:])
+            a, c = one[0, :, :, 4:4 + kept[b]].double(), t_out[b, :, :, 4:4 + kept[b]].double()
+            assert ((a - c).norm() / c.norm()).item() < 5e-3
+        for t_in, t_out, l, h in ((k_in, k, 0, 0), (v_in, v, 1, 9)):
+            want = oracle.compress_matrix(parity.to_f64(t_in[b, l, h, 4:lens[b]]), kept[b])
+            parity.check_matrix(parity.to_f64(t_out[b, l, h, 4:4 + kept[b]]), want, torch.bfloat16, f"sequence {b}")
 
 
 @pytest.mark.parametrize("n_in,kept,hd,H", [(68, 34, 128, 2), (65, 33, 8, 1), (67, 1, 128, 1), (252, 64, 72, 3), (510, 254, 128, 2), (1001, 500, 256, 2),
