@@ -246,15 +246,15 @@ def test_context_creation_does_not_wait_for_enqueued_work():
 def test_attend_work_area_follows_growing_lengths_once():
     """A batch whose lengths grow, as a decode stream's do, is split into more and more CTAs: the work area grows once for all
     of it (every time would mean a device synchronisation in the middle of the stream)."""
-    ctx = fk.Context(0)
     k = torch.zeros(64, 1, 8, 2048, 128, device="cuda", dtype=torch.bfloat16)
     q = torch.zeros(64, 64, 128, device="cuda", dtype=torch.bfloat16)
     v, out = torch.ones_like(k), torch.empty_like(q)
-    free = []
-    for n in (100, 250, 500, 900, 1400, 2048):
-        ctx.attend_decode(k, v, 0, q, [n] * 64, out=out)
-        torch.cuda.synchronize()
-        free.append(torch.cuda.mem_get_info()[0])
-        assert (out == 1).all()
+    for attempt in range(2):     # the first also loads the kernels, which takes memory of its own
+        ctx, free = fk.Context(0), []
+        for n in (100, 250, 500, 900, 1400, 2048):
+            ctx.attend_decode(k, v, 0, q, [n] * 64, out=out)
+            torch.cuda.synchronize()
+            free.append(torch.cuda.mem_get_info()[0])
+            assert (out == 1).all()
+        ctx.close()
     assert len(set(free)) <= 2, free
-    ctx.close()
