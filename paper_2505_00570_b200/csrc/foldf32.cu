@@ -12,7 +12,13 @@
 //                        the order they are read in).  Bound by FFMA issue: a thread owns 8 x 8 products, 64 FFMA for
 //                        four 16-byte shared-memory loads, and a warp reads 4 x 8 distinct vectors of each operand.
 //   unfold_f32_kernel    combines the blocks and stores the 2 or 4 output rows of each folded row into the cache.
-// Only the first kernel reads the cache and only the last one writes it: safe in place.
+// Only the last kernel writes the cache, and the ones before it are done reading it by then: safe in place.
+//
+// Large values.  An infinite element is infinite in every folded row it enters, so sums and differences of these would be NaN where
+// the plain product has an infinity, and values near the end of the range would overflow in a sum of four.  The fold therefore looks at
+// the magnitudes that pass through it (free: it waits for memory), and a matrix with an element of 2^100 or more takes the
+// plain product after all, with its entries evaluated on the spot.  Below that nothing overflows: entries are below 1, |p|, |q| and
+// a sum of four below 2^102, and four sums of 2^23 of these below the end of the range.
 //
 // Measured against the plain product (64 matrices of 128 channels unless said): 2044 -> 1022 959 -> 212 us, odd lengths
 // 2043 -> 1021 959 -> 387 us, 4000 -> 2000 3655 -> 1040 us, 2 matrices 2044 -> 1022 107 -> 23 us; error against 64 bits
@@ -20,17 +26,34 @@
 // products of each and took 253 us.)
 #include <algorithm>
 
+#include "basis.cuh"
 #include "common.cuh"
 
 namespace freqkv {
 namespace {
 
 constexpr int TK = 16, STAGES = 3;
+constexpr int MOST_SHARES = 64;                 // blocks per matrix of the first and the last kernel
+constexpr float LARGE = 1.2676506002282294e30f;  // 2^100
+
+__device__ __forceinline__ float largest(float m, const float4& v)
+{
+    return fmaxf(fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));  // a NaN is no obstacle to folding
+}
+
+// Has a block of the fold seen a large value of this matrix?  The same answer for all threads of the block.
+__device__ __forceinline__ bool any_large(const int32_t* flags, int32_t mat, int32_t shares)
+{
+    int32_t f = 0;
+    for (int32_t i = threadIdx.x; i < shares; i += blockDim.x) f |= __ldg(flags + (size_t)mat * MOST_SHARES + i);
+    return __syncthreads_or(f);
+}
 
 // Planes of one matrix: [blocks][rows of a plane][head_dim]; rows = ceil(n_in / blocks).
 template <int BLOCKS>
 __global__ void __launch_bounds__(256) fold_f32_kernel(const CacheView view, int32_t first, int32_t n_in, int32_t sink,
-                                                       const float2* __restrict__ turns, float4* __restrict__ planes)
+                                                       const float2* __restrict__ turns, float4* __restrict__ planes,
+                                                       int32_t* __restrict__ flags)
 {
     const uint32_t vecs = (uint32_t)view.head_dim / 4;
     const uint32_t rows = (uint32_t)(n_in + BLOCKS - 1) / BLOCKS, plane = rows * vecs;
@@ -39,10 +62,12 @@ __global__ void __launch_bounds__(256) fold_f32_kernel(const CacheView view, int
                      (int64_t)sink * view.stride_token;
     float4* out = planes + (size_t)blockIdx.x * BLOCKS * plane;
     auto row = [&](int32_t n, uint32_t vec) { return __ldg(reinterpret_cast<const float4*>(x + (int64_t)n * view.stride_token) + vec); };
+    float most = 0.f;
     for (uint32_t i = blockIdx.y * blockDim.x + threadIdx.x; i < plane; i += gridDim.y * blockDim.x) {
         const int32_t n = (int32_t)(i / vecs);
         const uint32_t vec = i - (uint32_t)n * vecs;
         const float4 a = row(n, vec), b = row(n_in - 1 - n, vec);
+        most = largest(largest(most, a), b);
         const float4 u = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
         const float4 v = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
         if constexpr (BLOCKS == 2) {
@@ -51,6 +76,7 @@ __global__ void __launch_bounds__(256) fold_f32_kernel(const CacheView view, int
             out[plane + i] = v;
         } else {
             const float4 c = row(n_in / 2 - 1 - n, vec), d = row(n_in / 2 + n, vec);
+            most = largest(largest(most, c), d);
             const float4 u2 = make_float4(c.x + d.x, c.y + d.y, c.z + d.z, c.w + d.w);
             const float4 v2 = make_float4(c.x - d.x, c.y - d.y, c.z - d.z, c.w - d.w);
             const float2 t = __ldg(turns + n);
@@ -62,6 +88,8 @@ __global__ void __launch_bounds__(256) fold_f32_kernel(const CacheView view, int
                                              fmaf(t.x, v.w, t.y * v2.w));   // p
         }
     }
+    const int32_t large = __syncthreads_or(most >= LARGE);
+    if (threadIdx.x == 0) flags[(size_t)blockIdx.x * MOST_SHARES + blockIdx.y] = large;
 }
 
 struct ProductParams {
@@ -70,6 +98,11 @@ struct ProductParams {
     float* out;              // [matrix][blocks][rows_out][head_dim]
     int32_t head_dim, blocks, m_pad, basis_k;
     int32_t rows, rows_last, rows_out;  // folded rows of a plane; rows the last block's product runs over (q, or q and then p)
+    const int32_t* flags;    // [matrix][MOST_SHARES]: large values seen by the fold's blocks, of which there are `shares`
+    int32_t shares;
+    // the plain product of a matrix with large values
+    CacheView view;
+    int32_t first, n_in, n_keep, sink;
 };
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid)
@@ -78,10 +111,60 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 
+// The plain product for this CTA's share of a matrix with large values: of the blocks * rows_out rows that the matrix has in `out`,
+// the first n_keep are its output rows as they are.  Entries, order of the sums and rounding are project_simt_kernel's.
+template <int TM, int TN, int M, int N>
+__device__ __noinline__ void plain_product(const ProductParams& p, float (*As)[TM], float (*Bs)[TN], int32_t mat, int32_t block, int32_t m0, int32_t c0,
+                                           int ty, int tx)
+{
+    constexpr int THREADS = TM / M * TN / N;
+    const int32_t index = p.first + mat, tensor = index / p.view.mats_per_tensor;
+    const float* x = static_cast<const float*>(tensor_base(p.view, tensor)) + matrix_offset(p.view, index % p.view.mats_per_tensor) +
+                     (int64_t)p.sink * p.view.stride_token;
+    const int32_t row0 = block * p.rows_out + m0;
+    float acc[M][N] = {};
+#pragma unroll 1
+    for (int32_t k0 = 0; k0 < p.n_in; k0 += TK) {
+        __syncthreads();
+#pragma unroll 1
+        for (int idx = threadIdx.x; idx < TK * TM; idx += THREADS) {
+            const int k = idx / TM, m = idx % TM;
+            const bool ok = k0 + k < p.n_in && m0 + m < p.rows_out && row0 + m < p.n_keep;
+            As[k][m] = ok ? (float)basis_entry(row0 + m, k0 + k, p.n_in, p.n_keep, 0) : 0.f;
+        }
+#pragma unroll 1
+        for (int idx = threadIdx.x; idx < TK * TN / 4; idx += THREADS) {
+            const int k = idx / (TN / 4), c = idx % (TN / 4) * 4;
+            const bool ok = k0 + k < p.n_in && c0 + c < p.head_dim;
+            *reinterpret_cast<float4*>(&Bs[k][c]) =
+                ok ? *reinterpret_cast<const float4*>(x + (int64_t)(k0 + k) * p.view.stride_token + c0 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int k = 0; k < min(TK, p.n_in - k0); ++k) {
+#pragma unroll
+            for (int i = 0; i < M; ++i)
+#pragma unroll
+                for (int j = 0; j < N; ++j) acc[i][j] = fmaf(As[k][ty + i / 4 * 16 + i % 4], Bs[k][tx + j / 4 * 32 + j % 4], acc[i][j]);
+        }
+    }
+    float* out = p.out + (size_t)(mat * p.blocks + block) * p.rows_out * p.head_dim;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        const int32_t m = m0 + ty + i / 4 * 16 + i % 4;
+        if (m >= p.rows_out) continue;
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const int32_t c = c0 + tx + j / 4 * 32 + j % 4;
+            if (c < p.head_dim) out[(size_t)m * p.head_dim + c] = acc[i][j];
+        }
+    }
+}
+
 // grid: x = matrix * blocks + block, y = TM folded output rows, z = TN channels.  A warp covers 4 M x 8 N products: lane
 // (ly, lx) has rows ly * 4 + 16 i and channels lx * 4 + 32 j, four of each.
 template <int TM, int TN, int M, int N>
-__global__ void __launch_bounds__(TM / M * TN / N) product_f32_kernel(const ProductParams p)
+__global__ void __launch_bounds__(TM / M * TN / N) product_f32_kernel(const __grid_constant__ ProductParams p)
 {
     constexpr int THREADS = TM / M * TN / N, WARPS_N = TN / (8 * N);
     constexpr int A_VECS = TK * TM / 4, B_VECS = TK * TN / 4;  // 16-byte vectors of a stage
@@ -123,6 +206,11 @@ __global__ void __launch_bounds__(TM / M * TN / N) product_f32_kernel(const Prod
     float acc[M][N] = {};
 #pragma unroll
     for (int s = 0; s < STAGES - 1; ++s) fetch(s);
+    if (any_large(p.flags, mat, p.shares)) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        plain_product<TM, TN, M, N>(p, As[0], Bs[0], mat, block, m0, c0, ty, tx);
+        return;
+    }
     int stage = 0;
 #pragma unroll 1
     for (int32_t st = 0; st < steps; ++st) {
@@ -160,7 +248,7 @@ __global__ void __launch_bounds__(TM / M * TN / N) product_f32_kernel(const Prod
 // One thread per folded row and four channels; grid as fold_f32_kernel's.
 template <int BLOCKS>
 __global__ void __launch_bounds__(256) unfold_f32_kernel(const CacheView view, int32_t first, int32_t n_keep, int32_t sink,
-                                                         const float4* __restrict__ sums)
+                                                         const float4* __restrict__ sums, const int32_t* __restrict__ flags, int32_t shares)
 {
     const uint32_t vecs = (uint32_t)view.head_dim / 4;
     const int32_t rows_half = (n_keep + 1) / 2, rows_out = BLOCKS == 2 ? rows_half : (rows_half + 1) / 2;
@@ -169,6 +257,14 @@ __global__ void __launch_bounds__(256) unfold_f32_kernel(const CacheView view, i
     float* y = static_cast<float*>(tensor_base(view, tensor)) + matrix_offset(view, mat % view.mats_per_tensor) +
                (int64_t)sink * view.stride_token;
     const float4* in = sums + (size_t)blockIdx.x * BLOCKS * plane;
+    if (any_large(flags, (int32_t)blockIdx.x, shares)) {  // the output rows themselves
+        const uint32_t total = (uint32_t)n_keep * vecs;
+        for (uint32_t i = blockIdx.y * blockDim.x + threadIdx.x; i < total; i += gridDim.y * blockDim.x) {
+            const uint32_t m = i / vecs;
+            reinterpret_cast<float4*>(y + (int64_t)m * view.stride_token)[i - m * vecs] = __ldg(in + i);
+        }
+        return;
+    }
     for (uint32_t i = blockIdx.y * blockDim.x + threadIdx.x; i < plane; i += gridDim.y * blockDim.x) {
         const int32_t m = (int32_t)(i / vecs);
         const uint32_t vec = i - (uint32_t)m * vecs;
@@ -219,9 +315,17 @@ cudaError_t launch_blocks(const CacheView& view, int32_t first, int32_t count, c
     p.rows_last = BLOCKS == 4 && basis.n_keep / 2 % 2 == 0 ? 2 * p.rows : p.rows;
     p.rows_out = BLOCKS == 2 ? rows_half : (rows_half + 1) / 2;
     p.out = scratch + (size_t)count * BLOCKS * p.rows * view.head_dim;
-    auto share = [&](int32_t rows) { return (unsigned)std::min<int64_t>(((int64_t)rows * (view.head_dim / 4) + 255) / 256, 64); };
+    auto share = [&](int32_t rows) { return (unsigned)std::min<int64_t>(((int64_t)rows * (view.head_dim / 4) + 255) / 256, MOST_SHARES); };
+    int32_t* flags = reinterpret_cast<int32_t*>(p.out + (size_t)count * BLOCKS * p.rows_out * view.head_dim);
+    p.flags = flags;
+    p.shares = (int32_t)share(p.rows);
+    p.view = view;
+    p.first = first;
+    p.n_in = basis.n_in;
+    p.n_keep = basis.n_keep;
+    p.sink = sink;
     fold_f32_kernel<BLOCKS><<<dim3((unsigned)count, share(p.rows)), 256, 0, stream>>>(view, first, basis.n_in, sink, basis.f32_turns,
-                                                                                    reinterpret_cast<float4*>(scratch));
+                                                                                    reinterpret_cast<float4*>(scratch), flags);
     // 8 x 8 products a thread take the fewest shared-memory loads, 4 x 4 spread few matrices over more SMs (2 matrices of
     // 2044 -> 1022: 41 and 23 us).  Tiles of 128 rows read the folded inputs least often; where they would leave much of
     // the last one empty, tiles of 32 (64 matrices of 256 rows a block 212 and 222 us, 16 of 281 rows 75 and 58 us).
@@ -234,7 +338,7 @@ cudaError_t launch_blocks(const CacheView& view, int32_t first, int32_t count, c
     else
         launch_product<32, 64, 8, 8>(p, count, stream);
     unfold_f32_kernel<BLOCKS><<<dim3((unsigned)count, share(p.rows_out)), 256, 0, stream>>>(view, first, basis.n_keep, sink,
-                                                                                         reinterpret_cast<const float4*>(p.out));
+                                                                                         reinterpret_cast<const float4*>(p.out), flags, p.shares);
     return cudaGetLastError();
 }
 
@@ -247,7 +351,8 @@ size_t fold_f32_scratch_bytes(int32_t n_in, int32_t n_keep, int32_t head_dim)
 {
     const int32_t blocks = fold_f32_blocks(n_in, n_keep), rows_half = (n_keep + 1) / 2;
     const int32_t rows = (n_in + blocks - 1) / blocks, rows_out = blocks == 2 ? rows_half : (rows_half + 1) / 2;
-    return (size_t)blocks * (rows + rows_out) * head_dim * sizeof(float);  // the folded inputs, the blocks' products
+    // the folded inputs, the blocks' products, the fold's flags
+    return (size_t)blocks * (rows + rows_out) * head_dim * sizeof(float) + MOST_SHARES * sizeof(int32_t);
 }
 
 cudaError_t launch_fold_f32(const CacheView& view, int32_t first, int32_t count, const Basis& basis, int32_t sink, void* scratch,

@@ -328,6 +328,41 @@ def test_folded_fp32(ctx, n_in, kept, hd, H):
     parity.check_compress(ctx, w, n_in + 3, kept, 3, fk.AUTO, sample=6, row_pad=8)
 
 
+@pytest.mark.parametrize("n_in,kept,hd,H", [(68, 34, 128, 2), (255, 127, 72, 3), (1001, 500, 256, 2), (1004, 502, 64, 40), (777, 389, 128, 80)])
+def test_folded_fp32_infinities_and_large_values(ctx, n_in, kept, hd, H):
+    """What the plain product makes of infinities, NaN and values that overflow in a sum of mirrored rows is what the folded one makes
+    of them, bit for bit; matrices without any keep the bits they have without those neighbours.  Four blocks and one level, the three
+    tiles of the product, head sizes that are no whole tile."""
+    sink, cap = 3, n_in + 5
+    w = small(cap=cap, hd=hd, sink=sink, Ly=1, H=H)
+    k0, v0 = synth.make_cache(w, "cuda")
+    planted = [(k0, 0, 0, 5, float("inf")), (k0, 0, n_in - 1, hd - 1, -float("inf")), (v0, 0, n_in // 2, 1, 3.0e38), (v0, 0, n_in - 1 - n_in // 2, 1, 3.0e38),
+               (v0, H - 1, 7, 0, float("inf")), (v0, H - 1, 9, 0, float("nan")), (k0, H - 1, 3, 2, -3.0e38), (k0, H - 1, n_in - 4, 2, 3.0e38)]
+    out = {}
+    for plant in (False, True):
+        for variant in (fk.AUTO, fk.SIMT):
+            k, v = k0.clone(), v0.clone()
+            if plant:
+                for src, h, n, c, x in planted:
+                    (k if src is k0 else v)[0, 0, h, sink + n, c] = x
+            ctx.set_variant(variant)
+            ctx.compress(k, v, n_in + sink, kept, sink)
+            out[plant, variant] = torch.stack([k, v])[:, 0, 0].view(torch.int32)
+    ctx.set_variant(fk.AUTO)
+    got, plain, clean = out[True, fk.AUTO], out[True, fk.SIMT], out[False, fk.AUTO]
+    assert not torch.equal(clean, out[False, fk.SIMT])          # two different products
+    touched = {0, H - 1}
+    for h in range(H):
+        for t in range(2):
+            a, b = got[t, h].view(torch.float32), plain[t, h].view(torch.float32)
+            if h in touched:
+                assert torch.equal(torch.isnan(a), torch.isnan(b))
+                assert torch.equal(a.nan_to_num(nan=0.0, posinf=1.0, neginf=-1.0), b.nan_to_num(nan=0.0, posinf=1.0, neginf=-1.0)), (t, h)
+            else:
+                assert torch.equal(got[t, h], clean[t, h])
+    assert torch.isinf(got[0, 0, sink:sink + kept, 5].view(torch.float32)).all()
+
+
 def test_gemm_batch_layers_heads_and_padding(ctx):
     w = small(cap=333, dtype=torch.bfloat16, sink=4, outliers=2, B=2, Ly=3, H=2)
     parity.check_compress(ctx, w, 330, 163, 4, fk.GEMM)
