@@ -728,10 +728,13 @@ freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_
     }
     if (variant == FREQKV_GEMM && dtype != FREQKV_BF16) return FREQKV_ERR_UNSUPPORTED;
     Basis b;
-    const bool gemm = variant == FREQKV_GEMM;
-    const bool both = variant == FREQKV_AUTO;
-    const bool folded = !gemm && fold_f32_applies(ctx, dtype, n_in, 0);
-    return get_basis(ctx, n_in, n_keep, 0, (!gemm && !folded) || both, (gemm || both) && dtype == FREQKV_BF16, stream, &b, folded);
+    if (dtype == FREQKV_F32) {
+        // the folded planes serve every call but one that asks for the CUDA-core variant by name (now or, on a context that does not
+        // force it yet, later): a plan of that variant has the plain matrix too
+        const bool folded = fold_f32_applies(ctx, dtype, n_in, 0);
+        return get_basis(ctx, n_in, n_keep, 0, !folded || variant == FREQKV_SIMT, false, stream, &b, folded);
+    }
+    return get_basis(ctx, n_in, n_keep, 0, variant != FREQKV_GEMM, variant != FREQKV_SIMT, stream, &b);
 }
 
 freqkv_status freqkv_check_compress(const freqkv_layout* layout, const void* k, const void* v, int32_t cache_len,

@@ -579,3 +579,23 @@ def test_auto_picks_documented_variants(ctx):
     assert ctx.resolve_variant(f32, 512, 256) == fk.FDCT
     assert ctx.resolve_variant(f32, 500, 250) == fk.SIMT
     assert ctx.resolve_variant(bf, 100, 50) == fk.SIMT
+
+
+def test_fp32_plans_hold_what_the_calls_read():
+    """The kernels that a plan launches are its table builders: AUTO's calls read the folded planes alone; a plan of the CUDA-core
+    variant by name serves both the unforced call and the forced one, which must build nothing more."""
+    k, v = (torch.randn(1, 1, 2, 2044, 128, device="cuda") for _ in range(2))
+    ctx = fk.Context(0)
+
+    def launches(call):
+        before = ctx.get_timing()[2]
+        call()
+        return ctx.get_timing()[2] - before
+
+    compress = lambda: ctx.compress(k, v, 2044, 1022, 0)  # noqa: E731
+    assert launches(lambda: ctx.plan(2044, 1022, fk.F32, fk.AUTO)) == 1 and launches(compress) == 3    # fold, product, unfold
+    assert launches(lambda: ctx.plan(2044, 1020, fk.F32, fk.SIMT)) == 2
+    assert launches(lambda: ctx.compress(k, v, 2044, 1020, 0)) == 3
+    ctx.set_variant(fk.SIMT)
+    assert launches(lambda: ctx.compress(k, v, 2044, 1020, 0)) == 2                                    # product, copy back
+    ctx.close()
