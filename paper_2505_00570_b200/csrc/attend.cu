@@ -839,12 +839,17 @@ cudaError_t launch_typed(const AttendParams& prm, int32_t g, int32_t nb, int32_t
         auto* kernel = prm.tickets ? with_tickets : without;
         launch_attention(kernel, grid, THREADS, 0, stream, prm, overlap);
     };
-    switch (g) {
-        case 1: launch(attend_partial_kernel<T, 1, true>, attend_partial_kernel<T, 1, false>); break;
-        case 2: launch(attend_partial_kernel<T, 2, true>, attend_partial_kernel<T, 2, false>); break;
-        case 4: launch(attend_partial_kernel<T, 4, true>, attend_partial_kernel<T, 4, false>); break;
-        case 8: launch(attend_partial_kernel<T, 8, true>, attend_partial_kernel<T, 8, false>); break;
-        default: return cudaErrorInvalidValue;
+    if (g == 1) {
+        launch(attend_partial_kernel<T, 1, true>, attend_partial_kernel<T, 1, false>);
+    } else if constexpr (sizeof(T) == 4) {  // grouped queries of bf16 caches take launch_mma
+        switch (g) {
+            case 2: launch(attend_partial_kernel<T, 2, true>, attend_partial_kernel<T, 2, false>); break;
+            case 4: launch(attend_partial_kernel<T, 4, true>, attend_partial_kernel<T, 4, false>); break;
+            case 8: launch(attend_partial_kernel<T, 8, true>, attend_partial_kernel<T, 8, false>); break;
+            default: return cudaErrorInvalidValue;
+        }
+    } else {
+        return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
