@@ -64,7 +64,9 @@ typedef enum { FREQKV_BF16 = 0, FREQKV_F32 = 1 } freqkv_dtype;
  *         <= 128: 4096 -> 2048), complex with twiddles.  fp32 caches: a radix-16 kernel for
  *         power-of-two lengths;
  *   SIMT  the same projection on the fp32 CUDA cores (any shape; the only path for fp32
- *         caches of non-power-of-two length);
+ *         caches of non-power-of-two length).  Where AUTO comes to it for an fp32 cache of at least
+ *         64 rows it runs a form with half or a quarter of the multiply-adds (the symmetries of
+ *         the basis taken out first, all in fp32); asked for by name it is the plain product;
  *   AUTO  picks per shape from a table filled from measurements. */
 typedef enum { FREQKV_AUTO = 0, FREQKV_GEMM = 1, FREQKV_FDCT = 2, FREQKV_SIMT = 3 } freqkv_variant;
 
@@ -106,13 +108,15 @@ freqkv_status freqkv_set_variant(freqkv_ctx* ctx, freqkv_variant variant);
 freqkv_status freqkv_set_fast_family(freqkv_ctx* ctx, int32_t family);
 
 /* Which variant AUTO (or the forced setting) resolves to for this shape; FREQKV_AUTO is never
- * returned.  Returns FREQKV_ERR_UNSUPPORTED through *out_variant = -1 when none applies. */
+ * returned (SIMT stands for both of its forms).  Returns FREQKV_ERR_UNSUPPORTED through *out_variant = -1 when none applies. */
 freqkv_status freqkv_resolve_variant(freqkv_ctx* ctx, const freqkv_layout* layout, int32_t n_in, int32_t n_keep,
                                      int32_t* out_variant);
 
 /* Optional warm-up: build and cache whatever tables the given variant needs to compress
  * n_in non-sink rows to n_keep rows (the projection basis of Eq. 2-3 folded with the
- * definitions of Appendix A, or the transform twiddles).  Work is enqueued on `cuda_stream`.
+ * definitions of Appendix A, or the transform twiddles).  For fp32, AUTO builds what AUTO's calls
+ * read and SIMT what they and the calls that ask for SIMT by name read.  Work is enqueued on
+ * `cuda_stream`.
  * Calling freqkv_compress without it builds the plan on first use. */
 freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_dtype dtype,
                           freqkv_variant variant, void* cuda_stream);
@@ -124,7 +128,9 @@ freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_
  *     y = sqrt(L/N) * IDCT_L(z[0:L])               (L-point orthonormal inverse).
  * y is rounded once (nearest even) to the cache dtype and written to rows [sink, sink+L).
  * Nothing else is written: sink rows, rows >= sink+L and any stride padding keep their bytes.
- * The caller's new cache length is sink + kept_len.  Arithmetic: fp32 accumulation.
+ * The caller's new cache length is sink + kept_len.  Arithmetic: fp32 accumulation.  Infinities and
+ * NaN stay in their channel; in bf16 caches an infinity may come out as NaN, and so may values
+ * whose sum over four mirrored rows leaves the range (above a quarter of the largest value).
  * kept_len == cache_len - sink is the identity and enqueues nothing; kept_len == 0 or
  * cache_len == sink enqueue nothing.
  * Errors: INVALID_ARG (null pointers, sink < 0, sink > cache_len, cache_len > capacity,
@@ -235,7 +241,13 @@ freqkv_status freqkv_compress_host(freqkv_ctx* ctx, const freqkv_layout* layout,
  *           must then stay below 65504 in magnitude (larger values give infinities).
  *   scale   score scale; <= 0 selects 1/sqrt(head_dim).
  *   lens    HOST array of `batch` cache lengths, each in [1, capacity].
- * Nothing in the cache is written.  Errors: INVALID_ARG (null pointers, q == out, layer out of
+ * Nothing in the cache is written.  The launches of a call let a following launch start early that asks for it
+ * (programmatic stream serialization): a kernel launched so behind this call has to wait for its
+ * predecessor itself (griddepcontrol.wait) before it reads `out`; any other launch is ordered as usual.
+ * The call may be captured into a graph, on the stream of the context's last call and after a call that
+ * allocated what it needs; replays use the context's work areas, so the caller keeps them apart from its
+ * other calls, and a later call of a larger batch or of longer lengths may move them.
+ * Errors: INVALID_ARG (null pointers, q == out, layer out of
  * range, a length outside [1, capacity], NaN scale or base), UNSUPPORTED (head_dim != 128,
  * q_heads_per_kv not 1, 2, 4 or 8, misaligned pointers, layout rules), ALLOC, CUDA.  The first call
  * with a new rope_base builds a cos/sin table (capacity x head_dim/2 entries) the context keeps. */
@@ -268,7 +280,7 @@ freqkv_status freqkv_attend_prefill(freqkv_ctx* ctx, const freqkv_layout* layout
 
 /* Instrumentation for benchmarks.  With timing enabled every compression records a CUDA event
  * pair on the caller's stream around its transform kernel (the projection / fast-transform
- * launch, not the copy-back or table builders).  freqkv_get_timing waits for the recorded
+ * launch, not the copy-back or table builders; the folded fp32 product's three launches together).  freqkv_get_timing waits for the recorded
  * events, returns the number of timed transform launches and their summed device time in
  * milliseconds since the last call, plus the number of kernels of any kind this context has
  * launched since creation, and resets the timing sums.  Any output pointer may be NULL. */
