@@ -397,7 +397,8 @@ __device__ __forceinline__ void fold8_quad(const uint4& a, const uint4& b, const
     *q = make_uint4(o[3][0], o[3][1], o[3][2], o[3][3]);
 }
 
-// Four blocks: as fold_one_level; job.n_half = N' rows per plane; a thread folds two vectors per round.
+// Four blocks: as fold_one_level; job.n_half = N' rows per plane; a thread folds VECS vectors per round.
+template <int VECS>
 __device__ __forceinline__ void fold_four_blocks(const CacheView& view, const FoldJob& job, uint32_t pt, const float2* __restrict__ turns)
 {
     const char* x = static_cast<const char*>(tensor_base(view, pt & 1)) +
@@ -407,11 +408,11 @@ __device__ __forceinline__ void fold_four_blocks(const CacheView& view, const Fo
     const uint32_t total = (uint32_t)n_quarter * 16u;                // vectors of uu (= of uv, q, p)
     uint4* plane0 = job.dst + (int64_t)pt * 2 * ((int64_t)job.n_half * 16);
     uint4* plane1 = plane0 + (int64_t)job.n_half * 16;
-    for (uint32_t c0 = blockIdx.y * 512u; c0 < total; c0 += gridDim.y * 512u) {
-        uint4 a[2], b[2], c[2], d[2];
-        float2 cs[2];
+    for (uint32_t c0 = blockIdx.y * (VECS * 256u); c0 < total; c0 += gridDim.y * (VECS * 256u)) {
+        uint4 a[VECS], b[VECS], c[VECS], d[VECS];
+        float2 cs[VECS];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
+        for (int j = 0; j < VECS; ++j) {
             const uint32_t i = c0 + j * 256u + threadIdx.x;
             if (i < total) {
                 const int32_t n = (int32_t)(i >> 4);
@@ -423,7 +424,7 @@ __device__ __forceinline__ void fold_four_blocks(const CacheView& view, const Fo
             }
         }
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
+        for (int j = 0; j < VECS; ++j) {
             const uint32_t i = c0 + j * 256u + threadIdx.x;
             if (i < total) {
                 uint4 uu, uv, p, q;
@@ -444,14 +445,16 @@ __global__ void __launch_bounds__(256) fold_kernel(const CacheView view, const F
 // less, and 0.02 ms of a 7B-shaped fold.)
 __global__ void __launch_bounds__(256) fold_quad_kernel(const CacheView view, const FoldJob job, const float2* __restrict__ turns)
 {
-    fold_four_blocks(view, job, blockIdx.x, turns);
+    fold_four_blocks<2>(view, job, blockIdx.x, turns);
 }
 
+// (Four blocks of 256 threads an SM leave 64 registers, with which two vectors a round of the four-block branch spill; with one,
+// ragged batches take 1 to 3 % less: 64 matrices 1027 -> 513 41.9 -> 40.7 us, 512 matrices 8188 -> 4094 1108 -> 1087 us.)
 __global__ void __launch_bounds__(256, 4) fold_ragged_kernel(const CacheView view, const FoldJob* jobs, int32_t mats_per_seq)
 {
     const FoldJob job = jobs[blockIdx.x / mats_per_seq];
     if (job.turns)
-        fold_four_blocks(view, job, blockIdx.x % mats_per_seq, job.turns);
+        fold_four_blocks<1>(view, job, blockIdx.x % mats_per_seq, job.turns);
     else
         fold_one_level(view, job, blockIdx.x % mats_per_seq);
 }
