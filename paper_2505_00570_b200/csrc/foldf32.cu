@@ -18,7 +18,9 @@
 // the plain product has an infinity, and values near the end of the range would overflow in a sum of four.  The fold therefore looks at
 // the magnitudes that pass through it (free: it waits for memory), and a matrix with an element of 2^100 or more takes the
 // plain product after all, with its entries evaluated on the spot.  Below that nothing overflows: entries are below 1, |p|, |q| and
-// a sum of four below 2^102, and four sums of 2^23 of these below the end of the range.
+// a sum of four below 2^102, and four sums of 2^23 of these below the end of the range.  What the look at the flags costs: 64
+// matrices 2044 -> 1022 nothing (229 us with the append), few kept rows in tiles of one warp up to a tenth (4000 -> 16 161 -> 183 us, the
+// plain product 281; 66 -> 64 of 2048 matrices 50 -> 55, 62).
 //
 // Measured against the plain product (64 matrices of 128 channels unless said): 2044 -> 1022 959 -> 212 us, odd lengths
 // 2043 -> 1021 959 -> 387 us, 4000 -> 2000 3655 -> 1040 us, 2 matrices 2044 -> 1022 107 -> 23 us; error against 64 bits
