@@ -194,8 +194,8 @@ def test_ragged_batch_in_two_launches(ctx):
     and ONE tensor-core launch (the kernel counter says so); odd and even lengths, one sequence
     left alone (kept == length), one with more than one tile of rows.  Against the oracle, against
     the bytes outside the rewritten rows, and against compressing each sequence on its own: bit
-    for bit where that call runs the same arithmetic (one level of the symmetry fold), and to well
-    inside the tolerance where the lengths halve twice and the single call folds twice."""
+    for bit where both run one level of the symmetry fold, and to well inside the tolerance where the
+    lengths halve twice, so that larger calls would run four blocks."""
     w = small(cap=1400, dtype=torch.bfloat16, sink=4, B=6, Ly=2, H=3, outliers=2)
     k, v = synth.make_cache(w, "cuda")
     k_in, v_in = k.clone(), v.clone()
@@ -218,7 +218,7 @@ def test_ragged_batch_in_two_launches(ctx):
     for b in range(6):
         one_k, one_v = k_in[b:b + 1].clone(), v_in[b:b + 1].clone()
         ctx.compress(one_k, one_v, lens[b], kept[b], 4)
-        if (lens[b] - 4) % 4 == 0 and kept[b] % 2 == 0 and kept[b] > 256:   # the single call folds twice
+        if (lens[b] - 4) % 4 == 0 and kept[b] % 2 == 0 and kept[b] > 256:   # lengths of four blocks
             for one, both in ((one_k, k), (one_v, v)):
                 a, c = one[0, :, :, 4:4 + kept[b]].double(), both[b, :, :, 4:4 + kept[b]].double()
                 assert ((a - c).norm() / c.norm()).item() < 5e-3
