@@ -15,6 +15,7 @@
 
 #include "common.cuh"
 #include "gemm.cuh"
+#include "nearfar.cuh"
 #include "fdct.cuh"
 #include "dctmm.cuh"
 #include "attend.cuh"
@@ -253,6 +254,7 @@ void free_bases(freqkv_ctx* ctx)
         if (kv.second.fold) cudaFree(kv.second.fold);
         if (kv.second.dense) cudaFree(kv.second.dense);
         if (kv.second.f32_fold) cudaFree(kv.second.f32_fold);
+        if (kv.second.nearfar) cudaFree(kv.second.nearfar);
     }
     ctx->bases.clear();
     ctx->basis_bytes = 0;
@@ -277,9 +279,12 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
     if (it != ctx->bases.end()) b = it->second;
     // the tensor-core path wants the folded pair, or, for few kept rows, the dense bf16 matrix
     const bool direct = need_fold && first != kDctRows && gemm_is_direct(n_keep);
-    const bool make_f32 = need_f32 && !b.f32, make_fold = need_fold && !direct && !b.fold, make_dense = direct && !b.dense;
+    // (a plain compression: in one pass, nearfar.cu; retained bands and the spectrum: the folded pair)
+    const bool one_pass = need_fold && !direct && first == 0;
+    const bool make_f32 = need_f32 && !b.f32, make_fold = need_fold && !direct && !one_pass && !b.fold, make_dense = direct && !b.dense;
+    const bool make_nearfar = one_pass && !b.nearfar;
     const bool make_f32_fold = need_f32_fold && !b.f32_fold;
-    if (make_f32 || make_fold || make_dense || make_f32_fold) {
+    if (make_f32 || make_fold || make_dense || make_f32_fold || make_nearfar) {
         auto shape = [&](Basis& x) {
             x.n_in = n_in;
             x.n_keep = n_keep;
@@ -305,7 +310,9 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
         const int32_t f32_blocks = fold_f32_blocks(n_in, n_keep);
         const size_t f32_plane_elems = (size_t)f32_blocks * b.f32_fold_k * b.f32_fold_m;
         const size_t f32_fold_elems = f32_plane_elems + (f32_blocks == 4 ? (size_t)(n_in / 4) * 2 : 0);
-        const size_t want = (make_f32_fold ? f32_fold_elems * 4 : 0) + (make_f32 ? elems * 4 : 0) + (make_fold ? fold_elems * 2 : 0) + (make_dense ? dense_elems * 2 : 0);
+        const size_t nearfar_bytes = one_pass ? nearfar_shape(n_in, n_keep).bytes : 0;
+        const size_t want = (make_f32_fold ? f32_fold_elems * 4 : 0) + (make_f32 ? elems * 4 : 0) + (make_fold ? fold_elems * 2 : 0) + (make_dense ? dense_elems * 2 : 0) +
+                            (make_nearfar ? nearfar_bytes : 0);
         if (ctx->basis_bytes + want > kBasisBudgetBytes) {
             FREQKV_CUDA(ctx, cudaDeviceSynchronize());  // bases may be in use by enqueued kernels
             free_bases(ctx);
@@ -323,7 +330,7 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
                 return cuda_fail(ctx, e, "cudaMalloc(basis)");
             }
         }
-        if (need_fold && !direct && !b.fold) {
+        if (need_fold && !direct && !one_pass && !b.fold) {
             const cudaError_t e = cudaMalloc(&pb, fold_elems * 2);
             if (e != cudaSuccess) {
                 if (pf) cudaFree(pf);
@@ -340,8 +347,23 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
                 return cuda_fail(ctx, e, "cudaMalloc(basis)");
             }
         }
+        void* pn = nullptr;
+        if (one_pass && !b.nearfar) {
+            const cudaError_t e = cudaMalloc(&pn, nearfar_bytes);
+            if (e != cudaSuccess) {
+                if (pf) cudaFree(pf);
+                if (pb) cudaFree(pb);
+                if (pd) cudaFree(pd);
+                if (pq) cudaFree(pq);
+                return cuda_fail(ctx, e, "cudaMalloc(basis)");
+            }
+        }
         cudaError_t e = cudaSuccess;
-        if (pq) {
+        if (pn) {
+            e = launch_build_nearfar(pn, n_in, n_keep, stream);
+            ctx->kernels_launched += 2;
+        }
+        if (e == cudaSuccess && pq) {
             e = launch_build_fold_f32(pq, reinterpret_cast<float2*>(pq + f32_plane_elems), n_in, n_keep, f32_blocks, b.f32_fold_k,
                                       b.f32_fold_m, stream);
             ctx->kernels_launched += 1;
@@ -369,7 +391,13 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
             if (pb) cudaFree(pb);
             if (pd) cudaFree(pd);
             if (pq) cudaFree(pq);
+            if (pn) cudaFree(pn);
             return cuda_fail(ctx, e, "build_basis");
+        }
+        if (pn) {
+            b.nearfar = pn;
+            b.nearfar_bytes = (int64_t)nearfar_bytes;
+            ctx->basis_bytes += nearfar_bytes;
         }
         if (pq) {
             b.f32_fold = pq;
@@ -395,7 +423,8 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
 size_t basis_device_bytes(const Basis& b)
 {
     return (b.f32 ? (size_t)b.ld * b.rows_pad * 4 : 0) + (b.fold ? (size_t)b.fold_alloc_elems * 2 : 0) +
-           (b.dense ? (size_t)256 * b.ld * 2 : 0) + (b.f32_fold ? (size_t)b.f32_fold_alloc_elems * 4 : 0);
+           (b.dense ? (size_t)256 * b.ld * 2 : 0) + (b.f32_fold ? (size_t)b.f32_fold_alloc_elems * 4 : 0) +
+           (b.nearfar ? (size_t)b.nearfar_bytes : 0);
 }
 
 // Remove the plan of (n_in, n_keep, first) from the cache without freeing it: the caller owns its
@@ -415,6 +444,7 @@ void free_basis(Basis* b)
     if (b->fold) cudaFree(b->fold);
     if (b->dense) cudaFree(b->dense);
     if (b->f32_fold) cudaFree(b->f32_fold);
+    if (b->nearfar) cudaFree(b->nearfar);
     *b = Basis();
 }
 
@@ -535,9 +565,9 @@ freqkv_status compress_group(freqkv_ctx* ctx, const freqkv_layout& l, void* k, v
         hooks.before = [](void* u, cudaStream_t) { static_cast<TransformTimer*>(u)->begin(); };
         hooks.after = [](void* u, cudaStream_t) { static_cast<TransformTimer*>(u)->end(); };
         const cudaError_t e =
-            gemm_is_direct(n_keep)
-                ? launch_gemm_direct(gs, view, basis, sink, ctx->status_dev, ctx->sm_count, hooks, stream)
-                : launch_gemm(gs, view, basis, sink, ctx->status_dev, ctx->sm_count, hooks, stream);
+            gemm_is_direct(n_keep) ? launch_gemm_direct(gs, view, basis, sink, ctx->status_dev, ctx->sm_count, hooks, stream)
+            : first == 0 ? launch_nearfar(gs, view, {{0, batch_count, n_in, n_keep, basis.nearfar}}, sink, ctx->status_dev, ctx->sm_count, hooks, stream)
+                         : launch_gemm(gs, view, basis, sink, ctx->status_dev, ctx->sm_count, hooks, stream);
         if (e != cudaSuccess) return cuda_fail(ctx, e, gs->last_error ? gs->last_error : "launch_gemm");
         ctx->kernels_launched += gs->kernels_last_call;
         return FREQKV_OK;
@@ -874,7 +904,7 @@ freqkv_status freqkv_compress_ragged(freqkv_ctx* ctx, const freqkv_layout* layou
             if (variant[b] != FREQKV_GEMM || gemm_is_direct(kept_len[b])) all_folded = false;
         }
         if (all_folded && active > 1) {
-            std::vector<RaggedItem> items;
+            std::vector<NearFarItem> items;
             bool ok = true;
             for (int pass = 0; pass < 2 && ok; ++pass) {  // second pass: a flush of the plan cache may have dropped earlier plans
                 items.clear();
@@ -883,12 +913,12 @@ freqkv_status freqkv_compress_ragged(freqkv_ctx* ctx, const freqkv_layout* layou
                     Basis basis;
                     st = get_basis(ctx, lens[b] - sink, kept_len[b], 0, false, true, stream, &basis);
                     if (st != FREQKV_OK) return st;  // nothing enqueued but plan builders
-                    items.push_back({b, basis});
+                    items.push_back({b, 1, basis.n_in, basis.n_keep, basis.nearfar});
                 }
                 bool intact = true;
-                for (const RaggedItem& it : items) {
-                    auto found = ctx->bases.find(std::make_tuple(it.basis.n_in, it.basis.n_keep, (int32_t)0));
-                    if (found == ctx->bases.end() || found->second.fold != it.basis.fold) intact = false;
+                for (const NearFarItem& it : items) {
+                    auto found = ctx->bases.find(std::make_tuple(it.n_in, it.n_keep, (int32_t)0));
+                    if (found == ctx->bases.end() || found->second.nearfar != it.plan) intact = false;
                 }
                 if (intact) break;
                 if (pass == 1) ok = false;
@@ -901,14 +931,14 @@ freqkv_status freqkv_compress_ragged(freqkv_ctx* ctx, const freqkv_layout* layou
                 hooks.before = [](void* u, cudaStream_t) { static_cast<TransformTimer*>(u)->begin(); };
                 hooks.after = [](void* u, cudaStream_t) { static_cast<TransformTimer*>(u)->end(); };
                 ctx->gemm.last_error = nullptr;
-                const cudaError_t e = launch_gemm_ragged(&ctx->gemm, view, items, sink, ctx->status_dev, ctx->sm_count, hooks, stream);
+                const cudaError_t e = launch_nearfar(&ctx->gemm, view, items, sink, ctx->status_dev, ctx->sm_count, hooks, stream);
                 if (e == cudaSuccess) {
                     ctx->kernels_launched += ctx->gemm.kernels_last_call;
                     for (int32_t b = 0; b < layout->batch; ++b) lens[b] = sink + kept_len[b];
                     return FREQKV_OK;
                 }
                 if (e != cudaErrorMemoryAllocation || ctx->gemm.kernels_last_call != 0)
-                    return cuda_fail(ctx, e, ctx->gemm.last_error ? ctx->gemm.last_error : "launch_gemm_ragged");
+                    return cuda_fail(ctx, e, ctx->gemm.last_error ? ctx->gemm.last_error : "launch_nearfar");
                 cudaGetLastError();  // the folded batch does not fit: go sequence by sequence
             }
         }
@@ -1308,7 +1338,8 @@ freqkv_status freqkv_decode_graph_create(freqkv_ctx* ctx, const freqkv_layout* l
     }
     cudaError_t e = st == FREQKV_OK ? cudaStreamSynchronize(cs) : cudaSuccess;
     if (st == FREQKV_OK && e == cudaSuccess)
-        e = gemm_prepare(&dg->gemm, gemm_is_direct(kept_len) ? 0 : l.batch * l.layers * l.kv_heads, basis, ctx->sm_count);
+        e = gemm_is_direct(kept_len) ? gemm_prepare(&dg->gemm, 0, basis, ctx->sm_count)
+                                     : nearfar_prepare(&dg->gemm, make_view(l, k, v, 0, l.batch), {{0, l.batch, n_in, kept_len, basis.nearfar}}, ctx->sm_count);
     auto fail = [&](freqkv_status code, cudaError_t ce, const char* where) {
         if (ce != cudaSuccess) code = cuda_fail(ctx, ce, where);
         if (dg) {

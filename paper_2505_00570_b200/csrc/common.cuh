@@ -58,6 +58,9 @@ struct Basis {
     float2* f32_turns = nullptr;
     int32_t f32_fold_k = 0, f32_fold_m = 0;
     int64_t f32_fold_alloc_elems = 0;
+    // Near blocks, far blocks and tables of the one-pass form (nearfar.cu).
+    void* nearfar = nullptr;
+    int64_t nearfar_bytes = 0;
     // Tensor-core path for at most 256 kept rows: the whole P in bf16, dense_rows_pad (256) x ld.
     __nv_bfloat16* dense = nullptr;
     int32_t dense_rows_pad = 0;
