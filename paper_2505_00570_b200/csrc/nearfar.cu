@@ -23,10 +23,11 @@
 // (near slices, then 16 more columns that add the far part).  Every job is a product of 128 rows x 256 columns; both read
 // x as it lies in the cache, so nothing is folded or copied, and the second reading comes out of L2, since the groups
 // between a far job and its tiles are few.  In each CTA:
-//   warp 0       takes tickets, TMA: per slice 16 KB of basis (stored as the shared-memory image) and 64 rows x 256 channels
+//   warps 0,2,3  tickets; TMA: per slice 16 KB of basis (stored as the shared-memory image) and 64 rows x 256 channels
 //   warp 1       tcgen05.mma 128 x 256 x 16, two accumulators of 256 columns of tensor memory in turn
 //   warps 4-11   epilogue: partial far sums to the ring, or rows rounded to bf16 into the cache
 //   warps 12-15  the far operand of the tiles: sums of the parts, as bf16 and its remainder in bf16 (16 rows of the product)
+//   warps 16,17  far sums written and read: one release for all warps
 // A tile overwrites rows that other tiles of its group read.  It waits until those have them in shared memory (flags):
 // only tiles before it and the one after it can be among them, so every wait is for a job whose ticket is lower, or the
 // very next one, which nothing keeps from loading (its accumulator is the other one, its far jobs have lower tickets).
@@ -56,8 +57,9 @@ constexpr int FAR_CHUNK = FAR_COLS * 128;   // 16 rows x 64 channels
 constexpr int FAR_BYTES = 4 * FAR_CHUNK;
 constexpr int JOBS = 4;                     // ring of jobs between the producer and the other roles
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 2 * FAR_BYTES + 1024 + 512;
-constexpr int THREADS = 512;
-constexpr int EPI_WARPS = 8, FAR_WARPS = 4;
+constexpr int EPI_WARPS = 8, FAR_WARPS = 4, LOAD_WARPS = 3;
+constexpr int EPI_WARP0 = 4, FAR_WARP0 = EPI_WARP0 + EPI_WARPS, WRITTEN_WARP = FAR_WARP0 + FAR_WARPS, READ_WARP = WRITTEN_WARP + 1;
+constexpr int THREADS = 32 * (READ_WARP + 1);
 constexpr int MAX_RANK = 8;
 constexpr int TABLE = 4;                    // int32 per tile: first near column, first and last tile that reads its rows, -
 constexpr unsigned long long LANDING_NS = 1000000ull;
@@ -85,7 +87,7 @@ struct Params {
     const CUtensorMap* maps;    // K and V of every item
     int32_t n_runs, tickets, ahead, ring;
     int32_t sink, wide;
-    float* far;                 // [ring][parts x far_tiles][128][256]
+    float* far;                 // [ring][far_tiles x parts][tile][64][rank][4 columns]
     int64_t far_stride;         // floats per group
     uint32_t* flags;            // ticket | far sums written [groups] | far sums read [groups] | rows read [tiles]
     int32_t groups;
@@ -112,15 +114,17 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// (The hint lets the hardware put the warp to sleep: twenty warps that spin leave the epilogue a fifth of the issue slots.)
+constexpr uint32_t SUSPEND_NS = 20000;
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity)
+        : "r"(bar), "r"(parity), "r"(SUSPEND_NS)
         : "memory");
     return ok != 0;
 }
@@ -149,6 +153,23 @@ __device__ __forceinline__ uint32_t load_acquire(const uint32_t* p)
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ uint32_t load_relaxed(const uint32_t* p)
+{
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// For waits on other CTAs: relaxed looks, one acquiring load at the end (an acquiring load empties the SM's L1).
+template <class F>
+__device__ __forceinline__ bool seen(const uint32_t* p, F&& good)
+{
+    if (!good(load_relaxed(p))) return false;
+    return good(load_acquire(p));
+}
+__device__ __forceinline__ void store_relaxed(uint32_t* p, uint32_t v)
+{
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 __device__ __forceinline__ void store_release(uint32_t* p, uint32_t v)
 {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -158,6 +179,14 @@ __device__ __forceinline__ uint32_t add_acq_rel(uint32_t* p, uint32_t v)
     uint32_t old;
     asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
     return old;
+}
+// Counters in shared memory, one for each warp: the warp that publishes for all of them waits for every one.
+__device__ __forceinline__ void count_up(uint32_t* p, uint32_t n) { asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(n) : "memory"); }
+__device__ __forceinline__ uint32_t counted(const uint32_t* p)
+{
+    uint32_t v;
+    asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
 }
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t c0, int32_t c1, int32_t c2,
                                             int32_t c3, int32_t c4)
@@ -243,6 +272,8 @@ __device__ __forceinline__ Chunk chunk_of(int32_t head_dim, int32_t group, int32
 
 struct Job {
     int32_t kind, seq, group, idx;  // group: over the whole call; idx: tile, or far tile * parts + part
+    int32_t row, first, last;       // tiles: their entry of the plan's table; far jobs: first input row
+    int32_t steps;
 };
 constexpr int32_t JOB_FAR = 0, JOB_TILE = 1, JOB_STOP = 2;
 
@@ -270,11 +301,13 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     Job* jobs = reinterpret_cast<Job*>(bars + N_BARS);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(jobs + JOBS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    uint32_t* written = tmem_slot + 2;          // per epilogue warp: far jobs whose sums it has stored
+    uint32_t* read = written + EPI_WARPS;       // per far warp: tiles whose sums it has read
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(full_bar(s), 1);
+            mbar_init(full_bar(s), LOAD_WARPS);
             mbar_init(empty_bar(s), 1);
         }
         for (int s = 0; s < 2; ++s) {
@@ -285,9 +318,10 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         }
         for (int s = 0; s < JOBS; ++s) {
             mbar_init(job_full(s), 1);
-            mbar_init(job_empty(s), 1 + EPI_WARPS + FAR_WARPS);
+            mbar_init(job_empty(s), (LOAD_WARPS - 1) + 1 + EPI_WARPS + FAR_WARPS + 2);
         }
         *abort_flag = 0;
+        for (int i = 0; i < EPI_WARPS + FAR_WARPS; ++i) written[i] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -311,83 +345,96 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     // by every lane of a warp, with one outcome for all of them
     auto warp_wait_bar = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, wait_bar(bar, parity)) != 0; };
 
-    if (warp == 0) {
+    if (warp == 0 || warp == 2 || warp == 3) {
+        // ---------------- loads: warp 0 takes the tickets and brings the basis, warps 2 and 3 half of the group's chunks each ----------------
+        // (A thread issues a bulk or tensor copy every 250 to 300 cycles, whatever its size: five of them a slice from one thread
+        // took twice as long as the slice's products.)
         if (lane == 0) {
             uint32_t it = 0;
             int32_t run_idx = 0;
             Run run = RAGGED ? prm.runs[0] : prm.run[0];
-            int32_t ticket = (int32_t)atomicAdd(prm.flags, 1u);
+            int32_t ticket = warp == 0 ? (int32_t)atomicAdd(prm.flags, 1u) : 0;
             bool alive = true;
             for (uint32_t n = 0; alive; ++n) {
-                Job job = {JOB_STOP, 0, 0, 0};
-                if (ticket < prm.tickets) {
-                    while (run_idx + 1 < prm.n_runs) {
-                        const Run next = RAGGED ? prm.runs[run_idx + 1] : prm.run[run_idx + 1 < 3 ? run_idx + 1 : 2];
-                        if (ticket < next.ticket0) break;
-                        run = next;
-                        ++run_idx;
-                    }
-                    const int32_t per_block = run.far_jobs + run.tiles;
-                    const int32_t block = (ticket - run.ticket0) / per_block, at = (ticket - run.ticket0) % per_block;
-                    if (at < run.far_jobs)
-                        job = {JOB_FAR, run.far_seq, run.block0 + block + prm.ahead, at};
-                    else
-                        job = {JOB_TILE, run.tile_seq, run.block0 + block, at - run.far_jobs};
-                }
                 const int slot = n % JOBS;
-                if (n >= JOBS && !wait_bar(job_empty(slot), (n / JOBS - 1) & 1)) break;
-                jobs[slot] = job;
-                mbar_arrive(job_full(slot));
+                Job job = {JOB_STOP, 0, 0, 0, 0, 0, 0, 0};
+                if (warp == 0) {
+                    if (ticket < prm.tickets) {
+                        while (run_idx + 1 < prm.n_runs) {
+                            const Run next = RAGGED ? prm.runs[run_idx + 1] : prm.run[run_idx + 1 < 3 ? run_idx + 1 : 2];
+                            if (ticket < next.ticket0) break;
+                            run = next;
+                            ++run_idx;
+                        }
+                        const int32_t per_block = run.far_jobs + run.tiles;
+                        const int32_t block = (ticket - run.ticket0) / per_block, at = (ticket - run.ticket0) % per_block;
+                        if (at < run.far_jobs) {
+                            const Seq& s = seq_of(run.far_seq);
+                            const int32_t s0 = at % s.parts * s.part_slices;
+                            job = {JOB_FAR, run.far_seq, run.block0 + block + prm.ahead, at, s0 * BK, 0, 0, min(s.part_slices, s.k_slices - s0)};
+                        } else {
+                            const Seq& s = seq_of(run.tile_seq);
+                            const int32_t tile = at - run.far_jobs;
+                            const int4 t = *reinterpret_cast<const int4*>(s.table + tile * TABLE);
+                            job = {JOB_TILE, run.tile_seq, run.block0 + block, tile, t.x, t.y, t.z, s.slices};
+                        }
+                    }
+                    if (n >= JOBS && !wait_bar(job_empty(slot), (n / JOBS - 1) & 1)) break;
+                    jobs[slot] = job;
+                    mbar_arrive(job_full(slot));
+                } else {
+                    if (!wait_bar(job_full(slot), (n / JOBS) & 1)) break;
+                    job = jobs[slot];
+                    mbar_arrive(job_empty(slot));
+                }
                 if (job.kind == JOB_STOP) break;
 
                 const Seq& s = seq_of(job.seq);
-                const CUtensorMap* mk = RAGGED ? prm.maps + 2 * job.seq : &map_k;
-                const CUtensorMap* mv = RAGGED ? prm.maps + 2 * job.seq + 1 : &map_v;
-                int32_t steps, row;
-                const uint8_t* a;
-                if (job.kind == JOB_FAR) {
-                    const int32_t s0 = job.idx % s.parts * s.part_slices;
-                    steps = min(s.part_slices, s.k_slices - s0);
-                    row = s0 * BK;
-                    a = s.blocks + (size_t)s.tiles * s.slices * A_BYTES + ((size_t)(job.idx / s.parts) * s.k_slices + s0) * A_BYTES;
-                } else {
-                    steps = s.slices;
-                    row = s.table[job.idx * TABLE];
-                    a = s.blocks + (size_t)job.idx * s.slices * A_BYTES;
+                if (warp == 0) {
+                    const size_t block0 = job.kind == JOB_FAR ? (size_t)s.tiles * s.slices + (size_t)(job.idx / s.parts) * s.k_slices + job.row / BK
+                                                              : (size_t)job.idx * s.slices;
+                    const uint8_t* a = s.blocks + block0 * A_BYTES;
+                    int32_t next = 0;
+                    for (int32_t ks = 0; ks < job.steps; ++ks, ++it) {
+                        if (ks == max(0, job.steps - 4)) next = (int32_t)atomicAdd(prm.flags, 1u);
+                        const int st = it % STAGES;
+                        if (it >= STAGES && !wait_bar(empty_bar(st), (it / STAGES - 1) & 1)) {
+                            alive = false;
+                            break;
+                        }
+                        mbar_expect_tx(full_bar(st), A_BYTES);
+                        bulk_load(base + st * STAGE_BYTES, a + (size_t)ks * A_BYTES, A_BYTES, full_bar(st));
+                    }
+                    ticket = next;
+                    continue;
                 }
-                // the group's chunks: coordinates of their (kv_head, layer, batch)
-                const int32_t group = job.group - s.group0;
-                int32_t ch[4], h[4], l[4], b[4], valid = 0;
-                const CUtensorMap* map[4];
+                // chunks 2 (warp - 2) and the one after it: coordinates of their (kv_head, layer, batch)
+                int32_t ch[2], h[2], l[2], b[2], valid = 0;
+                const CUtensorMap* map[2];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const Chunk c = chunk_of(view.head_dim, group, j);
+                for (int j = 0; j < 2; ++j) {
+                    const Chunk c = chunk_of(view.head_dim, job.group - s.group0, 2 * (warp - 2) + j);
                     if (c.triple < s.triples) valid |= 1 << j;
                     const int32_t t = s.triple0 + min(c.triple, s.triples - 1);
                     ch[j] = c.channel;
                     h[j] = t % view.kv_heads;
                     l[j] = t / view.kv_heads % view.layers;
                     b[j] = t / (view.kv_heads * view.layers);
-                    map[j] = c.tensor ? mv : mk;
+                    map[j] = RAGGED ? prm.maps + 2 * job.seq + c.tensor : c.tensor ? &map_v : &map_k;
                 }
-                const uint32_t tx = A_BYTES + __popc(valid) * CHUNK_BYTES;
-                int32_t next = 0;
-                for (int32_t ks = 0; ks < steps; ++ks, ++it) {
-                    if (ks == max(0, steps - 4)) next = (int32_t)atomicAdd(prm.flags, 1u);
+                for (int32_t ks = 0; ks < job.steps; ++ks, ++it) {
                     const int st = it % STAGES;
                     if (it >= STAGES && !wait_bar(empty_bar(st), (it / STAGES - 1) & 1)) {
                         alive = false;
                         break;
                     }
-                    const uint32_t stage = base + st * STAGE_BYTES;
-                    mbar_expect_tx(full_bar(st), tx);
-                    bulk_load(stage, a + (size_t)ks * A_BYTES, A_BYTES, full_bar(st));
+                    const uint32_t dst = base + st * STAGE_BYTES + A_BYTES + 2 * (warp - 2) * CHUNK_BYTES;
+                    mbar_expect_tx(full_bar(st), __popc(valid) * CHUNK_BYTES);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
+                    for (int j = 0; j < 2; ++j)
                         if (valid >> j & 1)
-                            tma_load_5d(stage + A_BYTES + j * CHUNK_BYTES, map[j], full_bar(st), ch[j], row + ks * BK, h[j], l[j], b[j]);
+                            tma_load_5d(dst + j * CHUNK_BYTES, map[j], full_bar(st), ch[j], job.row + ks * BK, h[j], l[j], b[j]);
                 }
-                ticket = next;
             }
             if (*abort_flag) {  // let the copies in flight land before the shared memory goes away
                 const unsigned long long t0 = global_timer_ns();
@@ -406,7 +453,7 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                 if (job.kind == JOB_STOP) break;
                 const Seq& s = seq_of(job.seq);
                 const bool tile = job.kind == JOB_TILE;
-                const int32_t steps = tile ? s.slices : min(s.part_slices, s.k_slices - job.idx % s.parts * s.part_slices);
+                const int32_t steps = job.steps;
                 const uint32_t acc = n & 1, use = n >> 1;
                 if (use > 0 && !wait_bar(acc_empty(acc), (use - 1) & 1)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -426,8 +473,10 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                         umma(d, smem_desc(a0 + kk * 32, 16, 1024), smem_desc(b0 + kk * 2048, CHUNK_BYTES, 1024), (ks | kk) != 0);
                     }
                     if (last) {
-                        // every row of the window is in shared memory: they may be overwritten
-                        store_release(rows_read + s.read0 + (job.group - s.group0) * s.tiles + job.idx, 1u);
+                        // Every row of the window is in shared memory (this thread has seen the barriers of its copies): they may be
+                        // overwritten.  Nothing was written that the flag would have to publish, so it needs no release, which
+                        // takes 4000 cycles here (it waits for the stores of the other warps).
+                        store_relaxed(rows_read + s.read0 + (job.group - s.group0) * s.tiles + job.idx, 1u);
                         const uint32_t buf = tiles & 1;
                         if (!wait_bar(far_full(buf), (tiles >> 1) & 1)) {
                             alive = false;
@@ -443,10 +492,11 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                 if (alive) umma_commit(acc_full(acc));
             }
         }
-    } else if (warp >= 4 && warp < 4 + EPI_WARPS) {
-        const int quarter = warp % 4, half = (warp - 4) / 4;
+    } else if (warp >= EPI_WARP0 && warp < EPI_WARP0 + EPI_WARPS) {
+        const int quarter = warp % 4, half = (warp - EPI_WARP0) / 4;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * 128;
         const int32_t row = quarter * 32 + lane;
+        uint32_t far_jobs = 0;
         for (uint32_t n = 0;; ++n) {
             const int slot = n % JOBS;
             if (!warp_wait_bar(job_full(slot), (n / JOBS) & 1)) break;
@@ -467,12 +517,14 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                 // the ring's place is free once the tiles of the group before have read it
                 if (job.group >= prm.ring) {
                     const uint32_t* p = far_read + job.group - prm.ring;
-                    if (!__all_sync(0xffffffffu, wait_flag([&] { return (load_acquire(p) & FAR_READ) != 0; }))) break;
+                    if (!__all_sync(0xffffffffu, wait_flag([&] { return seen(p, [](uint32_t v) { return (v & FAR_READ) != 0; }); }))) break;
                 }
                 if (!warp_wait_bar(acc_full(acc), (n >> 1) & 1)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                // [tile][4 columns][value]: a warp stores whole lines, and what a tile reads lies together
+                float4* out = reinterpret_cast<float4*>(prm.far + (int64_t)(job.group % prm.ring) * prm.far_stride + (int64_t)job.idx * BM * BN) +
+                              (row / s.rank * (BN / 4) + half * 32) * s.rank + row % s.rank;
                 const bool used = job.idx / s.parts * BM + row < s.rank * s.tiles;
-                float* out = prm.far + (int64_t)(job.group % prm.ring) * prm.far_stride + ((int64_t)job.idx * BM + row) * BN + half * 128;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     tmem_ld32(addr + c * 32, r);
@@ -480,24 +532,23 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                     if (c == 3) release();
                     if (used)
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) store32(out + c * 32 + i * 8, r + i * 8, true);
+                        for (int i = 0; i < 8; ++i)
+                            __stcg(out + (c * 8 + i) * s.rank, make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
+                                                                           __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3])));
                 }
                 __syncwarp();
-                if (lane == 0) {
-                    __threadfence();
-                    add_acq_rel(far_written + job.group, 1u);
-                }
+                if (lane == 0) count_up(written + warp - EPI_WARP0, ++far_jobs);
                 continue;
             }
             if (!warp_wait_bar(acc_full(acc), (n >> 1) & 1)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             {
                 // the tiles that read the rows this one writes must have them
-                const int32_t other = s.table[job.idx * TABLE + 1] + lane;
+                const int32_t other = job.first + lane;
                 bool ok = true;
-                if (other <= s.table[job.idx * TABLE + 2] && other != job.idx) {
+                if (other <= job.last && other != job.idx) {
                     const uint32_t* p = rows_read + s.read0 + group * s.tiles + other;
-                    ok = wait_flag([&] { return load_acquire(p) != 0; });
+                    ok = wait_flag([&] { return seen(p, [](uint32_t v) { return v != 0; }); });
                 }
                 if (!__all_sync(0xffffffffu, ok)) break;
             }
@@ -520,8 +571,8 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                 }
             }
         }
-    } else if (warp >= 4 + EPI_WARPS) {
-        const int32_t col = (threadIdx.x - 32 * (4 + EPI_WARPS)) * 2;  // this thread's two columns
+    } else if (warp >= FAR_WARP0 && warp < FAR_WARP0 + FAR_WARPS) {
+        const int32_t tid = threadIdx.x - 32 * FAR_WARP0, i = tid % MAX_RANK;  // value i of columns 4 (tid / 8 + 16 j) and the three after
         uint32_t tiles = 0;
         for (uint32_t n = 0;; ++n) {
             const int slot = n % JOBS;
@@ -534,43 +585,72 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             const Seq& s = seq_of(job.seq);
             const uint32_t buf = tiles & 1;
             if (tiles >= 2 && !warp_wait_bar(far_empty(buf), ((tiles >> 1) - 1) & 1)) break;
-            const uint32_t want = (uint32_t)(EPI_WARPS * s.parts * s.far_tiles);
+            const uint32_t want = (uint32_t)(s.parts * s.far_tiles);
             bool ok = true;
-            if (lane == 0) ok = wait_flag([&] { return load_acquire(far_written + job.group) >= want; });
+            if (lane == 0) ok = wait_flag([&] { return seen(far_written + job.group, [&](uint32_t v) { return v >= want; }); });
             if (!__all_sync(0xffffffffu, ok)) break;
             const int32_t row0 = job.idx * s.rank;
-            const float* in = prm.far + (int64_t)(job.group % prm.ring) * prm.far_stride +
-                              ((int64_t)(row0 / BM) * s.parts * BM + row0 % BM) * BN + col;
-            float2 e[MAX_RANK];
+            const float4* in = reinterpret_cast<const float4*>(prm.far + (int64_t)(job.group % prm.ring) * prm.far_stride +
+                                                               (int64_t)(row0 / BM) * s.parts * BM * BN) +
+                               (row0 % BM) * (BN / 4) + tid / MAX_RANK * s.rank + i;
+            float4 e[4];
 #pragma unroll
-            for (int i = 0; i < MAX_RANK; ++i) e[i] = make_float2(0.f, 0.f);
-            for (int32_t p = 0; p < s.parts; ++p, in += BM * BN) {
+            for (int j = 0; j < 4; ++j) e[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (i < s.rank) {
+#pragma unroll 2
+                for (int32_t p = 0; p < s.parts; ++p, in += BM * BN / 4) {
 #pragma unroll
-                for (int i = 0; i < MAX_RANK; ++i)
-                    if (i < s.rank) {
-                        const float2 x = __ldcg(reinterpret_cast<const float2*>(in + i * BN));
-                        e[i].x += x.x;
-                        e[i].y += x.y;
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 x = __ldcg(in + j * 16 * s.rank);
+                        e[j].x += x.x;
+                        e[j].y += x.y;
+                        e[j].z += x.z;
+                        e[j].w += x.w;
                     }
+                }
             }
-            uint8_t* dst = far_smem + buf * FAR_BYTES + col / 64 * FAR_CHUNK;
-            const uint32_t piece = (col % 64) / 8, within = col % 8 * 2;
+            uint8_t* dst = far_smem + buf * FAR_BYTES + i * 128;
 #pragma unroll
-            for (int i = 0; i < MAX_RANK; ++i) {
-                const uint32_t hi = pack_bf16(e[i].x, e[i].y);
-                const uint32_t lo = pack_bf16(e[i].x - __uint_as_float(hi << 16), e[i].y - __uint_as_float(hi & 0xffff0000u));
-                const uint32_t at = i * 128 + ((piece ^ (uint32_t)i) << 4) + within;
-                *reinterpret_cast<uint32_t*>(dst + at) = hi;
-                *reinterpret_cast<uint32_t*>(dst + MAX_RANK * 128 + at) = lo;
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t col = 4 * (tid / MAX_RANK + 16 * j);
+                const uint32_t at = col / 64 * FAR_CHUNK + ((col % 64 / 8 ^ (uint32_t)i) << 4) + col % 8 * 2;
+                const uint2 hi = make_uint2(pack_bf16(e[j].x, e[j].y), pack_bf16(e[j].z, e[j].w));
+                const uint2 lo = make_uint2(pack_bf16(e[j].x - __uint_as_float(hi.x << 16), e[j].y - __uint_as_float(hi.x & 0xffff0000u)),
+                                            pack_bf16(e[j].z - __uint_as_float(hi.y << 16), e[j].w - __uint_as_float(hi.y & 0xffff0000u)));
+                *reinterpret_cast<uint2*>(dst + at) = hi;
+                *reinterpret_cast<uint2*>(dst + MAX_RANK * 128 + at) = lo;
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(far_full(buf));
-                const uint32_t old = add_acq_rel(far_read + job.group, 1u);
-                if (old + 1 == (uint32_t)(FAR_WARPS * s.tiles)) store_release(far_read + job.group, FAR_READ);
+                count_up(read + warp - FAR_WARP0, tiles + 1);
             }
             ++tiles;
+        }
+    } else if (warp == WRITTEN_WARP || warp == READ_WARP) {
+        // ---------------- far sums written, far sums read: told to the other CTAs for all warps of this one ----------------
+        const bool writes = warp == WRITTEN_WARP;
+        const uint32_t* counter = (writes ? written : read) + lane;
+        uint32_t done = 0;
+        for (uint32_t n = 0;; ++n) {
+            const int slot = n % JOBS;
+            if (!warp_wait_bar(job_full(slot), (n / JOBS) & 1)) break;
+            const Job job = jobs[slot];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(job_empty(slot));
+            if (job.kind == JOB_STOP) break;
+            if (job.kind != (writes ? JOB_FAR : JOB_TILE)) continue;
+            ++done;
+            bool ok = true;
+            if (lane < (writes ? EPI_WARPS : FAR_WARPS)) ok = wait_flag([&] { return counted(counter) >= done; });
+            if (!__all_sync(0xffffffffu, ok)) break;
+            __syncwarp();
+            if (lane == 0) {
+                uint32_t* p = (writes ? far_written : far_read) + job.group;
+                const uint32_t old = add_acq_rel(p, 1u);
+                if (!writes && old + 1 == (uint32_t)seq_of(job.seq).tiles) store_release(p, FAR_READ);
+            }
         }
     }
 
@@ -799,7 +879,7 @@ Schedule schedule(const CacheView& view, const std::vector<NearFarItem>& items, 
     s.groups = (int32_t)groups;
     s.tickets = jobs;
     // A group's far jobs are over when its tiles begin: between them lie more jobs than the chip takes at once.
-    s.ahead = (int32_t)std::min<int64_t>(groups, 1 + (sm_count * groups * 5 / 4) / std::max<int64_t>(jobs, 1) + 1);
+    s.ahead = (int32_t)std::min<int64_t>(groups, 1 + (sm_count * groups * 3 / 2) / std::max<int64_t>(jobs, 1) + 1);
     s.ring = (int32_t)std::min<int64_t>(groups, 2 * (int64_t)s.ahead);
     s.flags = (16 + 2 * groups + reads + 3) / 4 * 4;
     s.far_offset = ((size_t)s.flags * 4 + 255) / 256 * 256;
@@ -890,7 +970,7 @@ NearFarShape nearfar_shape(int32_t n_in, int32_t n_keep)
     s.slices = (rows + 2 * least + FAR_COLS + BK - 1) / BK;
     s.margin = (s.slices * BK - FAR_COLS - rows) / 2;
     s.k_slices = (n_in + BK - 1) / BK;
-    s.parts = (s.k_slices + 15) / 16;
+    s.parts = (s.k_slices + 23) / 24;  // 16 or 32 slices a job: 7B shape 1.03 and 1.01 times as long, ragged batches 1.08 and 0.98
     s.part_slices = (s.k_slices + s.parts - 1) / s.parts;
     s.parts = (s.k_slices + s.part_slices - 1) / s.part_slices;
     s.far_tiles = (s.tiles * s.rank + BM - 1) / BM;
