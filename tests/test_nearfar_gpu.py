@@ -1,0 +1,67 @@
+"""GPU parity of the one-pass compression (near rows exactly, far rows by interpolation) at the edges of its tiles, against
+the fp64 CPU oracle.  Its own error beside the roundings is below 2e-4 of the matrix (4 nodes a tile; 3e-6 with 8), so the
+bounds of the other bf16 paths hold unchanged: 1e-2 a matrix, 3e-2 a row."""
+import pytest
+import torch
+
+from paper_2505_00570_b200 import binding as fk
+from paper_2505_00570_b200 import synth
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = fk.Context(0)
+    yield c
+    c.close()
+
+
+def workload(cap, sink, B=1, Ly=1, H=2, rho=0.9):
+    return synth.Workload("t", B, Ly, H, 128, cap, torch.bfloat16, sink, rho, 2, synth.BASE_SEED + 11)
+
+
+# kept rows: two tiles and a row, three whole tiles; 16 and 17 tiles (8 and 6 nodes each), 21 and 22 (6 and 4), 33 (two blocks
+# of far rows); nearly all rows kept (a tile then writes rows the next one reads); a wide window (one row in 30)
+@pytest.mark.parametrize("n_in,kept,sink", [(514, 257, 4), (1001, 384, 0), (2731, 2048, 4), (3000, 2049, 1), (5376, 2688, 4),
+                                            (3001, 2689, 0), (4500, 4097, 4), (300, 299, 2), (1500, 1409, 4), (8000, 267, 4)])
+def test_edges_of_the_tiles(ctx, n_in, kept, sink):
+    parity.check_compress(ctx, workload(n_in + sink + 3, sink), n_in + sink, kept, sink, fk.GEMM)
+    parity.check_compress(ctx, workload(n_in + sink + 3, sink, rho=0.0), n_in + sink, kept, sink, fk.GEMM, row_pad=8, sample=2)
+
+
+@pytest.mark.parametrize("n_in,kept", [(1028, 514), (700, 650), (3001, 749)])
+def test_many_groups_repeat_bit_for_bit(ctx, n_in, kept):
+    """More groups of channels than the ring of far sums has places; the tiles of all CTAs overwrite each other's input in
+    place, and the result is the same every time, and that of each matrix pair alone."""
+    w = workload(n_in + 4, 4, B=2, Ly=9, H=13)
+    k0, v0 = synth.make_cache(w, "cuda")
+    ctx.set_variant(fk.AUTO)
+    first = None
+    for _ in range(6):
+        k, v = k0.clone(), v0.clone()
+        ctx.compress(k, v, n_in + 4, kept, 4)
+        if first is None:
+            first = (k, v)
+        assert torch.equal(k, first[0]) and torch.equal(v, first[1])
+    assert ctx.last_device_status() == fk.OK
+    for b, layer, h in ((0, 0, 0), (1, 8, 12), (1, 3, 7)):
+        k, v = k0[b:b + 1, layer:layer + 1, h:h + 1].clone(), v0[b:b + 1, layer:layer + 1, h:h + 1].clone()
+        ctx.compress(k, v, n_in + 4, kept, 4)
+        assert torch.equal(k[0, 0, 0], first[0][b, layer, h]) and torch.equal(v[0, 0, 0], first[1][b, layer, h])
+
+
+def test_ragged_batch_of_different_ranks(ctx):
+    """Sequences of 8, 6 and 4 nodes a tile in one launch, each as on its own, bit for bit."""
+    lens, kept = [1300, 4500, 5200, 700], [640, 2500, 2900, 690]
+    w = workload(5200, 4, B=4, Ly=2, H=3)
+    k0, v0 = synth.make_cache(w, "cuda")
+    ctx.set_variant(fk.AUTO)
+    k, v = k0.clone(), v0.clone()
+    ctx.compress_ragged(k, v, lens, kept, 4)
+    assert ctx.last_device_status() == fk.OK
+    for b, (n, m) in enumerate(zip(lens, kept)):
+        one_k, one_v = k0[b:b + 1].clone(), v0[b:b + 1].clone()
+        ctx.compress(one_k, one_v, n, m, 4)
+        assert torch.equal(one_k[0], k[b]) and torch.equal(one_v[0], v[b]), b
