@@ -49,10 +49,9 @@ typedef enum { FREQKV_BF16 = 0, FREQKV_F32 = 1 } freqkv_dtype;
 /* Which kernel family executes the compression.
  *   GEMM  the DCT-II -> truncate -> IDCT -> rescale chain folded into one precomputed
  *         kept_len x n_in projection basis and run on the tcgen05 tensor cores (bf16 caches,
- *         head_dim 128 only); halved by the even/odd symmetry of the cosines after a fold pass
- *         over the cache (to a quarter where n_in is a multiple of 4, kept_len even and the call
- *         large enough, see freqkv_gemm_blocks), or, for kept_len <= 256, straight from the cache
- *         without that pass;
+ *         head_dim 128 only): the rows near a tile of the output exactly, all others through a few
+ *         interpolated values, in one pass over the cache; for kept_len <= 256 the plain product;
+ *         for retained bands halved by the even/odd symmetry of the cosines after a fold pass;
  *   FDCT  fast transform, O(N log N) (Appendix A: the DCT "can be computed using the FFT"): for
  *         bf16 caches the transform pair is factored into four small dense stages that run on
  *         the tensor cores, in place with no scratch, for every n_in = N1 N2 and kept_len = L1 L2
@@ -169,11 +168,9 @@ freqkv_status freqkv_power_spectrum(freqkv_ctx* ctx, const freqkv_layout* layout
  * N = lens[b] - sink, L = kept_len[b]).  `lens` and `kept_len` are host arrays of
  * layout->batch entries; on success lens[b] is updated to sink + kept_len[b].  All arguments
  * are validated for every sequence before anything is enqueued.  When every sequence that needs
- * work takes the folded tensor-core form (bf16, head_dim 128, more than 256 kept rows) the whole
- * batch is ONE fold launch and ONE tensor-core launch over a host-built work list (longest
- * sequences first), all plans built and all memory allocated before the first of them; the folded
- * inputs of the whole batch then live in the context's scratch (as many bytes as the non-sink
- * rows; beyond 64 GiB, or with other variants in the batch, the call goes run by run). */
+ * work takes the one-pass tensor-core form (bf16, head_dim 128, more than 256 kept rows) the whole
+ * batch is one tensor-core launch over a host-built table, behind a small one that clears its counters, all plans
+ * built and all memory allocated before the first of them; with other variants in the batch, the call goes run by run. */
 freqkv_status freqkv_compress_ragged(freqkv_ctx* ctx, const freqkv_layout* layout, void* k, void* v, int32_t* lens,
                                      const int32_t* kept_len, int32_t sink, void* cuda_stream);
 
@@ -370,10 +367,11 @@ freqkv_status freqkv_fast_plan_apply_host(int32_t n_in, int32_t n_keep, int32_t 
  * multiple of 4, kept_len even, first_component 0, and fewer 64-row slices of 256-row tiles that way).  With one
  * level the multiply-adds per matrix are 2 * ceil(L/2) * ceil(N/2) * head_dim, with two of the mirror symmetry alone
  * 3 * ceil(L/4) * (N/2) * head_dim.  -1 for invalid lengths.  Retained bands that start higher and the power
- * spectrum always use one level.  (Where this says 2 the library can split the odd part as well: freqkv_gemm_blocks.) */
+ * spectrum always use one level.  (A count of what the symmetry would save: plain compressions of more than 256 kept rows run in
+ * one pass over the cache instead, whose work grows with n_in alone.) */
 int32_t freqkv_gemm_fold_levels(int32_t n_in, int32_t kept_len, int32_t first_component);
 
-/* Host-only: in how many blocks variant GEMM runs such a compression of `triples` (batch, layer, kv_head) triples:
+/* Host-only: in how many blocks the symmetries would cut such a compression of `triples` (batch, layer, kv_head) triples:
  * 1 = the dense kept_len x n_in product straight from the cache (kept_len <= 256); 2 = one level of the mirror
  * symmetry; 4 = both levels and the odd part split by a rotation, 4 * ceil(L/4) * (N/4) * head_dim multiply-adds per
  * matrix (5 instead of 4 for even L/2), for lengths of two levels where there is work enough for its longer

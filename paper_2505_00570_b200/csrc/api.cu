@@ -298,14 +298,10 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
             // four blocks: columns up to n_in / 2 (the last block may run on through p), rows padded to the product's tiles
             x.f32_fold_k = (n_in / 2 + 1 + 15) / 16 * 16;
             x.f32_fold_m = ((n_keep + blocks - 1) / blocks + 127) / 128 * 128;
-            x.quad_rows_pad = first >= 0 && gemm_quad(n_in, n_keep, first) ? ((n_keep / 2 + 1) / 2 + 255) / 256 * 256 : 0;
         };
         shape(b);
         const size_t elems = (size_t)b.ld * b.rows_pad;
-        const size_t fold1_elems = (size_t)2 * b.fold_ld * b.fold_rows_pad;
-        const size_t quad_elems = (size_t)4 * b.fold_ld * b.quad_rows_pad;
-        const size_t turns_elems = b.quad_rows_pad ? (size_t)(n_in / 4) * (sizeof(float2) / 2) : 0;  // counted in bf16
-        const size_t fold_elems = fold1_elems + quad_elems + turns_elems;
+        const size_t fold_elems = (size_t)2 * b.fold_ld * b.fold_rows_pad;
         const size_t dense_elems = (size_t)256 * b.ld;
         const int32_t f32_blocks = fold_f32_blocks(n_in, n_keep);
         const size_t f32_plane_elems = (size_t)f32_blocks * b.f32_fold_k * b.f32_fold_m;
@@ -376,11 +372,6 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
             e = first == kDctRows ? launch_build_dct_folded(pb, n_in, b.fold_ld, b.fold_rows_pad, stream)
                                   : launch_build_folded_basis(pb, n_in, n_keep, first, b.fold_ld, b.fold_rows_pad, stream);
             ctx->kernels_launched += 1;
-            if (e == cudaSuccess && b.quad_rows_pad) {
-                e = launch_build_quad_basis(pb + fold1_elems, reinterpret_cast<float2*>(pb + fold1_elems + quad_elems), n_in, n_keep,
-                                            b.fold_ld, b.quad_rows_pad, stream);
-                ctx->kernels_launched += 1;
-            }
         }
         if (e == cudaSuccess && pd) {
             e = launch_build_basis(nullptr, pd, n_in, n_keep, first, b.ld, 256, stream);
@@ -409,8 +400,6 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
         if (pf) { b.f32 = pf; ctx->basis_bytes += elems * 4; }
         if (pb) {
             b.fold = pb;
-            b.quad = b.quad_rows_pad ? pb + fold1_elems : nullptr;
-            b.turns = b.quad_rows_pad ? reinterpret_cast<float2*>(pb + fold1_elems + quad_elems) : nullptr;
             b.fold_alloc_elems = (int64_t)fold_elems;
             ctx->basis_bytes += fold_elems * 2;
         }

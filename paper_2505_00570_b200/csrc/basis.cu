@@ -112,20 +112,6 @@ __device__ inline void store_turns(float2* turns, int64_t n_in, int64_t i0, int6
     }
 }
 
-__global__ void build_quad_basis_kernel(__nv_bfloat16* __restrict__ out, float2* __restrict__ turns, int32_t n_in, int32_t n_keep,
-                                        int32_t ld, int32_t rows_pad)
-{
-    const int64_t plane = (int64_t)rows_pad * ld;
-    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = i0; i < plane; i += step) {
-        double e[4];
-        quad_entries(i / ld, i % ld, n_in, n_keep, e);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) out[b * plane + i] = __double2bfloat16(e[b]);
-    }
-    store_turns(turns, n_in, i0, step);
-}
-
 // The same blocks, or the two of one level, in fp32 and transposed: [blocks][k_pad][m_pad], zero past the ends.
 __global__ void build_fold_f32_kernel(float* __restrict__ out, float2* __restrict__ turns, int32_t n_in, int32_t n_keep, int32_t blocks,
                                       int32_t k_pad, int32_t m_pad)
@@ -179,15 +165,6 @@ cudaError_t launch_build_dct_folded(__nv_bfloat16* out, int32_t n_in, int32_t ld
     const int64_t total = (int64_t)2 * rows_pad * ld;
     int64_t blocks = std::min<int64_t>((total + 255) / 256, 148 * 32);
     build_dct_folded_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, stream>>>(out, n_in, ld, rows_pad);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_build_quad_basis(__nv_bfloat16* out, float2* turns, int32_t n_in, int32_t n_keep, int32_t ld, int32_t rows_pad,
-                                    cudaStream_t stream)
-{
-    const int64_t total = (int64_t)rows_pad * ld;
-    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 148 * 32));
-    build_quad_basis_kernel<<<(unsigned)blocks, 256, 0, stream>>>(out, turns, n_in, n_keep, ld, rows_pad);
     return cudaGetLastError();
 }
 

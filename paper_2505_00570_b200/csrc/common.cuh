@@ -45,12 +45,6 @@ struct Basis {
     // m < ceil(n_keep/2), n < ceil(n_in/2), bf16, two planes of fold_rows_pad x fold_ld (see basis.cu).
     __nv_bfloat16* fold = nullptr;
     int32_t fold_ld = 0, fold_rows_pad = 0;
-    // The four-block form, where the lengths can take it (gemm_quad; a call chooses by its matrices, gemm_blocks): four planes of quad_rows_pad x fold_ld -- Pee, Peo,
-    // PA, PB -- stored behind the two planes above in the same allocation, then (cos, sin) of theta_n, n < n_in / 4
-    // (see basis.cu).
-    __nv_bfloat16* quad = nullptr;
-    float2* turns = nullptr;
-    int32_t quad_rows_pad = 0;
     int64_t fold_alloc_elems = 0;  // bf16 elements of the allocation `fold` points to
     // Folded fp32 product (foldf32.cu): fold_f32_blocks(n_in, n_keep) planes of f32_fold_k x f32_fold_m, transposed, then
     // (cos, sin) of theta_n, n < n_in / 4, where there are four.
@@ -72,10 +66,6 @@ struct Basis {
 // (`first` = index of the first retained DCT component; 0 for the method's low-pass compression)
 cudaError_t launch_build_basis(float* p_f32, __nv_bfloat16* p_bf16, int32_t n_in, int32_t n_keep, int32_t first,
                                int32_t ld, int32_t rows_pad, cudaStream_t stream);
-
-// Pee, Peo, PA and PB of the four-block form (four planes of rows_pad x ld) and the (cos, sin) that turn its odd rows.
-cudaError_t launch_build_quad_basis(__nv_bfloat16* out, float2* turns, int32_t n_in, int32_t n_keep, int32_t ld, int32_t rows_pad,
-                                    cudaStream_t stream);
 
 // The folded fp32 basis of foldf32.cu: `blocks` planes of k_pad x m_pad, transposed; `turns` for four blocks.
 cudaError_t launch_build_fold_f32(float* out, float2* turns, int32_t n_in, int32_t n_keep, int32_t blocks, int32_t k_pad,

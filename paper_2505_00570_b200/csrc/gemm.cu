@@ -9,13 +9,8 @@
 //     y_m = s_m + d_m,   y_{L-1-m} = s_m - d_m
 // which is the same linear map with half the multiply-adds.  (For odd N the middle row enters u
 // once and v as zero; for odd L the middle output row has d = 0 and is written once.)
-// For even L the even part Pe is itself the basis of a compression of N/2 rows to L/2, so where N is a
-// multiple of 4 it is folded once more (uu, uv; Pee, Peo); and the odd part Po, whose frequencies are
-// those of a DCT-IV, splits by a rotation of its mirrored rows into two blocks of the same quarter size
-// (p, q; PA, PB; see freqkv_fold_gemm_kernel and basis.cu): four blocks of ceil(L/4) x N/4, half of these multiply-adds
-// again.  The four-block form is what a plain compression of such lengths runs (the paper's
-// 4092 -> 2046 and 4096 -> 2048) where there is work enough (gemm_blocks), alone or in a ragged batch; the description below
-// is the one-level form, which serves everything else, retained bands and the power spectrum among it.
+// This folded form serves retained bands above the lowest component and the power spectrum; a plain compression of more than
+// 256 kept rows runs in one pass over the cache (nearfar.cu), of fewer as one dense product (MODE_DIRECT).
 //
 // Two kernels per call:
 //   fold_kernel         reads every non-sink cache row once and writes U and V (bf16) to a scratch
@@ -70,36 +65,24 @@ constexpr int NUM_THREADS = 320;                   // direct and spectrum modes:
 // registers unevenly.  The shares add up to what the block is launched with: 40 + 2 * 232 = 3 * 168.
 constexpr int FOLD_THREADS = 384, FOLD_LAUNCH_REGS = 168, CONTROL_REGS = 40, EPILOGUE_REGS = 232;
 static_assert(CONTROL_REGS + 2 * EPILOGUE_REGS <= 3 * FOLD_LAUNCH_REGS, "a larger sum would wait for registers for ever");
-constexpr size_t PARK_BYTES_PER_CTA = (size_t)BM * 256 * 8;  // four blocks: the pairs (s, s') of one tile, bf16 or fp32
 constexpr int EPI_WARPS = 8;
 constexpr unsigned long long LANDING_NS = 1000000ull;        // 1 ms: far longer than any copy in flight needs
 
 constexpr uint32_t ERR_FULL_WAIT = 1u, ERR_EMPTY_WAIT = 2u, ERR_ACC_FULL_WAIT = 4u, ERR_ACC_EMPTY_WAIT = 8u;
 
-// The matrices of one sequence (or of one pass of a uniform call): how they fold and what their tiles are.
-struct FoldSeq {
-    int32_t tile0;              // first tile in the launch
-    int32_t pair0;              // first (batch, layer, kv_head) triple
-    int32_t n_half, n_keep, rows_half;
-    int32_t quad;               // four blocks instead of one level
-    int32_t basis_rows_pad;     // row offset of one basis plane to the next inside the basis tensor map
-    int32_t k_steps, k_last;    // slices per phase; of the fourth phase of four
-    int32_t m_pairs;            // tiles of 256 folded rows per triple
-};
-
+// One pass of a call: how its matrices fold and what their tiles are.
 struct FoldParams {
     int32_t sink;
     int32_t mirror_sign;        // +1: y[L-1-m] = s - d;  -1: y[L-1-m] = d - s (a retained band that starts at an odd component)
     int32_t wide_rows;          // every row is 32-byte aligned
     int32_t total_tiles;
-    uint4* park;                // four blocks: work area of (s, s')
+    int32_t pair0;              // first (batch, layer, kv_head) triple
+    int32_t n_keep, rows_half;
+    int32_t basis_rows_pad;     // row offset of the Po plane inside the basis tensor map
+    int32_t k_steps;            // slices per phase
+    int32_t m_pairs;            // tiles of 256 folded rows per triple
     int32_t* status;
     unsigned long long wait_limit_ns;  // bound of every mbarrier wait
-    FoldSeq seq;                // uniform calls
-    // ragged batches: one entry per sequence, sorted by decreasing work, and one past the end that holds the total of
-    // tiles; two tensor maps per sequence (basis, planes)
-    const FoldSeq* seqs;
-    const CUtensorMap* seq_maps;
 };
 
 struct GemmParams {
@@ -323,7 +306,6 @@ __device__ __forceinline__ void fold8(const uint4& a, const uint4& b, uint4* u, 
 struct FoldJob {
     int32_t pair0, pair_count, n_in, n_half, sink;
     uint4* dst;
-    const float2* turns;  // four blocks: (cos, sin) of theta_n; null: one level
 };
 
 // One level: matrix pt of the job (pair_local * 2 + tensor), the y-th of gridDim.y shares of its n_half * 16 vectors.
@@ -366,98 +348,8 @@ __device__ __forceinline__ void fold_one_level(const CacheView& view, const Fold
     }
 }
 
-// The four-block fold (n_in a multiple of 4; see basis.cu): with N' = n_in / 2 and n < N' / 2 the four rows
-// n, N-1-n, N'-1-n and N'+n give u_n, u_{N'-1-n}, v_n, v_{N'-1-n}; from the two u's come
-// uu_n = u_n + u_{N'-1-n}, uv_n = u_n - u_{N'-1-n}, from the two v's, turned by theta_n = pi (2n+1) / (4 N'),
-// p_n = cos v_n + sin v_{N'-1-n}, q_n = sin v_n - cos v_{N'-1-n} (all in fp32, rounded once).  Plane 0 of a
-// matrix holds uu (rows 0 .. N'/2 - 1) followed by uv (rows N'/2 .. N' - 1), plane 1 holds q followed by p: the same
-// bytes as one level.
-__device__ __forceinline__ void fold8_quad(const uint4& a, const uint4& b, const uint4& c, const uint4& d, float2 cs, uint4* uu,
-                                           uint4* uv, uint4* p, uint4* q)
-{
-    const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w}, cw[4] = {c.x, c.y, c.z, c.w},
-                   dw[4] = {d.x, d.y, d.z, d.w};
-    uint32_t o[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float a0 = __uint_as_float(aw[i] << 16), a1 = __uint_as_float(aw[i] & 0xffff0000u);
-        const float b0 = __uint_as_float(bw[i] << 16), b1 = __uint_as_float(bw[i] & 0xffff0000u);
-        const float c0 = __uint_as_float(cw[i] << 16), c1 = __uint_as_float(cw[i] & 0xffff0000u);
-        const float d0 = __uint_as_float(dw[i] << 16), d1 = __uint_as_float(dw[i] & 0xffff0000u);
-        const float p0 = a0 + b0, p1 = a1 + b1, q0 = c0 + d0, q1 = c1 + d1;  // u_n, u_{N'-1-n}
-        const float r0 = a0 - b0, r1 = a1 - b1, s0 = c0 - d0, s1 = c1 - d1;  // v_n, v_{N'-1-n}
-        o[0][i] = pack_bf16(p0 + q0, p1 + q1);
-        o[1][i] = pack_bf16(p0 - q0, p1 - q1);
-        o[2][i] = pack_bf16(fmaf(cs.x, r0, cs.y * s0), fmaf(cs.x, r1, cs.y * s1));
-        o[3][i] = pack_bf16(fmaf(cs.y, r0, -cs.x * s0), fmaf(cs.y, r1, -cs.x * s1));
-    }
-    *uu = make_uint4(o[0][0], o[0][1], o[0][2], o[0][3]);
-    *uv = make_uint4(o[1][0], o[1][1], o[1][2], o[1][3]);
-    *p = make_uint4(o[2][0], o[2][1], o[2][2], o[2][3]);
-    *q = make_uint4(o[3][0], o[3][1], o[3][2], o[3][3]);
-}
-
-// Four blocks: as fold_one_level; job.n_half = N' rows per plane; a thread folds VECS vectors per round.
-template <int VECS>
-__device__ __forceinline__ void fold_four_blocks(const CacheView& view, const FoldJob& job, uint32_t pt, const float2* __restrict__ turns)
-{
-    const char* x = static_cast<const char*>(tensor_base(view, pt & 1)) +
-                    (matrix_offset(view, job.pair0 + (int32_t)(pt >> 1)) + (int64_t)job.sink * view.stride_token) * 2;
-    const int64_t row_bytes = view.stride_token * 2;
-    const int32_t n_quarter = job.n_half / 2;
-    const uint32_t total = (uint32_t)n_quarter * 16u;                // vectors of uu (= of uv, q, p)
-    uint4* plane0 = job.dst + (int64_t)pt * 2 * ((int64_t)job.n_half * 16);
-    uint4* plane1 = plane0 + (int64_t)job.n_half * 16;
-    for (uint32_t c0 = blockIdx.y * (VECS * 256u); c0 < total; c0 += gridDim.y * (VECS * 256u)) {
-        uint4 a[VECS], b[VECS], c[VECS], d[VECS];
-        float2 cs[VECS];
-#pragma unroll
-        for (int j = 0; j < VECS; ++j) {
-            const uint32_t i = c0 + j * 256u + threadIdx.x;
-            if (i < total) {
-                const int32_t n = (int32_t)(i >> 4);
-                a[j] = __ldcs(reinterpret_cast<const uint4*>(x + n * row_bytes) + (i & 15u));
-                b[j] = __ldcs(reinterpret_cast<const uint4*>(x + (job.n_in - 1 - n) * row_bytes) + (i & 15u));
-                c[j] = __ldcs(reinterpret_cast<const uint4*>(x + (job.n_half - 1 - n) * row_bytes) + (i & 15u));
-                d[j] = __ldcs(reinterpret_cast<const uint4*>(x + (job.n_half + n) * row_bytes) + (i & 15u));
-                cs[j] = __ldg(turns + n);
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < VECS; ++j) {
-            const uint32_t i = c0 + j * 256u + threadIdx.x;
-            if (i < total) {
-                uint4 uu, uv, p, q;
-                fold8_quad(a[j], b[j], c[j], d[j], cs[j], &uu, &uv, &p, &q);
-                __stcs(plane0 + i, uu);
-                __stcs(plane0 + total + i, uv);
-                __stcs(plane1 + i, q);
-                __stcs(plane1 + total + i, p);
-            }
-        }
-    }
-}
-
-// Block x: matrix x of the job, or, of a ragged batch (every sequence has the same number of matrices), of job x / mats_per_seq.
+// Block x: matrix x of the job.
 __global__ void __launch_bounds__(256) fold_kernel(const CacheView view, const FoldJob job) { fold_one_level(view, job, blockIdx.x); }
-
-// (`turns` = job.turns as a parameter of its own: read through the struct it costs 83 registers instead of 80, one block an SM
-// less, and 0.02 ms of a 7B-shaped fold.)
-__global__ void __launch_bounds__(256) fold_quad_kernel(const CacheView view, const FoldJob job, const float2* __restrict__ turns)
-{
-    fold_four_blocks<2>(view, job, blockIdx.x, turns);
-}
-
-// (Four blocks of 256 threads an SM leave 64 registers, with which two vectors a round of the four-block branch spill; with one,
-// ragged batches take 1 to 3 % less: 64 matrices 1027 -> 513 41.9 -> 40.7 us, 512 matrices 8188 -> 4094 1108 -> 1087 us.)
-__global__ void __launch_bounds__(256, 4) fold_ragged_kernel(const CacheView view, const FoldJob* jobs, int32_t mats_per_seq)
-{
-    const FoldJob job = jobs[blockIdx.x / mats_per_seq];
-    if (job.turns)
-        fold_four_blocks<1>(view, job, blockIdx.x % mats_per_seq, job.turns);
-    else
-        fold_one_level(view, job, blockIdx.x % mats_per_seq);
-}
 
 // The other two uses of the same tiles:
 // MODE_SPECTRUM: the basis holds the even and the odd rows of the plain N-point DCT-II instead of
@@ -496,51 +388,10 @@ __device__ __forceinline__ void store_row16(__nv_bfloat16* dst, const uint32_t (
 
 // ---- the product of the folded forms ----
 
-// Ragged batches: a role walks its tiles in increasing order, so the sequence a tile belongs to is found by moving a
-// cursor forward; the table in global memory is read only when a tile crosses into a new sequence.
-struct SeqCursor {
-    int32_t idx = -1, end_tile = 0;
-    FoldSeq s;
-};
-template <bool RAGGED>
-__device__ __forceinline__ const FoldSeq& seq_of_tile(const FoldParams& prm, int32_t tile, SeqCursor& cur)
-{
-    if constexpr (RAGGED) {
-        while (tile >= cur.end_tile) {
-            ++cur.idx;
-            cur.s = prm.seqs[cur.idx];
-            cur.end_tile = __ldg(&prm.seqs[cur.idx + 1].tile0);
-        }
-        return cur.s;
-    } else {
-        return prm.seq;
-    }
-}
-
-// FORM_ONE_LEVEL, FORM_FOUR_BLOCKS: the compression of one pair of lengths.
-// FORM_RAGGED: sequences of different lengths in one launch: a tile looks up its sequence (shapes, tensor
-//   maps) in a table built on the host; one-level and four-block sequences mix (FoldSeq::quad).  The pairs (s, s') below stay in
-//   fp32 here.
-// Four blocks (n_in a multiple of 4, n_keep even): a tile is 256 rows m < ceil(L/4) of all
-//   four blocks and runs four phases, each N/4 deep, alternating between the two halves of tensor memory:
-//   a = Pee uu, b = Peo uv, A = PA p, B = PB q (for even L/2 one retained component couples p into B: the last
-//   phase then runs on through p, with that component's column weights as its basis).  The epilogue
-//   parks a in registers, turns it with b into the pair s = a + b, s' = a - b (two bf16 in a word, or two words), which waits
-//   in a work area of this CTA that stays in L2 -- the accumulators of a tile would need twice the tensor memory there is --,
-//   parks A, and turns it with B by theta'_m = pi (2m+1) / (2L) into d = cos A + sin B and d' = sin A - cos B:
-//   y_m = s + d, y_{L-1-m} = s - d, y_{L/2-1-m} = s' + d', y_{L/2+m} = s' - d'.
-constexpr int FORM_ONE_LEVEL = 0, FORM_FOUR_BLOCKS = 1, FORM_RAGGED = 2;
-
-template <int FORM>
 __global__ void __launch_bounds__(FOLD_THREADS, 1)
 freqkv_fold_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_x, const CacheView view,
                         const __grid_constant__ FoldParams prm)
 {
-    constexpr bool RAGGED = FORM == FORM_RAGGED, WIDE = RAGGED;
-    // The next 16 columns (and their pairs) leave tensor memory while these are combined and stored, where the registers allow
-    // it (2997 -> 749 1.50 -> 1.48 ms with the append, 64 matrices 1497 -> 749 44.1 -> 42.1 us; with fp32 pairs 57 -> 61 us).
-    constexpr bool AHEAD = !WIDE;
-    constexpr bool FOUR = FORM == FORM_FOUR_BLOCKS;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // 128-byte swizzle atoms need 1024-byte alignment
@@ -591,22 +442,11 @@ freqkv_fold_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_
             if (lane == 0) {
                 uint32_t it = 0;  // global slice counter: stage = it % STAGES, phase = it / STAGES
                 bool alive = true;
-                SeqCursor cursor;
                 for (int32_t tile = cluster; tile < prm.total_tiles && alive; tile += n_clusters) {
-                    const FoldSeq& s = seq_of_tile<RAGGED>(prm, tile, cursor);
-                    const CUtensorMap* mp = RAGGED ? prm.seq_maps + 2 * cursor.idx : &map_p;
-                    const CUtensorMap* mx = RAGGED ? prm.seq_maps + 2 * cursor.idx + 1 : &map_x;
-                    const int32_t local = tile - s.tile0, pair = local / s.m_pairs;
-                    const int32_t m0 = (local % s.m_pairs * 2 + (int32_t)rank) * BM;
-                    const bool quad = RAGGED ? s.quad != 0 : FOUR;
-                    const int32_t phases = quad ? 4 : 2;
-                    for (int eo = 0; eo < phases && alive; ++eo) {
-                        // rank 0: K channels, rank 1: V.  Four blocks: phases 0, 1 read uu and uv (both in plane 0, uv
-                        // n_half / 2 rows down), phases 2, 3 read p (n_half / 2 rows down in plane 1) and q
-                        const int32_t plane = (pair * 2 + (int32_t)rank) * 2 + (quad ? eo >> 1 : eo);
-                        const int32_t row0 = (quad && (eo == 1 || eo == 2)) ? s.n_half / 2 : 0;
-                        const int32_t steps = eo == 3 ? s.k_last : s.k_steps;
-                        for (int32_t ks = 0; ks < steps; ++ks, ++it) {
+                    const int32_t pair = tile / prm.m_pairs, m0 = (tile % prm.m_pairs * 2 + (int32_t)rank) * BM;
+                    for (int eo = 0; eo < 2 && alive; ++eo) {
+                        const int32_t plane = (pair * 2 + (int32_t)rank) * 2 + eo;  // rank 0: K channels, rank 1: V
+                        for (int32_t ks = 0; ks < prm.k_steps; ++ks, ++it) {
                             const int st = it % STAGES;
                             if (it >= STAGES &&
                                 !mbar_wait(empty_bar(st), ((it / STAGES) - 1) & 1, abort_flag, prm.status, ERR_EMPTY_WAIT, prm.wait_limit_ns)) {
@@ -617,9 +457,9 @@ freqkv_fold_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_
                             const uint32_t leader_full = cluster_addr(full_bar(st), 0);
                             if (rank == 0) mbar_expect_tx(full_bar(st), 2 * STAGE_BYTES);
                             const int32_t k0 = ks * BK;
-                            tma_load_2d(stage, mp, leader_full, k0, eo * s.basis_rows_pad + m0);
-                            tma_load_3d(stage + A_BYTES, mx, leader_full, 0, row0 + k0, plane);
-                            tma_load_3d(stage + A_BYTES + B_CHUNK_BYTES, mx, leader_full, 64, row0 + k0, plane);
+                            tma_load_2d(stage, &map_p, leader_full, k0, eo * prm.basis_rows_pad + m0);
+                            tma_load_3d(stage + A_BYTES, &map_x, leader_full, 0, k0, plane);
+                            tma_load_3d(stage + A_BYTES + B_CHUNK_BYTES, &map_x, leader_full, 64, k0, plane);
                         }
                     }
                 }
@@ -633,11 +473,8 @@ freqkv_fold_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_
             if (lane == 0 && rank == 0) {
                 uint32_t it = 0, phase = 0;  // phase: over all tiles; half of tensor memory = phase % 2
                 bool alive = true;
-                SeqCursor cursor;
                 for (int32_t tile = cluster; tile < prm.total_tiles && alive; tile += n_clusters) {
-                    const FoldSeq& s = seq_of_tile<RAGGED>(prm, tile, cursor);
-                    const int32_t phases = (RAGGED ? s.quad != 0 : FOUR) ? 4 : 2, k_steps = s.k_steps, k_last = s.k_last;
-                    for (int eo = 0; eo < phases && alive; ++eo, ++phase) {
+                    for (int eo = 0; eo < 2 && alive; ++eo, ++phase) {
                         const uint32_t acc = phase & 1, use = phase >> 1;  // use: how often that half was filled before
                         if (use > 0) {  // both CTAs' epilogues must have read what this half held last
                             if (!mbar_wait(acc_empty_bar(acc), (use - 1) & 1, abort_flag, prm.status, ERR_ACC_EMPTY_WAIT, prm.wait_limit_ns)) {
@@ -646,8 +483,7 @@ freqkv_fold_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_
                             }
                             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         }
-                        const int32_t steps = eo == 3 ? k_last : k_steps;
-                        for (int32_t ks = 0; ks < steps; ++ks, ++it) {
+                        for (int32_t ks = 0; ks < prm.k_steps; ++ks, ++it) {
                             const int st = it % STAGES;
                             if (!mbar_wait(full_bar(st), (it / STAGES) & 1, abort_flag, prm.status, ERR_FULL_WAIT, prm.wait_limit_ns)) {
                                 alive = false;
@@ -675,8 +511,6 @@ freqkv_fold_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_
         // ---------------- epilogue (both CTAs, each on its own 128 rows) ----------------
         const int ew = warp - 4, quarter = warp % 4, tensor = ew / 4;  // tensor: 0 = K columns, 1 = V columns
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + tensor * 128;
-        // this thread's vectors of the work area: vector i of lane l at (i * 32 + l), so that a warp's access is dense
-        uint4* park = prm.park + ((size_t)blockIdx.x * EPI_WARPS + ew) * (64 * 32) + lane;
         uint32_t phase = 0;  // as the MMA issuer counts
         // wait for the accumulator that is complete next
         auto next_full = [&]() -> bool {
@@ -691,153 +525,46 @@ freqkv_fold_gemm_kernel(const __grid_constant__ CUtensorMap map_p, const __grid_
             if (lane == 0) mbar_arrive_cluster(cluster_addr(acc_empty_bar(phase & 1), 0));
             ++phase;
         };
-        SeqCursor cursor;
         for (int32_t tile = cluster; tile < prm.total_tiles; tile += n_clusters) {
-            const FoldSeq& sq = seq_of_tile<RAGGED>(prm, tile, cursor);
             uint32_t s[128];
-            auto park_all = [&](uint32_t addr) {
-                tmem_ld32<0>(addr + 0, s);
-                tmem_ld32<32>(addr + 32, s);
-                tmem_ld32<64>(addr + 64, s);
-                tmem_ld32<96>(addr + 96, s);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            };
-            // S = Pe U, or a = Pee uu: park this thread's row (128 columns) in registers, hand that half back
+            // S = Pe U: park this thread's row (128 columns) in registers, hand that half back
             if (!next_full()) break;
-            park_all(lane_addr + (phase & 1) * 256);
+            tmem_ld32<0>(lane_addr + (phase & 1) * 256 + 0, s);
+            tmem_ld32<32>(lane_addr + (phase & 1) * 256 + 32, s);
+            tmem_ld32<64>(lane_addr + (phase & 1) * 256 + 64, s);
+            tmem_ld32<96>(lane_addr + (phase & 1) * 256 + 96, s);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             release();
-            const int32_t local = tile - sq.tile0, n_keep = sq.n_keep;
-            const int32_t m = (local % sq.m_pairs * 2 + (int32_t)rank) * BM + quarter * 32 + lane;
+            const int32_t n_keep = prm.n_keep;
+            const int32_t m = (tile % prm.m_pairs * 2 + (int32_t)rank) * BM + quarter * 32 + lane;
             __nv_bfloat16* mat = static_cast<__nv_bfloat16*>(tensor_base(view, tensor)) +
-                                 matrix_offset(view, sq.pair0 + local / sq.m_pairs) + (int64_t)prm.sink * view.stride_token;
-            if (RAGGED ? !sq.quad : FORM == FORM_ONE_LEVEL) {
-                // D = Po V: combine and store rows m and L-1-m
-                if (!next_full()) break;
-                const uint32_t addr = lane_addr + (phase & 1) * 256;
-                const bool row_ok = m < sq.rows_half, mirror_ok = row_ok && n_keep - 1 - m != m;
-                const float sgn = (float)prm.mirror_sign;
-                __nv_bfloat16* out_p = mat + (int64_t)m * view.stride_token;
-                __nv_bfloat16* out_m = mat + (int64_t)(n_keep - 1 - m) * view.stride_token;
-                uint32_t d2[2][16];
-                if (AHEAD) tmem_ld16(addr, d2[0]);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    if (!AHEAD) tmem_ld16(addr + c * 16, d2[0]);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (AHEAD && c < 7) tmem_ld16(addr + (c + 1) * 16, d2[(c + 1) & 1]);
-                    if (c == 7) release();
-                    const uint32_t(&d)[16] = d2[AHEAD ? c & 1 : 0];
-                    uint32_t p[8], q[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float s0 = __uint_as_float(s[c * 16 + 2 * j]), s1 = __uint_as_float(s[c * 16 + 2 * j + 1]);
-                        const float d0 = __uint_as_float(d[2 * j]), d1 = __uint_as_float(d[2 * j + 1]);
-                        p[j] = pack_bf16(s0 + d0, s1 + d1);
-                        q[j] = pack_bf16(sgn * (s0 - d0), sgn * (s1 - d1));
-                    }
-                    if (row_ok) store_row16(out_p + c * 16, p, prm.wide_rows);
-                    if (mirror_ok) store_row16(out_m + c * 16, q, prm.wide_rows);
-                }
-                continue;
-            }
-            // b = Peo uv: s = a + b and s' = a - b go to the work area (bf16: s in the low half of a word)
-            if (!next_full()) break;
-            {
-                const uint32_t addr = lane_addr + (phase & 1) * 256;
-                uint32_t b2[2][16];
-                if (AHEAD) tmem_ld16(addr, b2[0]);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    if (!AHEAD) tmem_ld16(addr + c * 16, b2[0]);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (AHEAD && c < 7) tmem_ld16(addr + (c + 1) * 16, b2[(c + 1) & 1]);
-                    const uint32_t(&b)[16] = b2[AHEAD ? c & 1 : 0];
-                    if constexpr (WIDE) {
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const float a0 = __uint_as_float(s[c * 16 + 2 * j]), a1 = __uint_as_float(s[c * 16 + 2 * j + 1]);
-                            const float b0 = __uint_as_float(b[2 * j]), b1 = __uint_as_float(b[2 * j + 1]);
-                            __stcg(reinterpret_cast<float4*>(park) + (c * 8 + j) * 32, make_float4(a0 + b0, a0 - b0, a1 + b1, a1 - b1));
-                        }
-                    } else {
-                        uint32_t w[16];
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const float av = __uint_as_float(s[c * 16 + j]), bv = __uint_as_float(b[j]);
-                            w[j] = pack_bf16(av + bv, av - bv);
-                        }
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            __stcg(park + (c * 4 + j) * 32, make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]));
-                    }
-                }
-            }
-            release();
-            const int32_t rows_half = sq.rows_half, mh = rows_half - 1 - m;  // mh: the row whose even part is s'
-            const bool row_ok = m < (rows_half + 1) / 2;
-            const bool second_ok = row_ok && mh != m;  // the middle row of an odd L/2 is its own mirror
-            float ct, st;                              // theta'_m = pi (2m+1) / (2L)
-            sincospif((float)(2 * m + 1) / (float)(2 * n_keep), &st, &ct);
-            __nv_bfloat16* rows[4] = {mat + (int64_t)m * view.stride_token, mat + (int64_t)(n_keep - 1 - m) * view.stride_token,
-                                      mat + (int64_t)mh * view.stride_token, mat + (int64_t)(rows_half + m) * view.stride_token};
-            // A = PA p: park it
-            if (!next_full()) break;
-            park_all(lane_addr + (phase & 1) * 256);
-            release();
-            // B = PB q: turn (A, B), combine with (s, s') and store the four rows
-            constexpr int WORDS = WIDE ? 32 : 16;  // pairs of 16 columns
-            uint32_t b2[2][16], w2[2][WORDS];
-            auto pairs = [&](int c, uint32_t(&v)[WORDS]) {
-#pragma unroll
-                for (int j = 0; j < WORDS / 4; ++j) {
-                    // volatile: hoisting the loads of every chunk to the front would cost more registers than there are
-                    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(v[4 * j]), "=r"(v[4 * j + 1]), "=r"(v[4 * j + 2]), "=r"(v[4 * j + 3])
-                                 : "l"(park + (c * (WORDS / 4) + j) * 32)
-                                 : "memory");
-                }
-            };
-            if (AHEAD) pairs(0, w2[0]);
+                                 matrix_offset(view, prm.pair0 + tile / prm.m_pairs) + (int64_t)prm.sink * view.stride_token;
+            // D = Po V: combine and store rows m and L-1-m
             if (!next_full()) break;
             const uint32_t addr = lane_addr + (phase & 1) * 256;
-            if (AHEAD) tmem_ld16(addr, b2[0]);
+            const bool row_ok = m < prm.rows_half, mirror_ok = row_ok && n_keep - 1 - m != m;
+            const float sgn = (float)prm.mirror_sign;
+            __nv_bfloat16* out_p = mat + (int64_t)m * view.stride_token;
+            __nv_bfloat16* out_m = mat + (int64_t)(n_keep - 1 - m) * view.stride_token;
+            // The next 16 columns leave tensor memory while these are combined and stored (64 matrices 1497 -> 749 44.1 -> 42.1 us).
+            uint32_t d2[2][16];
+            tmem_ld16(addr, d2[0]);
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                if (!AHEAD) tmem_ld16(addr + c * 16, b2[0]);
-                if (!AHEAD) pairs(c, w2[0]);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (AHEAD && c < 7) tmem_ld16(addr + (c + 1) * 16, b2[(c + 1) & 1]);
-                if (AHEAD && c < 7) pairs(c + 1, w2[(c + 1) & 1]);
+                if (c < 7) tmem_ld16(addr + (c + 1) * 16, d2[(c + 1) & 1]);
                 if (c == 7) release();
-                const uint32_t(&b)[16] = b2[AHEAD ? c & 1 : 0];
-                const uint32_t(&w)[WORDS] = w2[AHEAD ? c & 1 : 0];
-                uint32_t y[4][8];
+                const uint32_t(&d)[16] = d2[c & 1];
+                uint32_t p[8], q[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    float lo[4], hi[4];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const float s0 = __uint_as_float(WIDE ? w[(4 * j + 2 * e) % WORDS] : w[2 * j + e] << 16);
-                        const float s1 = __uint_as_float(WIDE ? w[(4 * j + 2 * e + 1) % WORDS] : w[2 * j + e] & 0xffff0000u);
-                        const float A = __uint_as_float(s[c * 16 + 2 * j + e]), B = __uint_as_float(b[2 * j + e]);
-                        const float d0 = fmaf(ct, A, st * B), d1 = fmaf(st, A, -ct * B);
-                        float(&o)[4] = e ? hi : lo;
-                        o[0] = s0 + d0;
-                        o[1] = s0 - d0;
-                        o[2] = s1 + d1;
-                        o[3] = s1 - d1;
-                    }
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) y[r][j] = pack_bf16(lo[r], hi[r]);
+                    const float s0 = __uint_as_float(s[c * 16 + 2 * j]), s1 = __uint_as_float(s[c * 16 + 2 * j + 1]);
+                    const float d0 = __uint_as_float(d[2 * j]), d1 = __uint_as_float(d[2 * j + 1]);
+                    p[j] = pack_bf16(s0 + d0, s1 + d1);
+                    q[j] = pack_bf16(sgn * (s0 - d0), sgn * (s1 - d1));
                 }
-                if (row_ok) {
-                    store_row16(rows[0] + c * 16, y[0], prm.wide_rows);
-                    store_row16(rows[1] + c * 16, y[1], prm.wide_rows);
-                }
-                if (second_ok) {
-                    store_row16(rows[2] + c * 16, y[2], prm.wide_rows);
-                    store_row16(rows[3] + c * 16, y[3], prm.wide_rows);
-                }
+                if (row_ok) store_row16(out_p + c * 16, p, prm.wide_rows);
+                if (mirror_ok) store_row16(out_m + c * 16, q, prm.wide_rows);
             }
         }
     }
@@ -1108,18 +835,6 @@ bool encode_basis_map(CUtensorMap* map, const Basis& basis)
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The four blocks of the basis stacked: 4 * quad_rows_pad rows x fold_ld columns.
-bool encode_quad_map(CUtensorMap* map, const Basis& basis)
-{
-    const cuuint64_t dims[2] = {(cuuint64_t)basis.fold_ld, (cuuint64_t)4 * basis.quad_rows_pad};
-    const cuuint64_t strides[1] = {(cuuint64_t)basis.fold_ld * 2};
-    const cuuint32_t box[2] = {BK, BM};
-    const cuuint32_t elem[2] = {1, 1};
-    return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, basis.quad, dims, strides, box, elem,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // The scratch planes as a 3-D tensor (channel, folded row, plane); rows past n_half read as zero.
 bool encode_scratch_map(CUtensorMap* map, void* scratch, int32_t n_half, int32_t planes)
 {
@@ -1132,11 +847,10 @@ bool encode_scratch_map(CUtensorMap* map, void* scratch, int32_t n_half, int32_t
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// 64-row slices of one phase of the four-block form; the last phase runs on through p where L/2 is even.
+// 64-row slices of one block of the four (gemm_blocks); the last runs on where L/2 is even.
 int32_t quad_steps(int32_t n_in) { return (n_in / 4 + BK - 1) / BK; }
 int32_t quad_last_steps(int32_t n_in, int32_t n_keep) { return n_keep / 2 % 2 ? quad_steps(n_in) : (n_in / 2 + BK - 1) / BK; }
 
-constexpr size_t kRaggedScratchLimit = size_t(64) << 30;  // a ragged batch is folded whole: beyond this it goes sequence by sequence
 constexpr size_t kFoldBufferBytes = size_t(2304) << 20;  // scratch for the folded inputs: a 7B-shaped cache of 4096 tokens fits in one pass
 
 }  // namespace
@@ -1196,19 +910,18 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
         return cudaErrorNotSupported;
     }
     if (!state->attr_set) {
-        const void* kernels[5] = {(const void*)freqkv_gemm_kernel<MODE_SPECTRUM>, (const void*)freqkv_gemm_kernel<MODE_DIRECT>,
-                                  (const void*)freqkv_fold_gemm_kernel<FORM_ONE_LEVEL>, (const void*)freqkv_fold_gemm_kernel<FORM_FOUR_BLOCKS>,
-                                  (const void*)freqkv_fold_gemm_kernel<FORM_RAGGED>};
-        for (int i = 0; i < 5; ++i) {
+        const void* kernels[3] = {(const void*)freqkv_gemm_kernel<MODE_SPECTRUM>, (const void*)freqkv_gemm_kernel<MODE_DIRECT>,
+                                  (const void*)freqkv_fold_gemm_kernel};
+        for (int i = 0; i < 3; ++i) {
             const cudaError_t e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
             if (e != cudaSuccess) {
                 state->last_error = "cudaFuncSetAttribute(max dynamic shared memory)";
                 return e;
             }
         }
-        for (int i = 2; i < 5; ++i) {  // the register shares are of what the block is launched with
+        {  // the register shares are of what the block is launched with
             cudaFuncAttributes fa;
-            const cudaError_t e = cudaFuncGetAttributes(&fa, kernels[i]);
+            const cudaError_t e = cudaFuncGetAttributes(&fa, kernels[2]);
             if (e != cudaSuccess || fa.numRegs < FOLD_LAUNCH_REGS) {
                 state->last_error = "the kernel of the folded forms was not built with the registers it shares out";
                 return e != cudaSuccess ? e : cudaErrorLaunchOutOfResources;
@@ -1217,21 +930,13 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
         // how many CTA pairs the device can hold at once (one CTA per SM; SMs pair up inside a GPC)
         PairLaunch launch(2 * (sm_count / 2), FOLD_THREADS, SMEM_BYTES, nullptr);
         int n = 0;
-        const cudaError_t q = cudaOccupancyMaxActiveClusters(&n, freqkv_fold_gemm_kernel<FORM_ONE_LEVEL>, &launch.cfg);
+        const cudaError_t q = cudaOccupancyMaxActiveClusters(&n, freqkv_fold_gemm_kernel, &launch.cfg);
         if (q != cudaSuccess || n < 1) {
             state->last_error = "cudaOccupancyMaxActiveClusters: no CTA pair fits on this device";
             return q != cudaSuccess ? q : cudaErrorLaunchOutOfResources;
         }
         state->max_clusters = std::min(n, sm_count / 2);
         state->attr_set = true;
-    }
-    if (basis.quad && !state->park) {  // once: it depends on the device alone
-        const cudaError_t e = cudaMalloc(&state->park, (size_t)2 * state->max_clusters * PARK_BYTES_PER_CTA);
-        if (e != cudaSuccess) {
-            state->park = nullptr;
-            state->last_error = "cudaMalloc(work area of the four-block epilogue)";
-            return e;
-        }
     }
     const int32_t n_half = (basis.n_in + 1) / 2;
     const size_t per_pair = (size_t)4 * n_half * 128 * 2;  // K and V, U and V planes
@@ -1242,60 +947,45 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
     return e;
 }
 
-// The shapes of one sequence: everything but its place in the launch.
-static FoldSeq fold_seq(const Basis& b, int32_t pair0, bool quad)
-{
-    FoldSeq s = {};
-    s.pair0 = pair0;
-    s.n_half = (b.n_in + 1) / 2;
-    s.n_keep = b.n_keep;
-    s.rows_half = (b.n_keep + 1) / 2;
-    s.quad = quad;
-    s.basis_rows_pad = s.quad ? b.quad_rows_pad : b.fold_rows_pad;
-    s.k_steps = s.quad ? quad_steps(b.n_in) : (s.n_half + BK - 1) / BK;
-    s.k_last = s.quad ? quad_last_steps(b.n_in, b.n_keep) : 0;
-    const int32_t rows = s.quad ? (s.rows_half + 1) / 2 : s.rows_half;
-    s.m_pairs = (rows + 2 * BM - 1) / (2 * BM);
-    return s;
-}
-
-static FoldParams fold_params(const GemmState* state, const CacheView& view, int32_t sink, int32_t* status_dev)
+static FoldParams fold_params(const GemmState* state, const CacheView& view, const Basis& b, int32_t sink, int32_t* status_dev)
 {
     FoldParams prm = {};
     prm.sink = sink;
-    prm.mirror_sign = 1;
+    prm.mirror_sign = (b.first & 1) ? -1 : 1;
     prm.wide_rows = (((uintptr_t)view.base[0] | (uintptr_t)view.base[1]) & 31) == 0 &&
                     ((view.stride_token | view.stride_head | view.stride_layer | view.stride_batch) & 15) == 0;
-    prm.park = static_cast<uint4*>(state->park);
+    prm.n_keep = b.n_keep;
+    prm.rows_half = (b.n_keep + 1) / 2;
+    prm.basis_rows_pad = b.fold_rows_pad;
+    prm.k_steps = ((b.n_in + 1) / 2 + BK - 1) / BK;
+    prm.m_pairs = (prm.rows_half + 2 * BM - 1) / (2 * BM);
     prm.status = status_dev;
     prm.wait_limit_ns = state->wait_limit_ns;
     return prm;
 }
 
-static FoldJob fold_job(const Basis& b, const FoldSeq& s, int32_t pairs, int32_t sink, void* planes)
+static FoldJob fold_job(const Basis& b, int32_t pair0, int32_t pairs, int32_t sink, void* planes)
 {
     FoldJob job;
-    job.pair0 = s.pair0;
+    job.pair0 = pair0;
     job.pair_count = pairs;
     job.n_in = b.n_in;
-    job.n_half = s.n_half;
+    job.n_half = (b.n_in + 1) / 2;
     job.sink = sink;
     job.dst = static_cast<uint4*>(planes);
-    job.turns = s.quad ? b.turns : nullptr;
     return job;
 }
 
-// Blocks per matrix of a fold launch: each takes rounds of 1024 vectors of one level, or 512 of the four blocks.
+// Blocks per matrix of a fold launch: each takes rounds of 1024 vectors.
 static unsigned fold_blocks(int32_t n_half) { return (unsigned)std::min<int64_t>(((int64_t)n_half * 16 + 1023) / 1024, 64); }
 
 // The product, after its fold launch.
-template <int FORM>
 static cudaError_t launch_product(GemmState* state, const CUtensorMap& map_p, const CUtensorMap& map_x, const CacheView& view,
                                   const FoldParams& prm, const LaunchHooks& hooks, cudaStream_t stream)
 {
     PairLaunch launch(2 * std::min<int32_t>(prm.total_tiles, state->max_clusters), FOLD_THREADS, SMEM_BYTES, stream);
     if (hooks.before) hooks.before(hooks.user, stream);
-    const cudaError_t e = cudaLaunchKernelEx(&launch.cfg, freqkv_fold_gemm_kernel<FORM>, map_p, map_x, view, prm);
+    const cudaError_t e = cudaLaunchKernelEx(&launch.cfg, freqkv_fold_gemm_kernel, map_p, map_x, view, prm);
     if (hooks.after) hooks.after(hooks.user, stream);
     if (e != cudaSuccess) {
         state->last_error = "freqkv_fold_gemm_kernel launch";
@@ -1315,38 +1005,31 @@ cudaError_t launch_gemm(GemmState* state, const CacheView& view, const Basis& ba
     const size_t per_pair = (size_t)4 * ((basis.n_in + 1) / 2) * 128 * 2;
     // One pass when the folded inputs fit the scratch buffer, else several passes of `chunk` pairs.
     const int64_t chunk = std::min<int64_t>(std::max<int64_t>(1, (int64_t)(kFoldBufferBytes / per_pair)), pairs);
-    FoldSeq seq = fold_seq(basis, 0, basis.quad && gemm_blocks(basis.n_in, basis.n_keep, basis.first, chunk, false) == 4);
     CUtensorMap map_p;
-    if (!(seq.quad ? encode_quad_map(&map_p, basis) : encode_basis_map(&map_p, basis))) {
+    if (!encode_basis_map(&map_p, basis)) {
         state->last_error = "tensor map encoding rejected the basis";
         return cudaErrorInvalidValue;
     }
-    FoldParams prm = fold_params(state, view, sink, status_dev);
-    prm.mirror_sign = (basis.first & 1) ? -1 : 1;
+    const int32_t n_half = (basis.n_in + 1) / 2;
+    FoldParams prm = fold_params(state, view, basis, sink, status_dev);
     for (int64_t p0 = 0; p0 < pairs; p0 += chunk) {
         const int32_t count = (int32_t)std::min<int64_t>(chunk, pairs - p0);
         CUtensorMap map_x;
-        if (!encode_scratch_map(&map_x, state->scratch, seq.n_half, count * 4)) {
+        if (!encode_scratch_map(&map_x, state->scratch, n_half, count * 4)) {
             state->last_error = "tensor map encoding rejected the scratch planes";
             return cudaErrorInvalidValue;
         }
-        seq.pair0 = (int32_t)p0;
-        prm.seq = seq;
-        if ((int64_t)count * seq.m_pairs > 0x7fffffff) return cudaErrorInvalidValue;
-        prm.total_tiles = count * seq.m_pairs;
-        const FoldJob job = fold_job(basis, seq, count, sink, state->scratch);
-        const dim3 grid((unsigned)count * 2, fold_blocks(seq.n_half));
-        if (seq.quad)
-            fold_quad_kernel<<<grid, 256, 0, stream>>>(view, job, job.turns);
-        else
-            fold_kernel<<<grid, 256, 0, stream>>>(view, job);
+        prm.pair0 = (int32_t)p0;
+        if ((int64_t)count * prm.m_pairs > 0x7fffffff) return cudaErrorInvalidValue;
+        prm.total_tiles = count * prm.m_pairs;
+        fold_kernel<<<dim3((unsigned)count * 2, fold_blocks(n_half)), 256, 0, stream>>>(
+            view, fold_job(basis, (int32_t)p0, count, sink, state->scratch));
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) {
             state->last_error = "fold_kernel launch";
             return e;
         }
-        e = seq.quad ? launch_product<FORM_FOUR_BLOCKS>(state, map_p, map_x, view, prm, hooks, stream)
-                     : launch_product<FORM_ONE_LEVEL>(state, map_p, map_x, view, prm, hooks, stream);
+        e = launch_product(state, map_p, map_x, view, prm, hooks, stream);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1376,7 +1059,6 @@ cudaError_t launch_gemm_spectrum(GemmState* state, const CacheView& view, const 
         job.n_half = n_half;
         job.sink = sink;
         job.dst = static_cast<uint4*>(state->scratch);
-        job.turns = nullptr;
         fold_kernel<<<dim3((unsigned)job.pair_count * 2, fold_blocks(n_half)), 256, 0, stream>>>(view, job);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) {
@@ -1413,84 +1095,6 @@ cudaError_t launch_gemm_spectrum(GemmState* state, const CacheView& view, const 
         state->kernels_last_call += 2;
     }
     return cudaSuccess;
-}
-
-// A ragged batch in two launches: one fold pass and one tensor-core pass over every sequence, longest first.
-// Everything that can fail for lack of memory happens before the first launch.
-cudaError_t launch_gemm_ragged(GemmState* state, const CacheView& view, const std::vector<RaggedItem>& items_in, int32_t sink,
-                               int32_t* status_dev, int sm_count, const LaunchHooks& hooks, cudaStream_t stream)
-{
-    state->kernels_last_call = 0;
-    if (items_in.empty()) return cudaSuccess;
-    const int32_t lh = view.layers * view.kv_heads;  // (layer, kv_head) pairs per sequence
-    std::vector<RaggedItem> items = items_in;
-    auto work = [](const RaggedItem& it) { return (int64_t)it.basis.n_in * it.basis.n_keep; };
-    std::stable_sort(items.begin(), items.end(), [&](const RaggedItem& a, const RaggedItem& b) { return work(a) > work(b); });
-    const size_t n = items.size();
-    for (const RaggedItem& it : items) {
-        const cudaError_t prepared = gemm_prepare(state, 0, it.basis, sm_count);
-        if (prepared != cudaSuccess) return prepared;
-    }
-    // the table's entries; scratch: the folded planes of every sequence, back to back
-    std::vector<FoldSeq> seqs(n + 1);
-    std::vector<size_t> offset(n);
-    size_t scratch = 0;
-    int64_t tiles = 0;
-    int32_t max_half = 0;
-    for (size_t i = 0; i < n; ++i) {
-        const Basis& b = items[i].basis;
-        const bool quad = b.quad && gemm_blocks(b.n_in, b.n_keep, 0, (int64_t)n * lh, true) == 4;
-        FoldSeq& s = seqs[i] = fold_seq(b, items[i].batch_index * lh, quad);
-        s.tile0 = (int32_t)tiles;
-        tiles += (int64_t)lh * s.m_pairs;
-        max_half = std::max(max_half, s.n_half);
-        if (tiles > 0x7fffffff || (int64_t)n * 2 * lh > 0x7fffffff) return cudaErrorInvalidValue;
-        offset[i] = scratch;
-        scratch += (size_t)lh * 4 * s.n_half * 256;
-    }
-    seqs[n].tile0 = (int32_t)tiles;
-    if (scratch > kRaggedScratchLimit) {
-        state->last_error = "folded inputs of the ragged batch exceed the scratch limit";
-        return cudaErrorMemoryAllocation;
-    }
-    const size_t maps_bytes = n * 2 * sizeof(CUtensorMap), seqs_bytes = ((n + 1) * sizeof(FoldSeq) + 15) / 16 * 16,
-                 jobs_bytes = n * sizeof(FoldJob);
-    cudaError_t e = grow(&state->scratch, &state->scratch_bytes, scratch);
-    if (e == cudaSuccess) e = grow(&state->ragged_meta, &state->ragged_meta_bytes, maps_bytes + seqs_bytes + jobs_bytes);
-    if (e != cudaSuccess) {
-        state->last_error = "cudaMalloc(scratch and tables of a ragged batch)";
-        return e;
-    }
-    std::vector<CUtensorMap> maps(2 * n);
-    std::vector<FoldJob> jobs(n);
-    for (size_t i = 0; i < n; ++i) {
-        char* planes = static_cast<char*>(state->scratch) + offset[i];
-        const Basis& b = items[i].basis;
-        jobs[i] = fold_job(b, seqs[i], lh, sink, planes);
-        if (!(seqs[i].quad ? encode_quad_map(&maps[2 * i], b) : encode_basis_map(&maps[2 * i], b)) ||
-            !encode_scratch_map(&maps[2 * i + 1], planes, seqs[i].n_half, lh * 4)) {
-            state->last_error = "tensor map encoding rejected a sequence of the ragged batch";
-            return cudaErrorInvalidValue;
-        }
-    }
-    char* meta = static_cast<char*>(state->ragged_meta);
-    // pageable sources: each copy has left its host buffer when the call returns
-    e = cudaMemcpyAsync(meta, maps.data(), maps_bytes, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(meta + maps_bytes, seqs.data(), (n + 1) * sizeof(FoldSeq), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(meta + maps_bytes + seqs_bytes, jobs.data(), jobs_bytes, cudaMemcpyHostToDevice, stream);
-    if (e != cudaSuccess) return e;
-    fold_ragged_kernel<<<dim3((unsigned)(n * 2 * lh), fold_blocks(max_half)), 256, 0, stream>>>(
-        view, reinterpret_cast<const FoldJob*>(meta + maps_bytes + seqs_bytes), 2 * lh);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        state->last_error = "fold_ragged_kernel launch";
-        return e;
-    }
-    FoldParams prm = fold_params(state, view, sink, status_dev);
-    prm.total_tiles = (int32_t)tiles;
-    prm.seq_maps = reinterpret_cast<const CUtensorMap*>(meta);
-    prm.seqs = reinterpret_cast<const FoldSeq*>(meta + maps_bytes);
-    return launch_product<FORM_RAGGED>(state, maps[0], maps[1], view, prm, hooks, stream);
 }
 
 // The non-sink rows of one cache tensor as a 5-D tensor (channel, token, kv_head, layer, batch).
@@ -1530,17 +1134,10 @@ int32_t gemm_fold_levels(int32_t n_in, int32_t n_keep, int32_t first)
 
 bool gemm_quad(int32_t n_in, int32_t n_keep, int32_t first) { return gemm_fold_levels(n_in, n_keep, first) == 2; }
 
-// One level or four blocks, for lengths that halve twice.  Four blocks are half the multiply-adds, but a tile of theirs stands for
-// twice the output rows, and its epilogue -- four phases, the pairs' way through L2 -- outlasts its slices where these are few.  So
-// both forms are counted in slices of their longest CTA pair, with a tile of four blocks costing as many more as its epilogue
-// adds: 30, and 60 in a ragged launch, whose pairs are fp32 (8 more for the first of them).  Compression alone in us, one level and four blocks:
-//   512 matrices 1028 -> 514 109, 125; 2048 -> 1024 181, 203; 4092 -> 1022 329, 319; 4096 -> 2048 468, 436; 4092 -> 2046 476, 406;
-//   8188 -> 4094 1707, 1100.  80 matrices 4096 -> 2048 95, 103; 2200 -> 1650 60, 66; 8 matrices 4092 -> 2046 34, 42; 8188 -> 4094 55, 62.
-//   Ragged, 512 matrices of 1028 -> 514 127, 152; 4096 -> 2048 463, 477; 4092 -> 2046 465, 444; 8188 -> 4094 1590, 1094.
-// Compression and append of a 7B-shaped cache (2048 matrices, 4092 -> 2046) 2.52 ms with two levels of the mirror symmetry alone,
-// 2.21 ms with the four blocks; 8B-shaped (4096 matrices, 8188 -> 4094) 15.4 and 12.5 ms; error against 64 bits 1.7e-3 both.
-// (Where a second level means no fewer slices -- kept rows 1026 to 1536 when both lengths halve: two tiles instead of three --
-// four blocks lost up to a third: 512 matrices 2400 -> 1200 251, 331; 16 matrices 2052 -> 1026 25, 37.)
+// In how many blocks the symmetries of the cosines would cut a compression of these lengths, and a call of this size run them: 1, 2
+// (one level), or 4 (both levels, the odd part split by a rotation) where a count of 64-row slices, with 30 for the longer epilogue of a
+// four-block tile, says they pay.  What this file runs is one level; plain compressions of more than 256 kept rows take nearfar.cu, whose
+// work is not cut this way.
 int32_t gemm_blocks(int32_t n_in, int32_t n_keep, int32_t first, int64_t triples, bool ragged)
 {
     if (gemm_is_direct(n_keep)) return 1;
@@ -1617,8 +1214,6 @@ void gemm_release(GemmState* state)
     if (state->scratch) cudaFree(state->scratch);
     state->scratch = nullptr;
     state->scratch_bytes = 0;
-    if (state->park) cudaFree(state->park);
-    state->park = nullptr;
 }
 
 }  // namespace freqkv

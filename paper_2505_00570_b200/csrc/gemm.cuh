@@ -11,10 +11,9 @@ struct GemmState {
     int kernels_last_call = 0;
     bool attr_set = false;
     int max_clusters = 0;     // CTA pairs that can be resident at once
-    void* scratch = nullptr;  // folded inputs U, V: [pairs][K|V][U|V][ceil(n_in/2)][128] bf16 per pass
+    void* scratch = nullptr;  // folded inputs U, V: [pairs][K|V][U|V][ceil(n_in/2)][128] bf16 per pass; or nearfar.cu's flags and far sums
     size_t scratch_bytes = 0;
-    void* park = nullptr;     // four-block form: (s, s') of the tile each CTA works on (38 MB on 74 CTA pairs)
-    void* ragged_meta = nullptr;  // tensor maps, shapes and fold jobs of a ragged batch (device)
+    void* ragged_meta = nullptr;  // tensor maps and shapes of a ragged batch (device)
     size_t ragged_meta_bytes = 0;
     unsigned long long wait_limit_ns = 2000000000ull;  // bound of every mbarrier wait inside the kernel (2 s)
 };
@@ -46,21 +45,11 @@ cudaError_t gemm_prepare(GemmState* state, int32_t pairs, const Basis& basis, in
 bool gemm_is_direct(int32_t n_keep);
 // 0, 1 or 2 levels of the mirror symmetry for a plain compression of these lengths (see gemm.cu).
 int32_t gemm_fold_levels(int32_t n_in, int32_t n_keep, int32_t first);
-// Can a plain compression of these lengths run as four quarter-size blocks?
+// Do the symmetries cut these lengths into four quarter-size blocks?
 bool gemm_quad(int32_t n_in, int32_t n_keep, int32_t first);
-// Blocks that a launch of so many (batch, layer, kv_head) triples runs: 4, 2 (one level), or 1 (the direct mode).
+// Blocks the symmetries cut a call of so many (batch, layer, kv_head) triples into: 4, 2 (one level), or 1 (the direct mode).
 int32_t gemm_blocks(int32_t n_in, int32_t n_keep, int32_t first, int64_t triples, bool ragged);
 cudaError_t launch_gemm_direct(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink,
-                               int32_t* status_dev, int sm_count, const LaunchHooks& hooks, cudaStream_t stream);
-// One sequence of a ragged batch: its index in the cache and the (folded) basis of its lengths.
-struct RaggedItem {
-    int32_t batch_index;
-    Basis basis;
-};
-// Every listed sequence in one fold launch and one tensor-core launch (each needs more than 256 kept
-// rows: the folded form).  `view` covers the whole cache.  cudaErrorMemoryAllocation before anything is
-// enqueued when the folded inputs do not fit: the caller then goes sequence by sequence.
-cudaError_t launch_gemm_ragged(GemmState* state, const CacheView& view, const std::vector<RaggedItem>& items, int32_t sink,
                                int32_t* status_dev, int sm_count, const LaunchHooks& hooks, cudaStream_t stream);
 void gemm_release(GemmState* state);
 // A one-thread kernel that waits, with the tensor-core kernel's own bounded wait, on an mbarrier
