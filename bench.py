@@ -159,8 +159,8 @@ def workload_numbers(w, cache_len, kept, sink, first=0):
         folded = 2.0 * ((kept // 2 + 1) // 2) * 3 * (n_in // 2) * w.head_dim * m
     else:
         folded = 2.0 * 2 * ((kept + 1) // 2) * ((n_in + 1) // 2) * w.head_dim * m
-    # What the library executes: one level, or four blocks of ceil(L/4) x N/4 (the last N/2 deep for even L/2), or the
-    # dense product for few kept rows.
+    # The multiply-adds of the symmetry's blocks: one level, or four of ceil(L/4) x N/4 (the last N/2 deep for even L/2), or the
+    # dense product for few kept rows.  (Plain compressions run fewer: near rows and far values, nearfar.cu.)
     blocks = _fk.gemm_blocks(n_in, kept, m // 2, first)
     executed = {1: 2.0 * kept * n_in, 2: 2.0 * 2 * ((kept + 1) // 2) * ((n_in + 1) // 2),
                 4: 2.0 * ((kept // 2 + 1) // 2) * (4 if kept // 2 % 2 else 5) * (n_in // 4)}[blocks] * w.head_dim * m
@@ -666,9 +666,8 @@ def main():
     per_call = max(t_launches, 1) / args.steps             # launches per compression (large caches take several passes)
     for key in ("executed_flops", "projection_flops", "algorithmic_bytes"):
         nums[key + "_per_launch"] = nums[key] / per_call
-    if chosen == fk.GEMM and kept <= 256:
-        # few kept rows: the tensor-core variant reads the cache directly (no fold pass, one tile per
-        # matrix pair) and is bound by that one read of the cache
+    if chosen == fk.GEMM and (kept <= 256 or not first):
+        # a plain compression reads the cache once and writes the kept rows, with no fold pass: bound by those bytes
         achieved = nums["algorithmic_bytes_per_launch"] / (kernel_ms * 1e-3) / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "peak_kind": "copy, of " + peaks["source"]}
