@@ -107,7 +107,8 @@ freqkv_status freqkv_set_variant(freqkv_ctx* ctx, freqkv_variant variant);
 freqkv_status freqkv_set_fast_family(freqkv_ctx* ctx, int32_t family);
 
 /* Which variant AUTO (or the forced setting) resolves to for this shape; FREQKV_AUTO is never
- * returned (SIMT stands for both of its forms).  Returns FREQKV_ERR_UNSUPPORTED through *out_variant = -1 when none applies. */
+ * returned (SIMT stands for both of its forms; FDCT, under AUTO and for bf16 heads of 64 or 256 channels, also for the one-pass
+ * kernel of variant GEMM, which takes the larger of those calls).  Returns FREQKV_ERR_UNSUPPORTED through *out_variant = -1 when none applies. */
 freqkv_status freqkv_resolve_variant(freqkv_ctx* ctx, const freqkv_layout* layout, int32_t n_in, int32_t n_keep,
                                      int32_t* out_variant);
 

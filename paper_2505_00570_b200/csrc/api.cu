@@ -247,6 +247,18 @@ int32_t resolve(freqkv_ctx* ctx, const freqkv_layout& l, int32_t n_in, int32_t n
     return FREQKV_SIMT;
 }
 
+// bf16 caches with heads of 64 or 256 channels, where AUTO resolves to the fast transform as tensor-core stages: with more than 256
+// kept rows the one-pass kernel takes those, too (a group is four chunks of 64 channels, whatever matrix each belongs to), where
+// the transform would need more than one slab of 8 channels an SM -- below that both wait for a single chain.  Compression in us,
+// fast transform and one pass: heads of 64, 4092 -> 2046, 8 of them 22.5, 25.7; 16 33.7, 29.7; 64 90, 54; 144 194, 100; 1024 -> 512, 8
+// 16.4, 21.5; 16 25.5, 21.5; 144 128, 36; heads of 256, 3000 -> 1500, 2 21.5, 25.6; 4 30.7, 25.6; 32 148, 73.  Error against 64 bits
+// 2.8e-3 and 1.3e-3.  (What runs on the CUDA cores or in the fp32 transform stays there: those round to bf16 once.)
+bool one_pass_heads(freqkv_ctx* ctx, const freqkv_layout& l, int32_t n_in, int32_t n_keep, int64_t triples)
+{
+    return ctx->forced == FREQKV_AUTO && ctx->fast_family == 0 && l.dtype == FREQKV_BF16 && (l.head_dim == 64 || l.head_dim == 256) &&
+           !gemm_is_direct(n_keep) && triples * (l.head_dim / 4) > ctx->sm_count && dctmm_applicable(ctx, l, n_in, n_keep);
+}
+
 void free_bases(freqkv_ctx* ctx)
 {
     for (auto& kv : ctx->bases) {
@@ -494,6 +506,7 @@ freqkv_status compress_group(freqkv_ctx* ctx, const freqkv_layout& l, void* k, v
     const CacheView view = make_view(l, k, v, batch0, batch_count);
     const int32_t n_mat = 2 * view.mats_per_tensor;
 
+    if (variant == FREQKV_FDCT && first == 0 && one_pass_heads(ctx, l, n_in, n_keep, view.mats_per_tensor)) variant = FREQKV_GEMM;
     if (variant == FREQKV_FDCT && first == 0 && dctmm_applicable(ctx, l, n_in, n_keep)) {
         DctmmPlan plan;
         const auto key = std::make_tuple(n_in, n_keep, ctx->fast_family);
@@ -724,6 +737,12 @@ freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_
     DeviceGuard g(ctx->device);
     if (!g.ok) return FREQKV_ERR_CUDA;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    if (variant == FREQKV_FDCT && dtype == FREQKV_BF16 && ctx->forced == FREQKV_AUTO && ctx->fast_family == 0 && n_keep < n_in &&
+        !gemm_is_direct(n_keep) && dctmm_supported(dtype, 64, n_in, n_keep, 0)) {
+        Basis b;  // a plan does not know the heads: one_pass_heads decides with the call
+        const freqkv_status st = get_basis(ctx, n_in, n_keep, 0, false, true, stream, &b);
+        if (st != FREQKV_OK) return st;
+    }
     if (variant == FREQKV_FDCT && dtype == FREQKV_BF16 && n_keep < n_in && dctmm_supported(dtype, 128, n_in, n_keep, ctx->fast_family)) {
         const auto key = std::make_tuple(n_in, n_keep, ctx->fast_family);
         if (ctx->dctmm_plans.find(key) == ctx->dctmm_plans.end()) {

@@ -65,3 +65,16 @@ def test_ragged_batch_of_different_ranks(ctx):
         one_k, one_v = k0[b:b + 1].clone(), v0[b:b + 1].clone()
         ctx.compress(one_k, one_v, n, m, 4)
         assert torch.equal(one_k[0], k[b]) and torch.equal(one_v[0], v[b]), b
+
+
+@pytest.mark.parametrize("hd,H,n_in,kept", [(64, 11, 1030, 515), (64, 19, 2046, 1023), (256, 3, 1028, 514), (256, 5, 700, 350)])
+def test_other_head_sizes(ctx, hd, H, n_in, kept):
+    """Heads of 64 channels (two matrix pairs a group, the last group half empty) and of 256 (one matrix a group), in calls
+    large enough for the one-pass kernel: against the oracle, and more accurate than the fast transform."""
+    w = synth.Workload("t", 1, 2, H, hd, n_in + 7, torch.bfloat16, 4, 0.9, 2, synth.BASE_SEED + 12)
+    err = parity.check_compress(ctx, w, n_in + 4, kept, 4, fk.AUTO, sample=8)
+    parity.check_compress(ctx, w, n_in + 4, kept, 4, fk.AUTO, row_pad=8, sample=4)
+    lay = fk.layout_contiguous(fk.BF16, 1, 2, H, n_in + 7, hd)[1]
+    ctx.set_variant(fk.AUTO)
+    if ctx.resolve_variant(lay, n_in, kept) == fk.FDCT:
+        assert err < parity.check_compress(ctx, w, n_in + 4, kept, 4, fk.FDCT, sample=8)
