@@ -197,6 +197,12 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
         : "memory");
 }
+// A tensor map that a copy has put into global memory, before this thread's loads use it: what the SM holds of the map that lay
+// there before (the call before had other lengths, another cache) is not read again.
+__device__ __forceinline__ void map_acquire(const CUtensorMap* map)
+{
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
+}
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
@@ -354,6 +360,7 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         if (lane == 0) {
             uint32_t it = 0;
             int32_t run_idx = 0;
+            int32_t acquired_far = -1, acquired_tile = -1;  // ragged: sequences whose maps this thread acquired last
             Run run = RAGGED ? prm.runs[0] : prm.run[0];
             int32_t ticket = warp == 0 ? (int32_t)atomicAdd(prm.flags, 1u) : 0;
             bool alive = true;
@@ -411,6 +418,14 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                     }
                     ticket = next;
                     continue;
+                }
+                if (RAGGED) {
+                    if (job.seq != acquired_far && job.seq != acquired_tile)
+                        for (int t = 0; t < 2; ++t) map_acquire(prm.maps + 2 * job.seq + t);
+                    if (job.kind == JOB_FAR)
+                        acquired_far = job.seq;
+                    else
+                        acquired_tile = job.seq;
                 }
                 // chunks 2 (warp - 2) and the one after it: coordinates of their (kv_head, layer, batch)
                 int32_t ch[2], h[2], l[2], b[2], valid = 0;

@@ -69,6 +69,31 @@ def test_ragged_batch_of_different_ranks(ctx):
         assert torch.equal(one_k[0], k[b]) and torch.equal(one_v[0], v[b]), b
 
 
+def test_ragged_calls_in_turn(ctx):
+    """Ragged calls of other lengths, sinks, layouts and caches one after the other, with nothing waited for in between: the tables
+    of each call lie where those of the call before lay.  Every sequence as on its own, bit for bit."""
+    ctx.set_variant(fk.AUTO)
+    calls = []
+    for i, (cap, sink, lens) in enumerate([(2100, 4, [2100, 700, 1300]), (1500, 0, [601, 1500]), (2100, 1, [999, 2048, 2100]),
+                                           (1600, 4, [1600, 1200, 900, 1500, 600, 1001])] * 2):
+        w = workload(cap, sink, B=len(lens), Ly=2, H=2 + i % 3)
+        k, v = synth.make_cache(w, "cuda")
+        if i % 2:  # rows 8 elements apart from the next
+            k, v = (torch.nn.functional.pad(t, (0, 8))[..., :128] for t in (k, v))
+        calls.append((k, v, k.clone(), v.clone(), lens, [(n - sink) // 2 for n in lens], sink))
+        for n, m in zip(lens, calls[-1][5]):
+            ctx.plan(n - sink, m, fk.BF16, fk.GEMM)
+    torch.cuda.synchronize()
+    for k, v, _, _, lens, kept, sink in calls:
+        ctx.compress_ragged(k, v, lens, kept, sink)
+    assert ctx.last_device_status() == fk.OK
+    for k, v, k0, v0, lens, kept, sink in calls:
+        for b, (n, m) in enumerate(zip(lens, kept)):
+            one_k, one_v = k0[b:b + 1].clone(), v0[b:b + 1].clone()
+            ctx.compress(one_k, one_v, n, m, sink)
+            assert torch.equal(one_k[0], k[b]) and torch.equal(one_v[0], v[b]), (lens, b)
+
+
 @pytest.mark.parametrize("hd,H,n_in,kept", [(64, 11, 1030, 515), (64, 19, 2046, 1023), (256, 3, 1028, 514), (256, 5, 700, 350)])
 def test_other_head_sizes(ctx, hd, H, n_in, kept):
     """Heads of 64 channels (two matrix pairs a group, the last group half empty) and of 256 (one matrix a group), in calls
