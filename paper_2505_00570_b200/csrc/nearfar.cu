@@ -570,6 +570,7 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                     ok = wait_flag([&] { return seen(p, [](uint32_t v) { return v != 0; }); });
                 }
                 if (!__all_sync(0xffffffffu, ok)) break;
+                __syncwarp();  // what a lane has acquired holds for all of them (a vote alone orders no memory)
             }
             const int32_t m = job.idx * BM + row;
 #pragma unroll
@@ -608,6 +609,7 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             bool ok = true;
             if (lane == 0 && !job.ready) ok = wait_flag([&] { return seen(far_written + job.group, [&](uint32_t v) { return v >= want; }); });
             if (!__all_sync(0xffffffffu, ok)) break;
+            __syncwarp();  // lane 0 has acquired the sums, every lane reads them (a vote alone orders no memory)
             const int32_t row0 = job.idx * s.rank;
             const float4* in = reinterpret_cast<const float4*>(prm.far + (int64_t)(job.group % prm.ring) * prm.far_stride +
                                                                (int64_t)(row0 / BM) * s.parts * BM * BN) +
