@@ -305,7 +305,8 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     auto far_empty = [&](int s) { return bar0 + 8 * (2 * STAGES + 6 + s); };
     auto job_full = [&](int s) { return bar0 + 8 * (2 * STAGES + 8 + s); };
     auto job_empty = [&](int s) { return bar0 + 8 * (2 * STAGES + 8 + JOBS + s); };
-    constexpr int N_BARS = 2 * STAGES + 8 + 2 * JOBS;
+    constexpr int N_BARS = 2 * STAGES + 9 + 2 * JOBS;
+    const uint32_t drained = bar0 + 8 * (N_BARS - 1);
     Job* jobs = reinterpret_cast<Job*>(bars + N_BARS);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(jobs + JOBS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -328,6 +329,7 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             mbar_init(job_full(s), 1);
             mbar_init(job_empty(s), (LOAD_WARPS - 1) + 1 + EPI_WARPS + FAR_WARPS + 2);
         }
+        mbar_init(drained, 1);
         *abort_flag = 0;
         for (int i = 0; i < EPI_WARPS + FAR_WARPS; ++i) written[i] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -454,10 +456,6 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                         if (valid >> j & 1)
                             tma_load_5d(dst + j * CHUNK_BYTES, map[j], full_bar(st), ch[j], job.row + ks * BK, h[j], l[j], b[j]);
                 }
-            }
-            if (*abort_flag) {  // let the copies in flight land before the shared memory goes away
-                const unsigned long long t0 = global_timer_ns();
-                while (global_timer_ns() - t0 < LANDING_NS) __nanosleep(1000);
             }
         }
     } else if (warp == 1) {
@@ -677,6 +675,16 @@ freqkv_nearfar_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (*abort_flag) {
+        // Some role gave up, whichever: copies that were issued may still be on their way to shared memory and products in the tensor
+        // cores.  Both are waited for, with a limit, before either memory goes away.  (Every role is here, so none issues more.)
+        if (threadIdx.x == 32) umma_commit(drained);
+        if (threadIdx.x == 0 || threadIdx.x == 32) {
+            const unsigned long long t0 = global_timer_ns();
+            while (global_timer_ns() - t0 < LANDING_NS && !(threadIdx.x == 32 && mbar_try_wait(drained, 0))) __nanosleep(1000);
+        }
+        __syncthreads();
+    }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));
 }

@@ -51,3 +51,28 @@ def test_wait_limit_arguments():
         assert ctx.last_device_status() == fk.OK
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("n_in,kept,heads", [(4092, 2046, 1), (1024, 512, 64), (4092, 2046, 64)])
+def test_the_one_pass_compression_gives_up_and_the_next_call_is_right(n_in, kept, heads):
+    """With a limit of a microsecond a healthy call's own waits run out (a tile waits ten microseconds for its far sums): every CTA
+    gives up and returns, the status says so, and the same call with the usual limit gives what it gave before."""
+    ctx = fk.Context(0)
+    try:
+        w = synth.Workload("limit", 1, 1, heads, 128, n_in, torch.bfloat16, 0, 0.9, 2, synth.BASE_SEED + 92)
+        k0, v0 = synth.make_cache(w, "cuda")
+        k, v = k0.clone(), v0.clone()
+        ctx.compress(k, v, n_in, kept, 0)
+        assert ctx.last_device_status() == fk.OK
+        for _ in range(3):
+            ctx.set_wait_limit(1000)
+            ctx.compress(k0.clone(), v0.clone(), n_in, kept, 0)
+            assert ctx.last_device_status() == fk.ERR_TIMEOUT
+            assert "00001000" in ctx.last_error()     # the bit of this kernel
+            ctx.set_wait_limit(2_000_000_000)
+            again_k, again_v = k0.clone(), v0.clone()
+            ctx.compress(again_k, again_v, n_in, kept, 0)
+            assert ctx.last_device_status() == fk.OK
+            assert torch.equal(again_k, k) and torch.equal(again_v, v)
+    finally:
+        ctx.close()
