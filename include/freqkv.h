@@ -133,6 +133,9 @@ freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_
  * whose sum over four mirrored rows leaves the range (above a quarter of the largest value).
  * kept_len == cache_len - sink is the identity and enqueues nothing; kept_len == 0 or
  * cache_len == sink enqueue nothing.
+ * Capture into a graph: a call that runs the fast transform (variant FDCT; under AUTO so do captured calls of bf16 heads of 64
+ * and 256 channels whatever their size) may be captured after freqkv_plan or an earlier call of its lengths.  The other
+ * variants use work areas that a later, larger call may move: freqkv_decode_graph owns its own.
  * Errors: INVALID_ARG (null pointers, sink < 0, sink > cache_len, cache_len > capacity,
  * kept_len < 0, kept_len > cache_len - sink, k == v), UNSUPPORTED (layout rules above, forced
  * variant not applicable), ALLOC, CUDA. */

@@ -259,6 +259,18 @@ bool one_pass_heads(freqkv_ctx* ctx, const freqkv_layout& l, int32_t n_in, int32
            !gemm_is_direct(n_keep) && triples * (l.head_dim / 4) > ctx->sm_count && dctmm_applicable(ctx, l, n_in, n_keep);
 }
 
+// A captured call keeps the fast transform, whose kernel reads nothing but its plan: a capture may not allocate, and a later, larger
+// call would move the one-pass kernel's work area away under the replays.
+bool is_capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &status) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return status != cudaStreamCaptureStatusNone;
+}
+
 void free_bases(freqkv_ctx* ctx)
 {
     for (auto& kv : ctx->bases) {
@@ -506,7 +518,8 @@ freqkv_status compress_group(freqkv_ctx* ctx, const freqkv_layout& l, void* k, v
     const CacheView view = make_view(l, k, v, batch0, batch_count);
     const int32_t n_mat = 2 * view.mats_per_tensor;
 
-    if (variant == FREQKV_FDCT && first == 0 && one_pass_heads(ctx, l, n_in, n_keep, view.mats_per_tensor)) variant = FREQKV_GEMM;
+    if (variant == FREQKV_FDCT && first == 0 && one_pass_heads(ctx, l, n_in, n_keep, view.mats_per_tensor) && !is_capturing(stream))
+        variant = FREQKV_GEMM;
     if (variant == FREQKV_FDCT && first == 0 && dctmm_applicable(ctx, l, n_in, n_keep)) {
         DctmmPlan plan;
         const auto key = std::make_tuple(n_in, n_keep, ctx->fast_family);

@@ -132,3 +132,42 @@ def test_every_row_of_the_basis(ctx, n_in, kept):
     error = (got - want).norm(dim=1) / want.norm(dim=1)
     assert error.max().item() < 2.5e-3, f"row {error.argmax().item()}: {error.max().item():.2e}"
     assert v.abs().max().item() == 0
+
+
+def test_heads_of_64_captured_after_a_plan():
+    """A compression of 64-channel heads, large enough for the one-pass kernel, captured as the context's first call after
+    freqkv_plan: the capture allocates nothing and the replays give what the fast transform gives, also after a larger call of
+    the context."""
+    w = synth.Workload("t", 1, 3, 13, 64, 1024, torch.bfloat16, 0, 0.9, 2, synth.BASE_SEED + 13)
+    k0, v0 = synth.make_cache(w, "cuda")
+    c, stream = fk.Context(0), torch.cuda.Stream()
+    try:
+        c.set_variant(fk.FDCT)
+        want_k, want_v = k0.clone(), v0.clone()
+        c.compress(want_k, want_v, 1024, 512, 0)
+        torch.cuda.synchronize()
+    finally:
+        c.close()
+    c = fk.Context(0)
+    try:
+        lay = fk.layout_of(k0)
+        with torch.cuda.stream(stream):
+            c.plan(1024, 512, fk.BF16, c.resolve_variant(lay, 1024, 512))
+        torch.cuda.synchronize()
+        k, v = k0.clone(), v0.clone()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            c.compress(k, v, 1024, 512, 0)
+        for _ in range(2):
+            with torch.cuda.stream(stream):
+                k.copy_(k0)
+                v.copy_(v0)
+                graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(k, want_k) and torch.equal(v, want_v)
+            with torch.cuda.stream(stream):
+                big = torch.zeros(1, 8, 64, 4092, 64, device="cuda", dtype=torch.bfloat16)
+                c.compress(big, big.clone(), 4092, 2046, 0)
+        del graph
+    finally:
+        c.close()
