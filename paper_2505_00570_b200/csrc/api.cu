@@ -518,8 +518,10 @@ freqkv_status compress_group(freqkv_ctx* ctx, const freqkv_layout& l, void* k, v
     const CacheView view = make_view(l, k, v, batch0, batch_count);
     const int32_t n_mat = 2 * view.mats_per_tensor;
 
-    if (variant == FREQKV_FDCT && first == 0 && one_pass_heads(ctx, l, n_in, n_keep, view.mats_per_tensor) && !is_capturing(stream))
-        variant = FREQKV_GEMM;
+    if (variant == FREQKV_FDCT && first == 0 && one_pass_heads(ctx, l, n_in, n_keep, view.mats_per_tensor) && !is_capturing(stream)) {
+        const freqkv_status st = compress_group(ctx, l, k, v, batch0, batch_count, n_in, n_keep, sink, FREQKV_GEMM, stream);
+        if (st != FREQKV_ERR_ALLOC) return st;  // no memory for its plan or work area, nothing enqueued: the transform needs neither
+    }
     if (variant == FREQKV_FDCT && first == 0 && dctmm_applicable(ctx, l, n_in, n_keep)) {
         DctmmPlan plan;
         const auto key = std::make_tuple(n_in, n_keep, ctx->fast_family);
@@ -752,9 +754,9 @@ freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     if (variant == FREQKV_FDCT && dtype == FREQKV_BF16 && ctx->forced == FREQKV_AUTO && ctx->fast_family == 0 && n_keep < n_in &&
         !gemm_is_direct(n_keep) && dctmm_supported(dtype, 64, n_in, n_keep, 0)) {
-        Basis b;  // a plan does not know the heads: one_pass_heads decides with the call
+        Basis b;  // a plan does not know the heads: one_pass_heads decides with the call, which without this plan runs the transform
         const freqkv_status st = get_basis(ctx, n_in, n_keep, 0, false, true, stream, &b);
-        if (st != FREQKV_OK) return st;
+        if (st != FREQKV_OK && st != FREQKV_ERR_ALLOC) return st;
     }
     if (variant == FREQKV_FDCT && dtype == FREQKV_BF16 && n_keep < n_in && dctmm_supported(dtype, 128, n_in, n_keep, ctx->fast_family)) {
         const auto key = std::make_tuple(n_in, n_keep, ctx->fast_family);

@@ -171,3 +171,36 @@ def test_heads_of_64_captured_after_a_plan():
         del graph
     finally:
         c.close()
+
+
+def test_heads_of_64_without_memory_for_a_work_area():
+    """A call large enough for the one-pass kernel on a device with a few MB free: it runs the fast transform, which needs none."""
+    w = synth.Workload("t", 1, 4, 36, 64, 4092, torch.bfloat16, 0, 0.9, 2, synth.BASE_SEED + 14)
+    k0, v0 = synth.make_cache(w, "cuda")
+    small = torch.zeros(1, 1, 40, 1024, 64, device="cuda", dtype=torch.bfloat16)
+    c, filler = fk.Context(0), []
+    try:
+        c.compress(small, small.clone(), 1024, 512, 0)          # loads the kernels
+        c.set_variant(fk.FDCT)
+        want_k, want_v = k0.clone(), v0.clone()
+        c.compress(want_k, want_v, 4092, 2046, 0)
+        c.set_variant(fk.AUTO)
+        k, v = k0.clone(), v0.clone()
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        size = torch.cuda.mem_get_info()[0] >> 20 << 20
+        while size >= 2 << 20:
+            try:
+                filler.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            except torch.cuda.OutOfMemoryError:
+                size //= 2
+        assert torch.cuda.mem_get_info()[0] < 8 << 20           # its far sums alone take 10 MB
+        c.plan(4092, 2046, fk.BF16, fk.FDCT)
+        c.compress(k, v, 4092, 2046, 0)
+        assert c.last_device_status() == fk.OK
+        filler.clear()
+        assert torch.equal(k, want_k) and torch.equal(v, want_v)
+    finally:
+        filler.clear()
+        torch.cuda.empty_cache()
+        c.close()
