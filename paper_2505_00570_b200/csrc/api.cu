@@ -757,6 +757,11 @@ freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_
         Basis b;  // a plan does not know the heads: one_pass_heads decides with the call, which without this plan runs the transform
         const freqkv_status st = get_basis(ctx, n_in, n_keep, 0, false, true, stream, &b);
         if (st != FREQKV_OK && st != FREQKV_ERR_ALLOC) return st;
+        if (st == FREQKV_OK) {
+            const cudaError_t e = nearfar_reserve(&ctx->gemm, n_in, n_keep);
+            if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(ctx, e, "work area");
+            cudaGetLastError();
+        }
     }
     if (variant == FREQKV_FDCT && dtype == FREQKV_BF16 && n_keep < n_in && dctmm_supported(dtype, 128, n_in, n_keep, ctx->fast_family)) {
         const auto key = std::make_tuple(n_in, n_keep, ctx->fast_family);

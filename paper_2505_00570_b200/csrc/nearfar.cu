@@ -879,6 +879,9 @@ struct Schedule {
     size_t far_offset = 0, bytes = 0;
 };
 
+// Groups of so many rows that the far jobs run ahead of the tiles (of calls with as many).
+int64_t lead(int64_t rows) { return std::max<int64_t>(2, AHEAD_BYTES / (rows * BN * 2)); }
+
 Schedule schedule(const CacheView& view, const std::vector<NearFarItem>& items, int sm_count)
 {
     Schedule s;
@@ -913,7 +916,7 @@ Schedule schedule(const CacheView& view, const std::vector<NearFarItem>& items, 
     // shape 1.10 against 0.93 ms, 8B shape 4.7 and 4.3 ms; 7B with 20 MB 1.57 ms, 30 1.05, 60 0.97, 90 1.00).
     int64_t rows = 0;
     for (const NearFarItem& item : items) rows += (int64_t)groups_of(view.head_dim, item.batch_count * view.layers * view.kv_heads) * item.n_in;
-    s.ahead = (int32_t)std::min<int64_t>(groups, std::max<int64_t>(2, (int64_t)AHEAD_BYTES / (rows / groups * BN * 2)));
+    s.ahead = (int32_t)std::min<int64_t>(groups, lead(rows / groups));
     s.ring = (int32_t)std::min<int64_t>(groups, 2 * (int64_t)s.ahead);
     s.flags = (16 + 2 * groups + reads + 3) / 4 * 4;
     s.far_offset = ((size_t)s.flags * 4 + 255) / 256 * 256;
@@ -1034,6 +1037,13 @@ cudaError_t launch_build_nearfar(void* out, int32_t n_in, int32_t n_keep, cudaSt
     if (e != cudaSuccess) return e;
     build_nearfar_kernel<<<(unsigned)(s.tiles * s.slices + s.far_tiles * s.k_slices), 256, 0, stream>>>(job);
     return cudaGetLastError();
+}
+
+cudaError_t nearfar_reserve(GemmState* state, int32_t n_in, int32_t n_keep)
+{
+    const NearFarShape sh = nearfar_shape(n_in, n_keep);
+    const size_t flags = size_t(1) << 20;
+    return grow(&state->scratch, &state->scratch_bytes, flags + (size_t)(2 * lead(n_in)) * sh.parts * sh.far_tiles * BM * BN * sizeof(float));
 }
 
 cudaError_t nearfar_prepare(GemmState* state, const CacheView& view, const std::vector<NearFarItem>& items, int sm_count)

@@ -35,6 +35,9 @@ struct NearFarItem {
 // Everything a launch needs that is not a stream operation; launch_nearfar calls it itself, a caller that must not
 // allocate later (stream capture) calls it first.
 cudaError_t nearfar_prepare(GemmState* state, const CacheView& view, const std::vector<NearFarItem>& items, int sm_count);
+// The work area of any uniform call of these lengths with up to some 15000 groups of 16 tiles (about 15 MB for each block of 128 far
+// rows), so that the calls after a plan allocate nothing.
+cudaError_t nearfar_reserve(GemmState* state, int32_t n_in, int32_t n_keep);
 cudaError_t launch_nearfar(GemmState* state, const CacheView& view, const std::vector<NearFarItem>& items, int32_t sink,
                            int32_t* status_dev, int sm_count, const LaunchHooks& hooks, cudaStream_t stream);
 

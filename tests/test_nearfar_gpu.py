@@ -204,3 +204,22 @@ def test_heads_of_64_without_memory_for_a_work_area():
         filler.clear()
         torch.cuda.empty_cache()
         c.close()
+
+
+@pytest.mark.parametrize("hd,B,H,n_in,kept", [(64, 2, 72, 4092, 2046), (64, 1, 41, 1024, 512), (256, 1, 300, 3000, 1500)])
+def test_calls_after_a_plan_allocate_nothing(hd, B, H, n_in, kept):
+    w = synth.Workload("t", B, 2, H, hd, n_in, torch.bfloat16, 0, 0.9, 2, synth.BASE_SEED + 15)
+    free = []
+    for _ in range(2):      # the first also loads the kernels, which takes memory of its own
+        k, v = synth.make_cache(w, "cuda")
+        c = fk.Context(0)
+        c.plan(n_in, kept, fk.BF16, c.resolve_variant(fk.layout_of(k), n_in, kept))
+        torch.cuda.synchronize()
+        free.append(torch.cuda.mem_get_info()[0])
+        before = c.get_timing()[2]
+        c.compress(k, v, n_in, kept, 0)
+        torch.cuda.synchronize()
+        free.append(torch.cuda.mem_get_info()[0])
+        assert c.get_timing()[2] - before == 2                  # the one-pass kernel and the one that clears its counters
+        c.close()
+    assert free[2] == free[3], free
