@@ -63,6 +63,7 @@ constexpr int THREADS = 32 * (READ_WARP + 1);
 constexpr int MAX_RANK = 8;
 constexpr int TABLE = 4;                    // int32 per tile: first near column, first and last tile that reads its rows, -
 constexpr int64_t AHEAD_BYTES = 40000000;
+constexpr int64_t RING_BYTES = 256 << 20;   // the far sums of a call whose places are not all of one size (four places may take more)
 constexpr unsigned long long LANDING_NS = 1000000ull;
 constexpr uint32_t FAR_READ = 0x80000000u;  // in the counter of a group: every tile has read the far sums
 
@@ -916,7 +917,9 @@ Schedule schedule(const CacheView& view, const std::vector<NearFarItem>& items, 
     // shape 1.10 against 0.93 ms, 8B shape 4.7 and 4.3 ms; 7B with 20 MB 1.57 ms, 30 1.05, 60 0.97, 90 1.00).
     int64_t rows = 0;
     for (const NearFarItem& item : items) rows += (int64_t)groups_of(view.head_dim, item.batch_count * view.layers * view.kv_heads) * item.n_in;
-    s.ahead = (int32_t)std::min<int64_t>(groups, lead(rows / groups));
+    // The ring's places are as large as the longest sequence needs, their number follows the mean: a long sequence among many short ones
+    // would ask for many large places (131072 -> 65536 beside 31 of 600 -> 300: 33 of 180 MB), so there the lead gives way.
+    s.ahead = (int32_t)std::min<int64_t>({groups, lead(rows / groups), std::max<int64_t>(2, RING_BYTES / (2 * s.far_stride * 4))});
     s.ring = (int32_t)std::min<int64_t>(groups, 2 * (int64_t)s.ahead);
     s.flags = (16 + 2 * groups + reads + 3) / 4 * 4;
     s.far_offset = ((size_t)s.flags * 4 + 255) / 256 * 256;

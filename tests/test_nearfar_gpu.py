@@ -69,6 +69,45 @@ def test_ragged_batch_of_different_ranks(ctx):
         assert torch.equal(one_k[0], k[b]) and torch.equal(one_v[0], v[b]), b
 
 
+def test_a_long_sequence_among_short_ones():
+    """Sixteen blocks of far rows beside sequences of one: the work area is hardly larger than that of the long sequence alone, and
+    every sequence comes out as on its own, bit for bit."""
+    lens, kept = [600] * 32, [300] * 32
+    lens[5], kept[5] = 131072, 65536
+    k0 = torch.zeros(32, 1, 1, 131072, 128, device="cuda", dtype=torch.bfloat16)
+    for b, n in enumerate(lens):
+        k0[b, :, :, :n].normal_()
+    k, v = k0.clone(), k0.clone()
+    one_k, one_v = k0[5:6].clone(), k0[5:6].clone()
+    spare = torch.zeros(4, 1, 1, 600, 128, device="cuda", dtype=torch.bfloat16)
+    c = fk.Context(0)
+    c.compress_ragged(spare, spare.clone(), [600, 560, 580, 600], [300, 270, 290, 300], 0)    # loads the kernels
+    c.close()
+    used = []
+    for _ in range(2):
+        c = fk.Context(0)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        if not used:
+            c.compress(one_k, one_v, 131072, 65536, 0)
+        else:
+            c.compress_ragged(k, v, lens, kept, 0)
+        assert c.last_device_status() == fk.OK
+        used.append(before - torch.cuda.mem_get_info()[0])
+        c.close()
+    assert torch.equal(one_k[0], k[5]) and torch.equal(one_v[0], v[5])
+    c = fk.Context(0)
+    try:
+        for b in (0, 4, 6, 31):
+            one_k, one_v = k0[b:b + 1].clone(), k0[b:b + 1].clone()
+            c.compress(one_k, one_v, 600, 300, 0)
+            assert torch.equal(one_k[0], k[b]) and torch.equal(one_v[0], v[b]), b
+    finally:
+        c.close()
+    print(used)
+    assert used[1] < used[0] + (800 << 20)     # four places of 180 MB instead of one
+
+
 def test_ragged_calls_in_turn(ctx):
     """Ragged calls of other lengths, sinks, layouts and caches one after the other, with nothing waited for in between: the tables
     of each call lie where those of the call before lay.  Every sequence as on its own, bit for bit."""
