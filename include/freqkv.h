@@ -129,8 +129,10 @@ freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_
  * y is rounded once (nearest even) to the cache dtype and written to rows [sink, sink+L).
  * Nothing else is written: sink rows, rows >= sink+L and any stride padding keep their bytes.
  * The caller's new cache length is sink + kept_len.  Arithmetic: fp32 accumulation.  Infinities and
- * NaN stay in their channel; in bf16 caches an infinity may come out as NaN, and so may values
- * whose sum over four mirrored rows leaves the range (above a quarter of the largest value).
+ * NaN stay in their channel; in bf16 caches an infinity may come out as NaN in every row of its channel, and so may values
+ * whose partial sums leave the range.  Variant GEMM: weights of up to 2 in magnitude in all (3 at 131072 rows), so that no
+ * partial sum does for values up to a third of the largest; retained bands: sums of four mirrored rows; variant FDCT: sums over
+ * a factor of the length, so that values above a hundredth of the largest may.
  * kept_len == cache_len - sink is the identity and enqueues nothing; kept_len == 0 or
  * cache_len == sink enqueue nothing.
  * Capture into a graph: a call that runs the fast transform (variant FDCT; under AUTO so do captured calls of bf16 heads of 64

@@ -262,3 +262,30 @@ def test_calls_after_a_plan_allocate_nothing(hd, B, H, n_in, kept):
         assert c.get_timing()[2] - before == 2                  # the one-pass kernel and the one that clears its counters
         c.close()
     assert free[2] == free[3], free
+
+
+@pytest.mark.parametrize("hd,H,n_in,kept", [(128, 3, 1028, 514), (128, 2, 5376, 2689), (64, 41, 1024, 512)])
+def test_infinities_and_nan_stay_in_their_channel(ctx, hd, H, n_in, kept):
+    """An infinity near the first row, one under a middle tile, a NaN: nothing of their channels is claimed but that a NaN is in
+    every row; all other channels keep their bits.  A channel of values just below a third of the range stays finite."""
+    w = synth.Workload("t", 1, 1, H, hd, n_in + 4, torch.bfloat16, 4, 0.9, 2, synth.BASE_SEED + 16)
+    k0, v0 = synth.make_cache(w, "cuda")
+    ctx.set_variant(fk.AUTO)
+    clean_k, clean_v = k0.clone(), v0.clone()
+    ctx.compress(clean_k, clean_v, n_in + 4, kept, 4)
+    top = torch.finfo(torch.bfloat16).max
+    k, v = k0.clone(), v0.clone()
+    k[0, 0, 1, 4 + 7, 9] = float("inf")
+    k[0, 0, 0, 4 + n_in // 2, 0] = float("-inf")
+    v[0, 0, 1, 4 + n_in - 1, hd - 1] = float("nan")
+    v[0, 0, 0, 4:, 17] = top / 3.1
+    ctx.compress(k, v, n_in + 4, kept, 4)
+    assert ctx.last_device_status() == fk.OK
+    assert not torch.isfinite(k[0, 0, 1, 4:4 + kept, 9]).all() and not torch.isfinite(k[0, 0, 0, 4:4 + kept, 0]).all()
+    assert torch.isnan(v[0, 0, 1, 4:4 + kept, hd - 1]).all()
+    steady = v[0, 0, 0, 4:4 + kept, 17].double() / (top / 3.1) - 1
+    assert steady.abs().max().item() < 3e-2
+    for got, want, touched in ((k, clean_k, ((1, 9), (0, 0))), (v, clean_v, ((1, hd - 1), (0, 17)))):
+        for head, channel in touched:
+            got[0, 0, head, :, channel] = want[0, 0, head, :, channel] = 0
+        assert torch.equal(got, want)
