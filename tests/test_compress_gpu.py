@@ -190,12 +190,10 @@ def test_ragged_batch_small(ctx):
 
 
 def test_ragged_batch_in_two_launches(ctx):
-    """A ragged batch whose sequences all take the folded tensor-core form runs as ONE fold launch
-    and ONE tensor-core launch (the kernel counter says so); odd and even lengths, one sequence
-    left alone (kept == length), one with more than one tile of rows.  Against the oracle, against
-    the bytes outside the rewritten rows, and against compressing each sequence on its own: bit
-    for bit where both run one level of the symmetry fold, and to well inside the tolerance where the
-    lengths halve twice, so that larger calls would run four blocks."""
+    """A ragged batch whose sequences all take the one-pass tensor-core form runs as ONE launch that
+    clears its counters and ONE tensor-core launch (the kernel counter says so); odd and even lengths,
+    one sequence left alone (kept == length).  Against the oracle, against the bytes outside the
+    rewritten rows, and bit for bit against compressing each sequence on its own."""
     w = small(cap=1400, dtype=torch.bfloat16, sink=4, B=6, Ly=2, H=3, outliers=2)
     k, v = synth.make_cache(w, "cuda")
     k_in, v_in = k.clone(), v.clone()
@@ -218,13 +216,7 @@ def test_ragged_batch_in_two_launches(ctx):
     for b in range(6):
         one_k, one_v = k_in[b:b + 1].clone(), v_in[b:b + 1].clone()
         ctx.compress(one_k, one_v, lens[b], kept[b], 4)
-        if (lens[b] - 4) % 4 == 0 and kept[b] % 2 == 0 and kept[b] > 256:   # lengths of four blocks
-            for one, both in ((one_k, k), (one_v, v)):
-                a, c = one[0, :, :, 4:4 + kept[b]].double(), both[b, :, :, 4:4 + kept[b]].double()
-                assert ((a - c).norm() / c.norm()).item() < 5e-3
-                assert torch.equal(one[0, :, :, :4], both[b, :, :, :4]) and torch.equal(one[0, :, :, 4 + kept[b]:], both[b, :, :, 4 + kept[b]:])
-        else:
-            assert torch.equal(one_k[0], k[b]) and torch.equal(one_v[0], v[b]), f"sequence {b} differs from its own compression"
+        assert torch.equal(one_k[0], k[b]) and torch.equal(one_v[0], v[b]), f"sequence {b} differs from its own compression"
         for t_in, t_out in ((k_in, k), (v_in, v)):
             assert torch.equal(t_out[b, :, :, :4], t_in[b, :, :, :4])
             assert torch.equal(t_out[b, :, :, 4 + kept[b]:], t_in[b, :, :, 4 + kept[b]:])
@@ -242,40 +234,35 @@ def test_gemm_lengths(ctx, n_in, kept, sink):
 
 
 @pytest.mark.parametrize("n_in,kept,sink", [(2048, 1024, 0), (4092, 2728, 4), (1396, 698, 4), (4092, 2046, 4), (2732, 1366, 0)])
-def test_gemm_two_fold_levels(ctx, n_in, kept, sink):
-    """Lengths that halve twice (n_in a multiple of 4, kept even), in calls too small for four blocks: a whole
-    number of 256-row tiles (2048 -> 1024), a ragged last tile (2728 kept rows: 682 twice-folded ones), an odd
-    kept / 2 whose middle row is its own mirror (698, 2046, 1366), several sequences, layers and heads, padded rows."""
+def test_gemm_lengths_that_halve_twice(ctx, n_in, kept, sink):
+    """Lengths that halve twice (n_in a multiple of 4, kept even): a whole number of 128-row tiles (2048 -> 1024), ragged
+    last tiles, several sequences, layers and heads, padded rows."""
     w = small(cap=n_in + sink + 3, dtype=torch.bfloat16, sink=sink, outliers=2, B=2, Ly=2, H=3)
     parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM)
     parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM, row_pad=8)
 
 
 @pytest.mark.parametrize("n_in,kept,sink", [(1028, 514, 4), (1032, 516, 0), (2048, 1028, 4), (3000, 1500, 4), (2064, 1026, 1)])
-def test_gemm_four_blocks(ctx, n_in, kept, sink):
-    """Lengths the four blocks could take at their edges, in calls too small for them: the fewest kept rows, a row more than one
-    tile of 256, even and odd kept / 2, inputs that are no whole number of 64-row slices."""
+def test_gemm_few_rows_in_the_last_tile(ctx, n_in, kept, sink):
+    """Two and four rows in the last tile of 128 and most of a tile, inputs that are no whole number of 64-row slices."""
     w = small(cap=n_in + sink + 3, dtype=torch.bfloat16, sink=sink, outliers=2, B=1, Ly=2, H=2)
     parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM)
     parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM, row_pad=8)
 
 
 @pytest.mark.parametrize("n_in,kept,sink,H", [(2044, 1022, 4, 20), (4096, 1024, 0, 20), (3076, 1538, 4, 10), (4096, 2048, 4, 10), (2200, 1650, 1, 10), (8188, 4094, 4, 5)])
-def test_gemm_runs_four_blocks(ctx, n_in, kept, sink, H):
-    """Calls that run four blocks, at the edges of their tiles: one whole tile of 256 quarter rows (511 and 512 half rows), a tile and
-    129 rows, two whole tiles, four; even and odd kept / 2 (an even one leaves a component without a partner, so the last phase
-    runs on; the middle row of an odd one is its own mirror); rows that are 16- but not 32-byte aligned."""
-    assert fk.gemm_blocks(n_in, kept, 2 * H) == 4
+def test_gemm_lengths_in_larger_calls(ctx, n_in, kept, sink, H):
+    """Calls of many groups, ratios of a half, a quarter and three quarters, whole and ragged tiles; rows that are 16- but not
+    32-byte aligned."""
     w = small(cap=n_in + sink + 3, dtype=torch.bfloat16, sink=sink, outliers=2, B=1, Ly=2, H=H)
     parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM, sample=6)
     parity.check_compress(ctx, w, n_in + sink, kept, sink, fk.GEMM, row_pad=8, sample=6)
 
 
 @pytest.mark.parametrize("pairs,n_in,kept", [(256, 2400, 1200), (256, 1028, 514), (8, 4092, 2046)])
-def test_one_level_where_it_is_faster(ctx, pairs, n_in, kept):
-    """Lengths and sizes of call at which four blocks cost 15 to 35 % more than one level of the fold, which a retained band above
-    the lowest component always runs: the compression takes no longer than such a band (median of alternating
-    runs; the two launch the same work)."""
+def test_plain_compressions_are_no_slower_than_a_band(ctx, pairs, n_in, kept):
+    """A retained band above the lowest component runs a fold pass and one level of the symmetry: the plain compression of the
+    same lengths takes no longer (median of alternating runs)."""
     ctx.set_variant(fk.AUTO)
     k, v = (torch.randn(1, 1, pairs, n_in, 128, device="cuda").bfloat16() for _ in range(2))
     times = {0: [], 1: []}
@@ -296,10 +283,9 @@ def test_one_level_where_it_is_faster(ctx, pairs, n_in, kept):
 
 
 @pytest.mark.parametrize("row_pad", [0, 8])
-def test_ragged_batch_mixes_four_blocks_and_one_level(ctx, row_pad):
-    """Sequences of four blocks with even kept / 2 (their last phase runs on through p) and with odd, beside one-level ones: phase
-    counts and depths change from tile to tile.  Whole rows and rows that are 16- but not 32-byte aligned; against the oracle and,
-    sequence by sequence, against the call on its own, which keeps the four blocks' pairs in bf16."""
+def test_ragged_batch_of_long_and_short_sequences(ctx, row_pad):
+    """Sequences of four and of eight nodes a tile, even and odd lengths: the depth of the jobs changes from tile to tile.  Whole
+    rows and rows that are 16- but not 32-byte aligned; against the oracle and, bit for bit, against each sequence on its own."""
     w = small(cap=8200, dtype=torch.bfloat16, sink=4, B=4, Ly=2, H=10, outliers=2)
     (_, k), (_, v) = parity.guarded_cache(w, torch.device("cuda"), fill_len=8200, row_pad=row_pad)
     k_in, v_in = k.clone(), v.clone()
@@ -311,8 +297,7 @@ def test_ragged_batch_mixes_four_blocks_and_one_level(ctx, row_pad):
         ctx.compress(one_k, one_v, lens[b], kept[b], 4)
         for t_in, t_out, one in ((k_in, k, one_k), (v_in, v, one_v)):
             assert torch.equal(t_out[b, :, :, :4], t_in[b, :, :, :4]) and torch.equal(t_out[b, :, :, 4 + kept[b]:], t_in[b, :, :, 4 + kept[b]:])
-            a, c = one[0, :, :, 4:4 + kept[b]].double(), t_out[b, :, :, 4:4 + kept[b]].double()
-            assert ((a - c).norm() / c.norm()).item() < 5e-3
+            assert torch.equal(one[0], t_out[b]), b
         for t_in, t_out, l, h in ((k_in, k, 0, 0), (v_in, v, 1, 9)):
             want = oracle.compress_matrix(parity.to_f64(t_in[b, l, h, 4:lens[b]]), kept[b])
             parity.check_matrix(parity.to_f64(t_out[b, l, h, 4:4 + kept[b]]), want, torch.bfloat16, f"sequence {b}")

@@ -18,7 +18,7 @@ def ctx():
     c.close()
 
 
-@pytest.mark.parametrize("cap,sink,kept,T", [(300, 4, 148, 1000), (132, 0, 33, 500)])
+@pytest.mark.parametrize("cap,sink,kept,T", [(300, 4, 148, 1000), (132, 0, 33, 500), (700, 4, 348, 1800)])
 def test_decode_graph_equals_host_driven_stream(ctx, cap, sink, kept, T):
     w = synth.Workload("dg", 2, 2, 2, 128, cap, torch.bfloat16, sink, 0.9, 2, synth.BASE_SEED + 41)
     gen = torch.Generator(device="cuda")
@@ -62,12 +62,12 @@ def test_decode_graph_equals_host_driven_stream(ctx, cap, sink, kept, T):
         graph.close()
 
 
-def test_decode_graph_survives_larger_calls_on_its_context(ctx):
-    """The graph's kernels have the addresses of the fold scratch and of the basis baked in.  Other
-    calls on the same context that need a larger scratch (a bigger cache) or rebuild plans must not
+@pytest.mark.parametrize("cap,sink,kept,T", [(300, 4, 148, 700), (640, 4, 300, 1400)])
+def test_decode_graph_survives_larger_calls_on_its_context(ctx, cap, sink, kept, T):
+    """The graph's kernels have the addresses of the work area and of the plan baked in.  Other
+    calls on the same context that need a larger work area (a bigger cache) or rebuild plans must not
     move or free what a live graph replays from: the graph owns its own.  The stream through the
     graph, with such calls in between, must still be bit-identical to the host-driven one."""
-    cap, sink, kept, T = 300, 4, 148, 700
     w = synth.Workload("dg", 2, 2, 2, 128, cap, torch.bfloat16, sink, 0.9, 2, synth.BASE_SEED + 43)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(w.seed)
@@ -92,7 +92,7 @@ def test_decode_graph_survives_larger_calls_on_its_context(ctx):
     graph = fk.DecodeGraph(ctx, k2, v2, stage_k, stage_v, lens_dev, kept, sink)
     try:
         for t in range(T):
-            if t in (10, 350):   # a call that needs a much larger fold scratch, and the graph's own shape again
+            if t in (10, 350):   # a call that needs a much larger work area, and the graph's own shape again
                 kb, vb = synth.make_cache(big, "cuda")
                 ctx.compress(kb, vb, 1500, 748, sink)
                 ks, vs = synth.make_cache(w, "cuda")
