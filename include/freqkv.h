@@ -108,7 +108,8 @@ freqkv_status freqkv_set_fast_family(freqkv_ctx* ctx, int32_t family);
 
 /* Which variant AUTO (or the forced setting) resolves to for this shape; FREQKV_AUTO is never
  * returned (SIMT stands for both of its forms; FDCT, under AUTO and for bf16 heads of 64 or 256 channels, also for the one-pass
- * kernel of variant GEMM, which takes the larger of those calls).  Returns FREQKV_ERR_UNSUPPORTED through *out_variant = -1 when none applies. */
+ * kernel of variant GEMM, which takes the larger of those calls; freqkv_plan makes its work area, too, and where there is no
+ * memory for it, or in a capture, they run the transform).  Returns FREQKV_ERR_UNSUPPORTED through *out_variant = -1 when none applies. */
 freqkv_status freqkv_resolve_variant(freqkv_ctx* ctx, const freqkv_layout* layout, int32_t n_in, int32_t n_keep,
                                      int32_t* out_variant);
 
@@ -130,9 +131,9 @@ freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_
  * Nothing else is written: sink rows, rows >= sink+L and any stride padding keep their bytes.
  * The caller's new cache length is sink + kept_len.  Arithmetic: fp32 accumulation.  Infinities and
  * NaN stay in their channel; in bf16 caches an infinity may come out as NaN in every row of its channel, and so may values
- * whose partial sums leave the range.  Variant GEMM: weights of up to 2 in magnitude in all (3 at 131072 rows), so that no
- * partial sum does for values up to a third of the largest; retained bands: sums of four mirrored rows; variant FDCT: sums over
- * a factor of the length, so that values above a hundredth of the largest may.
+ * whose partial sums leave the range.  Variant GEMM: values of up to a tenth of the largest never do, whatever their signs
+ * (measured: none up to 0.45 of it; retained bands add four mirrored rows first); variant FDCT sums over a factor of the length
+ * first, where values above a hundredth of the largest may.
  * kept_len == cache_len - sink is the identity and enqueues nothing; kept_len == 0 or
  * cache_len == sink enqueue nothing.
  * Capture into a graph: a call that runs the fast transform (variant FDCT; under AUTO so do captured calls of bf16 heads of 64
@@ -374,7 +375,7 @@ freqkv_status freqkv_fast_plan_apply_host(int32_t n_in, int32_t n_keep, int32_t 
  * level the multiply-adds per matrix are 2 * ceil(L/2) * ceil(N/2) * head_dim, with two of the mirror symmetry alone
  * 3 * ceil(L/4) * (N/2) * head_dim.  -1 for invalid lengths.  Retained bands that start higher and the power
  * spectrum always use one level.  (A count of what the symmetry would save: plain compressions of more than 256 kept rows run in
- * one pass over the cache instead, whose work grows with n_in alone.) */
+ * one pass over the cache instead, whose products grow with n_in, and from 4096 kept rows on with n_in * kept_len / 4096.) */
 int32_t freqkv_gemm_fold_levels(int32_t n_in, int32_t kept_len, int32_t first_component);
 
 /* Host-only: in how many blocks the symmetries would cut such a compression of `triples` (batch, layer, kv_head) triples:

@@ -39,7 +39,7 @@ struct freqkv_ctx {
     int32_t* status_dev = nullptr;
     GemmState gemm;
     std::string last_error;
-    // Work areas (fold scratch, staging, attention partials) are shared by all calls on this
+    // Work areas (folded rows, far sums, staging, attention partials) are shared by all calls on this
     // context: a call on another stream than the previous one first waits for that one's work.
     cudaEvent_t work_done = nullptr;
     cudaStream_t work_stream = nullptr;
@@ -225,13 +225,12 @@ bool dctmm_applicable(freqkv_ctx* ctx, const freqkv_layout& l, int32_t n_in, int
 }
 
 // Variant table, from measurements on B200 (7B shape, 2048 matrices of head_dim 128, bf16): the
-// tensor-core projection takes 1.75 ms at 4092 -> 2046 (fold pass included)
-// and the fast transform 2.49 ms (2.77 ms at 4096 -> 2048); at 4092 -> 1023, 3000 -> 1500 and 2046 -> 1023 the
-// projection is 1.5 to 2.3 times faster (its work shrinks with both lengths, the fast transform's
-// per-slab chain of steps does not), at 4092 -> 3069 they are level.  So bf16 caches with head_dim
-// 128 go to the projection whenever a tile can be filled; the fast transform serves what the
-// projection does not take (bf16 with other head sizes: 40 times faster there than the CUDA cores;
-// fp32 caches of power-of-two length); everything else runs as a projection on the CUDA cores (fp32: folded first).
+// tensor-core projection in one pass takes 0.92 ms at 4092 -> 2046, the fast transform 2.49 ms; where less is
+// kept the projection gains more (its work shrinks with the length, the fast transform's per-slab chain of
+// steps does not).  So bf16 caches with head_dim 128 go to the projection whenever a tile can be filled; the
+// fast transform serves what the projection does not take (bf16 with other head sizes, unless one_pass_heads below
+// says otherwise: 40 times faster there than the CUDA cores; fp32 caches of power-of-two length); everything else
+// runs as a projection on the CUDA cores (fp32: folded first).
 int32_t resolve(freqkv_ctx* ctx, const freqkv_layout& l, int32_t n_in, int32_t n_keep)
 {
     const bool g = gemm_applicable(l, n_in, n_keep);
@@ -293,7 +292,7 @@ bool fold_f32_applies(const freqkv_ctx* ctx, int32_t dtype, int32_t n_in, int32_
 }
 
 // Projection basis for (n_in, n_keep) holding at least the requested forms: the full fp32 matrix
-// (CUDA-core path), the folded bf16 pair Pe, Po (tensor-core path), the folded fp32 planes.
+// (CUDA-core path), what the tensor-core path reads for these lengths, the folded fp32 planes.
 freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t first, bool need_f32, bool need_fold,
                         cudaStream_t stream, Basis* out, bool need_f32_fold = false)
 {
@@ -301,7 +300,7 @@ freqkv_status get_basis(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, int32_t f
     Basis b;
     auto it = ctx->bases.find(key);
     if (it != ctx->bases.end()) b = it->second;
-    // the tensor-core path wants the folded pair, or, for few kept rows, the dense bf16 matrix
+    // the tensor-core path reads the dense bf16 matrix where few rows are kept
     const bool direct = need_fold && first != kDctRows && gemm_is_direct(n_keep);
     // (a plain compression: in one pass, nearfar.cu; retained bands and the spectrum: the folded pair)
     const bool one_pass = need_fold && !direct && first == 0;
@@ -920,18 +919,18 @@ freqkv_status freqkv_compress_ragged(freqkv_ctx* ctx, const freqkv_layout* layou
     if (!g.ok) return FREQKV_ERR_CUDA;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     WorkOrder order(ctx, stream);
-    // When every sequence that needs work takes the folded tensor-core form, the whole batch runs
-    // as one fold launch and one tensor-core launch; every plan is built and all memory is
-    // allocated before the first of them.
+    // When every sequence that needs work takes the one-pass tensor-core form, the whole batch runs
+    // as one tensor-core launch behind one that clears its counters; every plan is built and all
+    // memory is allocated before the first of them.
     {
-        bool all_folded = true;
+        bool all_one_pass = true;
         int32_t active = 0;
         for (int32_t b = 0; b < layout->batch; ++b) {
             if (variant[b] == 0) continue;
             ++active;
-            if (variant[b] != FREQKV_GEMM || gemm_is_direct(kept_len[b])) all_folded = false;
+            if (variant[b] != FREQKV_GEMM || gemm_is_direct(kept_len[b])) all_one_pass = false;
         }
-        if (all_folded && active > 1) {
+        if (all_one_pass && active > 1) {
             std::vector<NearFarItem> items;
             bool ok = true;
             for (int pass = 0; pass < 2 && ok; ++pass) {  // second pass: a flush of the plan cache may have dropped earlier plans
@@ -967,7 +966,7 @@ freqkv_status freqkv_compress_ragged(freqkv_ctx* ctx, const freqkv_layout* layou
                 }
                 if (e != cudaErrorMemoryAllocation || ctx->gemm.kernels_last_call != 0)
                     return cuda_fail(ctx, e, ctx->gemm.last_error ? ctx->gemm.last_error : "launch_nearfar");
-                cudaGetLastError();  // the folded batch does not fit: go sequence by sequence
+                cudaGetLastError();  // the work area of the whole batch does not fit: go run by run
             }
         }
     }
@@ -1310,7 +1309,7 @@ freqkv_status freqkv_attend_prefill(freqkv_ctx* ctx, const freqkv_layout* layout
     return FREQKV_OK;
 }
 
-// The graph's kernels have the addresses of the fold scratch and of the basis baked in, so the
+// The graph's kernels have the addresses of the work area and of the plan baked in, so the
 // graph owns both: no later call on the context can free or move them under a replay.
 struct freqkv_decode_graph {
     freqkv_ctx* ctx = nullptr;
@@ -1367,7 +1366,7 @@ freqkv_status freqkv_decode_graph_create(freqkv_ctx* ctx, const freqkv_layout* l
     cudaError_t e = st == FREQKV_OK ? cudaStreamSynchronize(cs) : cudaSuccess;
     if (st == FREQKV_OK && e == cudaSuccess)
         e = gemm_is_direct(kept_len) ? gemm_prepare(&dg->gemm, 0, basis, ctx->sm_count)
-                                     : nearfar_prepare(&dg->gemm, make_view(l, k, v, 0, l.batch), {{0, l.batch, n_in, kept_len, basis.nearfar}}, ctx->sm_count);
+                                     : nearfar_prepare(&dg->gemm, make_view(l, k, v, 0, l.batch), {{0, l.batch, n_in, kept_len, basis.nearfar}});
     auto fail = [&](freqkv_status code, cudaError_t ce, const char* where) {
         if (ce != cudaSuccess) code = cuda_fail(ctx, ce, where);
         if (dg) {
@@ -1386,7 +1385,7 @@ freqkv_status freqkv_decode_graph_create(freqkv_ctx* ctx, const freqkv_layout* l
     if (!dg) return fail(FREQKV_ERR_ALLOC, cudaSuccess, "");
     dg->ctx = ctx;
 
-    // graph: trigger -> IF (all sequences full) { fold, GEMM, lengths := sink + kept_len } -> append + advance
+    // graph: trigger -> IF (all sequences full) { compression, lengths := sink + kept_len } -> append + advance
     if ((e = cudaGraphCreate(&dg->graph, 0)) != cudaSuccess) return fail(FREQKV_ERR_CUDA, e, "cudaGraphCreate");
     cudaGraphConditionalHandle handle;
     if ((e = cudaGraphConditionalHandleCreate(&handle, dg->graph, 0, cudaGraphCondAssignDefault)) != cudaSuccess)
@@ -1551,7 +1550,7 @@ int32_t freqkv_gemm_fold_levels(int32_t n_in, int32_t kept_len, int32_t first_co
 int32_t freqkv_gemm_blocks(int32_t n_in, int32_t kept_len, int32_t first_component, int64_t triples)
 {
     if (n_in < 1 || kept_len < 1 || kept_len > n_in || first_component < 0 || first_component > n_in - kept_len || triples < 1) return -1;
-    return gemm_blocks(n_in, kept_len, first_component, triples, false);
+    return gemm_blocks(n_in, kept_len, first_component, triples);
 }
 
 const char* freqkv_last_error(freqkv_ctx* ctx) { return ctx ? ctx->last_error.c_str() : ""; }

@@ -1138,7 +1138,7 @@ bool gemm_quad(int32_t n_in, int32_t n_keep, int32_t first) { return gemm_fold_l
 // (one level), or 4 (both levels, the odd part split by a rotation) where a count of 64-row slices, with 30 for the longer epilogue of a
 // four-block tile, says they pay.  What this file runs is one level; plain compressions of more than 256 kept rows take nearfar.cu, whose
 // work is not cut this way.
-int32_t gemm_blocks(int32_t n_in, int32_t n_keep, int32_t first, int64_t triples, bool ragged)
+int32_t gemm_blocks(int32_t n_in, int32_t n_keep, int32_t first, int64_t triples)
 {
     if (gemm_is_direct(n_keep)) return 1;
     if (!gemm_quad(n_in, n_keep, first)) return 2;
@@ -1147,8 +1147,7 @@ int32_t gemm_blocks(int32_t n_in, int32_t n_keep, int32_t first, int64_t triples
     const int64_t tiles2 = (rows_half + 2 * BM - 1) / (2 * BM), tiles4 = (rows_quarter + 2 * BM - 1) / (2 * BM);
     const int64_t slices2 = 2 * ((n_in / 2 + BK - 1) / BK), slices4 = 3 * quad_steps(n_in) + quad_last_steps(n_in, n_keep);
     const int64_t waves2 = (triples * tiles2 + CLUSTERS - 1) / CLUSTERS, waves4 = (triples * tiles4 + CLUSTERS - 1) / CLUSTERS;
-    const int64_t cost4 = ragged ? waves4 * (slices4 + 60) + 8 : waves4 * (slices4 + 30);
-    return cost4 < waves2 * slices2 ? 4 : 2;
+    return waves4 * (slices4 + 30) < waves2 * slices2 ? 4 : 2;
 }
 
 cudaError_t launch_gemm_direct(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink,

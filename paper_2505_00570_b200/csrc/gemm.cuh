@@ -48,7 +48,7 @@ int32_t gemm_fold_levels(int32_t n_in, int32_t n_keep, int32_t first);
 // Do the symmetries cut these lengths into four quarter-size blocks?
 bool gemm_quad(int32_t n_in, int32_t n_keep, int32_t first);
 // Blocks the symmetries cut a call of so many (batch, layer, kv_head) triples into: 4, 2 (one level), or 1 (the direct mode).
-int32_t gemm_blocks(int32_t n_in, int32_t n_keep, int32_t first, int64_t triples, bool ragged);
+int32_t gemm_blocks(int32_t n_in, int32_t n_keep, int32_t first, int64_t triples);
 cudaError_t launch_gemm_direct(GemmState* state, const CacheView& view, const Basis& basis, int32_t sink,
                                int32_t* status_dev, int sm_count, const LaunchHooks& hooks, cudaStream_t stream);
 void gemm_release(GemmState* state);

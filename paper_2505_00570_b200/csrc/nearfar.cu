@@ -15,7 +15,9 @@
 //         (Beckermann, Townsend, "Bounds on the singular values of matrices with displacement structure", 2019) -- for
 //         which the error falls by a constant factor per node.  So a tile needs `rank` numbers per channel of all its far
 //         rows, E_i = sum_{n far} w_in x_n.
-// Work per matrix grows with N instead of N L, for every N and L: no length has to halve.
+// The near products grow with N instead of N L, for every N and L: no length has to halve.  The far products are N for each 128
+// far rows, `rank` of them a tile: one block up to 4096 kept rows, then N L / 4096 (16 blocks at 131072 -> 65536, with 0.5 GB of
+// far basis and 180 MB of sums for a group in flight).
 //
 // The kernel.  One persistent CTA per SM takes jobs in the order of a ticket counter; a group of columns is 256 channels,
 // the K and the V matrix of one (batch, layer, kv_head) of head_dim 128.  For every group come first its far jobs (a range of
@@ -32,7 +34,9 @@
 // only tiles before it and the one after it can be among them, so every wait is for a job whose ticket is lower, or the
 // very next one, which nothing keeps from loading (its accumulator is the other one, its far jobs have lower tickets).
 //
-// Bound by HBM: (N + L) rows in and out.
+// Its floor is HBM, (N + L) rows in and out; it runs at 0.46 to 0.59 of that: a job costs 7900 cycles and 770 for each of its slices
+// (48 KB at the 64 bytes a clock that an SM takes from L2), and the first part hides behind nothing (4092 -> 2046 x 1024 groups 0.92 ms,
+// 131 jobs an SM of 7.6 slices).
 #include <cuda.h>
 
 #include <algorithm>
@@ -883,7 +887,7 @@ struct Schedule {
 // Groups of so many rows that the far jobs run ahead of the tiles (of calls with as many).
 int64_t lead(int64_t rows) { return std::max<int64_t>(2, AHEAD_BYTES / (rows * BN * 2)); }
 
-Schedule schedule(const CacheView& view, const std::vector<NearFarItem>& items, int sm_count)
+Schedule schedule(const CacheView& view, const std::vector<NearFarItem>& items)
 {
     Schedule s;
     int64_t reads = 0, jobs = 0, groups = 0;
@@ -1049,16 +1053,16 @@ cudaError_t nearfar_reserve(GemmState* state, int32_t n_in, int32_t n_keep)
     return grow(&state->scratch, &state->scratch_bytes, flags + (size_t)(2 * lead(n_in)) * sh.parts * sh.far_tiles * BM * BN * sizeof(float));
 }
 
-cudaError_t nearfar_prepare(GemmState* state, const CacheView& view, const std::vector<NearFarItem>& items, int sm_count)
+cudaError_t nearfar_prepare(GemmState* state, const CacheView& view, const std::vector<NearFarItem>& items)
 {
-    return prepare(state, schedule(view, items, sm_count));
+    return prepare(state, schedule(view, items));
 }
 
 cudaError_t launch_nearfar(GemmState* state, const CacheView& view, const std::vector<NearFarItem>& items, int32_t sink,
                            int32_t* status_dev, int sm_count, const LaunchHooks& hooks, cudaStream_t stream)
 {
     state->kernels_last_call = 0;
-    const Schedule s = schedule(view, items, sm_count);
+    const Schedule s = schedule(view, items);
     cudaError_t e = prepare(state, s);
     if (e != cudaSuccess) return e;
     const bool ragged = items.size() > 1;

@@ -34,7 +34,7 @@ struct NearFarItem {
 };
 // Everything a launch needs that is not a stream operation; launch_nearfar calls it itself, a caller that must not
 // allocate later (stream capture) calls it first.
-cudaError_t nearfar_prepare(GemmState* state, const CacheView& view, const std::vector<NearFarItem>& items, int sm_count);
+cudaError_t nearfar_prepare(GemmState* state, const CacheView& view, const std::vector<NearFarItem>& items);
 // The work area of any uniform call of these lengths with up to some 15000 groups of 16 tiles (about 15 MB for each block of 128 far
 // rows), so that the calls after a plan allocate nothing.
 cudaError_t nearfar_reserve(GemmState* state, int32_t n_in, int32_t n_keep);
