@@ -508,16 +508,18 @@ struct TransformTimer {
     ~TransformTimer() { end(); }
 };
 
-// Compress `count` sequences starting at batch0, all with the same (n_in, n_keep).
+// Compress `count` sequences starting at batch0, all with the same (n_in, n_keep).  `of_triples`: the triples of the whole call where
+// this is a part of it that has to come out as the whole would (0: this is all of it).
 freqkv_status compress_group(freqkv_ctx* ctx, const freqkv_layout& l, void* k, void* v, int32_t batch0,
                              int32_t batch_count, int32_t n_in, int32_t n_keep, int32_t sink, int32_t variant,
                              cudaStream_t stream, int32_t first = 0, GemmState* own_gemm = nullptr,
-                             const Basis* own_basis = nullptr)
+                             const Basis* own_basis = nullptr, int64_t of_triples = 0)
 {
     const CacheView view = make_view(l, k, v, batch0, batch_count);
     const int32_t n_mat = 2 * view.mats_per_tensor;
 
-    if (variant == FREQKV_FDCT && first == 0 && one_pass_heads(ctx, l, n_in, n_keep, view.mats_per_tensor) && !is_capturing(stream)) {
+    if (variant == FREQKV_FDCT && first == 0 && one_pass_heads(ctx, l, n_in, n_keep, of_triples ? of_triples : view.mats_per_tensor) &&
+        !is_capturing(stream)) {
         const freqkv_status st = compress_group(ctx, l, k, v, batch0, batch_count, n_in, n_keep, sink, FREQKV_GEMM, stream);
         if (st != FREQKV_ERR_ALLOC) return st;  // no memory for its plan or work area, nothing enqueued: the transform needs neither
     }
@@ -1096,7 +1098,8 @@ freqkv_status freqkv_compress_host(freqkv_ctx* ctx, const freqkv_layout* layout,
                 const size_t off = ((size_t)b * l.stride_batch + (size_t)y0 * l.stride_layer) * elt;
                 const freqkv_status gs = compress_group(ctx, sub, static_cast<char*>(ctx->stage[0]) + off,
                                                         static_cast<char*>(ctx->stage[1]) + off, 0, 1, n_in, kept_len, sink,
-                                                        variant, ctx->pipe[1]);
+                                                        variant, ctx->pipe[1], 0, nullptr, nullptr,
+                                                        (int64_t)l.batch * l.layers * l.kv_heads);
                 if (gs != FREQKV_OK) return gs;
                 FREQKV_CUDA(ctx, cudaEventRecord(compressed, ctx->pipe[1]));
                 FREQKV_CUDA(ctx, cudaStreamWaitEvent(ctx->pipe[2], compressed, 0));

@@ -324,3 +324,18 @@ def test_infinities_and_nan_stay_in_their_channel(ctx, hd, H, n_in, kept):
         for head, channel in touched:
             got[0, 0, head, :, channel] = want[0, 0, head, :, channel] = 0
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("hd,B,Ly,H", [(64, 2, 9, 3), (64, 1, 8, 1), (256, 1, 8, 1)])
+def test_host_buffers_come_out_as_on_the_device(ctx, hd, B, Ly, H):
+    """The host-buffer form works through a call a few layers at a time: heads of 64 and 256 channels take the kernel that the whole
+    call would take, and come out bit for bit as on the device."""
+    w = synth.Workload("t", B, Ly, H, hd, 1028, torch.bfloat16, 4, 0.9, 2, synth.BASE_SEED + 18)
+    k, v = synth.make_cache(w, "cuda")
+    host_k, host_v = k.cpu().pin_memory(), v.cpu().pin_memory()
+    ctx.set_variant(fk.AUTO)
+    ctx.compress_host(host_k, host_v, 1028, 512, 4)
+    torch.cuda.synchronize()
+    ctx.compress(k, v, 1028, 512, 4)
+    torch.cuda.synchronize()
+    assert torch.equal(host_k, k.cpu()) and torch.equal(host_v, v.cpu())
