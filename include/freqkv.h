@@ -117,7 +117,7 @@ freqkv_status freqkv_resolve_variant(freqkv_ctx* ctx, const freqkv_layout* layou
  * n_in non-sink rows to n_keep rows (the projection basis of Eq. 2-3 folded with the
  * definitions of Appendix A, or the transform twiddles).  For fp32, AUTO builds what AUTO's calls
  * read and SIMT what they and the calls that ask for SIMT by name read.  Work is enqueued on
- * `cuda_stream`.
+ * `cuda_stream`; where the work area of an earlier, smaller plan or call grows, the device is synchronised.
  * Calling freqkv_compress without it builds the plan on first use. */
 freqkv_status freqkv_plan(freqkv_ctx* ctx, int32_t n_in, int32_t n_keep, freqkv_dtype dtype,
                           freqkv_variant variant, void* cuda_stream);
